@@ -35,7 +35,7 @@ ROTATE_BYTES = 4 * L2_BYTES          # bytes touched before an input copy is rea
 # The dominant kernel is the row statistics kernel: it is the only one that reads the logits from HBM
 # (every logit once), and both verifiers start with it.
 STAT_KERNEL = {False: "stream::spec_row_partial_kernel (row statistics: the one pass over the logits in HBM)",
-               True: "trunc::spec_row_trunc_kernel (+ rowstat::spec_row_stat_kernel for the rows it leaves over)"}
+               True: "trunc::spec_row_trunc_kernel (row statistics and cuts: the one pass over the logits in HBM)"}
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of that kernel from the ncu captures summarised
 # under profiles/ (cold L2).  Workloads without a capture: null.
 TRAFFIC_BYTES = {"cfg2_llama3_b8": 69_799_168 + 626_432}

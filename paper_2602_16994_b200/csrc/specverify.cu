@@ -1,6 +1,6 @@
 // libspecverify: batched draft-tree verification for sm_100a -- host side of the C ABI.
 //
-// Kernels: stream.cuh (row statistics, the one pass over HBM), rowstat.cuh (the same for top-k / top-p
+// Kernels: stream.cuh (row statistics, the one pass over HBM), trunc.cuh (the same for top-k / top-p
 // rows), walk.cuh (SpecInfer along the accepted path), tree.cuh (every node: Traversal Verification,
 // diagnostic outputs), rowops.cuh (materialised row distributions, stand-alone inverse CDF), and the
 // residual kernel below.  This file validates
@@ -16,7 +16,6 @@
 #include "common.cuh"
 #include "cut.cuh"
 #include "rowops.cuh"
-#include "rowstat.cuh"
 #include "tree.cuh"
 #include "trunc.cuh"
 #include "specverify.h"
@@ -171,7 +170,7 @@ inline int64_t up256(int64_t x) { return (x + 255) / 256 * 256; }
 
 // workspace layout: node records | published weights + arrival counters (cleared per call) | row cuts
 struct WsLayout {
-    int64_t rec, pub, fin, best, done, ticket, order, cut, todo, stat, gseq, total;
+    int64_t rec, pub, fin, best, done, ticket, order, cut, stat, gseq, total;
 };
 constexpr int MAX_PARTS = 4;      // parts a row may be split into by the streaming statistics kernel
 WsLayout ws_layout(const SpecIn *in, int slices = MAX_PARTS)   // slices = 0: one record per row only
@@ -191,7 +190,6 @@ WsLayout ws_layout(const SpecIn *in, int slices = MAX_PARTS)   // slices = 0: on
     L.order = o; o += nodes * 8;
     o = up256(o);
     L.cut = o; o += up256(nodes * 8);
-    L.todo = o; o += up256(4 + nodes * 8);          // count, then ids of the rows left to the general top-k / top-p kernel
     L.stat = o; o += up256(nodes * 2 * (slices + 1) * (int64_t)sizeof(RowPart));      // one record per row, then the parts
     L.gseq = o; o += up256(nodes * KMAX * 8);       // step coefficients of every node
     L.total = o;
@@ -319,58 +317,33 @@ int launch_tree(const VPlan &pl, TParams &tp, cudaStream_t st)
     return launch_clustered(kernel, nc * pl.C, pl.C, threads, pl.smem, st, &tp);
 }
 
-// row statistics (cut, reference, normaliser) of every row the verifiers read, or of every row of `z`
-// when no tree is given
-int launch_rowstat(const SpecIn *in, const void *zp, const void *zq, const int *parent, unsigned char *ws,
-                   const WsLayout &L, cudaStream_t st)
+// row statistics (cut, reference, normaliser) of every row the verifiers read, or of every row of `zp` when no
+// tree is given, under top-k / top-p
+int launch_trunc(const SpecIn *in, const void *zp, const void *zq, const int *parent, unsigned char *ws,
+                 const WsLayout &L, const stream::NodeInit &init, cudaStream_t st)
 {
-    const int esz = in->logits_dtype == SPEC_BF16 ? 2 : 4;
-    const int budget = 113 * 1024 - (int)sizeof(rowstat::Shared) - 2048;
-    int C = 1;
-    while (C <= rowstat::CMAXR && (long long)up((in->V + C - 1) / C, 8) * esz > budget) C <<= 1;
-    if (C > rowstat::CMAXR) return SPEC_ERR_UNSUPPORTED;
-    rowstat::RParams rp = {};
-    rp.B = in->B; rp.N = in->N; rp.V = in->V; rp.C = C; rp.dtype = in->logits_dtype;
-    rp.top_k = in->top_k; rp.top_p = in->top_p; rp.slice_len = up((in->V + C - 1) / C, 8);
+    trunc::RParams rp = {};
+    rp.B = in->B; rp.N = in->N; rp.V = in->V; rp.top_k = in->top_k; rp.top_p = in->top_p;
     rp.zp = zp; rp.zq = zq; rp.seq_stride = in->seq_stride; rp.node_stride = in->node_stride;
     rp.topo_stride = in->topo_seq_stride; rp.parent = parent; rp.T = in->temperature; rp.T_seq = in->temperature_per_seq;
-    rp.part = (RowPart *)(ws + L.stat); rp.cut = (float *)(ws + L.cut);
-    rp.todo = (int *)(ws + L.todo); rp.only_todo = 0;
-    const int smem = up(rp.slice_len * esz, 128);
+    rp.part = (RowPart *)(ws + L.stat); rp.cut = (float *)(ws + L.cut); rp.init = init;
+    const bool bf = in->logits_dtype == SPEC_BF16;
     const long long items = 2ll * in->B * in->N;
-    int rc, nc;
-    // fast path first: one CTA per row, selection on a candidate list; the rows it cannot settle are
-    // listed in the workspace and taken by the general kernel afterwards
-    if (cudaMemsetAsync(rp.todo, 0, 4, st) != cudaSuccess) { cudaGetLastError(); return SPEC_ERR_CUDA; }
-    {
-        const long long want = 2ll * sm_count();
-        const unsigned grid = (unsigned)(items < want ? items : want);
-        const bool total = in->top_p < 1.f && !(in->top_k > 0 && in->top_k < in->V);
-        if (in->logits_dtype == SPEC_BF16) {
-            if (total) trunc::spec_row_trunc_kernel<SPEC_BF16, true><<<grid, trunc::NT, 0, st>>>(rp);
-            else trunc::spec_row_trunc_kernel<SPEC_BF16, false><<<grid, trunc::NT, 0, st>>>(rp);
-        } else {
-            if (total) trunc::spec_row_trunc_kernel<SPEC_F32, true><<<grid, trunc::NT, 0, st>>>(rp);
-            else trunc::spec_row_trunc_kernel<SPEC_F32, false><<<grid, trunc::NT, 0, st>>>(rp);
-        }
-        if (cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
+    const long long want = (long long)sm_count() * (bf ? trunc::CTAS<SPEC_BF16> : trunc::CTAS<SPEC_F32>);
+    const unsigned grid = (unsigned)(items < want ? items : want);
+    const bool total = in->top_p < 1.f && !(in->top_k > 0 && in->top_k < in->V);
+    auto go = [&](auto kernel, int smem) {
+        const int rc = prepare_kernel(kernel, 1, smem);
+        if (rc) return rc;
+        kernel<<<grid, trunc::NT, smem, st>>>(rp);
         g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
-    }
-    rp.only_todo = 1;
-    if (in->logits_dtype == SPEC_BF16) {
-        auto k = rowstat::spec_row_stat_kernel<SPEC_BF16>;
-        if ((rc = prepare_kernel(k, C, smem))) return rc;
-        nc = resident_clusters(k, C, rowstat::NT, smem);
-        if (nc <= 0) return SPEC_ERR_UNSUPPORTED;
-        if (nc > items) nc = (int)items;
-        return launch_clustered(k, nc * C, C, rowstat::NT, smem, st, &rp);
-    }
-    auto k = rowstat::spec_row_stat_kernel<SPEC_F32>;
-    if ((rc = prepare_kernel(k, C, smem))) return rc;
-    nc = resident_clusters(k, C, rowstat::NT, smem);
-    if (nc <= 0) return SPEC_ERR_UNSUPPORTED;
-    if (nc > items) nc = (int)items;
-    return launch_clustered(k, nc * C, C, rowstat::NT, smem, st, &rp);
+        return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_ERR_CUDA;
+    };
+    if (bf)
+        return total ? go(trunc::spec_row_trunc_kernel<SPEC_BF16, true>, trunc::Layout<SPEC_BF16>::BYTES)
+                     : go(trunc::spec_row_trunc_kernel<SPEC_BF16, false>, trunc::Layout<SPEC_BF16>::BYTES);
+    return total ? go(trunc::spec_row_trunc_kernel<SPEC_F32, true>, trunc::Layout<SPEC_F32>::BYTES)
+                 : go(trunc::spec_row_trunc_kernel<SPEC_F32, false>, trunc::Layout<SPEC_F32>::BYTES);
 }
 
 // SpecInfer without diagnostic outputs: row statistics of every row, then one walk per sequence
@@ -396,14 +369,12 @@ int row_statistics(const SpecIn *in, const SpecOut *out, unsigned char *w, const
     int rc;
     int NSL = 1;
     RowPart *part = (RowPart *)(w + L.stat);
+    stream::NodeInit init = {};
+    if (init_nodes)
+        init = {(unsigned long long *)(w + L.pub), (unsigned int *)(w + L.done), (int *)(w + L.fin),
+                (unsigned int *)(w + L.best), (unsigned long long *)(w + L.order), (unsigned int *)(w + L.ticket)};
     if (trunc) {
-        if (init_nodes &&
-            (cudaMemsetAsync(w + L.pub, 0xFF, (size_t)(L.done - L.pub), st) != cudaSuccess ||
-             cudaMemsetAsync(w + L.done, 0, (size_t)(L.order - L.done) + (size_t)in->B * in->N * 8, st) != cudaSuccess)) {
-            cudaGetLastError();
-            return SPEC_ERR_CUDA;
-        }
-        rc = launch_rowstat(in, in->target_logits, in->draft_logits, in->parent, w, L, st);
+        rc = launch_trunc(in, in->target_logits, in->draft_logits, in->parent, w, L, init, st);
         if (rc) return rc;
     } else {
         // rows are split into parts only when there are fewer rows than resident CTAs
@@ -420,11 +391,7 @@ int row_statistics(const SpecIn *in, const SpecOut *out, unsigned char *w, const
         // in one part is final as written.  One CTA per item: those of unread rows retire at once.
         RowPart *parts = part + 2ll * in->B * in->N;
         sp.part = NSL > 1 ? parts : part;
-        if (init_nodes) {
-            sp.w_pub = (unsigned long long *)(w + L.pub); sp.done = (unsigned int *)(w + L.done);
-            sp.fin = (int *)(w + L.fin); sp.ticket = (unsigned int *)(w + L.ticket);
-            sp.best = (unsigned int *)(w + L.best); sp.order = (unsigned long long *)(w + L.order);
-        }
+        sp.init = init;
         const long long items = 2ll * in->B * in->N * NSL;
         const unsigned grid = (unsigned)(items < (1ll << 20) ? items : (1ll << 20));
         int prc;
@@ -821,7 +788,7 @@ int32_t spec_tree_probs(const SpecIn *in, int32_t which, float *probs, float *ro
         // the cuts of every row of the chosen side go to slot 0 of every pair in the workspace
         const WsLayout L = ws_layout(in);
         if (!ws || ((uintptr_t)ws & 255) || ws_bytes < L.total) return SPEC_ERR_WORKSPACE;
-        rc = launch_rowstat(in, z, z, nullptr, (unsigned char *)ws, L, (cudaStream_t)stream);
+        rc = launch_trunc(in, z, z, nullptr, (unsigned char *)ws, L, stream::NodeInit{}, (cudaStream_t)stream);
         if (rc) return rc;
         cutp = (const float *)((unsigned char *)ws + L.cut);
     }

@@ -22,13 +22,32 @@ struct __align__(16) RowPart {
     int bad;           // 1: NaN or +inf seen; -1: row not read (draft row of a node without children)
 };
 constexpr int ROWPART_EMPTY = -(1 << 30);
-constexpr int ROW_TIMEOUT = 3;          // RowPart::bad of a row whose copy into shared memory was given up on
 
 namespace stream {
 
 constexpr int NT = 256;
 constexpr int PER = 32;                  // logits per thread
-constexpr int SLICE = NT * PER;          // logits per CTA
+constexpr int SLICE = NT * PER;          // logits per CTA and slice
+
+// Per-call words of the workspace that an every-node verification wants set (w_pub NULL: none): the published
+// weights and the accepted nodes to pending, no acceptance known, counters and post-order table to zero.  The
+// statistics kernels set them, which saves the memset nodes of a call.
+struct NodeInit {
+    unsigned long long *w_pub;   // [B*N]
+    unsigned int *done;          // [B]
+    int *fin;                    // [B]
+    unsigned int *best;          // [B]
+    unsigned long long *order;   // [B*N]
+    unsigned int *ticket;        // [1]
+    __device__ __forceinline__ void set(long long node, int b, int a) const
+    {
+        if (!w_pub) return;
+        w_pub[node] = W_PENDING;
+        order[node] = 0ull;
+        if (a == 0) { done[b] = 0u; fin[b] = -1; best[b] = 0xFFFFFFFFu; }
+        if (node == 0) *ticket = 0u;
+    }
+};
 
 struct SParams {
     int B, N, V, NSL;        // NSL: parts a row is split into (more CTAs than rows)
@@ -38,20 +57,110 @@ struct SParams {
     float T;
     const float *T_seq;
     RowPart *part;           // [B*N*2][NSL]
-    // optional (every-node verification follows): the per-node weight slots and the per-sequence accepted-node
-    // slots are set to pending, the arrival counters and the item counter to zero here, which saves the memset
-    // nodes of a call
-    unsigned long long *w_pub;   // [B*N]
-    unsigned int *done;          // [B]
-    int *fin;                    // [B] set to -1 (no accepted node selected yet)
-    unsigned int *best;          // [B] set to all-ones (no acceptance known yet)
-    unsigned long long *order;   // [B*N] set to 0 (post-order table not computed yet)
-    unsigned int *ticket;        // [1] item counter of the every-node kernel
+    NodeInit init;
 };
+
+// A row as whole 16-byte units of memory: wherever the row starts, its logits are in the units from the one that
+// holds its first byte to the one that holds its last, and the statistics do not care about positions inside
+// the row -- so every row takes the 16-byte path, and only its first and last units are masked.
+struct RowSpan {
+    const unsigned char *base;   // 16-byte aligned
+    int units;
+    short head, last;            // first logit of the first unit; logits of the last unit, counted from its start
+};
+template <int DT>
+__device__ __forceinline__ RowSpan row_span(const void *z, long long first, int V)
+{
+    constexpr int ESZ = DT == SPEC_BF16 ? 2 : 4, E = 16 / ESZ;
+    const uintptr_t at = (uintptr_t)z + (uintptr_t)(first * ESZ);
+    RowSpan r;
+    r.base = (const unsigned char *)(at & ~(uintptr_t)15);
+    r.head = (short)((at & 15) / ESZ);
+    r.units = (r.head + V + E - 1) / E;
+    r.last = (short)(r.head + V - (r.units - 1) * E);
+    return r;
+}
+// the logits of unit u that are not the row's become -inf (all of them beyond the last unit)
+template <int DT>
+__device__ __forceinline__ void mask_unit(uint4 &r, int u, const RowSpan &row)
+{
+    constexpr int E = DT == SPEC_BF16 ? 8 : 4;
+    const int e0 = u == 0 ? row.head : 0, e1 = u < row.units - 1 ? E : (u == row.units - 1 ? row.last : 0);
+    if (e0 == 0 && e1 == E) return;
+    uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+        const bool out = k < e0 || k >= e1;
+        if (DT == SPEC_BF16) {
+            if (out) w[k >> 1] = (k & 1) ? (w[k >> 1] & 0xFFFFu) | 0xFF800000u : (w[k >> 1] & 0xFFFF0000u) | 0xFF80u;
+        } else {
+            if (out) w[k] = 0xFF800000u;
+        }
+    }
+    r = make_uint4(w[0], w[1], w[2], w[3]);
+}
+// the logits of a unit (8 bf16 or 4 fp32)
+template <int DT>
+__device__ __forceinline__ void unpack_unit(const uint4 &r, float (&z)[DT == SPEC_BF16 ? 8 : 4])
+{
+    if (DT == SPEC_BF16) {
+        z[0] = bf16_lo(r.x); z[1] = bf16_hi(r.x); z[2] = bf16_lo(r.y); z[3] = bf16_hi(r.y);
+        z[4 % (DT == SPEC_BF16 ? 8 : 4)] = bf16_lo(r.z); z[5 % (DT == SPEC_BF16 ? 8 : 4)] = bf16_hi(r.z);
+        z[6 % (DT == SPEC_BF16 ? 8 : 4)] = bf16_lo(r.w); z[7 % (DT == SPEC_BF16 ? 8 : 4)] = bf16_hi(r.w);
+    } else {
+        z[0] = __uint_as_float(r.x); z[1] = __uint_as_float(r.y); z[2] = __uint_as_float(r.z); z[3] = __uint_as_float(r.w);
+    }
+}
+// maxima that a NaN operand makes NaN
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float d;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ uint32_t max_nan_bf16x2(uint32_t a, uint32_t b)
+{
+    uint32_t d;
+    asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+// maximum of a unit, as the bits of an fp32 value or of a pair of bf16 values (fold_max: the larger of the pair)
+template <int DT>
+__device__ __forceinline__ uint32_t max_raw(uint32_t a, uint32_t b)
+{
+    return DT == SPEC_BF16 ? max_nan_bf16x2(a, b) : __float_as_uint(max_nan(__uint_as_float(a), __uint_as_float(b)));
+}
+template <int DT>
+__device__ __forceinline__ uint32_t unit_max_raw(const uint4 &r)
+{
+    return max_raw<DT>(max_raw<DT>(r.x, r.y), max_raw<DT>(r.z, r.w));
+}
+template <int DT>
+__device__ __forceinline__ float fold_max(uint32_t m)
+{
+    return DT == SPEC_BF16 ? max_nan(bf16_lo(m), bf16_hi(m)) : __uint_as_float(m);
+}
+// s = s_hi + s_lo in two floats, s_lo > 0 (so that a -inf logit gives an exponent of -inf, never NaN)
+__device__ __forceinline__ void split_scale(double s_d, float &s_hi, float &s_lo)
+{
+    s_hi = (float)s_d;
+    if ((double)s_hi > s_d) s_hi = __uint_as_float(__float_as_uint(s_hi) - 1u);
+    s_lo = (float)(s_d - (double)s_hi);
+    if (!(s_lo > 0.f)) s_lo = 1.0e-30f;
+}
+// whether node a of a tree has children (warp-collective)
+__device__ __forceinline__ bool has_children(const int *parent, int N, int a, int lane)
+{
+    for (int c0 = a + 1; c0 < N; c0 += 32) {
+        const int c = c0 + lane;
+        if (__any_sync(0xffffffffu, c < N && __ldg(parent + c) == a)) return true;
+    }
+    return false;
+}
 
 // depth of the per-thread staging ring and its size
 template <int DT> struct Ring {
-    static constexpr int NV = DT == SPEC_BF16 ? 1 : 2;         // 16-byte units per chunk of 8 logits
+    static constexpr int NV = DT == SPEC_BF16 ? 1 : 2;         // 16-byte units per 8 logits
     static constexpr int UNITS = (PER / 8) * NV;               // 16-byte units per thread and slice
     static constexpr int DEPTH = DT == SPEC_BF16 ? 5 : 3;
     static constexpr int BYTES = DEPTH * UNITS * NT * 16;
@@ -82,7 +191,6 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b)
 template <int DT, bool FEAT>
 __global__ void __launch_bounds__(NT, 2) spec_row_partial_kernel(const SParams P)
 {
-    constexpr int ESZ = DT == SPEC_BF16 ? 2 : 4;
     constexpr int NV = Ring<DT>::NV, UNITS = Ring<DT>::UNITS, DEPTH = Ring<DT>::DEPTH;
     __shared__ double sS[NT / 32], sX[NT / 32], sB[NT / 32];
     __shared__ int sO[NT / 32], sBad[NT / 32];
@@ -90,8 +198,6 @@ __global__ void __launch_bounds__(NT, 2) spec_row_partial_kernel(const SParams P
     const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const long long items = 2ll * P.B * P.N * P.NSL;
-    const int slices_row = (P.V + SLICE - 1) / SLICE;
-    const int slices_part = (slices_row + P.NSL - 1) / P.NSL;
     grid_launch_dependents();     // a dependent verifier's CTAs may take the places of CTAs that have finished
 
     for (long long id = blockIdx.x; id < items; id += gridDim.x) {
@@ -101,34 +207,19 @@ __global__ void __launch_bounds__(NT, 2) spec_row_partial_kernel(const SParams P
         const long long row = row2 >> 1;
         const int b = (int)(row / P.N), a = (int)(row % P.N);
         RowPart *out = P.part + row2 * P.NSL + h;
-        if (P.w_pub && which == 0 && h == 0 && tid == 0) {
-            P.w_pub[row] = W_PENDING;
-            P.order[row] = 0ull;
-            if (a == 0) { P.done[b] = 0u; P.fin[b] = -1; P.best[b] = 0xFFFFFFFFu; }
-            if (row == 0) *P.ticket = 0u;
+        if (which == 0 && h == 0 && tid == 0) P.init.set(row, b, a);
+        // a draft row is read only for nodes that have children (every warp finds out by itself)
+        if (which == 1 && !has_children(P.parent + (long long)b * P.topo_stride, P.N, a, lane)) {
+            if (tid == 0) { RowPart r = {}; r.O = ROWPART_EMPTY; r.cut = -CUDART_INF_F; r.bad = -1; *out = r; }
+            continue;
         }
-        if (which == 1) {
-            // a draft row is read only for nodes that have children (every warp finds out by itself)
-            const int *parent = P.parent + (long long)b * P.topo_stride;
-            bool any = false;
-            for (int c0 = a + 1; c0 < P.N && !any; c0 += 32) {
-                const int c = c0 + lane;
-                any = __any_sync(0xffffffffu, c < P.N && __ldg(parent + c) == a);
-            }
-            if (!any) {
-                if (tid == 0) { RowPart r = {}; r.O = ROWPART_EMPTY; r.cut = -CUDART_INF_F; r.bad = -1; *out = r; }
-                continue;
-            }
-        }
-        const unsigned char *rowp = (const unsigned char *)(which ? P.zq : P.zp) +
-                                    ((long long)b * P.seq_stride + (long long)a * P.node_stride) * ESZ;
-        const bool aligned = (((uintptr_t)rowp) & 15) == 0;
+        const RowSpan span = row_span<DT>(which ? P.zq : P.zp, (long long)b * P.seq_stride + (long long)a * P.node_stride, P.V);
+        const int slices_row = (span.units + NT * UNITS - 1) / (NT * UNITS);
+        const int slices_part = (slices_row + P.NSL - 1) / P.NSL;
         const int s_begin = h * slices_part, s_end = min(slices_row, s_begin + slices_part);
         const double s_d = 1.4426950408889634 / (double)(P.T_seq ? __ldg(P.T_seq + b) : P.T);
-        float s_hi = (float)s_d;
-        if ((double)s_hi > s_d) s_hi = __uint_as_float(__float_as_uint(s_hi) - 1u);
-        float s_lo = (float)(s_d - (double)s_hi);
-        if (!(s_lo > 0.f)) s_lo = 1.0e-30f;
+        float s_hi, s_lo;
+        split_scale(s_d, s_hi, s_lo);
 
         // the thread's running state
         float of = 0.f, S_t = 0.f, X_t = 0.f, xm_t = -CUDART_INF_F;
@@ -187,21 +278,19 @@ __global__ void __launch_bounds__(NT, 2) spec_row_partial_kernel(const SParams P
             a0 = a1 = a2 = a3 = b0 = b1 = 0.f;
         };
 
-        // ---- whole slices of an aligned row go through the ring ------------------------------------------------
-        const int tok_end = min(P.V, s_end * SLICE);                       // first token past this part
-        const int nfull = aligned ? max(0, (tok_end - s_begin * SLICE) / SLICE) : 0;
+        // ---- the part's slices through the ring; the units at the ends of the row are masked ----------------------
         {
-            const unsigned char *src = rowp + (size_t)s_begin * SLICE * ESZ + (size_t)tid * 16 * NV;
+            const unsigned char *src = span.base + ((size_t)s_begin * NT * UNITS + tid) * 16;
             const uint32_t dst0 = ring_s + (uint32_t)tid * 16u;
-            int isl = 0, ist = 0, cst = 0;
+            int isl = s_begin, ist = 0, cst = 0;
             auto issue = [&]() {
-                if (isl < nfull) {
+                if (isl < s_end) {
+                    const int u0 = isl * NT * UNITS + tid;
 #pragma unroll
-                    for (int c = 0; c < PER / 8; ++c)
-#pragma unroll
-                        for (int k = 0; k < NV; ++k)
-                            cp_async16(dst0 + (uint32_t)((ist * UNITS + c * NV + k) * NT) * 16u, src + (size_t)c * NT * 16 * NV + k * 16, 16);
-                    src += (size_t)SLICE * ESZ;
+                    for (int u = 0; u < UNITS; ++u)
+                        if (u0 + u * NT < span.units)
+                            cp_async16(dst0 + (uint32_t)((ist * UNITS + u) * NT) * 16u, src + (size_t)u * NT * 16, 16);
+                    src += (size_t)NT * UNITS * 16;
                     ++isl;
                     ist = ist + 1 == DEPTH ? 0 : ist + 1;
                 }
@@ -209,44 +298,7 @@ __global__ void __launch_bounds__(NT, 2) spec_row_partial_kernel(const SParams P
             };
 #pragma unroll
             for (int k = 0; k < DEPTH - 1; ++k) issue();
-            // ---- the ragged end of the part (and every slice of a misaligned row) by plain loads, while the ring fills
-            for (int t_base = (s_begin + nfull) * SLICE; t_base < tok_end; t_base += SLICE) {
-                const int n = min(SLICE, tok_end - t_base);
-                const unsigned char *src = rowp + (size_t)t_base * ESZ;
-                float z[PER];
-#pragma unroll
-                for (int c = 0; c < PER / 8; ++c) {
-                    const int t0 = (tid + c * NT) * 8;
-                    if (aligned && t0 + 8 <= n) {
-                        const uint4 *s4 = reinterpret_cast<const uint4 *>(src) + (size_t)(tid + c * NT) * NV;
-                        if (DT == SPEC_BF16) {
-                            const uint4 r = __ldg(s4);
-                            z[c * 8 + 0] = bf16_lo(r.x); z[c * 8 + 1] = bf16_hi(r.x); z[c * 8 + 2] = bf16_lo(r.y); z[c * 8 + 3] = bf16_hi(r.y);
-                            z[c * 8 + 4] = bf16_lo(r.z); z[c * 8 + 5] = bf16_hi(r.z); z[c * 8 + 6] = bf16_lo(r.w); z[c * 8 + 7] = bf16_hi(r.w);
-                        } else {
-                            const uint4 r0 = __ldg(s4), r1 = __ldg(s4 + NV - 1);
-                            z[c * 8 + 0] = __uint_as_float(r0.x); z[c * 8 + 1] = __uint_as_float(r0.y); z[c * 8 + 2] = __uint_as_float(r0.z); z[c * 8 + 3] = __uint_as_float(r0.w);
-                            z[c * 8 + 4] = __uint_as_float(r1.x); z[c * 8 + 5] = __uint_as_float(r1.y); z[c * 8 + 6] = __uint_as_float(r1.z); z[c * 8 + 7] = __uint_as_float(r1.w);
-                        }
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) z[c * 8 + k] = (t0 + k < n) ? load_logit(src, DT, t0 + k) : -CUDART_INF_F;
-                    }
-                }
-                float zm = -CUDART_INF_F;
-#pragma unroll
-                for (int k = 0; k < PER; ++k) zm = fmaxf(zm, z[k]);
-                new_reference(zm);
-#pragma unroll
-                for (int c = 0; c < PER / 8; ++c) {
-                    float z8[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) z8[k] = z[c * 8 + k];
-                    add8(z8);
-                }
-                flush();
-            }
-            for (int sl = 0; sl < nfull; ++sl) {
+            for (int sl = s_begin; sl < s_end; ++sl) {
                 cp_async_wait<DEPTH - 2>();
                 const uint4 *st = ring + (size_t)cst * UNITS * NT + tid;
                 uint4 raw[UNITS];
@@ -254,6 +306,10 @@ __global__ void __launch_bounds__(NT, 2) spec_row_partial_kernel(const SParams P
                 for (int u = 0; u < UNITS; ++u) raw[u] = st[u * NT];
                 cst = cst + 1 == DEPTH ? 0 : cst + 1;
                 issue();                                  // the stage read in the previous iteration is free again
+                if (sl == 0 || sl == slices_row - 1) {
+#pragma unroll
+                    for (int u = 0; u < UNITS; ++u) mask_unit<DT>(raw[u], (sl * UNITS + u) * NT + tid, span);
+                }
                 float zm;
                 if (DT == SPEC_BF16) {
                     uint32_t m2 = 0xFF80FF80u;            // the slice maximum on packed pairs

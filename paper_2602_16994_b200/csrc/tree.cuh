@@ -1,4 +1,4 @@
-// Whole-tree verification on top of the row statistics (stream.cuh / rowstat.cuh): every node of
+// Whole-tree verification on top of the row statistics (stream.cuh / trunc.cuh): every node of
 // every sequence is one work item of a thread-block cluster, as Traversal Verification needs (its
 // weights are defined for every node, top-down: Section 3.2) and as SpecInfer's diagnostic outputs
 // need (the threshold of every node, Algorithm 4).
@@ -152,7 +152,7 @@ __device__ __noinline__ void leaf_record(const VParams &P, const RowPart *part, 
     Rl.kappa = Zl; Rl.nsteps = 0;
     Rl.cut_p = __ldcg(&rpl->cut); Rl.cut_q = -CUDART_INF_F;
     Rl.next_child = -1;
-    Rl.status = badl ? (__ldcg(&rpl->bad) == ROW_TIMEOUT ? SPEC_DEV_TIMEOUT : SPEC_DEV_NONFINITE) : 0;
+    Rl.status = badl ? SPEC_DEV_NONFINITE : 0;
     Rl.bonus = -1; Rl.bonus_margin = 0.f;
     Rl.w_in = trav ? thr_c : 1.0;
     Rl.thr = thr_c;
@@ -442,13 +442,12 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW <= 7 ? 2 : 1) spec_tree_kern
                 int O_q = ROWPART_EMPTY;
                 float cut_q = -CUDART_INF_F;
                 bool bad = __ldcg(&rp[0].bad) != 0 || !(O_p > ROWPART_EMPTY) || !(Z_p > 0.0) || !(Z_p < CUDART_INF);
-                bool slow = __ldcg(&rp[0].bad) == ROW_TIMEOUT || (hq && __ldcg(&rp[1].bad) == ROW_TIMEOUT);
                 if (hq) {
                     Z_q = __ldcg(&rp[1].S); O_q = __ldcg(&rp[1].O); cut_q = __ldcg(&rp[1].cut);
                     bad = bad || __ldcg(&rp[1].bad) != 0 || !(O_q > ROWPART_EMPTY) || !(Z_q > 0.0) || !(Z_q < CUDART_INF);
                 }
                 err = __reduce_max_sync(0xffffffffu, err);
-                if (bad && !err) err = slow ? SPEC_DEV_TIMEOUT : SPEC_DEV_NONFINITE;
+                if (bad && !err) err = SPEC_DEV_NONFINITE;
                 kind = (hint_dead || err) ? ITEM_DEAD : (hq ? ITEM_NODE : ITEM_LEAF);
                 __syncwarp();
                 if (kind == ITEM_NODE) {

@@ -1,5 +1,5 @@
 // SpecInfer verification as a walk (Algorithm 4 composed top-down, Section 3.2), one thread-block
-// cluster per sequence, on top of the row statistics (stream.cuh / rowstat.cuh).
+// cluster per sequence, on top of the row statistics (stream.cuh / trunc.cuh).
 //
 // With every row's normaliser known, the decision about a node's FIRST child needs no vocabulary-wide
 // work: its threshold is min(1, p(x)/q(x)), two logits and two normalisers.  The cluster therefore walks
@@ -213,9 +213,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) spec_walk_kernel(const WP
                     const double Zr = __ldcg(&p->S);
                     const int Or = __ldcg(&p->O), bd = __ldcg(&p->bad);
                     // a row is not finite if it holds NaN / +inf, or no finite logit at all
-                    if (bd == ROW_TIMEOUT)
-                        st1 = max(st1, SPEC_DEV_TIMEOUT);
-                    else if (bd != -1 && (bd == 1 || !(Or > ROWPART_EMPTY) || !(Zr > 0.0) || !(Zr < CUDART_INF)))
+                    if (bd != -1 && (bd == 1 || !(Or > ROWPART_EMPTY) || !(Zr > 0.0) || !(Zr < CUDART_INF)))
                         st1 = max(st1, SPEC_DEV_NONFINITE);
                     S.t_Z[r2] = Zr; S.t_O[r2] = Or; S.t_cut[r2] = __ldcg(&p->cut);
                 }

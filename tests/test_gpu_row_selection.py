@@ -1,0 +1,70 @@
+"""top-k / top-p selection at the edges of its one-pass kernel: slices of 8192 bf16 or 4096 fp32 logits, rows that start
+on no 16-byte boundary, candidate lists and bins at their limits, first slices that say nothing about the rest."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2602_16994_b200 import binding
+from .parity import PROB_TOL
+
+pytestmark = pytest.mark.gpu
+BF, F32 = torch.bfloat16, torch.float32
+
+
+def check(z, trunc, T=1.0):
+    probs, stats = binding.tree_probs(z, 0, temperature=T, **trunc)
+    B, N, V = z.shape
+    zb = z.contiguous().cpu()
+    bits = zb.view(torch.int16).numpy().view(np.uint16) if z.dtype == BF else zb.numpy()
+    inp = oracle.TreeInputs(bits, bits, np.array([-1] + [0] * (N - 1), np.int32), np.zeros((B, N), np.int32),
+                            np.zeros((B, N), np.float32), np.zeros((B, N), np.float32), temperature=T,
+                            top_k=trunc.get("top_k", 0), top_p=trunc.get("top_p", 1.0))
+    rp, rs, _ = oracle.tree_probs(inp, 0)
+    sure = rs[..., 5] >= 1e-6                      # rows whose nucleus boundary is not within 1e-6 of top_p
+    assert sure.any()
+    st = stats.cpu().numpy()
+    assert np.abs(probs.cpu().numpy() - rp)[sure].max() < PROB_TOL
+    np.testing.assert_array_equal(st[..., 2][sure], rs[..., 2][sure])                          # kept count
+    np.testing.assert_array_equal(st[..., 5][sure], rs[..., 6][sure].astype(np.float32))       # threshold logit
+
+
+def rows(V, dtype, scale=3.0):
+    g = torch.Generator(device="cuda").manual_seed(11)
+    z = (torch.randn((2, 3, V), generator=g, device="cuda") * scale).to(dtype)
+    z[0, 0, : V // 2] = z[0, 0, V // 2: 2 * (V // 2)]          # exact ties everywhere in one row
+    z[1, 1, 5], z[1, 1, 6] = -0.0, 0.0
+    return z
+
+
+@pytest.mark.parametrize("V", [7, 4097, 8191, 8192, 8193, 24577])
+@pytest.mark.parametrize("dtype", [BF, F32], ids=["bf16", "f32"])
+@pytest.mark.parametrize("trunc", [dict(top_k=5), dict(top_p=0.9), dict(top_p=0.99)], ids=["k5", "p90", "p99"])
+def test_slice_edges(V, dtype, trunc):
+    check(rows(V, dtype), trunc)
+
+
+@pytest.mark.parametrize("V,dtype,scale,trunc", [
+    (40000, BF, 3.0, dict(top_k=1024)), (40000, BF, 3.0, dict(top_k=1025)),      # the last k a first slice bounds, and one more
+    (40000, F32, 3.0, dict(top_k=256)), (40000, F32, 3.0, dict(top_k=257)),
+    (40000, F32, 3.0, dict(top_p=0.97)),                                        # more candidates than the list of keys holds
+    (40000, BF, 300.0, dict(top_k=40)), (40000, BF, 300.0, dict(top_p=0.9)),     # values beyond the bins
+    (40000, BF, 0.2, dict(top_p=0.95)),                                         # a nucleus that reaches below zero
+    (131072, BF, 1.0, dict(top_p=0.999)),                                       # almost all of the row, counted densely
+])
+def test_limits(V, dtype, scale, trunc):
+    check(rows(V, dtype, scale), trunc)
+
+
+@pytest.mark.parametrize("dtype", [BF, F32], ids=["bf16", "f32"])
+@pytest.mark.parametrize("trunc", [dict(top_k=60), dict(top_p=0.95), dict(top_k=200, top_p=0.9)], ids=["k60", "p95", "k200p90"])
+@pytest.mark.parametrize("order", ["descending", "ascending", "minus_inf_first"])
+def test_first_slice_unlike_the_rest(dtype, trunc, order):
+    V = 50003
+    g = torch.Generator(device="cuda").manual_seed(3)
+    z = (torch.randn((1, 2, V), generator=g, device="cuda") * 2.5).to(dtype)
+    if order == "minus_inf_first":
+        z[..., :9000] = -float("inf")
+    else:
+        z = torch.sort(z.float(), dim=-1, descending=order == "descending").values.to(dtype)
+    check(z, trunc, T=0.7)
