@@ -1,8 +1,9 @@
-"""Thin ctypes binding of libspecverify.so: argument marshalling only.
+"""Thin binding of libspecverify.so: argument marshalling only.
 
 Every step of the verification path runs inside the CUDA library; this module turns torch tensors
 into the plain pointers of the C ABI (``include/specverify.h``), owns the scratch workspace and
-allocates output tensors.  There is no CPU fallback: a missing library or a missing CUDA device
+allocates output tensors.  The calls of a decoding loop do that in native code (``csrc/torch_calls.cpp``);
+the host-buffer call, the plan queries and the caller-allocated entry point go through ctypes.  There is no CPU fallback: a missing library or a missing CUDA device
 raises ``RuntimeError``.
 
 Device-resident API (inputs already in HBM, nothing is synchronised):
@@ -108,6 +109,23 @@ def load_library(path: str = LIB_PATH):
     lib.spec_test_hooks.argtypes = [C.c_int64, C.c_int32]
     _lib = lib
     return lib
+
+
+_native = None
+
+
+def _calls():
+    """The native host path (``_torch_calls.so``), bound to the library."""
+    global _native
+    if _native is None:
+        load_library()
+        try:
+            from . import _torch_calls
+        except ImportError as e:
+            raise RuntimeError(f"the native host path is missing: build it with `python -m paper_2602_16994_b200.build` ({e})")
+        _torch_calls.init(LIB_PATH, VerifyOutputs, AnalysisOutputs)
+        _native = _torch_calls
+    return _native
 
 
 def _check(rc: int, what: str):
@@ -222,7 +240,7 @@ class Workspace:
         if self.buf is None or self.buf.numel() < nbytes + 256:
             self.buf = torch.empty(nbytes + 256, dtype=torch.uint8, device=self.device)
         base = self.buf.data_ptr()
-        off = (-base) % 256
+        off = -base % 256
         return C.c_void_p(base + off), self.buf.numel() - off
 
 
@@ -230,26 +248,10 @@ _default_ws = {}
 
 
 def _ws_for(device) -> Workspace:
-    key = str(device)
-    if key not in _default_ws:
-        _default_ws[key] = Workspace(device)
-    return _default_ws[key]
-
-
-def _verify(fn_name, batch_or_in, outputs, workspace, stream, **alloc):
-    lib = load_library()
-    if not torch.cuda.is_available():
-        raise RuntimeError("no CUDA device: the verification path has no CPU fallback")
-    spec_in, keep = batch_or_in
-    B, N, V = spec_in.B, spec_in.N, spec_in.V
-    device = keep[0].device
-    if outputs is None:
-        outputs = alloc_outputs(B, N, V, device, **alloc)
-    ws = workspace or _ws_for(device)
-    ptr, size = ws.get(workspace_bytes(spec_in))
-    so = outputs.as_struct()
-    _check(getattr(lib, fn_name)(C.byref(spec_in), C.byref(so), ptr, size, _stream_ptr(stream)), fn_name)
-    return outputs
+    ws = _default_ws.get(device)
+    if ws is None:
+        ws = _default_ws.setdefault(device, Workspace(device))
+    return ws
 
 
 def _marshal(target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature, top_k, top_p,
@@ -263,10 +265,9 @@ def verify_specinfer(target_logits, draft_logits, parent, token, u_accept, u_bon
                      top_k=0, top_p=1.0, temperature_per_seq=None, outputs=None, workspace=None,
                      stream=None, residual=False, node_thr=False, features=False, margin=False):
     """SpecInfer verification of a batch of draft trees (enqueued on the stream; returns device tensors)."""
-    m = _marshal(target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature, top_k, top_p,
-                 temperature_per_seq)
-    return _verify("spec_verify_specinfer", m, outputs, workspace, stream, residual=residual,
-                   node_thr=node_thr, features=features, margin=margin)
+    return _calls().verify(0, target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature, top_k, top_p,
+                           temperature_per_seq, outputs, workspace or _ws_for(target_logits.device), stream,
+                           bool(residual) + 2 * bool(node_thr) + 8 * bool(features) + 16 * bool(margin))
 
 
 OTLP_SOLVERS = {"nss": 0, "naive": 1, "spectr": 2}
@@ -275,20 +276,8 @@ OTLP_SOLVERS = {"nss": 0, "naive": 1, "spectr": 2}
 def verify_otlp(solver, target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature=1.0, top_k=0,
                 top_p=1.0, temperature_per_seq=None, outputs=None, workspace=None, stream=None):
     """Top-down verification with NSS, NaiveTree or SpecTr (``solver``: "nss", "naive", "spectr")."""
-    lib = load_library()
-    if not torch.cuda.is_available():
-        raise RuntimeError("no CUDA device: the verification path has no CPU fallback")
-    spec_in, keep = _marshal(target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature, top_k, top_p,
-                             temperature_per_seq)
-    device = target_logits.device
-    if outputs is None:
-        outputs = alloc_outputs(spec_in.B, spec_in.N, spec_in.V, device)
-    ws = workspace or _ws_for(device)
-    ptr, size = ws.get(workspace_bytes(spec_in))
-    so = outputs.as_struct()
-    _check(lib.spec_verify_otlp(C.byref(spec_in), C.byref(so), OTLP_SOLVERS[solver], ptr, size, _stream_ptr(stream)),
-           "spec_verify_otlp")
-    return outputs
+    return _calls().verify(2 + OTLP_SOLVERS[solver], target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature,
+                           top_k, top_p, temperature_per_seq, outputs, workspace or _ws_for(target_logits.device), stream, 0)
 
 
 def verify_specinfer_static(target_logits, draft_logits, parent, token, u_accept, u_bonus, outputs,
@@ -315,10 +304,9 @@ def verify_traversal(target_logits, draft_logits, parent, token, u_accept, u_bon
                      stream=None, residual=False, node_thr=False, node_w_in=False, features=False,
                      margin=False):
     """Traversal Verification of a batch of draft trees."""
-    m = _marshal(target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature, top_k, top_p,
-                 temperature_per_seq)
-    return _verify("spec_verify_traversal", m, outputs, workspace, stream, residual=residual,
-                   node_thr=node_thr, node_w_in=node_w_in, features=features, margin=margin)
+    return _calls().verify(1, target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature, top_k, top_p,
+                           temperature_per_seq, outputs, workspace or _ws_for(target_logits.device), stream,
+                           bool(residual) + 2 * bool(node_thr) + 4 * bool(node_w_in) + 8 * bool(features) + 16 * bool(margin))
 
 
 class PreparedVerify:
@@ -335,9 +323,7 @@ class PreparedVerify:
         self.lib = load_library()
         if not torch.cuda.is_available():
             raise RuntimeError("no CUDA device: the verification path has no CPU fallback")
-        self.fn = getattr(self.lib, {"specinfer": "spec_verify_specinfer",
-                                     "traversal": "spec_verify_traversal"}[algorithm])
-        self.name = algorithm
+        code = {"specinfer": 0, "traversal": 1}[algorithm]
         self.spec_in, self.keep = _marshal(target_logits, draft_logits, parent, token, u_accept, u_bonus,
                                            temperature, top_k, top_p, temperature_per_seq)
         B, N, V = self.spec_in.B, self.spec_in.N, self.spec_in.V
@@ -346,12 +332,12 @@ class PreparedVerify:
         self.spec_out = self.outputs.as_struct()
         self.workspace = workspace or _ws_for(dev)
         self.ws_ptr, self.ws_size = self.workspace.get(workspace_bytes(self.spec_in))
-        self._in_ref, self._out_ref = C.byref(self.spec_in), C.byref(self.spec_out)
+        self._in_ref = C.byref(self.spec_in)
+        self._call = (code, C.addressof(self.spec_in), C.addressof(self.spec_out), self.ws_ptr.value, self.ws_size)
+        self._launch = _calls().launch
 
     def launch(self, stream=None):
-        rc = self.fn(self._in_ref, self._out_ref, self.ws_ptr, self.ws_size, _stream_ptr(stream))
-        if rc != 0:
-            _check(rc, "spec_verify_" + self.name)
+        self._launch(*self._call, stream)
         return self.outputs
 
     def launch_statistics_only(self, stream=None):
@@ -372,21 +358,8 @@ class AnalysisOutputs:
 def tree_analysis(target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature=1.0, top_k=0,
                   top_p=1.0, temperature_per_seq=None, stream=None) -> AnalysisOutputs:
     """Acceptance rates, divergences, branching probabilities and block efficiency of a batch of trees."""
-    lib = load_library()
-    si, keep = _marshal(target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature, top_k, top_p,
-                        temperature_per_seq)
-    B, N = si.B, si.N
-    dev = target_logits.device
-    f32 = dict(dtype=torch.float32, device=dev)
-    out = AnalysisOutputs(torch.empty((B, N, 4), **f32), torch.empty((B, N, 3), **f32), torch.empty((5, B, N), **f32),
-                          torch.empty((5, B, N), **f32), torch.empty((5, B), **f32))
-    n = C.c_int64()
-    _check(lib.spec_analysis_workspace_bytes(C.byref(si), C.byref(n)), "spec_analysis_workspace_bytes")
-    ptr, size = _ws_for(dev).get(int(n.value))
-    so = SpecAnalysisOut(_ptr(out.acceptance), _ptr(out.divergence), _ptr(out.branch), _ptr(out.reach),
-                         _ptr(out.block_eff))
-    _check(lib.spec_tree_analysis(C.byref(si), C.byref(so), ptr, size, _stream_ptr(stream)), "spec_tree_analysis")
-    return out
+    return _calls().tree_analysis(target_logits, draft_logits, parent, token, u_accept, u_bonus, temperature, top_k, top_p,
+                                  temperature_per_seq, _ws_for(target_logits.device), stream)
 
 
 def latency_model(t_q, t_p, ctx, actions, stream=None):
@@ -408,37 +381,13 @@ def latency_model(t_q, t_p, ctx, actions, stream=None):
 def tree_probs(logits, which=0, temperature=1.0, top_k=0, top_p=1.0, temperature_per_seq=None,
                want_probs=True, want_stats=True, stream=None):
     """Sampling distribution of every row of ``logits`` [B,N,V].  Returns (probs or None, stats or None)."""
-    lib = load_library()
-    _require_cuda(logits, "logits")
-    if logits.dim() != 3 or logits.stride(2) != 1 or logits.dtype not in (torch.float32, torch.bfloat16):
-        raise RuntimeError("logits must be [B,N,V] float32 / bfloat16 with a contiguous vocabulary axis")
-    B, N, V = logits.shape
-    si = SpecIn(B, N, V, SPEC_F32 if logits.dtype == torch.float32 else SPEC_BF16,
-                _ptr(logits), _ptr(logits), logits.stride(0), logits.stride(1), None, 0, None,
-                float(temperature), int(top_k), float(top_p), _ptr(temperature_per_seq), None, None)
-    probs = torch.empty((B, N, V), dtype=torch.float32, device=logits.device) if want_probs else None
-    stats = torch.empty((B, N, 6), dtype=torch.float32, device=logits.device) if want_stats else None
-    ws_ptr, ws_size = _ws_for(logits.device).get(workspace_bytes(si))       # holds the row cuts when truncating
-    _check(lib.spec_tree_probs(C.byref(si), int(which), _ptr(probs), _ptr(stats), ws_ptr, ws_size,
-                               _stream_ptr(stream)), "spec_tree_probs")
-    return probs, stats
+    return _calls().tree_probs(logits, which, temperature, top_k, top_p, temperature_per_seq, want_probs, want_stats,
+                               _ws_for(logits.device), stream)
 
 
 def sample_bonus(weights, u, want_margin=False, stream=None):
     """Inverse-CDF draw from each row of ``weights`` [R,V] float32 with uniforms ``u`` [R]."""
-    lib = load_library()
-    _require_cuda(weights, "weights")
-    _require_cuda(u, "u")
-    if weights.dtype != torch.float32 or not weights.is_contiguous() or weights.dim() != 2:
-        raise RuntimeError("weights must be a contiguous [R,V] float32 tensor")
-    if u.dtype != torch.float32 or not u.is_contiguous() or u.numel() != weights.shape[0]:
-        raise RuntimeError("u must be a contiguous float32 tensor with one entry per row")
-    R, V = weights.shape
-    token = torch.empty(R, dtype=torch.int32, device=weights.device)
-    margin = torch.empty(R, dtype=torch.float32, device=weights.device) if want_margin else None
-    _check(lib.spec_sample_bonus(_ptr(weights), R, V, _ptr(u), _ptr(token), _ptr(margin), None, 0,
-                                 _stream_ptr(stream)), "spec_sample_bonus")
-    return (token, margin) if want_margin else token
+    return _calls().sample_bonus(weights, u, want_margin, stream)
 
 
 class HostVerifier:
