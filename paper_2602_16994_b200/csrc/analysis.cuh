@@ -6,7 +6,7 @@
 //
 // Division of work.  The every-node kernel holds a node's e_p, e_q on chip with its dominant tokens
 // exact; in analysis mode it runs, before the SpecInfer recursion, read-only sweeps for the vocabulary-wide
-// sums (the functors below) and SpecTr's bisection for rho*, and dumps per node the scalars everything
+// sums (the functors below) and the search for SpecTr's rho*, and dumps per node the scalars everything
 // else follows from (AnRec).  spec_branch_kernel (one warp per node) turns them into branching
 // probabilities -- for SpecInfer with uniformly picked children the dynamic programme of Algorithm 14 over
 // the sets of remaining children -- and spec_reach_kernel multiplies them down the tree.
@@ -31,54 +31,85 @@ struct __align__(16) AnRec {
 };
 
 // ---- functors of the read-only sweeps: tail in fp32, listed tokens in fp64 -----------------------------------
-struct FnL1Min {        // a0: sum |p - q|, a1: sum min(p, q)
-    float ipf, iqf; double ip, iq;
-    __device__ __forceinline__ void tail(float ep, float eq, float &a0, float &a1) const
-    { const float p = ep * ipf, q = eq * iqf; a0 += fabsf(p - q); a1 += fminf(p, q); }
-    __device__ __forceinline__ void exact(double ep, double eq, double &a0, double &a1) const
-    { const double p = ep * ip, q = eq * iq; a0 += fabs(p - q); a1 += fmin(p, q); }
-};
-struct FnNssNaive {     // a0: sum p (1 - (1-q)^k)  (Algorithm 6), a1: sum (p-q)+ (1 - (1-q)^(k-1))  (Algorithm 7)
-    float ipf, iqf; double ip, iq; float kf; double kd;
-    __device__ __forceinline__ void tail(float ep, float eq, float &a0, float &a1) const
+// x (1 + r + ... + r^(k-1)) with r = 1 - x, that is 1 - (1 - x)^k without its cancellation (all terms positive)
+template <typename F>
+__device__ __forceinline__ F one_minus_power(F x, int k)
+{
+    const F r = (F)1 - x;
+    F s = (F)1;
+    for (int i = 1; i < k; ++i) s = s * r + (F)1;
+    return k > 0 ? x * s : (F)0;
+}
+struct FnFirst {        // sum |p - q|, sum min(p, q), sum p (1 - (1-q)^k)  (Algorithm 6), sum (p-q)+ (1 - (1-q)^(k-1))
+                        // (Algorithm 7), sum (p-q)+
+    float ipf, iqf; double ip, iq; int k;
+    template <typename F> __device__ __forceinline__ void add(F p, F q, F (&a)[5]) const
     {
-        const float p = ep * ipf, q = eq * iqf;
-        const float l = log1pf(-fminf(q, 1.f));
-        a0 += p * (-expm1f(kf * l));
-        a1 += fmaxf(p - q, 0.f) * (kf > 1.f ? -expm1f((kf - 1.f) * l) : 0.f);
+        const F d = p - q, dp = d > (F)0 ? d : (F)0, qc = q < (F)1 ? q : (F)1;
+        a[0] += d > (F)0 ? d : -d;
+        a[1] += p < q ? p : q;
+        a[2] += p * one_minus_power(qc, k);
+        a[3] += dp * one_minus_power(qc, k - 1);
+        a[4] += dp;
     }
-    __device__ __forceinline__ void exact(double ep, double eq, double &a0, double &a1) const
-    {
-        const double p = ep * ip, q = eq * iq;
-        const double l = log1p(-fmin(q, 1.0));
-        a0 += p * (-expm1(kd * l));
-        a1 += fmax(p - q, 0.0) * (kd > 1.0 ? -expm1((kd - 1.0) * l) : 0.0);
-    }
+    __device__ __forceinline__ void tail(float ep, float eq, float (&a)[5]) const { add(ep * ipf, eq * iqf, a); }
+    __device__ __forceinline__ void exact(double ep, double eq, double (&a)[5]) const { add(ep * ip, eq * iq, a); }
 };
-struct FnBeta {         // a0: beta(rho) = sum min(p / rho, q)   (Appendix B, above Algorithm 3)
+struct FnBeta {         // beta(rho) = sum min(p / rho, q)   (Appendix B, above Algorithm 3)
     float ipf, iqf; double ip, iq;   // ip already divided by rho
-    __device__ __forceinline__ void tail(float ep, float eq, float &a0, float &) const { a0 += fminf(ep * ipf, eq * iqf); }
-    __device__ __forceinline__ void exact(double ep, double eq, double &a0, double &) const { a0 += fmin(ep * ip, eq * iq); }
+    __device__ __forceinline__ void tail(float ep, float eq, float (&a)[2]) const { a[0] += fminf(ep * ipf, eq * iqf); }
+    __device__ __forceinline__ void exact(double ep, double eq, double (&a)[2]) const { a[0] += fmin(ep * ip, eq * iq); }
 };
-struct FnSpecTrRes {    // a0: sum d, a1: sum d (1 - (1-r)^k), d = (p - min(p/rho, q) gamma)+, r = (q - p/rho)+ / (1-beta)
-    float ipf, iqf, irf, gf, ibf, kf; double ip, iq, ir, g, ib, kd;     // ir = 1/rho, ib = 1/(1-beta) (0 when beta = 1)
-    __device__ __forceinline__ void tail(float ep, float eq, float &a0, float &a1) const
+struct FnSpecTrRes {    // sum d, sum d (1 - (1-r)^k), d = (p - min(p/rho, q) gamma)+, r = (q - p/rho)+ / (1-beta)
+    float ipf, iqf, irf, gf, ibf; double ip, iq, ir, g, ib; int k;     // ir = 1/rho, ib = 1/(1-beta) (0 when beta = 1)
+    __device__ __forceinline__ void tail(float ep, float eq, float (&a)[2]) const
     {
         const float p = ep * ipf, q = eq * iqf, pr = p * irf;
         const float d = fmaxf(p - fminf(pr, q) * gf, 0.f);
         const float r = fminf(fmaxf(q - pr, 0.f) * ibf, 1.f);
-        a0 += d;
-        a1 += d * (-expm1f(kf * log1pf(-r)));
+        a[0] += d;
+        a[1] += d * one_minus_power(r, k);
     }
-    __device__ __forceinline__ void exact(double ep, double eq, double &a0, double &a1) const
+    __device__ __forceinline__ void exact(double ep, double eq, double (&a)[2]) const
     {
         const double p = ep * ip, q = eq * iq, pr = p * ir;
         const double d = fmax(p - fmin(pr, q) * g, 0.0);
         const double r = fmin(fmax(q - pr, 0.0) * ib, 1.0);
-        a0 += d;
-        a1 += d * (-expm1(kd * log1p(-r)));
+        a[0] += d;
+        a[1] += d * one_minus_power(r, k);
     }
 };
+
+// SpecTr's division factor: the root of f(rho) = 1 - (1 - beta)^k - rho beta on [1, k] (Appendix B), f(1) >= 0 >= f(k).
+// Regula falsi with the Illinois rule (the value at an end that stays is halved), and the middle whenever two steps
+// have not halved the bracket -- so never more than about twice the steps of a bisection, and about ten where f is
+// smooth (a bisection to the same 1e-9 takes 31, each a sweep over the node and a sum over the cluster).
+template <typename F>
+__device__ __forceinline__ double spectr_root(double k, F beta)
+{
+    const auto f = [&](double r) { const double b = beta(r); return (1.0 - pow(1.0 - b, k)) - r * b; };
+    double lo = 1.0, hi = k, flo = f(lo), fhi = f(hi);
+    if (!(flo > 0.0)) return 1.0;
+    double was = hi - lo;
+    int side = 0;
+    for (int it = 0; it < 64 && hi - lo > 1.0e-9; ++it) {
+        double x = fhi < 0.0 ? (lo * fhi - hi * flo) / (fhi - flo) : hi;
+        if ((it & 1) && hi - lo > 0.5 * was) x = 0.5 * (lo + hi);
+        if (it & 1) was = hi - lo;
+        if (!(x > lo && x < hi)) x = 0.5 * (lo + hi);
+        const double fx = f(x);
+        if (fx > 0.0) {
+            lo = x; flo = fx;
+            if (side > 0) fhi *= 0.5;
+            side = 1;
+        } else {
+            hi = x; fhi = fx;
+            if (side < 0) flo *= 0.5;
+            side = -1;
+        }
+    }
+    return 0.5 * (lo + hi);
+}
 
 namespace analysis {
 

@@ -146,16 +146,16 @@ __device__ __forceinline__ double pow2d(int k)
     k = min(k, 1023);
     return k < -1022 ? 0.0 : __hiloint2double((k + 1023) << 20, 0);
 }
-// 2^f for |f| <= 0.5 to about 1e-15 (Taylor series of exp(f ln 2), degree 13)
+// 2^f for |f| <= 0.5 to about 1e-15 (Taylor series of exp(f ln 2), degree 13; evaluated in pairs, because its callers wait
+// for it: five dependent operations instead of thirteen)
 __device__ __forceinline__ double exp2_frac(double f)
 {
-    const double t = f * 0.6931471805599453094;
-    double p = 1.0 / 6227020800.0;
-    p = fma(p, t, 1.0 / 479001600.0); p = fma(p, t, 1.0 / 39916800.0); p = fma(p, t, 1.0 / 3628800.0);
-    p = fma(p, t, 1.0 / 362880.0); p = fma(p, t, 1.0 / 40320.0); p = fma(p, t, 1.0 / 5040.0);
-    p = fma(p, t, 1.0 / 720.0); p = fma(p, t, 1.0 / 120.0); p = fma(p, t, 1.0 / 24.0);
-    p = fma(p, t, 1.0 / 6.0); p = fma(p, t, 0.5); p = fma(p, t, 1.0); p = fma(p, t, 1.0);
-    return p;
+    const double t = f * 0.6931471805599453094, t2 = t * t, t4 = t2 * t2, t8 = t4 * t4;
+    const double p0 = 1.0 + t, p1 = fma(t, 1.0 / 6.0, 0.5), p2 = fma(t, 1.0 / 120.0, 1.0 / 24.0);
+    const double p3 = fma(t, 1.0 / 5040.0, 1.0 / 720.0), p4 = fma(t, 1.0 / 362880.0, 1.0 / 40320.0);
+    const double p5 = fma(t, 1.0 / 39916800.0, 1.0 / 3628800.0), p6 = fma(t, 1.0 / 6227020800.0, 1.0 / 479001600.0);
+    const double q0 = fma(t2, p1, p0), q1 = fma(t2, p3, p2), q2 = fma(t2, p5, p4);
+    return fma(t8, fma(t4, p6, q2), fma(t4, q1, q0));
 }
 // fp32 pairs in one 64-bit register: packed fused multiply-add and add (sm_100)
 __device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi)
@@ -227,9 +227,10 @@ struct __align__(16) NodeRec {
     int next_child;              // SpecInfer: accepted child or -1
     int bonus;                   // bonus token this node would emit, or -1
     int status;
-    int nsteps;                  // sibling steps its final state went through; STATE_IS_Q: the state equals q
+    int nsteps;                  // sibling steps its final state went through; STATE_IS_Q: the state equals q; STATE_FIRST
     int pad;
 };
 constexpr int STATE_IS_Q = -1;
+constexpr int STATE_FIRST = -2;  // one child, rejected: the step is taken by whoever needs the state (a FINISH item), from w_in
 
 }  // namespace specv

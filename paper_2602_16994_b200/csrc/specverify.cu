@@ -1,8 +1,8 @@
 // libspecverify: batched draft-tree verification for sm_100a -- host side of the C ABI.
 //
 // Kernels: stream.cuh (row statistics, the one pass over HBM), trunc.cuh (the same for top-k / top-p
-// rows), walk.cuh (SpecInfer along the accepted path), tree.cuh (every node: Traversal Verification,
-// diagnostic outputs), rowops.cuh (materialised row distributions, stand-alone inverse CDF), and the
+// rows), walk.cuh (SpecInfer along the accepted path), nodes.cuh (every node: Traversal Verification,
+// diagnostic outputs, analysis), rowops.cuh (materialised row distributions, stand-alone inverse CDF), and the
 // residual kernel below.  This file validates
 // arguments, chooses the launch plan and enqueues; it never allocates and, except for the
 // host-buffer entry point, never synchronises.
@@ -11,12 +11,13 @@
 
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "analysis.cuh"
 #include "common.cuh"
 #include "cut.cuh"
+#include "nodes.cuh"
 #include "rowops.cuh"
-#include "tree.cuh"
 #include "trunc.cuh"
 #include "specverify.h"
 #include "verify.cuh"
@@ -78,8 +79,7 @@ __global__ void spec_residual_kernel(const RParams P)
 // launch plans
 // ------------------------------------------------------------------------------------------------
 struct VPlan {
-    int C, NW, slice_len, NS, nsm, off_x, off_list, off_es, off_ring, smem;
-    int whole_sm;       // one CTA per SM: the kernel variant without a register limit may be used
+    int C, slice_len, off_es, smem;
 };
 
 constexpr int SMEM_1CTA = 227 * 1024;          // opt-in limit per CTA
@@ -87,46 +87,36 @@ constexpr int SMEM_2CTA = 113 * 1024;          // so that two CTAs share an SM
 
 inline int up(int x, int m) { return (x + m - 1) / m * m; }
 
-// Launch shape of the cluster kernels (walk, tree).  Smallest cluster whose slices fit on chip: seven
-// consumer warps + the producer warp (256 threads, two CTAs per SM, 128 registers each) while a slice
-// fits in TMAX tiles of 1792 tokens, fifteen consumer warps (one CTA per SM) above that.
-// Dynamic shared memory: header | exchange slots [2][C][NW][2] doubles | exact lists [NW] | resident e
-// of the tiles that do not fit in registers | ring stages.
-bool make_vplan(int V, int dtype, VPlan *p, int hdr_bytes = (int)sizeof(Hdr), bool whole_sm = false, int want_c = 0,
-                int want_nw = 0)
+// Launch shape of the cluster kernels (walk, tree) with NW consumer warps of RC register chunks per thread: the smallest
+// cluster in which a thread has at most `want` chunks, those beyond RC in shared memory; eight CTAs with as many as fit
+// before sixteen (a non-portable size, and fewer clusters fit the chip).  Dynamic shared memory: header | resident e
+// of the chunks that do not fit in registers.
+bool make_vplan(int V, int NW, int RC, int budget, int want, int hdr_bytes, VPlan *p)
 {
-    const int esz = dtype == SPEC_BF16 ? 2 : 4;
-    for (int pass = 0; pass < 2; ++pass) {
-        const int NW = pass == 0 ? 7 : 15;
-        if (want_nw && NW != want_nw) continue;
-        const int tile = NW * 32 * 8;
-        const int budget = (NW == 7 && !whole_sm) ? SMEM_2CTA : SMEM_1CTA;
-        for (int C = 1; C <= CMAX; C <<= 1) {
-            if (want_c && C != want_c) continue;
-            const int slice = up((V + C - 1) / C, 8);
-            const int tiles = (slice + tile - 1) / tile;
-            if (tiles > TMAX) continue;
-            if (pass == 0 && C > 8 && !want_c) continue;   // prefer one CTA per SM over a non-portable cluster
-            const int off_x = up(hdr_bytes, 128);
-            const int off_list = off_x + up(2 * C * NW * 2 * 8, 128);
-            const int off_es = off_list + up(NW * (int)sizeof(WarpList), 128);
-            const int stage = 2 * tile * esz;
-            const int nsm = tiles > RT ? tiles - RT : 0;
-            if (nsm > SMT) continue;
-            const int es_bytes = nsm * tile * 8;
-            const int off_ring = off_es + es_bytes;
-            int ns = (budget - off_ring) / stage;
-            if (ns > NSMAX) ns = NSMAX;
-            if (ns > 2 * tiles) ns = 2 * tiles;
-            if (ns < 2) continue;
-            p->C = C; p->NW = NW; p->slice_len = slice; p->NS = ns; p->nsm = nsm; p->whole_sm = 0;
-            p->off_x = off_x; p->off_list = off_list; p->off_es = off_es; p->off_ring = off_ring;
-            p->smem = off_ring + ns * stage;
-            return true;
-        }
+    const int chunk_bytes = NW * 32 * 64, off_es = up(hdr_bytes, 128);
+    const int most = RC + (budget - off_es) / chunk_bytes, cap = most < CHMAX ? most : CHMAX;
+    const int units = (int)(((long long)V + 14) / 8);          // chunks of a row, wherever it starts
+    for (int C = 1; C <= CMAX; C <<= 1) {
+        const int per = (units + C - 1) / C, nch = (per + NW * 32 - 1) / (NW * 32);
+        if (nch > (C < 8 ? (want < cap ? want : cap) : cap)) continue;
+        p->C = C; p->slice_len = per * 8; p->off_es = off_es;
+        p->smem = off_es + (nch > RC ? nch - RC : 0) * chunk_bytes;
+        return true;
     }
     return false;
 }
+// The kernels keep a node's e in shared memory and go through it in loops: their code runs a few times per sequence, and its first
+// run costs about 80 cycles per 128 bytes of instructions (unrolled over eight chunks in registers, a first pass took 7000
+// cycles and the analysis' sweeps ten times that).  Registers as well (big: RC = 8) only for vocabularies beyond
+// what the shared memory of 16 CTAs holds; the walk of a batch that fills the chip puts two CTAs on an SM (RC = 4).
+bool one_cta_plan(int V, int NW, int hdr_bytes, VPlan *p, bool *big)
+{
+    *big = false;
+    if (make_vplan(V, NW, 0, SMEM_1CTA, 9, hdr_bytes, p)) return true;
+    *big = true;
+    return make_vplan(V, NW, 8, SMEM_1CTA, 9, hdr_bytes, p);
+}
+bool two_cta_plan(int V, int hdr_bytes, VPlan *p) { return make_vplan(V, 8, 4, SMEM_2CTA, 8, hdr_bytes, p); }
 
 struct RowPlan {
     int C, SL, smem;
@@ -170,7 +160,7 @@ inline int64_t up256(int64_t x) { return (x + 255) / 256 * 256; }
 
 // workspace layout: node records | published weights + arrival counters (cleared per call) | row cuts
 struct WsLayout {
-    int64_t rec, pub, fin, best, done, ticket, order, cut, stat, gseq, total;
+    int64_t rec, pub, fin, done, ticket, chain, cut, stat, gseq, total;
 };
 constexpr int MAX_PARTS = 4;      // parts a row may be split into by the streaming statistics kernel
 WsLayout ws_layout(const SpecIn *in, int slices = MAX_PARTS)   // slices = 0: one record per row only
@@ -179,16 +169,13 @@ WsLayout ws_layout(const SpecIn *in, int slices = MAX_PARTS)   // slices = 0: on
     const int64_t nodes = (int64_t)in->B * in->N;
     int64_t o = 0;
     L.rec = o; o += up256(nodes * (int64_t)sizeof(NodeRec));
-    // set to all-ones per call: published weights, accepted nodes, earliest known acceptance; set to zero:
-    // arrival counters, item counter, post-order table
+    // set per call by the statistics kernels (NodeInit)
     L.pub = o; o += nodes * 8;
     L.fin = o; o += (int64_t)in->B * 4;
-    L.best = o; o += (int64_t)in->B * 4;
     L.done = o; o += (int64_t)in->B * 4;
     L.ticket = o; o += 4;
-    o = (o + 7) / 8 * 8;
-    L.order = o; o += nodes * 8;
     o = up256(o);
+    L.chain = o; o += up256(nodes * (int64_t)sizeof(ChainRec));
     L.cut = o; o += up256(nodes * 8);
     L.stat = o; o += up256(nodes * 2 * (slices + 1) * (int64_t)sizeof(RowPart));      // one record per row, then the parts
     L.gseq = o; o += up256(nodes * KMAX * 8);       // step coefficients of every node
@@ -244,7 +231,7 @@ int sm_count()
 // Kernel attributes are set once per (device, kernel): the largest dynamic shared memory asked for
 // so far and the permission for clusters above 8 CTAs.  Later calls only launch.
 template <typename K>
-int prepare_kernel(K kernel, int C, int smem)
+int prepare_kernel(K kernel, int C, int smem, bool overlap = false)
 {
     struct Entry { const void *k; int dev, smem, big; };
     static Entry cache[256];
@@ -259,6 +246,13 @@ int prepare_kernel(K kernel, int C, int smem)
         if (used >= 256) return SPEC_ERR_CUDA;
         ent = &cache[used++];
         *ent = Entry{(const void *)kernel, dev, -1, 0};
+        // The kernel's code is on the device from here on: loaded at its first launch it could wait for kernels that wait for it.
+        cudaFuncAttributes attr;
+        if (cudaFuncGetAttributes(&attr, (const void *)kernel) != cudaSuccess) { cudaGetLastError(); --used; return SPEC_ERR_CUDA; }
+        // overlap: as much of an SM's L1 as can be is shared memory, so that CTAs of the kernels that run at the same time
+        // find room beside this one
+        if (overlap && cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+            cudaGetLastError();
     }
     if (smem > ent->smem) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -303,18 +297,32 @@ int resident_clusters(K kernel, int C, int threads, int smem)
     return n;
 }
 
-template <int DT, int NW, bool AN>
-int launch_tree(const VPlan &pl, TParams &tp, cudaStream_t st)
+// nodes with several children (AN: with any): a cluster each
+template <int DT, int RC, bool AN>
+int launch_branch(const VPlan &pl, NParams &np, cudaStream_t st, bool prepare)
 {
-    auto kernel = spec_tree_kernel<DT, NW, AN>;
-    int rc = prepare_kernel(kernel, pl.C, pl.smem);
-    if (rc) return rc;
-    const int threads = (NW + 1) * 32;
-    int nc = resident_clusters(kernel, pl.C, threads, pl.smem);
+    auto kernel = spec_recursion_kernel<DT, 7, RC, AN>;
+    if (prepare) return prepare_kernel(kernel, pl.C, pl.smem, true);
+    int nc = resident_clusters(kernel, pl.C, 256, pl.smem);
     if (nc <= 0) return SPEC_ERR_UNSUPPORTED;
-    const long long items = (long long)tp.v.B * tp.v.N + tp.v.B;
+    // A few SMs stay free for the nodes with one child, which hand weights to these: they have to run whatever this
+    // kernel's clusters wait for (and an SM whose shared memory is split for a smaller kernel takes none of them).
+    while (!AN && nc > 1 && nc * pl.C > sm_count() - 4) --nc;
+    const long long items = (long long)np.v.B * np.v.N;
     if (nc > items) nc = (int)items;
-    return launch_clustered(kernel, nc * pl.C, pl.C, threads, pl.smem, st, &tp);
+    np.v.C = pl.C; np.v.off_es = pl.off_es;
+    return launch_clustered(kernel, nc * pl.C, pl.C, 256, pl.smem, st, &np);
+}
+template <int DT, int RC>
+int launch_finish(const VPlan &pl, NParams &np, cudaStream_t st, bool prepare)
+{
+    auto kernel = spec_finish_kernel<DT, 8, RC>;
+    if (prepare) return prepare_kernel(kernel, pl.C, pl.smem, true);
+    int nc = resident_clusters(kernel, pl.C, 256, pl.smem);
+    if (nc <= 0) return SPEC_ERR_UNSUPPORTED;
+    if (nc > np.v.B) nc = np.v.B;
+    np.v.C = pl.C; np.v.off_es = pl.off_es;
+    return launch_clustered(kernel, nc * pl.C, pl.C, 256, pl.smem, st, &np, true);
 }
 
 // row statistics (cut, reference, normaliser) of every row the verifiers read, or of every row of `zp` when no
@@ -347,13 +355,13 @@ int launch_trunc(const SpecIn *in, const void *zp, const void *zq, const int *pa
 }
 
 // SpecInfer without diagnostic outputs: row statistics of every row, then one walk per sequence
-template <int DT, int NW, int MINB, bool OT = false>
+template <int DT, int NW, int RC, int MINB, bool OT>
 int launch_walk(const VPlan &pl, WParams &wp, cudaStream_t st)
 {
-    auto kernel = spec_walk_kernel<DT, NW, MINB, OT>;
+    auto kernel = spec_walk_kernel<DT, NW, RC, MINB, OT>;
     int rc = prepare_kernel(kernel, pl.C, pl.smem);
     if (rc) return rc;
-    const int threads = (NW + 1) * 32;
+    const int threads = NW * 32;
     int nc = resident_clusters(kernel, pl.C, threads, pl.smem);
     if (nc <= 0) return SPEC_ERR_UNSUPPORTED;
     if (nc > wp.B) nc = wp.B;
@@ -372,7 +380,7 @@ int row_statistics(const SpecIn *in, const SpecOut *out, unsigned char *w, const
     stream::NodeInit init = {};
     if (init_nodes)
         init = {(unsigned long long *)(w + L.pub), (unsigned int *)(w + L.done), (int *)(w + L.fin),
-                (unsigned int *)(w + L.best), (unsigned long long *)(w + L.order), (unsigned int *)(w + L.ticket)};
+                (unsigned int *)(w + L.ticket), (ulonglong2 *)(w + L.chain)};
     if (trunc) {
         rc = launch_trunc(in, in->target_logits, in->draft_logits, in->parent, w, L, init, st);
         if (rc) return rc;
@@ -424,41 +432,42 @@ int row_statistics(const SpecIn *in, const SpecOut *out, unsigned char *w, const
     return SPEC_OK;
 }
 
-int verify_walk(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, const VPlan &pl,
-                bool trunc, bool parts, cudaStream_t st, int solver = -1)
+// solver: -1 SpecInfer, otherwise the OTLP solver of spec_verify_otlp
+int verify_walk(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, bool trunc, bool parts,
+                cudaStream_t st, int solver = -1)
 {
+    // The walk keeps one cluster per sequence busy.  While all of them fit on the chip with one CTA per SM, a CTA may use
+    // all of an SM's registers; larger batches share the SMs.
+    VPlan pl, one;
+    bool big;
+    const bool fits = one_cta_plan(in->V, 8, (int)sizeof(WHdr), &one, &big);
+    const bool whole = fits && ((long long)in->B * one.C <= sm_count() || !two_cta_plan(in->V, (int)sizeof(WHdr), &pl));
+    if (whole) pl = one;
+    else if (!fits) return SPEC_ERR_UNSUPPORTED;
     int rc = row_statistics(in, out, w, L, trunc, parts, st);
     if (rc) return rc;
-    const int NSL = 1;
-    RowPart *part = (RowPart *)(w + L.stat);
     WParams wp = {};
-    wp.B = in->B; wp.N = in->N; wp.V = in->V; wp.C = pl.C; wp.NSL = NSL;
-    wp.slice_len = pl.slice_len; wp.NS = pl.NS; wp.nsm = pl.nsm; wp.off_x = pl.off_x; wp.off_list = pl.off_list; wp.off_es = pl.off_es;
-    wp.off_ring = pl.off_ring;
+    wp.B = in->B; wp.N = in->N; wp.V = in->V; wp.C = pl.C; wp.off_es = pl.off_es;
     wp.zp = in->target_logits; wp.zq = in->draft_logits;
     wp.seq_stride = in->seq_stride; wp.node_stride = in->node_stride; wp.topo_stride = in->topo_seq_stride;
     wp.parent = in->parent; wp.token = in->token; wp.T = in->temperature; wp.T_seq = in->temperature_per_seq;
-    wp.part = part; wp.u_accept = in->u_accept; wp.u_bonus = in->u_bonus; wp.out = *out;
+    wp.part = (RowPart *)(w + L.stat); wp.u_accept = in->u_accept; wp.u_bonus = in->u_bonus; wp.out = *out;
+    wp.solver = solver;
     const bool bf = in->logits_dtype == SPEC_BF16;
-    if (solver >= 0) {
-        // the walk with another OTLP solver (Algorithms 1-3): its own instantiation, two CTAs per SM
-        wp.solver = solver;
-        if (pl.NW == 7) return bf ? launch_walk<SPEC_BF16, 7, 2, true>(pl, wp, st) : launch_walk<SPEC_F32, 7, 2, true>(pl, wp, st);
-        return bf ? launch_walk<SPEC_BF16, 15, 1, true>(pl, wp, st) : launch_walk<SPEC_F32, 15, 1, true>(pl, wp, st);
-    }
-    if (pl.NW == 7 && pl.whole_sm) return bf ? launch_walk<SPEC_BF16, 7, 1>(pl, wp, st) : launch_walk<SPEC_F32, 7, 1>(pl, wp, st);
-    if (pl.NW == 7) return bf ? launch_walk<SPEC_BF16, 7, 2>(pl, wp, st) : launch_walk<SPEC_F32, 7, 2>(pl, wp, st);
-    return bf ? launch_walk<SPEC_BF16, 15, 1>(pl, wp, st) : launch_walk<SPEC_F32, 15, 1>(pl, wp, st);
+    auto go = [&](auto ot) {
+        constexpr bool OT = decltype(ot)::value;
+        if (whole && big) return bf ? launch_walk<SPEC_BF16, 8, 8, 1, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 8, 1, OT>(pl, wp, st);
+        if (whole) return bf ? launch_walk<SPEC_BF16, 8, 0, 1, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 0, 1, OT>(pl, wp, st);
+        return bf ? launch_walk<SPEC_BF16, 8, 4, 2, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 4, 2, OT>(pl, wp, st);
+    };
+    return solver >= 0 ? go(std::true_type{}) : go(std::false_type{});
 }
 
-void fill_tparams(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, const VPlan &pl, int mode,
-                  TParams &tp)
+void fill_params(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, int mode, NParams &tp)
 {
     VParams &vp = tp.v;
-    vp.B = in->B; vp.N = in->N; vp.V = in->V; vp.C = pl.C; vp.mode = mode;
+    vp.B = in->B; vp.N = in->N; vp.V = in->V; vp.mode = mode;
     vp.all_thr = (out->node_thr != nullptr || out->margin != nullptr) ? 1 : 0;
-    vp.slice_len = pl.slice_len; vp.NS = pl.NS; vp.nsm = pl.nsm;
-    vp.off_x = pl.off_x; vp.off_list = pl.off_list; vp.off_es = pl.off_es; vp.off_ring = pl.off_ring;
     vp.zp = in->target_logits; vp.zq = in->draft_logits;
     vp.seq_stride = in->seq_stride; vp.node_stride = in->node_stride; vp.topo_stride = in->topo_seq_stride;
     vp.parent = in->parent; vp.token = in->token;
@@ -468,26 +477,48 @@ void fill_tparams(const SpecIn *in, const SpecOut *out, unsigned char *w, const 
     vp.w_pub = (unsigned long long *)(w + L.pub);
     vp.done = (unsigned int *)(w + L.done);
     vp.fin = (int *)(w + L.fin);
-    vp.best = (unsigned int *)(w + L.best);
-    vp.order = (unsigned long long *)(w + L.order);
-    // Traversal without per-node diagnostics: subtrees that come after a known acceptance in the traversal
-    // order are not evaluated
-    vp.prune = (mode == MODE_TRAVERSAL && !out->node_thr && !out->node_w_in && !out->margin) ? 1 : 0;
+    vp.chain = (ChainRec *)(w + L.chain);
     vp.out = *out;
     tp.part = (const RowPart *)(w + L.stat);
     tp.gseq = (double *)(w + L.gseq);
     tp.ticket = (unsigned int *)(w + L.ticket);
 }
 
-int launch_tree_any(const SpecIn *in, const VPlan &pl, TParams &tp, bool analysis, cudaStream_t st)
+// every node of every sequence, on top of the row statistics
+int launch_nodes(const SpecIn *in, NParams &np, bool analysis, cudaStream_t st)
 {
     const bool bf = in->logits_dtype == SPEC_BF16;
-    if (analysis) {
-        if (pl.NW == 7) return bf ? launch_tree<SPEC_BF16, 7, true>(pl, tp, st) : launch_tree<SPEC_F32, 7, true>(pl, tp, st);
-        return bf ? launch_tree<SPEC_BF16, 15, true>(pl, tp, st) : launch_tree<SPEC_F32, 15, true>(pl, tp, st);
+    VPlan br, fi;
+    bool big, bigf;
+    if (!one_cta_plan(in->V, 7, (int)sizeof(BHdr), &br, &big) || !one_cta_plan(in->V, 8, (int)sizeof(FHdr), &fi, &bigf)) return SPEC_ERR_UNSUPPORTED;
+    auto branch = [&](auto an, bool prepare) {
+        constexpr bool AN = decltype(an)::value;
+        if (big) return bf ? launch_branch<SPEC_BF16, 8, AN>(br, np, st, prepare) : launch_branch<SPEC_F32, 8, AN>(br, np, st, prepare);
+        return bf ? launch_branch<SPEC_BF16, 0, AN>(br, np, st, prepare) : launch_branch<SPEC_F32, 0, AN>(br, np, st, prepare);
+    };
+    // nodes with one child: as many CTAs per node as the chip has room for while all nodes run at once
+    int C = 1;
+    const long long nodes = (long long)in->B * in->N;
+    while (C < 8 && nodes * C * 2 <= 2 * sm_count() && in->V >= C * 8192) C <<= 1;
+    auto single = [&](bool prepare) {
+        np.v.C = C;
+        auto go = [&](auto kernel) {
+            return prepare ? prepare_kernel(kernel, C, 0, true) : launch_clustered(kernel, (int)nodes * C, C, 256, 0, st, &np, true);
+        };
+        return bf ? go(spec_single_kernel<SPEC_BF16>) : go(spec_single_kernel<SPEC_F32>);
+    };
+    auto finish = [&](bool prepare) {
+        if (bigf) return bf ? launch_finish<SPEC_BF16, 8>(fi, np, st, prepare) : launch_finish<SPEC_F32, 8>(fi, np, st, prepare);
+        return bf ? launch_finish<SPEC_BF16, 0>(fi, np, st, prepare) : launch_finish<SPEC_F32, 0>(fi, np, st, prepare);
+    };
+    // (everything that may wait for the device happens before the first of the kernels that wait for one another)
+    for (int prepare = 1; prepare >= 0; --prepare) {
+        int rc = analysis ? branch(std::true_type{}, prepare) : branch(std::false_type{}, prepare);
+        if (!rc && !analysis) rc = single(prepare);
+        if (!rc && !analysis) rc = finish(prepare);
+        if (rc) return rc;
     }
-    if (pl.NW == 7) return bf ? launch_tree<SPEC_BF16, 7, false>(pl, tp, st) : launch_tree<SPEC_F32, 7, false>(pl, tp, st);
-    return bf ? launch_tree<SPEC_BF16, 15, false>(pl, tp, st) : launch_tree<SPEC_F32, 15, false>(pl, tp, st);
+    return SPEC_OK;
 }
 
 int verify_common(const SpecIn *in, const SpecOut *out, void *ws, int64_t ws_bytes, void *stream, int mode,
@@ -501,29 +532,20 @@ int verify_common(const SpecIn *in, const SpecOut *out, void *ws, int64_t ws_byt
     const WsLayout L = ws_layout(in, parts ? MAX_PARTS : 0);
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < L.total) return SPEC_ERR_WORKSPACE;
     VPlan pl;
-    if (!make_vplan(in->V, in->logits_dtype, &pl)) return SPEC_ERR_UNSUPPORTED;
+    bool big;
+    if (!one_cta_plan(in->V, 7, (int)sizeof(BHdr), &pl, &big)) return SPEC_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)stream;
     unsigned char *w = (unsigned char *)ws;
     const bool diagnostics = out->residual || out->node_thr || out->node_w_in || out->margin;
-    if (mode == MODE_SPECINFER && !diagnostics && in->N <= NWALK) {
-        // the walk keeps one cluster per sequence busy: when all of them fit on the chip with one CTA
-        // per SM, each CTA may use the whole SM's shared memory for its ring and twice the registers
-        VPlan wpl;
-        if (!make_vplan(in->V, in->logits_dtype, &wpl, (int)sizeof(WHdr), false)) return SPEC_ERR_UNSUPPORTED;
-        if ((long long)in->B * wpl.C <= sm_count()) {
-            VPlan big;
-            if (make_vplan(in->V, in->logits_dtype, &big, (int)sizeof(WHdr), true, wpl.C, wpl.NW)) { wpl = big; wpl.whole_sm = 1; }
-        }
-        return verify_walk(in, out, w, L, wpl, trunc, parts, st);
-    }
+    if (mode == MODE_SPECINFER && !diagnostics && in->N <= NWALK) return verify_walk(in, out, w, L, trunc, parts, st);
     // every node of every sequence on chip once, on top of the row statistics (which also set the
     // published-weight slots to pending and the arrival counters to zero)
     rc = row_statistics(in, out, w, L, trunc, parts, st, true);
     if (rc) return rc;
-    TParams tp = {};
-    fill_tparams(in, out, w, L, pl, mode, tp);
+    NParams tp = {};
+    fill_params(in, out, w, L, mode, tp);
     VParams &vp = tp.v;
-    rc = launch_tree_any(in, pl, tp, false, st);
+    rc = launch_nodes(in, tp, false, st);
     if (rc) return rc;
     if (out->residual) {
         RParams rp = {};
@@ -619,12 +641,13 @@ int32_t spec_query_plan(int32_t V, int32_t logits_dtype, int32_t *cluster_size, 
 {
     if (V <= 0) return SPEC_ERR_SHAPE;
     if (logits_dtype != SPEC_F32 && logits_dtype != SPEC_BF16) return SPEC_ERR_DTYPE;
-    VPlan pl;
-    if (!make_vplan(V, logits_dtype, &pl)) return SPEC_ERR_UNSUPPORTED;
+    VPlan pl;          // the walk of a batch that fills the chip
+    bool big;
+    if (!two_cta_plan(V, (int)sizeof(WHdr), &pl) && !one_cta_plan(V, 8, (int)sizeof(WHdr), &pl, &big)) return SPEC_ERR_UNSUPPORTED;
     if (cluster_size) *cluster_size = pl.C;
     if (slice_len) *slice_len = pl.slice_len;
     if (smem_bytes) *smem_bytes = pl.smem;
-    if (threads) *threads = (pl.NW + 1) * 32;
+    if (threads) *threads = 256;
     return SPEC_OK;
 }
 
@@ -675,9 +698,7 @@ int32_t spec_verify_otlp(const SpecIn *in, const SpecOut *out, int32_t solver, v
     const bool trunc = (in->top_k > 0 && in->top_k < in->V) || in->top_p < 1.f;
     const WsLayout L = ws_layout(in);
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < L.total) return SPEC_ERR_WORKSPACE;
-    VPlan wpl;
-    if (!make_vplan(in->V, in->logits_dtype, &wpl, (int)sizeof(WHdr), false)) return SPEC_ERR_UNSUPPORTED;
-    return verify_walk(in, out, (unsigned char *)ws, L, wpl, trunc, true, (cudaStream_t)stream, solver);
+    return verify_walk(in, out, (unsigned char *)ws, L, trunc, true, (cudaStream_t)stream, solver);
 }
 
 int32_t spec_verify_specinfer_static(const SpecIn *in, const SpecOut *out, void *stream)
@@ -729,7 +750,8 @@ int32_t spec_tree_analysis(const SpecIn *in, const SpecAnalysisOut *out, void *w
     const AnLayout A = an_layout(in);
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < A.total) return SPEC_ERR_WORKSPACE;
     VPlan pl;
-    if (!make_vplan(in->V, in->logits_dtype, &pl)) return SPEC_ERR_UNSUPPORTED;
+    bool big;
+    if (!one_cta_plan(in->V, 7, (int)sizeof(BHdr), &pl, &big)) return SPEC_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)stream;
     unsigned char *w = (unsigned char *)ws;
     const int64_t nodes = (int64_t)in->B * in->N;
@@ -746,11 +768,11 @@ int32_t spec_tree_analysis(const SpecIn *in, const SpecAnalysisOut *out, void *w
     so.status = (int32_t *)(w + A.status);
     rc = row_statistics(in, &so, w, L, trunc, true, st, true);
     if (rc) return rc;
-    TParams tp = {};
-    fill_tparams(in, &so, w, L, pl, MODE_SPECINFER, tp);
+    NParams tp = {};
+    fill_params(in, &so, w, L, MODE_SPECINFER, tp);
     tp.v.all_thr = 1;
     tp.an = (AnRec *)(w + A.an); tp.an_acc = out->acceptance; tp.an_div = out->divergence;
-    rc = launch_tree_any(in, pl, tp, true, st);
+    rc = launch_nodes(in, tp, true, st);
     if (rc) return rc;
     analysis::BParams bp = {in->B, in->N, in->parent, in->token, in->topo_seq_stride, tp.an, out->acceptance, out->branch};
     analysis::spec_branch_kernel<<<(unsigned)((nodes + 3) / 4), 128, 0, st>>>(bp);

@@ -30,21 +30,20 @@ constexpr int PER = 32;                  // logits per thread
 constexpr int SLICE = NT * PER;          // logits per CTA and slice
 
 // Per-call words of the workspace that an every-node verification wants set (w_pub NULL: none): the published
-// weights and the accepted nodes to pending, no acceptance known, counters and post-order table to zero.  The
+// weights, first-child ratios and accepted nodes to pending, counters to zero.  The
 // statistics kernels set them, which saves the memset nodes of a call.
 struct NodeInit {
     unsigned long long *w_pub;   // [B*N]
     unsigned int *done;          // [B]
     int *fin;                    // [B]
-    unsigned int *best;          // [B]
-    unsigned long long *order;   // [B*N]
     unsigned int *ticket;        // [1]
+    ulonglong2 *chain;           // [B*N]
     __device__ __forceinline__ void set(long long node, int b, int a) const
     {
         if (!w_pub) return;
         w_pub[node] = W_PENDING;
-        order[node] = 0ull;
-        if (a == 0) { done[b] = 0u; fin[b] = -1; best[b] = 0xFFFFFFFFu; }
+        chain[node] = make_ulonglong2(W_PENDING, 0ull);
+        if (a == 0) { done[b] = 0u; fin[b] = -1; }
         if (node == 0) *ticket = 0u;
     }
 };

@@ -1,15 +1,21 @@
 // Pieces shared by the verification kernels (walk.cuh: SpecInfer along the accepted path, Algorithm 4
 // composed top-down, Section 3.2; tree.cuh: every node, Traversal Verification of Section 3.2 with the
 // block-verification weights of Section 3.1): constants and shared-memory layouts, the handling of
-// one chunk of 8 logits (unpack, mask, exponentiate), the residual pass over resident e, prefix picks,
+// one chunk of 8 logits (load, mask, exponentiate), the residual pass over resident e, prefix picks,
 // the inverse-CDF search for the bonus token, and the writing of a sequence's outputs from the node
 // records.
 //
-// Common ground of both kernels.  Each CTA of a cluster owns a contiguous vocabulary slice; each
-// consumer thread owns 8 consecutive tokens of every tile of that slice.  A logit becomes
-// e = 2^(z s - O) with s = log2(e)/T and O the row's integer reference, so every scale factor is an
-// exact power of two.  The e of the last RT tiles of a slice stay in registers, the others in shared
-// memory; nothing is written back to HBM.
+// Common ground of both kernels.  A row is cut into chunks of 8 logits that start on 16-byte boundaries (the first
+// chunk holds fewer where the row starts on none); each CTA of a cluster owns a contiguous range of chunks, each
+// consumer thread every NCONS-th chunk of that range.  A logit becomes e = 2^(z s - O) with s = log2(e)/T and O the
+// row's integer reference, so every scale factor is an exact power of two.  The e of a thread's first RC chunks stay
+// in registers, the others in shared memory; nothing is written back to HBM.
+//
+// A node on chip is a chain of short dependent phases (load, exponentials, a few sweeps, each ended by a sum over the
+// cluster), so it is bound by latency, not by bandwidth or arithmetic.  Hence: every consumer thread loads its own
+// logits, all of them at once (a ring filled by a producer warp kept 3 of 9 tiles in flight and cost a wait and a
+// hand-back per tile: 5 us for the first pass at V = 128256, 2 us now); 16 consumer warps where one CTA has an SM to
+// itself (a sweep is 32 logits per thread), 8 where two share it.
 //
 // The recursion is the paper's own, step by step.  A node's state after j rejected children is the
 // residual law P_j with P_0 = p, held as u_j(t) = kappa_j P_j(t) in place of the resident e_p:
@@ -34,23 +40,20 @@
 // accumulated in fp64 above a thread) + (fp64 over the lists), and so are the rows' normalisers, which
 // the cluster recomputes from the resident e instead of taking them from the statistics pass.
 //
-// Exchanges.  Every consumer warp of every CTA of the cluster sends its partial sum straight into
-// the shared memory of all CTAs (st.async, which counts the bytes on the receiver's mbarrier); every
-// warp waits on its own CTA's mbarrier and reduces all partials itself, in one fixed order, so all
-// warps of the cluster hold bit-identical totals and take identical decisions without any CTA-wide
-// barrier.
+// Sums over the cluster.  Every consumer warp leaves its partial sum in its CTA's shared memory; one warp adds them up
+// and sends the CTA's sum into the shared memory of all CTAs (st.async, which counts the bytes on the receiver's
+// mbarrier); every warp waits on its own CTA's mbarrier and reduces the C sums itself.  One fixed order everywhere,
+// so all warps of the cluster hold bit-identical totals and take identical decisions.
 #pragma once
 #include "common.cuh"
+#include "stream.cuh"
 
 namespace specv {
 
-constexpr int RT = 4;        // tiles per thread whose e may live in registers
-constexpr int SMT = 10;      // tiles per thread whose e may live in shared memory
-constexpr int TMAX = RT + SMT;
+constexpr int CHMAX = 24;    // chunks per thread, in registers (RC of them) and shared memory
 constexpr int CMAX = 16;     // CTAs per cluster (above 8: non-portable size)
-constexpr int NSMAX = 16;    // ring stages
-constexpr int NWMAX = 15;    // consumer warps
-constexpr int OMIN = -(1 << 30);
+constexpr int NWMAX = 8;     // consumer warps
+constexpr int NVMAX = 9;     // doubles per sum over the cluster
 constexpr int FAST_N = 32;   // trees up to this size are finished warp-parallel
 constexpr int FIN_PENDING = -1;     // VParams::fin of a sequence whose nodes are not all done
 constexpr int FIN_FAULTY = -2;      // ... of a sequence with a device-detected fault: no bonus draw
@@ -72,12 +75,16 @@ constexpr int DOM_B = 34;    // tokens above 2^-DOM_B of a row's mass are listed
 
 enum Mode { MODE_SPECINFER = 0, MODE_TRAVERSAL = 1 };
 
+// Traversal: a node of weight w hands its first child min(1, w ratio), with ratio = p(x) / q(x) of the unmodified rows
+struct __align__(16) ChainRec {
+    unsigned long long ratio;    // bits of the double; W_PENDING: not known
+    int child;
+    int pad;
+};
+
 struct VParams {
     int B, N, V, C, mode, all_thr;
-    int slice_len;            // tokens per CTA slice: a multiple of 8, at most TMAX tiles
-    int NS;                   // ring stages
-    int nsm;                  // tiles of a slice kept in shared memory (the others, at most RT, in registers)
-    int off_x, off_list, off_es, off_ring;   // byte offsets inside dynamic shared memory
+    int off_es;               // byte offset of the resident e inside dynamic shared memory
     const void *zp, *zq;
     long long seq_stride, node_stride, topo_stride;
     const int *parent, *token;
@@ -88,67 +95,99 @@ struct VParams {
     unsigned long long *w_pub;   // [B*N] weight handed to a node by its parent (Traversal), W_PENDING until known
     unsigned int *done;          // [B] arrivals per sequence (one per node); the last one selects the accepted node
     int *fin;                    // [B] the accepted node once it is selected (FIN_PENDING before, FIN_FAULTY for a faulty sequence)
-    unsigned int *best;          // [B] smallest post-order rank of a node known to be accepted if reached (all-ones: none)
-    unsigned long long *order;   // [B*N] low word: 0x80000000 | post-order rank << 8 | nodes wholly before the node's
-                                 // subtree; high word: the node's ancestors (itself included) as a bit mask; 0: not computed
-    int prune;                   // Traversal: skip subtrees that lie wholly after a known acceptance
+    ChainRec *chain;             // [B*N] the node's first child and its ratio
     SpecOut out;
 };
 
-// per consumer warp: the children of the current node and the scalar state of its recursion
 struct __align__(16) WarpList {
     double ep[MW], eq[MW];         // exact 2^(z s - O) of the token in the target / draft row (0: cut, or no draft row)
-    int pos[MW];                   // (slot << 8) | (lane << 3) | position in the chunk; slot as in bonus_search
+    int pos[MW];                   // (chunk of the thread << 8) | (lane << 3) | position in the chunk
 };
 
-// the e of the RT register tiles of a thread
-struct Resident {
-    float p[RT][8], q[RT][8];
+// the e of the RC register chunks of a thread
+template <int RC> struct Resident {
+    float p[RC > 0 ? RC : 1][8], q[RC > 0 ? RC : 1][8];
 };
 
-struct __align__(16) WarpArea {
-    double cpm[KMAX], cqm[KMAX];   // exact 2^(z s - O) of the children's tokens in the node's target and draft rows
-    float cu[KMAX];
-    int child[KMAX];
-    double c, E, G;                // committed state (see the file header); identical in every warp of the cluster
-    double A, w_in, invZp, invZq;  // A = w_in / Z_p
-    double Rg;                     // pass coefficient g = (c + G) Rg, Rg = Z_p / (w_in Z_q)
-    double g_commit;               // coefficient of the pass the committed state came from (0: none)
-    double Z_p, Z_q;
-    int O_p, O_q;
-};
-
-struct __align__(16) Hdr {
-    uint64_t full[NSMAX], empty[NSMAX], xbar[2], cbar;
-    double wtile[NWMAX + 1][TMAX];
-    WarpArea wa[NWMAX];
+// shared memory of the consumer warps' common work
+struct __align__(16) Common {
+    uint64_t xbar[2], cbar;
+    double part[2][NVMAX][NWMAX];  // the warps' partial sums, by parity of the sum
+    double xsum[2][NVMAX][CMAX];   // the CTAs' sums
+    double wtile[NWMAX + 1][CHMAX];
+    WarpList list[NWMAX];
     int poison;
 };
+// a consumer warp's view of it
+struct Team {
+    Common &M;
+    int C, warp, lane, n;          // n: sums so far
+    unsigned rank;
+    uint32_t cph;                  // phase of the consumers' barrier
+};
+__device__ __forceinline__ void common_init(Common &M, int nw)
+{
+    mbar_init(&M.xbar[0], 1);
+    mbar_init(&M.xbar[1], 1);
+    mbar_init(&M.cbar, nw);
+    M.poison = 0;
+}
 
 // ------------------------------------------------------------------------------------------------
 // small helpers
 // ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ bool warp_has_children(const int *parent, int N, int a, int lane)
+// the CTA's chunks of a node's two rows
+struct Slice {
+    const unsigned char *p, *q;    // 16-byte boundaries at which chunk 0 of the rows starts
+    int u0, nu;                    // first chunk and number of chunks of this CTA
+    int h, V;                      // chunk u holds the row's logits 8 u - h .. 8 u - h + 7
+    bool vec;                      // both rows start at the same offset from a 16-byte boundary
+};
+template <int DT>
+__device__ __forceinline__ Slice make_slice(const void *zp, const void *zq, long long first, int V, int C, unsigned rank)
 {
-    for (int c0 = a + 1; c0 < N; c0 += 32) {
-        int c = c0 + lane;
-        bool is = c < N && __ldg(parent + c) == a;
-        if (__any_sync(0xffffffffu, is)) return true;
-    }
-    return false;
+    constexpr int ESZ = DT == SPEC_BF16 ? 2 : 4;
+    const uintptr_t ap = (uintptr_t)zp + (uintptr_t)(first * ESZ), aq = (uintptr_t)zq + (uintptr_t)(first * ESZ);
+    Slice s;
+    s.vec = ((ap ^ aq) & 15) == 0 && (ap & (ESZ - 1)) == 0;
+    const int off = s.vec ? (int)(ap & 15) : 0;
+    s.h = off / ESZ;
+    s.p = (const unsigned char *)(ap - off);
+    s.q = (const unsigned char *)(aq - off);
+    s.V = V;
+    const int units = (s.h + V + 7) >> 3, per = (units + C - 1) / C;
+    s.u0 = (int)rank * per;
+    s.nu = max(0, min(per, units - s.u0));
+    return s;
 }
-
-// the 8 logits a thread owns in one tile of one row, as they sit in the ring
+// the 8 logits of a chunk as they sit in memory
 template <int DT>
 struct RawChunk {
     uint4 a, b;      // bf16: a only
 };
+// chunk u of one row; what lies outside the row may be anything (mask_chunk).  Rows at different offsets from a 16-byte
+// boundary (two tensors of their own odd alignment) are read logit by logit, out of line.
 template <int DT>
-__device__ __forceinline__ RawChunk<DT> read_raw(const unsigned char *sp)
+__device__ __noinline__ RawChunk<DT> load_raw_scalar(const unsigned char *row, int u, int V)
 {
     RawChunk<DT> r;
-    r.a = *reinterpret_cast<const uint4 *>(sp);
-    if (DT == SPEC_F32) r.b = reinterpret_cast<const uint4 *>(sp)[1];
+    uint32_t w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int t = min(u * 8 + k, V - 1);
+        w[k] = DT == SPEC_BF16 ? (uint32_t)__ldg((const unsigned short *)row + t) : __ldg((const uint32_t *)row + t);
+    }
+    if (DT == SPEC_BF16) r.a = make_uint4(w[0] | w[1] << 16, w[2] | w[3] << 16, w[4] | w[5] << 16, w[6] | w[7] << 16);
+    else { r.a = make_uint4(w[0], w[1], w[2], w[3]); r.b = make_uint4(w[4], w[5], w[6], w[7]); }
+    return r;
+}
+template <int DT>
+__device__ __forceinline__ RawChunk<DT> load_raw(const unsigned char *row, int u, const Slice &s)
+{
+    RawChunk<DT> r;
+    const uint4 *src = reinterpret_cast<const uint4 *>(row) + (size_t)u * (DT == SPEC_BF16 ? 1 : 2);
+    r.a = __ldg(src);
+    if (DT == SPEC_F32) r.b = u * 8 - s.h + 4 < s.V ? __ldg(src + 1) : r.a;
     return r;
 }
 template <int DT>
@@ -162,13 +201,13 @@ __device__ __forceinline__ void unpack_chunk(const RawChunk<DT> &r, float (&z)[8
         z[4] = __uint_as_float(r.b.x); z[5] = __uint_as_float(r.b.y); z[6] = __uint_as_float(r.b.z); z[7] = __uint_as_float(r.b.w);
     }
 }
-// logits beyond the slice (nvalid < 8) or below the row's cut become -inf
-__device__ __forceinline__ void mask_chunk(float (&z)[8], int nvalid, bool has_cut, float cut)
+// logits outside the row (positions of the chunk outside lo .. hi - 1) or below the row's cut become -inf
+__device__ __forceinline__ void mask_chunk(float (&z)[8], int lo, int hi, bool has_cut, float cut)
 {
-    if (nvalid < 8) {
+    if (lo > 0 || hi < 8) {
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-            if (k >= nvalid) z[k] = -CUDART_INF_F;
+            if (k < lo || k >= hi) z[k] = -CUDART_INF_F;
     }
     if (has_cut) {
 #pragma unroll
@@ -248,7 +287,7 @@ __device__ __forceinline__ double exp2_exact(float z, double s_d, int O)
 }
 
 // ------------------------------------------------------------------------------------------------
-// pass 1: a node's rows from the ring into resident e, its dominant tokens into the warp's exact list
+// pass 1: a node's rows into resident e, its dominant tokens into the warp's exact list
 // ------------------------------------------------------------------------------------------------
 // what pass 1 has to know about the two rows of a node
 struct NodeRows {
@@ -278,73 +317,67 @@ __device__ __forceinline__ void set_list_thresholds(NodeRows &nr, double Z_p, do
     nr.thrA_q = nr.hq ? (float)(Z_q * a) : CUDART_INF_F;
     nr.thrB_q = nr.hq ? (flat ? nr.thrA_q : (float)(Z_q * b)) : CUDART_INF_F;
 }
-struct RingCtx {
-    uint64_t *full, *empty;
-    unsigned char *ring;
-    int NS;
-    int *poison;
-};
-
-// the e of the 8 tokens a thread owns in one tile, both rows (passed by value to list_append)
+// the e of the 8 tokens a thread owns in one chunk, both rows (passed by value to list_append)
 struct Chunk16 {
     float p[8], q[8];
 };
 
-// Warp-collective, and out of line on purpose (it runs on a few per cent of the tiles, and the kernels
+// logit k of a chunk
+template <int DT>
+__device__ __forceinline__ float raw_logit(const RawChunk<DT> &r, int k)
+{
+    const int j = DT == SPEC_BF16 ? k >> 1 : k & 3;
+    const uint32_t x = (DT == SPEC_F32 && k >= 4) ? r.b.x : r.a.x, y = (DT == SPEC_F32 && k >= 4) ? r.b.y : r.a.y;
+    const uint32_t z = (DT == SPEC_F32 && k >= 4) ? r.b.z : r.a.z, w = (DT == SPEC_F32 && k >= 4) ? r.b.w : r.a.w;
+    const uint32_t v = j & 2 ? (j & 1 ? w : z) : (j & 1 ? y : x);
+    return DT == SPEC_BF16 ? ((k & 1) ? bf16_hi(v) : bf16_lo(v)) : __uint_as_float(v);
+}
+
+// Warp-collective, and out of line on purpose (it runs on a few per cent of the chunks, and the kernels
 // are short of instruction cache): the tokens of the lane's chunk whose e exceeds the always-listed
 // threshold (thrA), or the while-there-is-room threshold (tp, tq), are appended to the warp's list while
-// it has room, as raw logits (pass1 evaluates the exponentials in fp64 once all tiles are in).  n is the
-// list's fill, the same in every lane.  Returns (new fill << 8) | the lane's mask of appended tokens
-// (the caller zeroes their fp32 copies).
+// it has room, as raw logits (pass1 evaluates the exponentials in fp64 once all chunks are in).  Places are dealt by
+// one scan over the lanes (position by position, with its ballots, it was the longest part of pass 1: 4 of 8.7
+// thousand cycles at V = 1000).  n is the list's fill, the same in every lane.  Returns (new fill << 8) | the lane's
+// mask of appended tokens (the caller zeroes their fp32 copies).
 template <int DT>
 __device__ __noinline__ unsigned list_append(WarpList &L, int n, const RawChunk<DT> raw_p, const RawChunk<DT> raw_q,
-                                             const Chunk16 e, float thrA_p, float thrA_q, float tp, float tq, int nvalid,
+                                             const Chunk16 e, float thrA_p, float thrA_q, float tp, float tq, int lo, int hi,
                                              float cut_p, float cut_q, bool hq, int slot)
 {
     const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    unsigned m_any = 0, m_a = 0;
+    unsigned m_a = 0, m_b = 0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        const bool a = e.p[k] > thrA_p || e.q[k] > thrA_q;
-        const bool any = a || e.p[k] > tp || e.q[k] > tq;
-        m_any |= (any ? 1u : 0u) << k;
-        m_a |= (a ? 1u : 0u) << k;
+        if (e.p[k] > thrA_p || e.q[k] > thrA_q) m_a |= 1u << k;
+        if (e.p[k] > tp || e.q[k] > tq) m_b |= 1u << k;
     }
-    float zp[8], zq[8];
-    unpack_chunk<DT>(raw_p, zp);
-    unpack_chunk<DT>(raw_q, zq);
-    unsigned adm = 0;
-#pragma unroll 1
-    for (int k = 0; k < 8; ++k) {
-        if (n >= MW - MW_RES) m_any &= m_a;           // no room left in the second tier
-        if (!__any_sync(0xffffffffu, (m_any >> k) != 0u)) break;
-        const bool a = (m_a >> k) & 1u, b = ((m_any >> k) & 1u) && !a;
-        const unsigned balA = __ballot_sync(0xffffffffu, a), balB = __ballot_sync(0xffffffffu, b);
-        if (!(balA | balB)) continue;
-        const int nA = min(n + __popc(balA), MW);
-        const int capB = MW - MW_RES;
-        const int nB = max(nA, min(nA + __popc(balB), capB));
-        int idx = -1;
-        if (a) { const int i = n + __popc(balA & lt); if (i < MW) idx = i; }
-        else if (b) { const int i = nA + __popc(balB & lt); if (i < capB) idx = i; }
-        n = nB;
-        if (idx >= 0) {
-            float z0 = zp[0], z1 = zq[0];
+    m_b &= ~m_a;
+    const unsigned mine = (unsigned)__popc(m_a) | (unsigned)__popc(m_b) << 16;
+    unsigned incl = mine;
 #pragma unroll
-            for (int kk = 1; kk < 8; ++kk)
-                if (kk == k) { z0 = zp[kk]; z1 = zq[kk]; }
-            // the raw logits for now (-inf: cut, or no draft row); pass1 turns every entry into its
-            // exponential at the end, all lanes at once, instead of one long fp64 chain per admission
-            const bool valid = k < nvalid;
-            L.ep[idx] = (valid && z0 >= cut_p) ? (double)z0 : -CUDART_INF;
-            L.eq[idx] = (valid && hq && z1 >= cut_q) ? (double)z1 : -CUDART_INF;
-            L.pos[idx] = (slot << 8) | (lane << 3) | k;
-            adm |= 1u << k;
-        }
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const unsigned tot = __shfl_sync(0xffffffffu, incl, 31), before = incl - mine;
+    const int capB = MW - MW_RES, nA = min(n + (int)(tot & 0xFFFFu), MW);
+    int iA = n + (int)(before & 0xFFFFu), iB = nA + (int)(before >> 16);
+    unsigned adm = 0;
+    for (unsigned m = m_a | m_b; m; m &= m - 1u) {
+        const int k = __ffs(m) - 1;
+        const bool a = (m_a >> k) & 1u;
+        const int idx = a ? iA++ : iB++;
+        if (idx >= (a ? MW : capB)) continue;
+        const float z0 = raw_logit<DT>(raw_p, k), z1 = raw_logit<DT>(raw_q, k);
+        const bool valid = k >= lo && k < hi;
+        L.ep[idx] = (valid && z0 >= cut_p) ? (double)z0 : -CUDART_INF;      // (-inf: cut, or no draft row)
+        L.eq[idx] = (valid && hq && z1 >= cut_q) ? (double)z1 : -CUDART_INF;
+        L.pos[idx] = (slot << 8) | (lane << 3) | k;
+        adm |= 1u << k;
     }
     __syncwarp();
-    return ((unsigned)n << 8) | adm;
+    return (unsigned)max(nA, min(nA + (int)(tot >> 16), capB)) << 8 | adm;
 }
 
 // cross sums of the two rows for the Kullback-Leibler divergences (analysis instantiation only):
@@ -354,40 +387,43 @@ struct KlSums {
     float pp, pq, qp, qq;
 };
 
-// One tile: wait for the stage, take the thread's 8 logits of both rows, hand the stage back, turn them
-// into e (EP, EQ), move dominant tokens to the list.  The thread's tail sums of e go to zs_p / zs_q.
-template <int DT, int NW, bool KLS = false>
-__device__ __forceinline__ void pass1_tile(const RingCtx &rc, int &stage, uint32_t &phase, bool &poisoned,
-                                           const NodeRows &nr, int tile_index, int slot, int n_slice, int tid,
-                                           float (&EP)[8], float (&EQ)[8], WarpList &L, int &nl, float &zs_p, float &zs_q,
-                                           KlSums *kl = nullptr)
+// chunk i of the CTA in both rows (zeros beyond the CTA's chunks)
+template <int DT>
+__device__ __forceinline__ void fetch_pair(const Slice &sl, bool hq, int i, RawChunk<DT> &p, RawChunk<DT> &q)
 {
-    constexpr int NCONS = NW * 32;
-    constexpr int TILE = NCONS * 8;
-    constexpr int ESZ = DT == SPEC_BF16 ? 2 : 4;
-    constexpr int ROWB = TILE * ESZ;
-    constexpr int STAGE = 2 * ROWB;
-    if (!poisoned && !mbar_wait(&rc.full[stage], phase)) { *rc.poison = 1; poisoned = true; }
-    const unsigned char *sp = rc.ring + (size_t)stage * STAGE + (size_t)tid * 8 * ESZ;
-    const RawChunk<DT> raw_p = read_raw<DT>(sp);
-    RawChunk<DT> raw_q = raw_p;
-    if (nr.hq) raw_q = read_raw<DT>(sp + ROWB);
-    __syncwarp();
-    if ((tid & 31) == 0) mbar_arrive(&rc.empty[stage]);
-    if (++stage == rc.NS) { stage = 0; phase ^= 1u; }
-    const int nvalid = poisoned ? 0 : n_slice - (tile_index * TILE + tid * 8);
+    p.a = q.a = make_uint4(0, 0, 0, 0);
+    if (DT == SPEC_F32) p.b = q.b = make_uint4(0, 0, 0, 0);
+    if (i >= sl.nu) return;
+    if (sl.vec) {
+        p = load_raw<DT>(sl.p, sl.u0 + i, sl);
+        if (hq) q = load_raw<DT>(sl.q, sl.u0 + i, sl);
+    } else {
+        p = load_raw_scalar<DT>(sl.p, sl.u0 + i, sl.V);
+        if (hq) q = load_raw_scalar<DT>(sl.q, sl.u0 + i, sl.V);
+    }
+}
+
+// One chunk: its 8 logits of both rows into e (EP, EQ), dominant tokens to the list.  The thread's tail sums of e go to
+// zs_p / zs_q.  c: the chunk's index in the thread.
+template <int DT, int NW, bool KLS = false>
+__device__ __forceinline__ void pass1_chunk(const Slice &sl, const NodeRows &nr, const RawChunk<DT> &raw_p, const RawChunk<DT> &raw_q,
+                                            int c, int tid, float (&EP)[8], float (&EQ)[8], WarpList &L, int &nl, float &zs_p,
+                                            float &zs_q, KlSums *kl = nullptr)
+{
+    const int i = c * NW * 32 + tid, t0 = (sl.u0 + i) * 8 - sl.h;
+    const int lo = -t0, hi = i < sl.nu ? sl.V - t0 : 0;          // positions that are the row's
     float z[8], dsx = 0.f;
     float sum_p, sum_q = 0.f;
     if (KLS) {
         // the exponents themselves are needed: scalar form
         float xp[8], xq[8];
         unpack_chunk<DT>(raw_p, z);
-        mask_chunk(z, nvalid, nr.cut_p > -CUDART_INF_F, nr.cut_p);
+        mask_chunk(z, lo, hi, nr.cut_p > -CUDART_INF_F, nr.cut_p);
         sum_p = 0.f;
 #pragma unroll
         for (int k = 0; k < 8; ++k) { xp[k] = fmaf(z[k], nr.s_lo, fmaf(z[k], nr.s_hi, -(float)nr.O_p)); EP[k] = ex2_approx(xp[k]); sum_p += EP[k]; }
         unpack_chunk<DT>(raw_q, z);
-        mask_chunk(z, nvalid, nr.cut_q > -CUDART_INF_F, nr.cut_q);
+        mask_chunk(z, lo, hi, nr.cut_q > -CUDART_INF_F, nr.cut_q);
 #pragma unroll
         for (int k = 0; k < 8; ++k) { xq[k] = fmaf(z[k], nr.s_lo, fmaf(z[k], nr.s_hi, -(float)nr.O_q)); EQ[k] = ex2_approx(xq[k]); sum_q += EQ[k]; }
 #pragma unroll
@@ -397,11 +433,11 @@ __device__ __forceinline__ void pass1_tile(const RingCtx &rc, int &stage, uint32
         }
     } else {
         unpack_chunk<DT>(raw_p, z);
-        mask_chunk(z, nvalid, nr.cut_p > -CUDART_INF_F, nr.cut_p);
+        mask_chunk(z, lo, hi, nr.cut_p > -CUDART_INF_F, nr.cut_p);
         sum_p = exp_chunk<false>(z, nr.s_hi, nr.s_lo, (float)nr.O_p, EP, dsx);
         if (nr.hq) {
             unpack_chunk<DT>(raw_q, z);
-            mask_chunk(z, nvalid, nr.cut_q > -CUDART_INF_F, nr.cut_q);
+            mask_chunk(z, lo, hi, nr.cut_q > -CUDART_INF_F, nr.cut_q);
             sum_q = exp_chunk<false>(z, nr.s_hi, nr.s_lo, (float)nr.O_q, EQ, dsx);
         } else {
 #pragma unroll
@@ -415,8 +451,8 @@ __device__ __forceinline__ void pass1_tile(const RingCtx &rc, int &stage, uint32
         Chunk16 e;
 #pragma unroll
         for (int k = 0; k < 8; ++k) { e.p[k] = EP[k]; e.q[k] = EQ[k]; }
-        const unsigned r = list_append<DT>(L, nl, raw_p, raw_q, e, nr.thrA_p, nr.thrA_q, tp, tq, nvalid, nr.cut_p,
-                                           nr.cut_q, nr.hq, slot);
+        const unsigned r = list_append<DT>(L, nl, raw_p, raw_q, e, nr.thrA_p, nr.thrA_q, tp, tq, lo, hi, nr.cut_p,
+                                           nr.cut_q, nr.hq, c);
         nl = (int)(r >> 8);
         const unsigned adm = r & 255u;
         if (adm) {
@@ -432,38 +468,12 @@ __device__ __forceinline__ void pass1_tile(const RingCtx &rc, int &stage, uint32
     zs_q += sum_q;
 }
 
-// Pass 1 of a node.  es: [slot][p lo, p hi, q lo, q hi][NCONS] for the nsm shared-memory tiles; the last
-// nrg tiles of the slice stay in R.  On return nl is the fill of the warp's list and zs_p / zs_q the
-// thread's sums of the fp32 e it keeps (listed tokens excluded).
-template <int DT, int NW, bool KLS = false>
-__device__ __forceinline__ void pass1(const RingCtx &rc, int &stage, uint32_t &phase, bool &poisoned, const NodeRows &nr,
-                                      float4 *es, int nsm, int nrg, int n_slice, int tid, Resident &R, WarpList &L,
-                                      int &nl, float &zs_p, float &zs_q, KlSums *kl = nullptr)
+// the listed tokens' exponentials in fp64, an entry per lane (list_append left the raw logits)
+__device__ __forceinline__ void list_exact(WarpList &L, int nl, const NodeRows &nr)
 {
-    constexpr int NCONS = NW * 32;
-    nl = 0; zs_p = 0.f; zs_q = 0.f;
-    for (int i = 0; i < nsm; ++i) {
-        float ep[8], eq[8];
-        pass1_tile<DT, NW, KLS>(rc, stage, phase, poisoned, nr, i, i, n_slice, tid, ep, eq, L, nl, zs_p, zs_q, kl);
-        float4 *d = es + (size_t)(i * 4) * NCONS + tid;
-        d[0] = make_float4(ep[0], ep[1], ep[2], ep[3]);
-        d[NCONS] = make_float4(ep[4], ep[5], ep[6], ep[7]);
-        d[2 * NCONS] = make_float4(eq[0], eq[1], eq[2], eq[3]);
-        d[3 * NCONS] = make_float4(eq[4], eq[5], eq[6], eq[7]);
-    }
-#pragma unroll
-    for (int j = 0; j < RT; ++j) {
-        if (j < nrg) {
-            pass1_tile<DT, NW, KLS>(rc, stage, phase, poisoned, nr, nsm + j, SMT + j, n_slice, tid, R.p[j], R.q[j], L, nl, zs_p, zs_q, kl);
-        } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) { R.p[j][k] = 0.f; R.q[j][k] = 0.f; }
-        }
-    }
-    // the listed tokens' exponentials in fp64, entry `lane` (list_append left the raw logits)
     __syncwarp();
-    if ((tid & 31) < nl) {
-        const int i = tid & 31;
+    const int i = threadIdx.x & 31;
+    if (i < nl) {
         const double zp = L.ep[i], zq = L.eq[i];
         L.ep[i] = zp > -CUDART_INF ? exp2_exact((float)zp, nr.s_d, nr.O_p) : 0.0;
         L.eq[i] = zq > -CUDART_INF ? exp2_exact((float)zq, nr.s_d, nr.O_q) : 0.0;
@@ -471,15 +481,48 @@ __device__ __forceinline__ void pass1(const RingCtx &rc, int &stage, uint32_t &p
     __syncwarp();
 }
 
-// hand a node's stages back unread (the node turned out not to need its rows)
-__device__ __forceinline__ void drain_tiles(const RingCtx &rc, int &stage, uint32_t &phase, bool &poisoned, int ntiles)
+// Pass 1 of a node.  es: [chunk - RC][p lo, p hi, q lo, q hi][NCONS].  On return nl is the fill of the warp's list and
+// zs_p / zs_q the thread's sums of the fp32 e it keeps (listed tokens excluded).
+template <int DT, int NW, int RC, bool KLS = false>
+__device__ __forceinline__ void pass1(const Slice &sl, const NodeRows &nr, float4 *es, int tid, Resident<RC> &R, WarpList &L,
+                                      int &nl, float &zs_p, float &zs_q, KlSums *kl = nullptr)
 {
-    for (int i = 0; i < ntiles; ++i) {
-        if (!poisoned && !mbar_wait(&rc.full[stage], phase)) { *rc.poison = 1; poisoned = true; }
-        __syncwarp();
-        if ((threadIdx.x & 31) == 0) mbar_arrive(&rc.empty[stage]);
-        if (++stage == rc.NS) { stage = 0; phase ^= 1u; }
+    constexpr int NCONS = NW * 32;
+    nl = 0; zs_p = 0.f; zs_q = 0.f;
+    if (RC > 0) {
+        // every load of the register chunks is issued before the first is used
+        RawChunk<DT> rp[RC > 0 ? RC : 1], rq[RC > 0 ? RC : 1];
+#pragma unroll
+        for (int c = 0; c < RC; ++c) fetch_pair<DT>(sl, nr.hq, c * NCONS + tid, rp[c], rq[c]);
+#pragma unroll
+        for (int c = 0; c < RC; ++c) {
+            if (c * NCONS < sl.nu) {
+                pass1_chunk<DT, NW, KLS>(sl, nr, rp[c], rq[c], c, tid, R.p[c], R.q[c], L, nl, zs_p, zs_q, kl);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) { R.p[c][k] = 0.f; R.q[c][k] = 0.f; }
+            }
+        }
     }
+    // the others, one piece of code for all of them, three chunks' loads ahead
+    RawChunk<DT> ap, aq, bp, bq, cp, cq;
+    fetch_pair<DT>(sl, nr.hq, RC * NCONS + tid, ap, aq);
+    fetch_pair<DT>(sl, nr.hq, (RC + 1) * NCONS + tid, bp, bq);
+    fetch_pair<DT>(sl, nr.hq, (RC + 2) * NCONS + tid, cp, cq);
+#pragma unroll 1
+    for (int c = RC; c * NCONS < sl.nu; ++c) {
+        const RawChunk<DT> xp = ap, xq = aq;
+        ap = bp; aq = bq; bp = cp; bq = cq;
+        fetch_pair<DT>(sl, nr.hq, (c + 3) * NCONS + tid, cp, cq);
+        float ep[8], eq[8];
+        pass1_chunk<DT, NW, KLS>(sl, nr, xp, xq, c, tid, ep, eq, L, nl, zs_p, zs_q, kl);
+        float4 *d = es + (size_t)((c - RC) * 4) * NCONS + tid;
+        d[0] = make_float4(ep[0], ep[1], ep[2], ep[3]);
+        d[NCONS] = make_float4(ep[4], ep[5], ep[6], ep[7]);
+        d[2 * NCONS] = make_float4(eq[0], eq[1], eq[2], eq[3]);
+        d[3 * NCONS] = make_float4(eq[4], eq[5], eq[6], eq[7]);
+    }
+    list_exact(L, nl, nr);
 }
 
 // One step on a chunk: u <- (g u - q)+ for its 8 tokens, g = gh + gl; returns the sum of the new u
@@ -504,27 +547,30 @@ __device__ __forceinline__ float sum_chunk(const float (&u)[8])
     return ((u[0] + u[1]) + (u[2] + u[3])) + ((u[4] + u[5]) + (u[6] + u[7]));
 }
 
-// One sibling step over the thread's share of the resident node, in place: u <- (g u - e_q)+ for its
+// One sibling step over the thread's share of the resident node (nu: the CTA's chunks), in place: u <- (g u - e_q)+ for its
 // fp32 tail tokens and for the entry of the warp's exact list that falls to its lane.  Returns the
 // thread's sum of the new u.
-template <int NW>
-__device__ __forceinline__ double step_sweep(float4 *es, int nsm, int tid, Resident &R, WarpList &L, int nl, double g)
+template <int NW, int RC>
+__device__ __forceinline__ double step_sweep(float4 *es, int nu, int tid, Resident<RC> &R, WarpList &L, int nl, double g)
 {
     constexpr int NCONS = NW * 32;
     float g_hi, g_lo;
     split_float(g, g_hi, g_lo);
     float tot = 0.f;
-    for (int i = 0; i < nsm; ++i) {
+#pragma unroll 1
+    for (int c = RC; c * NCONS < nu; ++c) {
         float u[8], q[8];
-        float4 *d = es + (size_t)(i * 4) * NCONS + tid;
+        float4 *d = es + (size_t)((c - RC) * 4) * NCONS + tid;
         load_e8(d, NCONS, u);
         load_e8(d + 2 * NCONS, NCONS, q);
         tot += step_chunk(u, q, g_hi, g_lo);
         d[0] = make_float4(u[0], u[1], u[2], u[3]);
         d[NCONS] = make_float4(u[4], u[5], u[6], u[7]);
     }
-    tot += (step_chunk(R.p[0], R.q[0], g_hi, g_lo) + step_chunk(R.p[1], R.q[1], g_hi, g_lo)) +
-           (step_chunk(R.p[2], R.q[2], g_hi, g_lo) + step_chunk(R.p[3], R.q[3], g_hi, g_lo));
+    float part[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int c = 0; c < RC; ++c) part[c & 3] += step_chunk(R.p[c], R.q[c], g_hi, g_lo);
+    tot += (part[0] + part[1]) + (part[2] + part[3]);
     double d = (double)tot;
     const int lane = tid & 31;
     if (lane < nl) {
@@ -538,16 +584,17 @@ __device__ __forceinline__ double step_sweep(float4 *es, int nsm, int tid, Resid
 // SpecTr's residual (Algorithm 3) in place, in the units of the resident e_p: u <- (u - gm min(u ir, e_q r))+
 // with ir = 1 / rho, r = Z_p / Z_q, gm = gamma, for the thread's fp32 tail tokens and for the entry of the
 // warp's exact list that falls to its lane.  Returns the thread's sum of the new u.
-template <int NW>
-__device__ __forceinline__ double spectr_sweep(float4 *es, int nsm, int tid, Resident &R, WarpList &L, int nl, double gm,
+template <int NW, int RC>
+__device__ __forceinline__ double spectr_sweep(float4 *es, int nu, int tid, Resident<RC> &R, WarpList &L, int nl, double gm,
                                                double ir, double r)
 {
     constexpr int NCONS = NW * 32;
     const float gf = (float)gm, irf = (float)ir, rf = (float)r;
     float tot = 0.f;
-    for (int i = 0; i < nsm; ++i) {
+#pragma unroll 1
+    for (int c = RC; c * NCONS < nu; ++c) {
         float u[8], q[8];
-        float4 *d = es + (size_t)(i * 4) * NCONS + tid;
+        float4 *d = es + (size_t)((c - RC) * 4) * NCONS + tid;
         load_e8(d, NCONS, u);
         load_e8(d + 2 * NCONS, NCONS, q);
 #pragma unroll
@@ -556,7 +603,7 @@ __device__ __forceinline__ double spectr_sweep(float4 *es, int nsm, int tid, Res
         d[NCONS] = make_float4(u[4], u[5], u[6], u[7]);
     }
 #pragma unroll
-    for (int j = 0; j < RT; ++j) {
+    for (int j = 0; j < RC; ++j) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             R.p[j][k] = fmaxf(R.p[j][k] - gf * fminf(R.p[j][k] * irf, R.q[j][k] * rf), 0.f);
@@ -573,178 +620,224 @@ __device__ __forceinline__ double spectr_sweep(float4 *es, int nsm, int tid, Res
     return d;
 }
 
-// A read-only sweep over the thread's share of the resident node for the offline analysis: f.tail(e_p, e_q,
-// a0, a1) on every fp32 token (two running sums), f.exact(...) in fp64 on the entry of the warp's exact
-// list that falls to the lane.  Listed tokens are zero in the fp32 arrays; every f maps (0, 0) to nothing.
-template <int NW, typename F>
-__device__ __forceinline__ void reduce_sweep(const float4 *es, int nsm, int tid, const Resident &R, const WarpList &L,
-                                             int nl, const F &f, double &o0, double &o1)
+// Sum over the CTA's part of a node of (g e_p - e_q)+ straight from the logits: nothing resident, no exact lists, one loop
+// that stays in the instruction cache.  For nodes that need this one sum only, to fp32 exponentials (tree.cuh).
+template <int DT, int NW>
+__device__ __forceinline__ double residual_sum(const Slice &sl, const NodeRows &nr, double g, int tid)
 {
     constexpr int NCONS = NW * 32;
-    float a0 = 0.f, a1 = 0.f;
-    for (int i = 0; i < nsm; ++i) {
+    float g_hi, g_lo, dsx = 0.f, tot = 0.f;
+    split_float(g, g_hi, g_lo);
+    RawChunk<DT> np = {}, nq = {};
+    auto fetch = [&](int i) {
+        if (i >= sl.nu) return;
+        np = sl.vec ? load_raw<DT>(sl.p, sl.u0 + i, sl) : load_raw_scalar<DT>(sl.p, sl.u0 + i, sl.V);
+        nq = sl.vec ? load_raw<DT>(sl.q, sl.u0 + i, sl) : load_raw_scalar<DT>(sl.q, sl.u0 + i, sl.V);
+    };
+    fetch(tid);
+#pragma unroll 1
+    for (int i = tid; i < sl.nu; i += NCONS) {
+        const RawChunk<DT> rp = np, rq = nq;
+        fetch(i + NCONS);
+        const int t0 = (sl.u0 + i) * 8 - sl.h, lo = -t0, hi = sl.V - t0;
+        float z[8], ep[8], eq[8];
+        unpack_chunk<DT>(rp, z);
+        mask_chunk(z, lo, hi, nr.cut_p > -CUDART_INF_F, nr.cut_p);
+        exp_chunk<false>(z, nr.s_hi, nr.s_lo, (float)nr.O_p, ep, dsx);
+        unpack_chunk<DT>(rq, z);
+        mask_chunk(z, lo, hi, nr.cut_q > -CUDART_INF_F, nr.cut_q);
+        exp_chunk<false>(z, nr.s_hi, nr.s_lo, (float)nr.O_q, eq, dsx);
+        tot += step_chunk(ep, eq, g_hi, g_lo);
+    }
+    return (double)tot;
+}
+
+// A read-only sweep over the thread's share of the resident node: f.tail(e_p, e_q, a) on every fp32 token (f's running
+// sums), f.exact(...) in fp64 on the entry of the warp's exact list that falls to the lane.  Listed tokens are zero
+// in the fp32 arrays; every f maps (0, 0) to nothing.
+template <int NW, int RC, int NO, typename F>
+__device__ __forceinline__ void reduce_sweep(const float4 *es, int nu, int tid, const Resident<RC> &R, const WarpList &L, int nl,
+                                             const F &f, double (&o)[NO])
+{
+    constexpr int NCONS = NW * 32;
+    float a[NO];
+#pragma unroll
+    for (int i = 0; i < NO; ++i) a[i] = 0.f;
+#pragma unroll 1
+    for (int c = RC; c * NCONS < nu; ++c) {
         float p[8], q[8];
-        const float4 *d = es + (size_t)(i * 4) * NCONS + tid;
+        const float4 *d = es + (size_t)((c - RC) * 4) * NCONS + tid;
         load_e8(d, NCONS, p);
         load_e8(d + 2 * NCONS, NCONS, q);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) f.tail(p[k], q[k], a0, a1);
+        for (int k = 0; k < 8; ++k) f.tail(p[k], q[k], a);
     }
 #pragma unroll
-    for (int j = 0; j < RT; ++j) {
+    for (int j = 0; j < RC; ++j) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) f.tail(R.p[j][k], R.q[j][k], a0, a1);
-    }
-    o0 = (double)a0;
-    o1 = (double)a1;
-    if ((tid & 31) < nl) f.exact(L.ep[tid & 31], L.eq[tid & 31], o0, o1);
-}
-
-// All-to-all of NV doubles per consumer warp of the cluster: tot[i] is the sum over every warp of every
-// CTA (bit-identical in all of them: one fixed order), mine[i] in lane r < C the sum over CTA r's warps.
-// xchg: [parity 2][rank C][warp NW][2] doubles in every CTA's shared memory, xbar: two mbarriers.
-template <int NW, int NV>
-__device__ __forceinline__ void cluster_exchange(double *xchg, uint64_t *xbar, int &xn, int C, unsigned rank, int warp,
-                                                 int lane, int *poison, const double (&v)[NV], double (&tot)[NV],
-                                                 double (&mine)[NV])
-{
-    static_assert(NV <= 2, "two doubles per warp and exchange at most");
-    const int par = xn & 1;
-    if (warp == 0 && lane == 0) mbar_arrive_expect_tx(&xbar[par], (uint32_t)(C * NW * 8 * NV));
-    if (lane < C) {
-#pragma unroll
-        for (int i = 0; i < NV; ++i)
-            st_async_f64(xchg + ((size_t)(par * C + rank) * NW + warp) * 2 + i, &xbar[par], (uint32_t)lane, v[i]);
-    }
-    if (!*(volatile int *)poison && !mbar_wait_cluster(&xbar[par], (uint32_t)((xn >> 1) & 1))) *poison = 1;
-    ++xn;
-#pragma unroll
-    for (int i = 0; i < NV; ++i) mine[i] = 0.0;
-    if (lane < C) {
-        const double *src = xchg + (size_t)(par * C + lane) * NW * 2;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-#pragma unroll
-            for (int i = 0; i < NV; ++i) mine[i] += src[w * 2 + i];
-        }
+        for (int k = 0; k < 8; ++k) f.tail(R.p[j][k], R.q[j][k], a);
     }
 #pragma unroll
-    for (int i = 0; i < NV; ++i) tot[i] = warp_sum_once(mine[i]);
+    for (int i = 0; i < NO; ++i) o[i] = (double)a[i];
+    if ((tid & 31) < nl) f.exact(L.ep[tid & 31], L.eq[tid & 31], o);
 }
 
 // barrier of the consumer warps of a CTA on an mbarrier (one arrival per warp), with a bounded wait
-__device__ __forceinline__ void consumer_sync(uint64_t *bar, uint32_t &ph, int *poison)
+__device__ __forceinline__ void consumer_sync(Team &T)
 {
     __syncwarp();
-    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
-    if (!*(volatile int *)poison && !mbar_wait(bar, ph)) *poison = 1;
-    ph ^= 1u;
+    if (T.lane == 0) mbar_arrive(&T.M.cbar);
+    if (!*(volatile int *)&T.M.poison && !mbar_wait(&T.M.cbar, T.cph)) T.M.poison = 1;
+    T.cph ^= 1u;
+}
+
+// Sums of NV doubles per consumer thread over the cluster: tot[i] over everything (bit-identical in all warps of all
+// CTAs: one fixed order), mine[i] in lane r < C the sum over CTA r.
+template <int NW, int NV>
+__device__ __forceinline__ void cluster_sum(Team &T, const double (&v)[NV], double (&tot)[NV], double (&mine)[NV])
+{
+    static_assert(NV <= NVMAX, "room for the partial sums");
+    Common &M = T.M;
+    const int par = T.n & 1;
+    double s[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) s[i] = v[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) s[i] += __shfl_xor_sync(0xffffffffu, s[i], o);
+    }
+    if (T.lane < NV) {
+        double x = s[0];
+#pragma unroll
+        for (int i = 1; i < NV; ++i) x = T.lane == i ? s[i] : x;
+        M.part[par][T.lane][T.warp] = x;
+    }
+    if (T.C > 1 && T.warp == 0 && T.lane == 0) mbar_arrive_expect_tx(&M.xbar[par], (uint32_t)(T.C * 8 * NV));
+    consumer_sync(T);
+    if (T.C == 1 || T.warp == 0) {
+        // every lane adds up all partial sums by itself: broadcast reads and a tree of additions, no shuffles
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            double x[8];
+#pragma unroll
+            for (int w = 0; w < 8; ++w) x[w] = w < NW ? M.part[par][i][w] : 0.0;
+#pragma unroll
+            for (int h = 4; h > 0; h >>= 1) {
+#pragma unroll
+                for (int w = 0; w < h; ++w) x[w] += x[w + h];
+            }
+            tot[i] = x[0];
+            mine[i] = T.lane == 0 ? x[0] : 0.0;
+            if (T.C > 1 && T.lane < T.C) st_async_f64(&M.xsum[par][i][T.rank], &M.xbar[par], (uint32_t)T.lane, x[0]);
+        }
+    }
+    if (T.C > 1) {
+        if (!*(volatile int *)&M.poison && !mbar_wait_cluster(&M.xbar[par], (uint32_t)((T.n >> 1) & 1))) M.poison = 1;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            double x[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) x[r] = r < T.C ? M.xsum[par][i][r] : 0.0;
+            if (T.C > 8) {
+#pragma unroll
+                for (int r = 0; r < 8; ++r) x[r] += M.xsum[par][i][r + 8];
+            }
+            tot[i] = ((x[0] + x[4]) + (x[2] + x[6])) + ((x[1] + x[5]) + (x[3] + x[7]));
+            mine[i] = T.lane < T.C ? M.xsum[par][i][T.lane] : 0.0;
+        }
+    }
+    ++T.n;
 }
 
 // Inverse-CDF search over one CTA's share of the node's current state u (from_q: of the draft row e_q
 // instead, for a state that equals q), run by all consumer warps of the CTA that owns the target
-// (tau_rel, in units of e).  Token order is (tile, warp, lane, position
-// in the chunk): the tile, then the warp inside the tile, then the lane, then the token.  The per-tile
-// totals of a warp are reduced together, so that the shuffles of the ten tiles overlap; warp 0 alone
-// picks tile and warp.  Listed tokens enter with their exact values.
-// role: 1 = this thread found the token (index inside the slice in `token`, distance to the nearer
-// CDF edge in `edge`, both in units of e); 2 = this thread reports that no token carries weight;
-// 3 = this thread reports that a bounded wait ran out; 0 = nothing to do.  wtile is [NW + 1][TMAX] in shared memory; cbar / cph: the consumers' barrier.
+// (tau_rel, in units of e).  Token order is (chunk of the thread, warp, lane, position in the chunk): that is also how
+// the search descends.  The per-chunk totals of a warp are reduced together, so that their shuffles overlap.  Listed
+// tokens enter with their exact values.
+// role: 1 = this thread found the token (index in the row in `token`, distance to the nearer
+// CDF edge in `edge`, in units of e); 2 = this thread reports that no token carries weight;
+// 3 = this thread reports that a bounded wait ran out; 0 = nothing to do. 
 struct BonusFind {
     int role, token;
     double edge;
 };
-template <int NW>
-__device__ __forceinline__ BonusFind bonus_search(double (*wtile)[TMAX], uint64_t *cbar, uint32_t &cph, int *poison,
-                                                  const float4 *es, int nsm, int tid, const Resident &R,
+template <int NW, int RC>
+__device__ __forceinline__ BonusFind bonus_search(Team &T, const Slice &sl, const float4 *es, int tid, const Resident<RC> &R,
                                                   const WarpList &L, int nl, bool from_q, double tau_rel)
 {
     constexpr int NCONS = NW * 32;
-    constexpr int TILE = NCONS * 8;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = T.warp, lane = T.lane;
+    double (*wtile)[CHMAX] = T.M.wtile;
     const int qoff = from_q ? 2 * NCONS : 0;
     BonusFind out = {0, -1, 0.0};
-    // slot s < SMT: shared-memory tile s (empty beyond nsm); slot SMT + j: register tile j
-    float r[TMAX];
+    // the warp's total of every chunk: fp32 sums of 8 in a lane, its listed tokens exactly, fp64 across lanes
+    const double lr = lane < nl ? (from_q ? L.eq[lane] : L.ep[lane]) : 0.0;
+    const int lpos = lane < nl ? L.pos[lane] : -1;
+    double r[RC > 0 ? RC : 1], mine = 0.0;
 #pragma unroll
-    for (int i = 0; i < SMT; ++i) {
-        r[i] = 0.f;
-        if (i < nsm) {
-            float p[8];
-            load_e8(es + (size_t)(i * 4) * NCONS + tid + qoff, NCONS, p);
-            r[i] = sum_chunk(p);
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < RT; ++j) r[SMT + j] = from_q ? sum_chunk(R.q[j]) : sum_chunk(R.p[j]);
-    // a warp's total of one tile: 256 tokens, summed in fp32 like the chunks themselves; every level
-    // above works in fp64 on these stored values, so the levels agree with each other exactly
+    for (int c = 0; c < RC; ++c) r[c] = (double)(from_q ? sum_chunk(R.q[c]) : sum_chunk(R.p[c])) + ((lpos >> 8) == c ? lr : 0.0);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-        for (int i = 0; i < TMAX; ++i) r[i] += __shfl_xor_sync(0xffffffffu, r[i], o);
+        for (int c = 0; c < RC; ++c) r[c] += __shfl_xor_sync(0xffffffffu, r[c], o);
     }
-    // the warp's listed tokens, exactly: entry `lane`
-    const double lr = lane < nl ? (from_q ? L.eq[lane] : L.ep[lane]) : 0.0;
-    const int lpos = lane < nl ? L.pos[lane] : -1;
-    double mine = 0.0;
 #pragma unroll
-    for (int i = 0; i < TMAX; ++i)
-        if (lane == i) mine = (double)r[i];
-    if (nl > 0) {
+    for (int c = 0; c < RC; ++c)
+        if (lane == c) mine = r[c];
 #pragma unroll 1
-        for (int i = 0; i < TMAX; ++i) {
-            const double add = warp_sum_once((lpos >= 0 && (lpos >> 8) == i) ? lr : 0.0);
-            if (lane == i) mine += add;
-        }
+    for (int c = RC; c * NCONS < sl.nu; ++c) {
+        float p[8];
+        load_e8(es + (size_t)((c - RC) * 4) * NCONS + tid + qoff, NCONS, p);
+        const double x = warp_sum_once((double)sum_chunk(p) + ((lpos >> 8) == c ? lr : 0.0));
+        if (lane == c) mine = x;
     }
-    if (lane < TMAX) wtile[warp][lane] = mine;
-    consumer_sync(cbar, cph, poison);
-    // warp 0 picks the tile and the warp inside it; the others wait for its answer in row NW
-    if (warp == 0) {
-        double Ti = 0.0;
-        if (lane < TMAX)
-            for (int w = 0; w < NW; ++w) Ti += wtile[w][lane];
-        double tau2, tau3;
-        const int s_pick = pick_lane(Ti, tau_rel, tau2);
-        const double Ww = (s_pick >= 0 && lane < NW) ? wtile[lane][s_pick] : 0.0;
-        const int w_pick = s_pick >= 0 ? pick_lane(Ww, tau2, tau3) : -1;
-        if (lane == 0) { wtile[NW][0] = (double)s_pick; wtile[NW][1] = (double)w_pick; wtile[NW][2] = tau3; }
-    }
-    consumer_sync(cbar, cph, poison);
-    if (*(volatile int *)poison) {
+    if (lane < CHMAX) wtile[warp][lane] = mine;
+    consumer_sync(T);
+    // every warp picks the chunk and the warp inside it for itself; the one that is picked goes on
+    if (*(volatile int *)&T.M.poison) {
         if (tid == 0) out.role = 3;
         return out;
     }
-    const int s_star = (int)wtile[NW][0], w_star = (int)wtile[NW][1];
-    const double tau3 = wtile[NW][2];
-    double tau4;
+    double Ti = 0.0;
+    if (lane < CHMAX) {
+        double x[NW];
+#pragma unroll
+        for (int w = 0; w < NW; ++w) x[w] = wtile[w][lane];
+#pragma unroll
+        for (int w = 1; w < NW; ++w) x[0] += x[w];
+        Ti = x[0];
+    }
+    double tau2, tau3 = 0.0, tau4;
+    const int s_star = pick_lane(Ti, tau_rel, tau2);
+    const int w_star = s_star >= 0 ? pick_lane(lane < NW ? wtile[lane][s_star] : 0.0, tau2, tau3) : -1;
     if (w_star < 0) {
         if (tid == 0) out.role = 2;
         return out;
     }
     if (warp != w_star) return out;
     float p[8];
-    if (s_star < SMT) {
-        load_e8(es + (size_t)(s_star * 4) * NCONS + tid + qoff, NCONS, p);
+    if (s_star >= RC) {
+        load_e8(es + (size_t)((s_star - RC) * 4) * NCONS + tid + qoff, NCONS, p);
     } else {
-        const int jr = s_star - SMT;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float pv = jr == 0 ? R.p[0][k] : (jr == 1 ? R.p[1][k] : (jr == 2 ? R.p[2][k] : R.p[3][k]));
-            const float qv = jr == 0 ? R.q[0][k] : (jr == 1 ? R.q[1][k] : (jr == 2 ? R.q[2][k] : R.q[3][k]));
-            p[k] = from_q ? qv : pv;
-        }
+        for (int k = 0; k < 8; ++k) p[k] = 0.f;
+#pragma unroll
+        for (int c = 0; c < RC; ++c)
+            if (c == s_star) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) p[k] = from_q ? R.q[c][k] : R.p[c][k];
+            }
     }
     double wk[8], v = 0.0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) wk[k] = (double)p[k];
-    // the listed tokens of this tile: each goes to the lane and position it was taken from
-#pragma unroll 1
-    for (int i = 0; i < nl; ++i) {
+    // the listed tokens of this chunk: each goes to the lane and position it was taken from
+    for (unsigned m = __ballot_sync(0xffffffffu, lpos >= 0 && (lpos >> 8) == s_star); m; m &= m - 1u) {
+        const int i = __ffs(m) - 1;
         const int ps = __shfl_sync(0xffffffffu, lpos, i);
         const double rv = __shfl_sync(0xffffffffu, lr, i);
-        if ((ps >> 8) == s_star && ((ps >> 3) & 31) == lane) {
+        if (((ps >> 3) & 31) == lane) {
 #pragma unroll
             for (int k = 0; k < 8; ++k)
                 if ((ps & 7) == k) wk[k] = rv;
@@ -768,9 +861,8 @@ __device__ __forceinline__ BonusFind bonus_search(double (*wtile)[TMAX], uint64_
             if (found < 0 && run > tau4) { found = k; dlo = tau4 - before; dhi = run - tau4; }
         }
         if (found < 0) { found = last_pos; dlo = 0.0; dhi = 0.0; }
-        const int tile = s_star < SMT ? s_star : nsm + (s_star - SMT);
         out.role = found >= 0 ? 1 : 2;
-        out.token = found >= 0 ? tile * TILE + tid * 8 + found : -1;
+        out.token = found >= 0 ? (sl.u0 + s_star * NCONS + tid) * 8 - sl.h + found : -1;
         out.edge = fmin(dlo, dhi);
     }
     return out;
