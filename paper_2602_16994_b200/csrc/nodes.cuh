@@ -169,53 +169,109 @@ __device__ __noinline__ void leaf_record(const VParams &P, const RowPart *part, 
 // ------------------------------------------------------------------------------------------------
 // nodes with one child
 // ------------------------------------------------------------------------------------------------
-// The sums of one node again, for a weight that needs more than fp32: tokens above 2^-DOM_S of a row's mass (at most 1024 per
-// row, about 120 on the synthetic logits) in fp64, the others in fp32, whose share of the error is then below 1e-8 of the mass.
-// A lower threshold makes this a pass in fp64 (2^-20: 23000 tokens of 128256, the call twice as long); the recursion's
-// lists instead cost a first pass of a branching node each time (traversal, batch 8: 212 instead of 92 us).
+// Sums over the CTA's share of a node's two rows, which come through a ring in shared memory: every thread copies and reads
+// its own chunks, NS - 1 of them ahead (one chunk ahead in registers, a pass of one CTA over V = 128256 took 33 us, nearly all of
+// it the latency of L2).
+// HEAVY: tokens above 2^-DOM_S of a row's mass (at most 1024 per row, about 120 on the synthetic logits) in fp64, the
+// others in fp32, whose share of the error is then below 1e-8 of the mass.  They are collected per warp and evaluated 32
+// at a time.
 // g < 0: the rows' normalisers (o[0], o[1]); otherwise o[0] = sum (g e_p - e_q)+.
 constexpr int DOM_S = 10;
-template <int DT, int NW>
-__device__ __noinline__ void careful_sums(const Slice sl, const NodeRows nr, double g, int tid, double (&o)[2])
+template <int DT> constexpr int NS = DT == SPEC_BF16 ? 4 : 3;                                  // stages of the ring
+template <int DT> constexpr int SUMS_RING = NS<DT> * (DT == SPEC_BF16 ? 2 : 4) * 256 * 16;     // bytes of it
+// (out of line: its registers would be spilled around every chunk of the loop below)
+__device__ __noinline__ double2 heavy_terms(float2 z, float cut_p, float cut_q, int O_p, int O_q, double s_d, double g)
 {
-    constexpr int NCONS = NW * 32;
+    const double xp = z.x >= cut_p ? exp2_exact(z.x, s_d, O_p) : 0.0, xq = z.y >= cut_q ? exp2_exact(z.y, s_d, O_q) : 0.0;
+    return g < 0.0 ? make_double2(xp, xq) : make_double2(fmax(fma(g, xp, -xq), 0.0), 0.0);
+}
+template <int DT, bool HEAVY>
+__device__ __noinline__ void node_sums(const Slice &sl, const NodeRows &nr, double g, uint4 *ring, float2 *heavy, double (&o)[2])
+{
+    constexpr int NT = 256, U = DT == SPEC_BF16 ? 1 : 2;         // threads, 16-byte units of a chunk
+    const int tid = threadIdx.x, lane = tid & 31, nu = sl.nu, V = sl.V;
+    const bool vec = sl.vec, norm = HEAVY && g < 0.0;
+    const float s_hi = nr.s_hi, s_lo = nr.s_lo, O_p = (float)nr.O_p, O_q = (float)nr.O_q, cut_p = nr.cut_p, cut_q = nr.cut_q;
+    const float thr_p = nr.thrB_p, thr_q = nr.thrB_q;
     float g_hi, g_lo, dsx = 0.f, ap = 0.f, aq = 0.f;
     split_float(g, g_hi, g_lo);
-    o[0] = o[1] = 0.0;
-    RawChunk<DT> np, nq;
-    fetch_pair<DT>(sl, true, tid, np, nq);
+    double o0 = 0.0, o1 = 0.0;
+    int n = 0;                             // entries of the warp's list (below 32 between chunks)
+    ring += tid;
+    auto issue = [&](int c) {
+        const int i = c * NT + tid;
+        if (vec && i < nu) {
+            const size_t u = (size_t)(sl.u0 + i) * U;
+            const uint4 *p = reinterpret_cast<const uint4 *>(sl.p) + u, *q = reinterpret_cast<const uint4 *>(sl.q) + u;
+            const uint32_t dst = smem_u32(ring + (c % NS<DT>) * 2 * U * NT);
+            stream::cp_async16(dst, p, 16);
+            stream::cp_async16(dst + U * NT * 16, q, 16);
+            if (U == 2 && (sl.u0 + i) * 8 - sl.h + 4 < V) {
+                stream::cp_async16(dst + NT * 16, p + 1, 16);
+                stream::cp_async16(dst + 3 * NT * 16, q + 1, 16);
+            }
+        }
+        stream::cp_async_commit();
+    };
 #pragma unroll 1
-    for (int i = tid; i < sl.nu; i += NCONS) {
-        const RawChunk<DT> rp = np, rq = nq;
-        fetch_pair<DT>(sl, true, i + NCONS, np, nq);
-        const int t0 = (sl.u0 + i) * 8 - sl.h, lo = -t0, hi = sl.V - t0;
+    for (int c = 0; c < NS<DT> - 1; ++c) issue(c);
+#pragma unroll 1
+    for (int c = 0; c * NT < nu; ++c) {
+        const int i = c * NT + tid, t0 = (sl.u0 + i) * 8 - sl.h, lo = -t0, hi = i < nu ? V - t0 : 0;
+        RawChunk<DT> rp, rq;
+        stream::cp_async_wait<NS<DT> - 2>();
+        const uint4 *st = ring + (c % NS<DT>) * 2 * U * NT;
+        rp.a = st[0];
+        rq.a = st[U * NT];
+        if (U == 2) { rp.b = st[NT]; rq.b = st[3 * NT]; }
+        if (!vec && i < nu) {
+            rp = load_raw_scalar<DT>(sl.p, sl.u0 + i, V);
+            rq = load_raw_scalar<DT>(sl.q, sl.u0 + i, V);
+        }
+        issue(c + NS<DT> - 1);             // into the stage read in the previous iteration
         float z[8], ep[8], eq[8];
         unpack_chunk<DT>(rp, z);
-        mask_chunk(z, lo, hi, nr.cut_p > -CUDART_INF_F, nr.cut_p);
-        exp_chunk<false>(z, nr.s_hi, nr.s_lo, (float)nr.O_p, ep, dsx);
+        mask_chunk(z, lo, hi, cut_p > -CUDART_INF_F, cut_p);
+        exp_chunk<false>(z, s_hi, s_lo, O_p, ep, dsx);
         unpack_chunk<DT>(rq, z);
-        mask_chunk(z, lo, hi, nr.cut_q > -CUDART_INF_F, nr.cut_q);
-        exp_chunk<false>(z, nr.s_hi, nr.s_lo, (float)nr.O_q, eq, dsx);
-        unsigned dom = 0;
+        mask_chunk(z, lo, hi, cut_q > -CUDART_INF_F, cut_q);
+        exp_chunk<false>(z, s_hi, s_lo, O_q, eq, dsx);
+        if (HEAVY) {
+            unsigned m = 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (ep[k] > nr.thrB_p || eq[k] > nr.thrB_q) { dom |= 1u << k; }
-        for (unsigned m = dom; m; m &= m - 1u) {
-            const int k = __ffs(m) - 1;
-            const float z0 = raw_logit<DT>(rp, k), z1 = raw_logit<DT>(rq, k);       // (a dominant token lies inside the row)
-            const double xp = z0 >= nr.cut_p ? exp2_exact(z0, nr.s_d, nr.O_p) : 0.0;
-            const double xq = z1 >= nr.cut_q ? exp2_exact(z1, nr.s_d, nr.O_q) : 0.0;
-            if (g < 0.0) { o[0] += xp; o[1] += xq; }
-            else o[0] += fmax(fma(g, xp, -xq), 0.0);
+            for (int k = 0; k < 8; ++k)
+                if (ep[k] > thr_p || eq[k] > thr_q) { m |= 1u << k; ep[k] = eq[k] = 0.f; }
+            for (;;) {
+                const unsigned bal = __ballot_sync(0xffffffffu, m != 0);
+                if (!bal) break;
+                if (m) {
+                    const int k = __ffs(m) - 1;           // (inside the row: the others' e are 0)
+                    heavy[n + __popc(bal & ((1u << lane) - 1u))] = make_float2(raw_logit<DT>(rp, k), raw_logit<DT>(rq, k));
+                    m &= m - 1u;
+                }
+                n += __popc(bal);
+                __syncwarp();
+                if (n >= 32) {
+                    n -= 32;
+                    const double2 x = heavy_terms(heavy[n + lane], cut_p, cut_q, nr.O_p, nr.O_q, nr.s_d, g);
+                    o0 += x.x;
+                    o1 += x.y;
+                    __syncwarp();
+                }
+            }
         }
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if ((dom >> k) & 1u) ep[k] = eq[k] = 0.f;
-        if (g < 0.0) { ap += sum_chunk(ep); aq += sum_chunk(eq); }
+        if (norm) { ap += sum_chunk(ep); aq += sum_chunk(eq); }
         else ap += step_chunk(ep, eq, g_hi, g_lo);
     }
-    o[0] += (double)ap;
-    o[1] += (double)aq;
+    stream::cp_async_wait<0>();
+    if (HEAVY && lane < n) {
+        const double2 x = heavy_terms(heavy[lane], cut_p, cut_q, nr.O_p, nr.O_q, nr.s_d, g);
+        o0 += x.x;
+        o1 += x.y;
+    }
+    __syncwarp();
+    o[0] = o0 + (double)ap;
+    o[1] = o1 + (double)aq;
 }
 
 // One cluster of P.C CTAs (one where the batch fills the chip) per node, node-major; nodes of other kinds leave at once, except
@@ -229,6 +285,8 @@ __global__ void __launch_bounds__(256, 3) spec_single_kernel(const NParams NP)
     __shared__ Common M;
     __shared__ int s_first, s_count, s_nonleaf;
     __shared__ unsigned long long s_w;
+    uint4 *ring = reinterpret_cast<uint4 *>(dyn_smem);
+    __shared__ float2 s_heavy[NW][64];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, C = P.C;
     const unsigned rank = C > 1 ? cluster_ctarank() : 0u;
     // the same order as the items of spec_recursion_kernel: windows of sequences, node by node
@@ -279,7 +337,7 @@ __global__ void __launch_bounds__(256, 3) spec_single_kernel(const NParams NP)
         bool careful = trav && kc && !err && !flat_rows(Z_p, Z_q);
         auto exact_normalisers = [&]() {
             double v[2], tot[2], mine[2];
-            careful_sums<DT, NW>(sl, nr, -1.0, tid, v);
+            node_sums<DT, true>(sl, nr, -1.0, ring, s_heavy[warp], v);
             cluster_sum<NW, 2>(T, v, tot, mine);
             Z_p = tot[0]; Z_q = tot[1];
         };
@@ -302,14 +360,16 @@ __global__ void __launch_bounds__(256, 3) spec_single_kernel(const NParams NP)
             double tot[1], mine[1];
             double Sm = 0.0;
             if (!careful) {
-                const double v[1] = {residual_sum<DT, NW>(sl, nr, w * Z_q / Z_p, tid)};
-                cluster_sum<NW, 1>(T, v, tot, mine);
+                double v[2];
+                node_sums<DT, false>(sl, nr, w * Z_q / Z_p, ring, s_heavy[warp], v);
+                const double v1[1] = {v[0]};
+                cluster_sum<NW, 1>(T, v1, tot, mine);
                 Sm = tot[0] / Z_q;
                 if (!(Sm + (1.0 - w) > SMALL_STEP)) { careful = true; exact_normalisers(); }
             }
             if (careful) {
                 double v[2];
-                careful_sums<DT, NW>(sl, nr, w * Z_q / Z_p, tid, v);
+                node_sums<DT, true>(sl, nr, w * Z_q / Z_p, ring, s_heavy[warp], v);
                 const double v1[1] = {v[0]};
                 cluster_sum<NW, 1>(T, v1, tot, mine);
                 Sm = tot[0] / Z_q;

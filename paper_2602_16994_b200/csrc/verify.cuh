@@ -620,38 +620,6 @@ __device__ __forceinline__ double spectr_sweep(float4 *es, int nu, int tid, Resi
     return d;
 }
 
-// Sum over the CTA's part of a node of (g e_p - e_q)+ straight from the logits: nothing resident, no exact lists, one loop
-// that stays in the instruction cache.  For nodes that need this one sum only, to fp32 exponentials (tree.cuh).
-template <int DT, int NW>
-__device__ __forceinline__ double residual_sum(const Slice &sl, const NodeRows &nr, double g, int tid)
-{
-    constexpr int NCONS = NW * 32;
-    float g_hi, g_lo, dsx = 0.f, tot = 0.f;
-    split_float(g, g_hi, g_lo);
-    RawChunk<DT> np = {}, nq = {};
-    auto fetch = [&](int i) {
-        if (i >= sl.nu) return;
-        np = sl.vec ? load_raw<DT>(sl.p, sl.u0 + i, sl) : load_raw_scalar<DT>(sl.p, sl.u0 + i, sl.V);
-        nq = sl.vec ? load_raw<DT>(sl.q, sl.u0 + i, sl) : load_raw_scalar<DT>(sl.q, sl.u0 + i, sl.V);
-    };
-    fetch(tid);
-#pragma unroll 1
-    for (int i = tid; i < sl.nu; i += NCONS) {
-        const RawChunk<DT> rp = np, rq = nq;
-        fetch(i + NCONS);
-        const int t0 = (sl.u0 + i) * 8 - sl.h, lo = -t0, hi = sl.V - t0;
-        float z[8], ep[8], eq[8];
-        unpack_chunk<DT>(rp, z);
-        mask_chunk(z, lo, hi, nr.cut_p > -CUDART_INF_F, nr.cut_p);
-        exp_chunk<false>(z, nr.s_hi, nr.s_lo, (float)nr.O_p, ep, dsx);
-        unpack_chunk<DT>(rq, z);
-        mask_chunk(z, lo, hi, nr.cut_q > -CUDART_INF_F, nr.cut_q);
-        exp_chunk<false>(z, nr.s_hi, nr.s_lo, (float)nr.O_q, eq, dsx);
-        tot += step_chunk(ep, eq, g_hi, g_lo);
-    }
-    return (double)tot;
-}
-
 // A read-only sweep over the thread's share of the resident node: f.tail(e_p, e_q, a) on every fp32 token (f's running
 // sums), f.exact(...) in fp64 on the entry of the warp's exact list that falls to the lane.  Listed tokens are zero
 // in the fp32 arrays; every f maps (0, 0) to nothing.
