@@ -389,7 +389,7 @@ def run_ours(args):
         dt_ms = shard.max_over_ranks(dt_ms, world, dev)
         first = hv[w.algorithms[0]]
         e2e = {"value": world * w.draft_nodes() * len(w.algorithms) * n_e2e / dt_ms * 1e3, "unit": UNIT,
-               "h2d_bytes_per_step": first.h2d_bytes() * len(w.algorithms),
+               "h2d_bytes_per_step": first.h2d_bytes(hb.parent) * len(w.algorithms),
                "d2h_bytes_per_step": first.d2h_bytes() * len(w.algorithms),
                "ms_per_step": dt_ms / n_e2e, "steps": n_e2e,
                "api": "spec_verify_host (C ABI, pinned host buffers in, host results out, one sync per call)"}

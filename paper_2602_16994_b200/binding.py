@@ -420,10 +420,26 @@ class HostVerifier:
                                           ("bonus_token", (B,)), ("status", (B,)))}
         self.stream = torch.cuda.Stream(device=self.device)
 
-    def h2d_bytes(self) -> int:
+    def h2d_bytes(self, parent=None) -> int:
         B, N, V = self.shape
         esz = 4 if self.dtype == torch.float32 else 2
-        return 2 * B * N * V * esz + (B if self.per_seq else 1) * N * 4 + 3 * B * N * 4
+        total = 2 * B * N * V * esz + (B if self.per_seq else 1) * N * 4 + 3 * B * N * 4
+        return total - self._rows_left(parent, V * esz) * V * esz if parent is not None else total
+
+    def _rows_left(self, parent, row):
+        """Draft rows that the library leaves on the host for these trees (``copy_draft_rows`` in specverify.cu)."""
+        if row < 64 << 10:
+            return 0
+        trees = parent.reshape(-1, parent.shape[-1]).tolist()
+        height = 1 if self.per_seq else self.shape[0]
+        left = 0
+        for tree in trees:
+            inner = sorted({p for p in tree if 0 <= p < len(tree)})
+            edges = [-1] + inner + [len(tree)]
+            for k, (x, y) in enumerate(zip(edges, edges[1:])):
+                gap, last = y - x - 1, k == 0 or k == len(edges) - 2
+                left += height * gap if last or gap * row * height >= 256 << 10 else 0
+        return left
 
     def d2h_bytes(self) -> int:
         return sum(t.numel() * t.element_size() for t in self.host_out.values())

@@ -6,6 +6,8 @@
 // residual kernel below.  This file validates
 // arguments, chooses the launch plan and enqueues; it never allocates and, except for the
 // host-buffer entry point, never synchronises.
+#include <algorithm>
+#include <vector>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -598,6 +600,44 @@ HostLayout host_layout(const SpecIn *in)
     return L;
 }
 
+// The draft rows to the device: those of childless nodes stay behind (a tree of 4 branches: 1 row in 5; B = 8, V = 128256: 1.51 ->
+// 1.38 ms a call, which is bound by the PCIe copies).  A gap is left out where its bytes take longer than the
+// copy that it makes necessary (a few us, 256 KB).  A stream that still has work may yet write the tree: then, all rows.
+constexpr int64_t GAP_BYTES = 256 << 10, GAP_ROW_BYTES = 64 << 10;
+cudaError_t copy_draft_rows(const SpecIn *in, const HostLayout &L, unsigned char *dst, cudaStream_t st)
+{
+    const unsigned char *src = (const unsigned char *)in->draft_logits;
+    const int64_t row = L.logit_bytes / ((int64_t)in->B * in->N), seq = row * in->N;
+    if (row < GAP_ROW_BYTES || cudaStreamQuery(st) != cudaSuccess) {
+        cudaGetLastError();
+        return cudaMemcpyAsync(dst, src, (size_t)L.logit_bytes, cudaMemcpyHostToDevice, st);
+    }
+    // one tree for all: a strided copy per run of nodes; a tree per sequence: copies per sequence
+    const int trees = in->topo_seq_stride ? in->B : 1, N = in->N;
+    const int64_t height = in->topo_seq_stride ? 1 : in->B;
+    std::vector<char> inner(N);
+    for (int t = 0; t < trees; ++t) {
+        std::fill(inner.begin(), inner.end(), 0);
+        for (int c = 0; c < N; ++c) {
+            const int pa = in->parent[(int64_t)t * in->topo_seq_stride + c];
+            if (pa >= 0 && pa < N) inner[pa] = 1;
+        }
+        for (int a = 0; a < N;) {
+            if (!inner[a]) { ++a; continue; }
+            int end = a + 1;                                  // the run a .. end - 1, short gaps included
+            for (int c = end; c < N && (c - end) * row * height < GAP_BYTES; ++c)
+                if (inner[c]) end = c + 1;
+            const int64_t off = t * seq + a * row;
+            const cudaError_t e = height > 1
+                ? cudaMemcpy2DAsync(dst + off, (size_t)seq, src + off, (size_t)seq, (size_t)((end - a) * row), (size_t)height, cudaMemcpyHostToDevice, st)
+                : cudaMemcpyAsync(dst + off, src + off, (size_t)((end - a) * row), cudaMemcpyHostToDevice, st);
+            if (e != cudaSuccess) return e;
+            a = end;
+        }
+    }
+    return cudaSuccess;
+}
+
 // ------------------------------------------------------------------------------------------------
 // scratch that lives inside the library image, for spec_verify_specinfer_static
 // ------------------------------------------------------------------------------------------------
@@ -869,8 +909,8 @@ int32_t spec_verify_host(const SpecIn *in, const SpecOut *out, int32_t algorithm
     cudaStream_t st = (cudaStream_t)stream;
     unsigned char *d = (unsigned char *)dev_buf;
     bool ok = true;
+    ok &= copy_draft_rows(in, L, d + L.zq, st) == cudaSuccess;
     ok &= cudaMemcpyAsync(d + L.zp, in->target_logits, (size_t)L.logit_bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    ok &= cudaMemcpyAsync(d + L.zq, in->draft_logits, (size_t)L.logit_bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
     ok &= cudaMemcpyAsync(d + L.parent, in->parent, (size_t)L.parent_bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
     ok &= cudaMemcpyAsync(d + L.token, in->token, (size_t)L.bn4, cudaMemcpyHostToDevice, st) == cudaSuccess;
     ok &= cudaMemcpyAsync(d + L.ua, in->u_accept, (size_t)L.bn4, cudaMemcpyHostToDevice, st) == cudaSuccess;
