@@ -1,4 +1,4 @@
-// Offline analysis of a draft tree on the resident node data of the every-node kernel (tree.cuh in its
+// Offline analysis of a draft tree on the resident node data of the every-node kernel (nodes.cuh in its
 // analysis instantiation): acceptance rates (Definition 5.1, Algorithms 6-9), the divergences between
 // target and draft (Section 5's L1, the selector's KL features of Section 6), branching probabilities
 // (Definition 5.3, Algorithms 11-14) and the block-efficiency sum of equation (3); and the forward-time

@@ -1,5 +1,5 @@
 // Pieces shared by the verification kernels (walk.cuh: SpecInfer along the accepted path, Algorithm 4
-// composed top-down, Section 3.2; tree.cuh: every node, Traversal Verification of Section 3.2 with the
+// composed top-down, Section 3.2; nodes.cuh: every node, Traversal Verification of Section 3.2 with the
 // block-verification weights of Section 3.1): constants and shared-memory layouts, the handling of
 // one chunk of 8 logits (load, mask, exponentiate), the residual pass over resident e, prefix picks,
 // the inverse-CDF search for the bonus token, and the writing of a sequence's outputs from the node
@@ -840,7 +840,7 @@ __device__ __forceinline__ BonusFind bonus_search(Team &T, const Slice &sl, cons
 // selecting the accepted node of one sequence: run by the whole warp whose lane made the last arrival
 // ------------------------------------------------------------------------------------------------
 // Writes every output of the sequence except the bonus token (accepted node, length, path tokens, status,
-// the per-node diagnostics) and publishes the accepted node in P.fin for the sequence's FINISH item.
+// the per-node diagnostics) and publishes the accepted node in P.fin for the sequence's finish kernel.
 __device__ __noinline__ void finalize_sequence(const VParams &P, int b)
 {
     const int lane = threadIdx.x & 31;
@@ -958,9 +958,9 @@ __device__ __noinline__ void finalize_sequence(const VParams &P, int b)
     if (lane == 0) {
         P.out.accepted_node[b] = acc;
         P.out.accept_len[b] = len;
-        P.out.bonus_token[b] = -1;         // the FINISH item draws it
+        P.out.bonus_token[b] = -1;         // the finish kernel draws it
         P.out.status[b] = status;
-        if (P.out.margin) P.out.margin[(long long)b * (N + 1) + N] = CUDART_NAN_F;   // (the FINISH item's slot)
+        if (P.out.margin) P.out.margin[(long long)b * (N + 1) + N] = CUDART_NAN_F;   // (the finish kernel's slot)
     }
     // publication: the outputs above are visible to whoever sees the accepted node (the diagnostics below
     // are read by nobody on the device)
