@@ -231,6 +231,6 @@ struct __align__(16) NodeRec {
     int pad;
 };
 constexpr int STATE_IS_Q = -1;
-constexpr int STATE_FIRST = -2;  // one child, rejected: the step is taken by whoever needs the state (a FINISH item), from w_in
+constexpr int STATE_FIRST = -2;  // one child, rejected: the step is taken by whoever needs the state (the finish kernel), from w_in
 
 }  // namespace specv

@@ -5,7 +5,7 @@
 // the inverse-CDF search for the bonus token, and the writing of a sequence's outputs from the node
 // records.
 //
-// Common ground of both kernels.  A row is cut into chunks of 8 logits that start on 16-byte boundaries (the first
+// Common ground of the kernels.  A row is cut into chunks of 8 logits that start on 16-byte boundaries (the first
 // chunk holds fewer where the row starts on none); each CTA of a cluster owns a contiguous range of chunks, each
 // consumer thread every NCONS-th chunk of that range.  A logit becomes e = 2^(z s - O) with s = log2(e)/T and O the
 // row's integer reference, so every scale factor is an exact power of two.  The e of a thread's first RC chunks stay
