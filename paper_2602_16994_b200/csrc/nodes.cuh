@@ -8,16 +8,26 @@
 //                 the two rows, nothing resident (spec_single_kernel, a CTA or a small cluster per node);
 //   two or more   the residual recursion of verify.cuh, step by step, over resident rows (spec_recursion_kernel, a cluster per
 //                 node; in the analysis every node with children).
-// Weights flow down without waiting for rows: whoever publishes a node's weight publishes those of its whole line of
-// first children (publish_weight), so the only chain of dependent vocabulary-wide work is from branching node to
-// branching node.  The accepted node of a sequence is selected by whoever makes its last arrival, and one more
-// kernel (spec_finish_kernel, a cluster per sequence) brings that node on chip, takes its recorded steps and draws the
-// bonus token.
+// Weights flow down without waiting for rows: a node hands its first child min(1, w ratio) with ratio the quotient of two
+// probabilities of the unmodified rows, and a kernel of their own writes all ratios (spec_ratio_kernel).  Whoever
+// publishes a node's weight publishes those of its whole line of first children (publish_weight), so the only chain of
+// dependent vocabulary-wide work is from branching node to branching node.  The accepted node of a sequence is selected by
+// whoever makes its last arrival, and one more kernel (spec_finish_kernel, a cluster per sequence) brings that node on chip,
+// takes its recorded steps and draws the bonus token.
 //
-// The three kernels overlap (programmatic dependent launch): a kernel's CTAs take the places that the one before leaves
-// free and poll, with a limit, for what it publishes.  A kernel starts only when all CTAs of the one before have
-// started, never waits for a later one, and ends only after the one before has ended, so nothing waits on work that
-// cannot run.
+// Order of the kernels: ratios (Traversal only), recursion, single, finish.  They overlap (programmatic dependent launch): a
+// kernel's CTAs take the places that the one before leaves free and poll, with a limit, for what is published.  A kernel
+// starts only when all CTAs of the one before have started, and polls only for words that its own smaller items or
+// EARLIER kernels write:
+//   ratio      polls for nothing;
+//   recursion  ratios: from the ratio kernel; weights: from it, or from a smaller item of its own (drawn before it, hence
+//              running);
+//   single     ratios (exact normalisers come with them): from the ratio kernel; weights: from it or the recursion, never
+//              from its own kind;
+//   finish     accepted nodes: from the recursion or the single kernel.
+// So the calls of a stream come out the same when nothing overlaps (kernels run one at a time by a profiler, a debugger or
+// CUDA_LAUNCH_BLOCKING), and when kernels of other streams hold any part of the chip.  A kernel ends only after the
+// one before it has ended.
 //
 // Measured at V = 128256, bf16, batch 8, trunk of 2 and 4 branches of 4 (one branching node per sequence): see the
 // kernels.  A single kernel in which every node was an item of a cluster took 74 to 80 us here: its items cost 7 us
@@ -52,6 +62,7 @@ __device__ __forceinline__ int window_seqs(const VParams &P)
     return P.topo_stride == 0 ? P.B : min(P.B, max(1, FEW_SEQS / P.N));
 }
 
+constexpr unsigned long long NO_CHILD = W_PENDING - 1;        // a childless node's ratio
 __device__ __forceinline__ double token_ratio(double Pp, double Pq)
 {
     return !(Pp > 0.0) ? 0.0 : (!(Pq > 0.0) ? CUDART_INF : Pp / Pq);
@@ -81,8 +92,23 @@ __device__ __forceinline__ RowStat load_stat(const RowPart *p)
 // unnormalised probability of a token in a row, in units of 2^O
 __device__ __forceinline__ double token_e(float z, const RowStat &r, double s_d) { return z >= r.cut ? exp2_exact(z, s_d, r.O) : 0.0; }
 
-// Publishes weight thr of node c (warp-collective), and with it the weights of c's line of first children as far as their
-// ratios are known: they depend on nothing else.  A line is mostly consecutive nodes, so one load brings 32 ratios.
+// The ratio record of a node, written and read in one piece.
+__device__ __forceinline__ void put_chain(const VParams &P, long long node, unsigned long long ratio, int child)
+{
+    asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(P.chain + node), "l"(ratio),
+                 "l"((unsigned long long)(unsigned)child)
+                 : "memory");
+}
+__device__ __forceinline__ ulonglong2 get_chain(const VParams &P, long long node)
+{
+    ulonglong2 e;
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}" : "=l"(e.x), "=l"(e.y) : "l"(P.chain + node) : "memory");
+    return e;
+}
+// Publishes weight thr of node c (warp-collective), and with it the weights of c's line of first children, down to the childless end
+// or to a node whose ratio is not known yet (only while the ratio kernel runs): there whoever writes that ratio goes
+// on.  Both write before they look (put_ratio), so one of them sees the other; if both do, they write the same weights.
+// A line is mostly consecutive nodes, so one load brings 32 ratios.
 __device__ __noinline__ void publish_weight(const VParams &P, int b, int c, double thr)
 {
     const int lane = threadIdx.x & 31;
@@ -92,16 +118,25 @@ __device__ __noinline__ void publish_weight(const VParams &P, int b, int c, doub
     for (int hop = 0; hop < P.N; ++hop) {
         const long long at = (long long)b * P.N + c;
         if ((int)at == c_hold_slot) return;               // (a test may ask for one slot to stay pending)
-        // (the slot carries all there is to know: nothing to fence)
+        // (the slot carries all there is to know: nothing to fence for its readers)
         if (lane == 0) *(volatile unsigned long long *)(P.w_pub + at) = (unsigned long long)__double_as_longlong(thr);
         if (!have || c - base > 31) {
             base = c;
             have = true;
-            if (c + lane < P.N) e = __ldcg(reinterpret_cast<const ulonglong2 *>(P.chain + at + lane));
+            if (c + lane < P.N) e = get_chain(P, at + lane);
         }
-        const unsigned long long ratio = __shfl_sync(0xffffffffu, e.x, c - base);
-        if (ratio == W_PENDING) return;
-        c = (int)__shfl_sync(0xffffffffu, e.y, c - base);
+        unsigned long long ratio = __shfl_sync(0xffffffffu, e.x, c - base), child = __shfl_sync(0xffffffffu, e.y, c - base);
+        if (ratio == W_PENDING) {
+            __syncwarp();
+            __threadfence();
+            const ulonglong2 again = get_chain(P, at);
+            ratio = again.x;
+            child = again.y;
+        }
+        ratio = __shfl_sync(0xffffffffu, ratio, 0);       // (one answer for all lanes)
+        child = __shfl_sync(0xffffffffu, child, 0);
+        if (ratio == W_PENDING || ratio == NO_CHILD) return;
+        c = (int)(unsigned)child;
         thr = handed_weight(thr, __longlong_as_double((long long)ratio));
     }
 }
@@ -118,35 +153,6 @@ __device__ __forceinline__ unsigned long long poll_weight(const unsigned long lo
         __nanosleep(32);
     }
     return bits;
-}
-
-// The ratios of one sequence's first children, by one warp, and the root's line of first children published.  Left out: nodes
-// whose normalisers have to be taken more exactly first (spec_single_kernel, spec_recursion_kernel), and nodes with
-// a fault of any kind, which report it themselves.
-__device__ __noinline__ void first_children(const VParams &P, const RowPart *part, int dtype, int b)
-{
-    const int lane = threadIdx.x & 31;
-    const int *parent = P.parent + (long long)b * P.topo_stride;
-    const int *token = P.token + (long long)b * P.N;
-    const double s_d = 1.4426950408889634 / (double)(P.T_seq ? __ldg(P.T_seq + b) : P.T);
-    for (int c = 1 + lane; c < P.N; c += 32) {
-        const int pa = __ldg(parent + c), x = __ldg(token + c);
-        bool ok = pa >= 0 && pa < c && x >= 0 && x < P.V;
-        for (int d = pa + 1; ok && d < c; ++d) ok = __ldg(parent + d) != pa;
-        if (!ok) continue;
-        const RowPart *rp = part + ((long long)b * P.N + pa) * 2;
-        const long long at = (long long)b * P.seq_stride + (long long)pa * P.node_stride + x;
-        const float zp = load_logit(P.zp, dtype, at), zq = load_logit(P.zq, dtype, at);
-        const RowStat p = load_stat(rp), q = load_stat(rp + 1);
-        if (!p.ok() || !q.ok() || !flat_rows(p.Z, q.Z)) continue;
-        const double ratio = token_ratio(token_e(zp, p, s_d) / p.Z, token_e(zq, q, s_d) / q.Z);
-        __stcg(reinterpret_cast<ulonglong2 *>(P.chain + (long long)b * P.N + pa),
-               make_ulonglong2((unsigned long long)__double_as_longlong(ratio), (unsigned long long)c));
-    }
-    __threadfence();
-    __syncwarp();
-    const ulonglong2 e = __ldcg(reinterpret_cast<const ulonglong2 *>(P.chain + (long long)b * P.N));
-    if (e.x != W_PENDING) publish_weight(P, b, (int)e.y, handed_weight(1.0, __longlong_as_double((long long)e.x)));
 }
 
 // The record of a childless node, finished by whoever hands it its weight thr (lane 0 of a converged warp writes; the node's
@@ -169,28 +175,40 @@ __device__ __noinline__ void leaf_record(const VParams &P, const RowPart *part, 
 // ------------------------------------------------------------------------------------------------
 // nodes with one child
 // ------------------------------------------------------------------------------------------------
-// Sums over the CTA's share of a node's two rows, which come through a ring in shared memory: every thread copies and reads
+// Sums of NT threads (a CTA, or a warp) over their share of a node's two rows, which come through a ring in shared memory: every thread copies and reads
 // its own chunks, NS - 1 of them ahead (one chunk ahead in registers, a pass of one CTA over V = 128256 took 33 us, nearly all of
 // it the latency of L2).
-// HEAVY: tokens above 2^-DOM_S of a row's mass (at most 1024 per row, about 120 on the synthetic logits) in fp64, the
-// others in fp32, whose share of the error is then below 1e-8 of the mass.  They are collected per warp and evaluated 32
-// at a time.
-// g < 0: the rows' normalisers (o[0], o[1]); otherwise o[0] = sum (g e_p - e_q)+.
+// Kinds of sums: SUM_STEP o[0] = sum (g e_p - e_q)+ in fp32; SUM_STEP_HEAVY the same and SUM_NORM the rows' normalisers (o[0],
+// o[1]) with the tokens above 2^-DOM_S of a row's mass (at most 1024 per row, about 120 on the synthetic logits) in fp64
+// and the others in fp32, whose share of the error is then below 1e-8 of the mass.  They are collected per warp and
+// evaluated 32 at a time.
+enum SumKind { SUM_STEP, SUM_STEP_HEAVY, SUM_NORM };
 constexpr int DOM_S = 10;
 template <int DT> constexpr int NS = DT == SPEC_BF16 ? 4 : 3;                                  // stages of the ring
 template <int DT> constexpr int SUMS_RING = NS<DT> * (DT == SPEC_BF16 ? 2 : 4) * 256 * 16;     // bytes of it
 // (out of line: its registers would be spilled around every chunk of the loop below)
+template <int KIND>
 __device__ __noinline__ double2 heavy_terms(float2 z, float cut_p, float cut_q, int O_p, int O_q, double s_d, double g)
 {
     const double xp = z.x >= cut_p ? exp2_exact(z.x, s_d, O_p) : 0.0, xq = z.y >= cut_q ? exp2_exact(z.y, s_d, O_q) : 0.0;
-    return g < 0.0 ? make_double2(xp, xq) : make_double2(fmax(fma(g, xp, -xq), 0.0), 0.0);
+    return KIND == SUM_NORM ? make_double2(xp, xq) : make_double2(fmax(fma(g, xp, -xq), 0.0), 0.0);
 }
-template <int DT, bool HEAVY>
+__device__ __forceinline__ void set_sum_rows(NodeRows &nr, const RowStat &p, const RowStat &q, double s_d)
+{
+    nr.s_d = s_d;
+    stream::split_scale(s_d, nr.s_hi, nr.s_lo);
+    nr.hq = true;
+    nr.cut_p = p.cut; nr.cut_q = q.cut; nr.O_p = p.O; nr.O_q = q.O;
+    nr.thrB_p = (float)(p.Z / (double)(1 << DOM_S));
+    nr.thrB_q = (float)(q.Z / (double)(1 << DOM_S));
+}
+template <int DT, int KIND, int NT = 256>
 __device__ __noinline__ void node_sums(const Slice &sl, const NodeRows &nr, double g, uint4 *ring, float2 *heavy, double (&o)[2])
 {
-    constexpr int NT = 256, U = DT == SPEC_BF16 ? 1 : 2;         // threads, 16-byte units of a chunk
-    const int tid = threadIdx.x, lane = tid & 31, nu = sl.nu, V = sl.V;
-    const bool vec = sl.vec, norm = HEAVY && g < 0.0;
+    constexpr int U = DT == SPEC_BF16 ? 1 : 2;         // 16-byte units of a chunk
+    const int tid = threadIdx.x & (NT - 1), lane = tid & 31, nu = sl.nu, V = sl.V;
+    constexpr bool HEAVY = KIND != SUM_STEP;
+    const bool vec = sl.vec;
     const float s_hi = nr.s_hi, s_lo = nr.s_lo, O_p = (float)nr.O_p, O_q = (float)nr.O_q, cut_p = nr.cut_p, cut_q = nr.cut_q;
     const float thr_p = nr.thrB_p, thr_q = nr.thrB_q;
     float g_hi, g_lo, dsx = 0.f, ap = 0.f, aq = 0.f;
@@ -253,25 +271,236 @@ __device__ __noinline__ void node_sums(const Slice &sl, const NodeRows &nr, doub
                 __syncwarp();
                 if (n >= 32) {
                     n -= 32;
-                    const double2 x = heavy_terms(heavy[n + lane], cut_p, cut_q, nr.O_p, nr.O_q, nr.s_d, g);
+                    const double2 x = heavy_terms<KIND>(heavy[n + lane], cut_p, cut_q, nr.O_p, nr.O_q, nr.s_d, g);
                     o0 += x.x;
                     o1 += x.y;
                     __syncwarp();
                 }
             }
         }
-        if (norm) { ap += sum_chunk(ep); aq += sum_chunk(eq); }
+        if (KIND == SUM_NORM) { ap += sum_chunk(ep); aq += sum_chunk(eq); }
         else ap += step_chunk(ep, eq, g_hi, g_lo);
     }
     stream::cp_async_wait<0>();
     if (HEAVY && lane < n) {
-        const double2 x = heavy_terms(heavy[lane], cut_p, cut_q, nr.O_p, nr.O_q, nr.s_d, g);
+        const double2 x = heavy_terms<KIND>(heavy[lane], cut_p, cut_q, nr.O_p, nr.O_q, nr.s_d, g);
         o0 += x.x;
         o1 += x.y;
     }
     __syncwarp();
     o[0] = o0 + (double)ap;
     o[1] = o1 + (double)aq;
+}
+
+// What a node hands its first child depends on: that child, its logits in the node's rows, and whether anything is wrong with
+// the node's own arguments (what spec_single_kernel and spec_recursion_kernel look at too).  Warp-collective.
+struct __align__(16) FirstChild {
+    int child;
+    unsigned short kc, err;
+    float zp, zq;
+};
+template <int DT>
+__device__ __noinline__ FirstChild first_child(const VParams &P, int b, int a)
+{
+    const int lane = threadIdx.x & 31;
+    const int *parent = P.parent + (long long)b * P.topo_stride, *token = P.token + (long long)b * P.N;
+    FirstChild f = {0, 0, 0, 0.f, 0.f};
+    for (int c0 = a + 1; c0 < P.N; c0 += 32) {
+        const int c = c0 + lane;
+        const bool is = c < P.N && __ldg(parent + c) == a;
+        const unsigned bal = __ballot_sync(0xffffffffu, is);
+        if (bal && !f.kc) f.child = c0 + __ffs(bal) - 1;
+        f.kc += __popc(bal);
+        if (is) { const int x = __ldg(token + c); f.err |= x < 0 || x >= P.V; }
+    }
+    if (!f.kc) return f;
+    const int pa = __ldg(parent + a), xa = __ldg(token + a), x = __ldg(token + f.child);
+    f.err |= f.kc > KMAX || (a == 0 ? pa != -1 : (pa < 0 || pa >= a || xa < 0 || xa >= P.V));
+    f.err = __any_sync(0xffffffffu, f.err);
+    if (!f.err) {
+        const long long at = (long long)b * P.seq_stride + (long long)a * P.node_stride + x;
+        f.zp = load_logit(P.zp, DT, at);
+        f.zq = load_logit(P.zq, DT, at);
+    }
+    return f;
+}
+
+// A node's ratio is known (in lane 0; warp-collective): written down, and the line below the node published if the node's weight has
+// been (the root's is 1, that of a node without a parent to hand it one is 0).
+__device__ __noinline__ void put_ratio(const VParams &P, int b, int a, double ratio, int child)
+{
+    const long long node = (long long)b * P.N + a;
+    ratio = __shfl_sync(0xffffffffu, ratio, 0);
+    unsigned long long bits = (unsigned long long)__double_as_longlong(1.0);
+    if ((threadIdx.x & 31) == 0) {
+        put_chain(P, node, (unsigned long long)__double_as_longlong(ratio), child);
+        __threadfence();
+        const int pa = a == 0 ? 0 : __ldg(P.parent + (long long)b * P.topo_stride + a);
+        if (a > 0) bits = pa < 0 || pa >= a ? 0ull : *(volatile unsigned long long *)(P.w_pub + node);
+    }
+    bits = __shfl_sync(0xffffffffu, bits, 0);
+    if (bits != W_PENDING) publish_weight(P, b, child, handed_weight(__longlong_as_double((long long)bits), ratio));
+}
+
+// Traversal: the ratio of every first child, and the line of first children below each root, so that the kernels below ask for no
+// weight that a kernel after them would have to hand on.  A node with a fault of any kind hands on 0 and reports it itself.
+//   flat rows    two logits over the normalisers of the statistics pass, a warp per node (from the last CTA on, so that the
+//                first ones are free for the others);
+//   peaked rows  (flat_rows) both rows are summed again, heavy tokens in fp64.
+//     few    every CTA makes the same list of these nodes from the statistics, and as many CTAs take one as there are for each
+//            (up to SPLIT_MAX).  They and the node's warp leave what they have in the node's record, unused until the
+//            node's ratio is known, and the last of them writes the ratio;
+//     many   the node's warp does it by itself (many: see there).
+//   A node with one child keeps the exact normalisers in its record.
+// Bound by latency: what the call was given is read while the statistics kernel's last rows are on their way, a warp's ratio
+// is then one round of loads, one store and one look at the node's weight; a peaked node at V = 128256 on 5 CTAs is 13
+// rounds of its ring (9 us, 2.5 before it for the list and 2 after it).
+struct __align__(16) PeakedNode {
+    static constexpr int MOST = 5;
+    double2 part[MOST];          // the rows' sums of each CTA
+    FirstChild f;
+};
+static_assert(sizeof(PeakedNode) <= sizeof(NodeRec), "a node's record holds its partial sums");
+constexpr int SPLIT_MAX = PeakedNode::MOST;
+constexpr int PEAKED_LIST = 4096;                    // nodes that every CTA goes through (beyond: many)
+
+// One of the C + 1 who contribute to a peaked node has written its part (lane 0 of a converged warp): the last one writes the
+// ratio.
+__device__ __noinline__ void arrive_peaked(const VParams &P, const RowPart *part, long long node, int C)
+{
+    const int lane = threadIdx.x & 31;
+    int prev = 0;
+    if (lane == 0) asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(prev) : "l"(&P.chain[node].parts) : "memory");
+    if (__shfl_sync(0xffffffffu, prev, 0) != C) return;
+    const int b = (int)(node / P.N);
+    double ratio = 0.0;
+    int child = 0;
+    if (lane == 0) {
+        PeakedNode *R = reinterpret_cast<PeakedNode *>(P.rec + node);
+        double Z_p = 0.0, Z_q = 0.0;
+        double2 x[SPLIT_MAX];
+#pragma unroll
+        for (int k = 0; k < SPLIT_MAX; ++k) x[k] = k < C ? __ldcg(R->part + k) : make_double2(0.0, 0.0);
+        const uint4 f4 = __ldcg(reinterpret_cast<const uint4 *>(&R->f));
+        const RowStat p = load_stat(part + node * 2), q = load_stat(part + node * 2 + 1);
+#pragma unroll
+        for (int k = 0; k < SPLIT_MAX; ++k) { Z_p += x[k].x; Z_q += x[k].y; }
+        const double s_d = 1.4426950408889634 / (double)(P.T_seq ? __ldg(P.T_seq + b) : P.T);
+        const int kc = (int)(f4.y & 0xFFFFu), err = (int)(f4.y >> 16);
+        const double e_p = token_e(__uint_as_float(f4.z), p, s_d), e_q = token_e(__uint_as_float(f4.w), q, s_d);
+        if (kc == 1) { __stcg(&P.rec[node].Z_p, Z_p); __stcg(&P.rec[node].Z_q, Z_q); __threadfence(); }
+        if (!err) ratio = token_ratio(e_p / Z_p, e_q / Z_q);
+        child = (int)f4.x;
+    }
+    put_ratio(P, b, (int)(node % P.N), ratio, __shfl_sync(0xffffffffu, child, 0));
+}
+
+template <int DT>
+__global__ void __launch_bounds__(256, 3) spec_ratio_kernel(const NParams NP)
+{
+    constexpr int NW = 8;
+    const VParams &P = NP.v;
+    __shared__ float2 s_heavy[NW][64];
+    __shared__ double s_sum[NW][2];
+    __shared__ int s_cnt[NW];
+    __shared__ unsigned short s_list[PEAKED_LIST];
+    uint4 *ring = reinterpret_cast<uint4 *>(dyn_smem);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ctas = (int)gridDim.x;
+    const long long nodes = (long long)P.B * P.N, step = (long long)ctas * NW;
+    const auto scale = [&](int b) { return 1.4426950408889634 / (double)(P.T_seq ? __ldg(P.T_seq + b) : P.T); };
+    const auto peaked_node = [&](long long node) {
+        // (a childless node's draft row has not been read: not ok)
+        const RowStat p = load_stat(NP.part + node * 2), q = load_stat(NP.part + node * 2 + 1);
+        return p.ok() && q.ok() && !flat_rows(p.Z, q.Z);
+    };
+
+    long long id = (long long)(ctas - 1 - (int)blockIdx.x) * NW + warp;
+    FirstChild f = {};
+    if (id < nodes) f = first_child<DT>(P, (int)(id / P.N), (int)(id % P.N));
+    grid_dependency_wait();
+    grid_launch_dependents();     // (from here on: the recursion finds the statistics complete)
+
+    // ---- the list of peaked nodes -----------------------------------------------------------------------------------------
+    int n = 0, C = 1;
+    bool many = nodes > PEAKED_LIST;
+    if (!many) {
+        for (int i0 = 0; i0 < (int)nodes; i0 += 256) {
+            const int i = i0 + tid;
+            const bool peaked = i < (int)nodes && peaked_node(i);
+            const unsigned bal = __ballot_sync(0xffffffffu, peaked);
+            __syncthreads();
+            if (lane == 0) s_cnt[warp] = __popc(bal);
+            __syncthreads();
+            int at = n;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) { if (w < warp) at += s_cnt[w]; n += s_cnt[w]; }
+            if (peaked) s_list[at + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)i;
+        }
+        __syncthreads();
+        // A node costs about as much as 30 rounds of a CTA's ring besides its rows: loads that wait for each other, a barrier, the
+        // handing over.  A warp takes eight times the rounds and overlaps seven others.
+        const int rounds = (P.V + 2047) >> 11;
+        many = (n + ctas - 1) / ctas * (30 + rounds) > (n + ctas * NW - 1) / (ctas * NW) * (30 + NW * rounds);
+    }
+    if (!many) {
+        C = max(1, min(min(SPLIT_MAX, ctas / max(n, 1)), P.V >> 12));        // (a part of a row is at least 4096 logits)
+        for (int it = (int)blockIdx.x; it < n * C; it += ctas) {
+            const long long node = s_list[it / C];
+            const int r = it % C, b = (int)(node / P.N), a = (int)(node % P.N);
+            const RowStat p = load_stat(NP.part + node * 2), q = load_stat(NP.part + node * 2 + 1);
+            NodeRows nr;
+            set_sum_rows(nr, p, q, scale(b));
+            const Slice sl = make_slice<DT>(P.zp, P.zq, (long long)b * P.seq_stride + (long long)a * P.node_stride, P.V, C, (unsigned)r);
+            double v[2];
+            node_sums<DT, SUM_NORM>(sl, nr, 0.0, ring, s_heavy[warp], v);
+            v[0] = warp_sum(v[0]);
+            v[1] = warp_sum(v[1]);
+            if (lane == 0) { s_sum[warp][0] = v[0]; s_sum[warp][1] = v[1]; }
+            __syncthreads();
+            if (warp == 0) {
+                double2 z = make_double2(0.0, 0.0);
+                for (int w = 0; w < NW; ++w) { z.x += s_sum[w][0]; z.y += s_sum[w][1]; }
+                if (lane == 0) __stcg(reinterpret_cast<PeakedNode *>(P.rec + node)->part + r, z);
+                arrive_peaked(P, NP.part, node, C);
+            }
+            __syncthreads();
+        }
+    }
+
+    // ---- a warp per node ------------------------------------------------------------------------------------------------
+    while (id < nodes) {
+        const int b = (int)(id / P.N);
+        if (f.kc && !many && peaked_node(id)) {
+            if (lane == 0)
+                __stcg(reinterpret_cast<uint4 *>(&reinterpret_cast<PeakedNode *>(P.rec + id)->f),
+                       make_uint4((unsigned)f.child, (unsigned)f.kc | (unsigned)f.err << 16, __float_as_uint(f.zp), __float_as_uint(f.zq)));
+            arrive_peaked(P, NP.part, id, C);
+        } else if (f.kc) {
+            const int a = (int)(id % P.N);
+            const RowStat p = load_stat(NP.part + id * 2), q = load_stat(NP.part + id * 2 + 1);
+            const double s_d = scale(b);
+            double ratio = 0.0;
+            if (!f.err && p.ok() && q.ok()) {
+                double Z_p = p.Z, Z_q = q.Z;
+                if (!flat_rows(Z_p, Z_q)) {
+                    NodeRows nr;
+                    set_sum_rows(nr, p, q, s_d);
+                    const Slice sl = make_slice<DT>(P.zp, P.zq, (long long)b * P.seq_stride + (long long)a * P.node_stride, P.V, 1, 0u);
+                    double v[2];
+                    node_sums<DT, SUM_NORM, 32>(sl, nr, 0.0, ring + warp * (SUMS_RING<DT> / (16 * NW)), s_heavy[warp], v);
+                    Z_p = warp_sum(v[0]);
+                    Z_q = warp_sum(v[1]);
+                    if (f.kc == 1 && lane == 0) { __stcg(&P.rec[id].Z_p, Z_p); __stcg(&P.rec[id].Z_q, Z_q); __threadfence(); }
+                }
+                ratio = token_ratio(token_e(f.zp, p, s_d) / Z_p, token_e(f.zq, q, s_d) / Z_q);
+            }
+            put_ratio(P, b, a, ratio, f.child);
+        } else if (lane == 0) {
+            put_chain(P, id, NO_CHILD, 0);
+        }
+        id += step;
+        if (id < nodes) f = first_child<DT>(P, (int)(id / P.N), (int)(id % P.N));
+    }
 }
 
 // One cluster of P.C CTAs (one where the batch fills the chip) per node, node-major; nodes of other kinds leave at once, except
@@ -310,8 +539,7 @@ __global__ void __launch_bounds__(256, 3) spec_single_kernel(const NParams NP)
         const RowStat p = load_stat(rp), q = kc ? load_stat(rp + 1) : p;
         if (kc) for (int d = c + 1 + tid; d < P.N; d += 256) if (__ldg(parent + d) == c) s_nonleaf = 1;
         NodeRows nr;
-        nr.s_d = 1.4426950408889634 / (double)(P.T_seq ? __ldg(P.T_seq + b) : P.T);
-        stream::split_scale(nr.s_d, nr.s_hi, nr.s_lo);
+        set_sum_rows(nr, p, q, 1.4426950408889634 / (double)(P.T_seq ? __ldg(P.T_seq + b) : P.T));
         double e_p = 0.0, e_q = 0.0;
         if (kc) {
             const int x = __ldg(token + c);
@@ -329,47 +557,51 @@ __global__ void __launch_bounds__(256, 3) spec_single_kernel(const NParams NP)
         if (C > 1) cluster_sync_all();
         Team T = {M, C, warp, lane, 0, rank, 0u};
         const Slice sl = make_slice<DT>(P.zp, P.zq, (long long)b * P.seq_stride + (long long)a * P.node_stride, P.V, C, rank);
-        nr.hq = true;
-        nr.cut_p = p.cut; nr.cut_q = q.cut; nr.O_p = p.O; nr.O_q = q.O;
-        nr.thrB_p = (float)(p.Z / (double)(1 << DOM_S));
-        nr.thrB_q = (float)(q.Z / (double)(1 << DOM_S));
         double Z_p = p.Z, Z_q = q.Z;
-        bool careful = trav && kc && !err && !flat_rows(Z_p, Z_q);
-        auto exact_normalisers = [&]() {
-            double v[2], tot[2], mine[2];
-            node_sums<DT, true>(sl, nr, -1.0, ring, s_heavy[warp], v);
-            cluster_sum<NW, 2>(T, v, tot, mine);
-            Z_p = tot[0]; Z_q = tot[1];
-        };
-        // (nothing here waits for the weight yet: all such nodes do this at once)
-        if (careful) exact_normalisers();
+        if (trav && kc && p.ok() && q.ok() && !flat_rows(Z_p, Z_q)) {
+            // left in the record by the ratio kernel, with its ratio (a faulty node waits as well: partial sums may be there)
+            const long long node = (long long)b * P.N + a;
+            if (tid == 0) s_w = poll_weight(&P.chain[node].ratio, &M.poison);
+            __syncthreads();
+            if (s_w == W_PENDING) err = SPEC_DEV_TIMEOUT;
+            __threadfence();
+            Z_p = __ldcg(&P.rec[node].Z_p);
+            Z_q = __ldcg(&P.rec[node].Z_q);
+            __syncthreads();
+        }
         const double ratio = token_ratio(e_p / Z_p, e_q / Z_q);
         if (tid == 0) {
             s_w = (trav && a > 0 && !err) ? poll_weight(P.w_pub + (long long)b * P.N + a, &M.poison) : (unsigned long long)__double_as_longlong(1.0);
         }
         __syncthreads();
         double w = __longlong_as_double((long long)s_w);
-        if (s_w == W_PENDING) { err = SPEC_DEV_TIMEOUT; M.poison = 1; }
+        if (s_w == W_PENDING || err == SPEC_DEV_TIMEOUT) { err = SPEC_DEV_TIMEOUT; M.poison = 1; }
         if (err) w = 0.0;
         const double thr = err ? 0.0 : (trav ? handed_weight(w, ratio) : fmin(1.0, ratio));
-        if (trav && kc && s_nonleaf && rank == 0 && warp == 0 &&
-            *(volatile unsigned long long *)(P.w_pub + (long long)b * P.N + c) == W_PENDING)
-            publish_weight(P, b, c, thr);
+        // (the child's weight has been published with this node's; after a wait that ran out, those below need not wait as well)
+        if (err == SPEC_DEV_TIMEOUT && kc && s_nonleaf && rank == 0 && warp == 0) publish_weight(P, b, c, 0.0);
         double w_fin = w;
         if (trav && kc && w > 0.0) {
             double tot[1], mine[1];
             double Sm = 0.0;
+            bool careful = !flat_rows(p.Z, q.Z);
             if (!careful) {
                 double v[2];
-                node_sums<DT, false>(sl, nr, w * Z_q / Z_p, ring, s_heavy[warp], v);
+                node_sums<DT, SUM_STEP>(sl, nr, w * Z_q / Z_p, ring, s_heavy[warp], v);
                 const double v1[1] = {v[0]};
                 cluster_sum<NW, 1>(T, v1, tot, mine);
                 Sm = tot[0] / Z_q;
-                if (!(Sm + (1.0 - w) > SMALL_STEP)) { careful = true; exact_normalisers(); }
+                if (!(Sm + (1.0 - w) > SMALL_STEP)) {
+                    double t2[2], m2[2];
+                    careful = true;
+                    node_sums<DT, SUM_NORM>(sl, nr, 0.0, ring, s_heavy[warp], v);
+                    cluster_sum<NW, 2>(T, v, t2, m2);
+                    Z_p = t2[0]; Z_q = t2[1];
+                }
             }
             if (careful) {
                 double v[2];
-                node_sums<DT, true>(sl, nr, w * Z_q / Z_p, ring, s_heavy[warp], v);
+                node_sums<DT, SUM_STEP_HEAVY>(sl, nr, w * Z_q / Z_p, ring, s_heavy[warp], v);
                 const double v1[1] = {v[0]};
                 cluster_sum<NW, 1>(T, v1, tot, mine);
                 Sm = tot[0] / Z_q;
@@ -480,8 +712,8 @@ __device__ __noinline__ int list_nodes(BHdr &S, const VParams &P, int b0, int G,
 }
 
 // One cluster per item, items drawn from a counter by the first CTA's helper warp and passed to the others through distributed
-// shared memory (an item waits only for weights that smaller items hand down, and an item that is drawn runs, so
-// whatever share of the grid is resident, the smallest unfinished one never waits on anything unfinished).
+// shared memory (an item waits only for weights that the ratio kernel or smaller items publish, and an item that is drawn
+// runs, so whatever share of the grid is resident, the smallest unfinished one never waits on anything unfinished).
 //   helper warp     draws items; gathers an item's scalars while the one before runs; in the first CTA publishes what the
 //                   children are handed, writes the record and makes the arrivals -- so that none of this holds up
 //                   the consumers, whose sums over the cluster wait for their slowest warp
@@ -525,20 +757,29 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) spec_recursion_kernel(const 
         uint32_t mph[2] = {0u, 0u}, eph = 0;      // phases of the mailboxes
         int prev = -1;                       // scalars block of the item the consumers are at
         bool going = true;
+        // A node's record is written once its ratio is known: until then it may hold partial sums of the ratio kernel's.
+        auto after_ratio = [&](int b, int a) {
+            int w = 1;
+            __syncwarp();
+            if (trav && lane == 0) w = poll_weight(&P.chain[(long long)b * P.N + a].ratio, &S.M.poison) != W_PENDING;
+            if (!__shfl_sync(0xffffffffu, w, 0)) S.M.poison = 1;
+        };
 
-        // rank 0: what the children of an item are handed, published as the consumers find it; the record; the arrivals
+        // rank 0: what the children of an item are handed, published as the consumers find it (the first child's has been, with the
+        // item's own); the record; the arrivals
         auto serve = [&](int sb) {
             const NodeScalars &W = S.sc[sb];
             const Outcome &O = S.out[sb];
             NodeRec *rec = P.rec + (long long)W.b * P.N;
             unsigned narr = 1u;
+            after_ratio(W.b, W.a);
             for (int j = 0; j < W.kc; ++j) {
                 if (!*(volatile int *)&S.M.poison && !mbar_wait(&S.mb[sb][j], (mph[sb] >> j) & 1u)) S.M.poison = 1;
                 mph[sb] ^= 1u << j;
                 const double thr = *(volatile int *)&S.M.poison ? 0.0 : *(volatile double *)&S.out[sb].thr[j];
                 const int c = W.child[j];
                 if ((W.leaf_mask >> j) & 1u) { leaf_record(P, NP.part, W.b, c, thr); ++narr; }
-                else if (trav) publish_weight(P, W.b, c, thr);
+                else if (trav) { if (j > 0 || *(volatile int *)&S.M.poison) publish_weight(P, W.b, c, thr); }
                 else if (lane == 0) rec[c].thr = thr;
             }
             if (!*(volatile int *)&S.M.poison && !mbar_wait(&S.mend[sb], (eph >> sb) & 1u)) S.M.poison = 1;
@@ -676,6 +917,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) spec_recursion_kernel(const 
                 }
                 if ((err || zero) && rank == 0 && !AN) {
                     // A faulty node, or one of weight 0, is finished here: every child gets weight / threshold 0.
+                    after_ratio(b, a);
                     NodeRec *rec = P.rec + (long long)b * P.N;
                     unsigned narr = 1u;
                     for (int c = a + 1; c < P.N; ++c) {
@@ -717,9 +959,6 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) spec_recursion_kernel(const 
         WarpList &L = S.M.list[warp];
         Team T = {S.M, C, warp, lane, 0, rank, 0u};
         Resident<RC> R;
-        // while the first item is being gathered: the first children of this CTA's share of the sequences, a warp each
-        if (trav)
-            for (int b = (int)blockIdx.x * NW + warp; b < P.B; b += (int)gridDim.x * NW) first_children(P, NP.part, DT, b);
         for (int kidx = 0;; ++kidx) {
             const int sb = kidx & 1;
             if (!*(volatile int *)&S.M.poison && !mbar_wait(&S.sfull[sb], (uint32_t)((kidx >> 1) & 1))) S.M.poison = 1;
@@ -902,6 +1141,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) spec_recursion_kernel(const 
     }
     __syncthreads();
     cluster_sync_all();        // nobody leaves while a peer may still write to its shared memory
+    if (blockIdx.x == 0) grid_dependency_wait();      // this kernel ends only after the one before it
 }
 
 // ------------------------------------------------------------------------------------------------

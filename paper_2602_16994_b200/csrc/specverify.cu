@@ -248,9 +248,6 @@ int prepare_kernel(K kernel, int C, int smem, bool overlap = false)
         if (used >= 256) return SPEC_ERR_CUDA;
         ent = &cache[used++];
         *ent = Entry{(const void *)kernel, dev, -1, 0};
-        // The kernel's code is on the device from here on: loaded at its first launch it could wait for kernels that wait for it.
-        cudaFuncAttributes attr;
-        if (cudaFuncGetAttributes(&attr, (const void *)kernel) != cudaSuccess) { cudaGetLastError(); --used; return SPEC_ERR_CUDA; }
         // overlap: as much of an SM's L1 as can be is shared memory, so that CTAs of the kernels that run at the same time
         // find room beside this one
         if (overlap && cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
@@ -301,25 +298,24 @@ int resident_clusters(K kernel, int C, int threads, int smem)
 
 // nodes with several children (AN: with any): a cluster each
 template <int DT, int RC, bool AN>
-int launch_branch(const VPlan &pl, NParams &np, cudaStream_t st, bool prepare)
+int launch_branch(const VPlan &pl, NParams &np, cudaStream_t st)
 {
     auto kernel = spec_recursion_kernel<DT, 7, RC, AN>;
-    if (prepare) return prepare_kernel(kernel, pl.C, pl.smem, true);
+    const int rc = prepare_kernel(kernel, pl.C, pl.smem, true);
+    if (rc) return rc;
     int nc = resident_clusters(kernel, pl.C, 256, pl.smem);
     if (nc <= 0) return SPEC_ERR_UNSUPPORTED;
-    // A few SMs stay free for the nodes with one child, which hand weights to these: they have to run whatever this
-    // kernel's clusters wait for (and an SM whose shared memory is split for a smaller kernel takes none of them).
-    while (!AN && nc > 1 && nc * pl.C > sm_count() - 4) --nc;
     const long long items = (long long)np.v.B * np.v.N;
     if (nc > items) nc = (int)items;
     np.v.C = pl.C; np.v.off_es = pl.off_es;
-    return launch_clustered(kernel, nc * pl.C, pl.C, 256, pl.smem, st, &np);
+    return launch_clustered(kernel, nc * pl.C, pl.C, 256, pl.smem, st, &np, np.v.mode == MODE_TRAVERSAL);
 }
 template <int DT, int RC>
-int launch_finish(const VPlan &pl, NParams &np, cudaStream_t st, bool prepare)
+int launch_finish(const VPlan &pl, NParams &np, cudaStream_t st)
 {
     auto kernel = spec_finish_kernel<DT, 8, RC>;
-    if (prepare) return prepare_kernel(kernel, pl.C, pl.smem, true);
+    const int rc = prepare_kernel(kernel, pl.C, pl.smem, true);
+    if (rc) return rc;
     int nc = resident_clusters(kernel, pl.C, 256, pl.smem);
     if (nc <= 0) return SPEC_ERR_UNSUPPORTED;
     if (nc > np.v.B) nc = np.v.B;
@@ -493,36 +489,42 @@ int launch_nodes(const SpecIn *in, NParams &np, bool analysis, cudaStream_t st)
     VPlan br, fi;
     bool big, bigf;
     if (!one_cta_plan(in->V, 7, (int)sizeof(BHdr), &br, &big) || !one_cta_plan(in->V, 8, (int)sizeof(FHdr), &fi, &bigf)) return SPEC_ERR_UNSUPPORTED;
-    auto branch = [&](auto an, bool prepare) {
-        constexpr bool AN = decltype(an)::value;
-        if (big) return bf ? launch_branch<SPEC_BF16, 8, AN>(br, np, st, prepare) : launch_branch<SPEC_F32, 8, AN>(br, np, st, prepare);
-        return bf ? launch_branch<SPEC_BF16, 0, AN>(br, np, st, prepare) : launch_branch<SPEC_F32, 0, AN>(br, np, st, prepare);
-    };
-    // nodes with one child: more CTAs per node while few waves hold them all (with one CTA a node its passes, not their sum, are the
-    // latency: traversal, batch 8, V = 128256, 152 nodes: 131 us with 1, 109 with 2, 94 with 4)
-    int C = 1;
     const long long nodes = (long long)in->B * in->N;
-    while (C < 8 && nodes * C * 2 <= 8 * sm_count() && in->V >= C * 8192) C <<= 1;
-    auto single = [&](bool prepare) {
-        np.v.C = C;
-        auto go = [&](auto kernel) {
-            const int smem = bf ? SUMS_RING<SPEC_BF16> : SUMS_RING<SPEC_F32>;
-            return prepare ? prepare_kernel(kernel, C, smem, true) : launch_clustered(kernel, (int)nodes * C, C, 256, smem, st, &np, true);
+    const int smem = bf ? SUMS_RING<SPEC_BF16> : SUMS_RING<SPEC_F32>;
+    int rc;
+    if (np.v.mode == MODE_TRAVERSAL) {
+        // A CTA per SM, so that the recursion's clusters, which wait for its results, find their places beside it; as many as fit (3)
+        // where there are the nodes for them.
+        const int ctas = nodes < 2 * sm_count() ? sm_count() : 3 * sm_count();
+        const auto go = [&](auto kernel) {
+            const int e = prepare_kernel(kernel, 1, smem, true);
+            return e ? e : launch_clustered(kernel, ctas, 1, 256, smem, st, &np, true);
         };
-        return bf ? go(spec_single_kernel<SPEC_BF16>) : go(spec_single_kernel<SPEC_F32>);
-    };
-    auto finish = [&](bool prepare) {
-        if (bigf) return bf ? launch_finish<SPEC_BF16, 8>(fi, np, st, prepare) : launch_finish<SPEC_F32, 8>(fi, np, st, prepare);
-        return bf ? launch_finish<SPEC_BF16, 0>(fi, np, st, prepare) : launch_finish<SPEC_F32, 0>(fi, np, st, prepare);
-    };
-    // (everything that may wait for the device happens before the first of the kernels that wait for one another)
-    for (int prepare = 1; prepare >= 0; --prepare) {
-        int rc = analysis ? branch(std::true_type{}, prepare) : branch(std::false_type{}, prepare);
-        if (!rc && !analysis) rc = single(prepare);
-        if (!rc && !analysis) rc = finish(prepare);
+        rc = bf ? go(spec_ratio_kernel<SPEC_BF16>) : go(spec_ratio_kernel<SPEC_F32>);
         if (rc) return rc;
     }
-    return SPEC_OK;
+    const auto branch = [&](auto an) {
+        constexpr bool AN = decltype(an)::value;
+        if (big) return bf ? launch_branch<SPEC_BF16, 8, AN>(br, np, st) : launch_branch<SPEC_F32, 8, AN>(br, np, st);
+        return bf ? launch_branch<SPEC_BF16, 0, AN>(br, np, st) : launch_branch<SPEC_F32, 0, AN>(br, np, st);
+    };
+    rc = analysis ? branch(std::true_type{}) : branch(std::false_type{});
+    if (rc || analysis) return rc;
+    {
+        // nodes with one child: more CTAs per node while few waves hold them all (with one CTA a node its passes, not their sum, are the
+        // latency: traversal, batch 8, V = 128256, 152 nodes: 131 us with 1, 109 with 2, 94 with 4)
+        int C = 1;
+        while (C < 8 && nodes * C * 2 <= 8 * sm_count() && in->V >= C * 8192) C <<= 1;
+        np.v.C = C;
+        const auto go = [&](auto kernel) {
+            const int e = prepare_kernel(kernel, C, smem, true);
+            return e ? e : launch_clustered(kernel, (int)nodes * C, C, 256, smem, st, &np, true);
+        };
+        rc = bf ? go(spec_single_kernel<SPEC_BF16>) : go(spec_single_kernel<SPEC_F32>);
+        if (rc) return rc;
+    }
+    if (bigf) return bf ? launch_finish<SPEC_BF16, 8>(fi, np, st) : launch_finish<SPEC_F32, 8>(fi, np, st);
+    return bf ? launch_finish<SPEC_BF16, 0>(fi, np, st) : launch_finish<SPEC_F32, 0>(fi, np, st);
 }
 
 int verify_common(const SpecIn *in, const SpecOut *out, void *ws, int64_t ws_bytes, void *stream, int mode,

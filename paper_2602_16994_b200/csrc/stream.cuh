@@ -397,6 +397,7 @@ struct MParams {
 
 __global__ void spec_row_merge_kernel(const MParams P)
 {
+    grid_launch_dependents();     // (one sequence: the ratio kernel's CTAs are in their places when the last row is merged)
     const long long r2 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (r2 >= P.rows2) return;

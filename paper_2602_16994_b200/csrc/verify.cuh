@@ -77,9 +77,9 @@ enum Mode { MODE_SPECINFER = 0, MODE_TRAVERSAL = 1 };
 
 // Traversal: a node of weight w hands its first child min(1, w ratio), with ratio = p(x) / q(x) of the unmodified rows
 struct __align__(16) ChainRec {
-    unsigned long long ratio;    // bits of the double; W_PENDING: not known
+    unsigned long long ratio;    // bits of the double; W_PENDING: not known; NO_CHILD
     int child;
-    int pad;
+    int parts;                   // of a peaked node's normalisers, while they are being summed (0 at launch)
 };
 
 struct VParams {

@@ -1,5 +1,9 @@
 """The node kernels at the sizes where they can go wrong: chains (every node has one child), rows at odd offsets from a 16-byte
 boundary, trees of more than 32 nodes, peaked rows (normalisers and weights retaken in fp64), vocabularies of one chunk."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -57,3 +61,60 @@ def test_host_call_leaves_childless_rows_behind(per_seq):
         for f in ("accepted_node", "accept_len", "out_tokens", "bonus_token", "status"):
             assert np.array_equal(getattr(want, f).cpu().numpy(), got[f].numpy()), (algo, f)
         assert hv.h2d_bytes(host[2]) < hv.h2d_bytes()
+
+
+# branching nodes below one-child nodes whose rows are peaked; the third batch has so many of them that each is left to one warp,
+# the last rows so long that the node kernels find no room for each other on an SM
+ORDER = [Workload("trunk", 3, 8193, "bf16", 3, 3, 2, 0.5, temperature=0.25),
+         Workload("trunk_cut", 2, 32000, "bf16", 2, 2, 2, 0.6, temperature=0.6, top_p=0.95),
+         Workload("many_peaked", 400, 2003, "f32", 3, 2, 2, 0.6, temperature=0.25),
+         Workload("no_room", 1, 151936, "f32", 2, 2, 2, 0.6, temperature=0.3)]
+
+
+def in_order():
+    """Every workload of ORDER against the oracle, plain and with diagnostics, and a batch with faults."""
+    for w in ORDER:
+        check_batch(make_batch(w, seed=8, device="cuda"), "traversal")
+    b = make_batch(ORDER[0], seed=8, device="cuda")
+    args = lambda parent, token: (b.target_logits, b.draft_logits, parent, token, b.u_accept, b.u_bonus)
+    want = binding.verify_traversal(*args(b.parent, b.token), temperature=0.25)
+    parent = b.parent.reshape(1, -1).repeat(3, 1).contiguous()
+    token = b.token.clone()
+    parent[0, 2] = 7                     # a trunk node without a parent, branching node below it
+    token[1, 1] = -1                     # a trunk node with a token outside the vocabulary
+    got = binding.verify_traversal(*args(parent, token), temperature=0.25, node_thr=True, node_w_in=True)
+    status = got.status.cpu().numpy()
+    assert status[0] == 1 and status[1] == 2 and status[2] == 0, status
+    for f in ("accepted_node", "accept_len", "out_tokens", "bonus_token"):
+        assert np.array_equal(getattr(want, f)[2].cpu().numpy(), getattr(got, f)[2].cpu().numpy()), f
+
+
+@pytest.mark.parametrize("blocking", ["0", "1"])
+def test_no_kernel_waits_for_a_later_one(blocking):
+    """The same results when every kernel has ended before the next one starts."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", "from tests.test_gpu_nodes import in_order; in_order()"], cwd=root,
+                       env=dict(os.environ, CUDA_LAUNCH_BLOCKING=blocking), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_two_streams():
+    """Calls of two streams at once, a workspace each, share the chip: the results of calls one after the other."""
+    batches = [make_batch(Workload("stream", 4, 128256, "bf16", 4, 2, 3, 0.8, temperature=t), seed=i, device="cuda")
+               for i, t in enumerate((1.0, 0.4))]
+    args = [(b.target_logits, b.draft_logits, b.parent, b.token, b.u_accept, b.u_bonus, b.workload.temperature) for b in batches]
+    fields = ("accepted_node", "accept_len", "out_tokens", "bonus_token", "status")
+    want = [binding.verify_traversal(*a) for a in args]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in batches]
+    ws = [binding.Workspace(a[0].device) for a in args]
+    got = [[], []]
+    for _ in range(20):
+        for i, s in enumerate(streams):
+            with torch.cuda.stream(s):
+                got[i].append(binding.verify_traversal(*args[i], workspace=ws[i]))
+    torch.cuda.synchronize()
+    for i in range(2):
+        for o in got[i]:
+            for f in fields:
+                assert np.array_equal(getattr(want[i], f).cpu().numpy(), getattr(o, f).cpu().numpy()), (i, f)
