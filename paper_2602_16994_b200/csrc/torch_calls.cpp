@@ -41,6 +41,13 @@ const char *error_name(int rc)
 
 // an error that has been set as a Python exception
 struct Raised {};
+// a reference of this module's own
+struct Owned {
+    PyObject *o;
+    explicit Owned(PyObject *p) : o(p) {}
+    ~Owned() { Py_XDECREF(o); }
+    Owned(const Owned &) = delete;
+};
 template <typename... A> [[noreturn]] void raise(const char *fmt, A... a)
 {
     PyErr_Format(PyExc_RuntimeError, fmt, a...);
@@ -97,21 +104,22 @@ at::Tensor empty(at::IntArrayRef sizes, at::ScalarType t, const at::Device &d)
     return at::Tensor(at::detail::empty_cuda(sizes, t, d, std::nullopt));
 }
 
-// the caller's Workspace: its buffer, grown by the object itself when too small
-struct Scratch { void *ptr; int64_t bytes; };
+// the caller's Workspace: its buffer, grown by the object itself when too small (held until the call has been enqueued: another
+// thread may grow the object meanwhile)
+struct Scratch { void *ptr; int64_t bytes; at::Tensor buf; };
 Scratch scratch_of(PyObject *workspace, int64_t bytes)
 {
     for (int attempt = 0;; ++attempt) {
         PyObject *buf = PyObject_GetAttr(workspace, n_buf);
         if (!buf) throw Raised{};
         if (buf != Py_None) {
-            const at::Tensor &t = tensor(buf, "buf");
+            const Owned held(buf);
+            const at::Tensor t = tensor(buf, "buf");
             const int64_t have = t.numel();
             char *base = (char *)t.data_ptr();
-            Py_DECREF(buf);                   // (the object keeps its buffer)
             if (have >= bytes + 256) {
                 const int64_t off = (256 - ((intptr_t)base & 255)) & 255;
-                return {base + off, have - off};
+                return {base + off, have - off, t};
             }
         } else {
             Py_DECREF(buf);
@@ -219,10 +227,11 @@ PyObject *py_verify(PyObject *, PyObject *const *a, Py_ssize_t n)
             for (int i = 0; i < 10; ++i) if (t[i].defined()) p[i] = t[i].data_ptr();
         } else {
             for (int i = 0; i < 10; ++i) {
-                PyObject *o = PyObject_GetAttr(given, n_out[i]);
-                if (!o) throw Raised{};
-                Py_DECREF(o);                 // (the outputs object keeps it)
-                p[i] = pointer_or_null(o, OUT_NAMES[i]);
+                const Owned o(PyObject_GetAttr(given, n_out[i]));
+                if (!o.o) throw Raised{};
+                if (o.o == Py_None) continue;
+                t[i] = tensor(o.o, OUT_NAMES[i]);          // (held until the call has been enqueued: the attribute may be computed)
+                p[i] = t[i].data_ptr();
             }
         }
         const SpecOut out = {(int32_t *)p[0], (int32_t *)p[1], (int32_t *)p[2], (int32_t *)p[3], (int32_t *)p[4],
