@@ -55,6 +55,17 @@ template <typename... A> [[noreturn]] void raise(const char *fmt, A... a)
 }
 void check(int rc, const char *what) { if (rc) raise("%s failed: %s", what, error_name(rc)); }
 
+// Calls f, which touches no Python object, with the interpreter's lock released: a launch may wait (a full queue, the first use of
+// a kernel), and other threads run meanwhile, as with ctypes.
+template <typename F> int unlocked(F f)
+{
+    struct Released {
+        PyThreadState *state = PyEval_SaveThread();
+        ~Released() { PyEval_RestoreThread(state); }
+    } released;
+    return f();
+}
+
 const at::Tensor &tensor(PyObject *o, const char *name)
 {
     if (!THPVariable_Check(o)) { PyErr_Format(PyExc_TypeError, "%s must be a tensor", name); throw Raised{}; }
@@ -237,9 +248,12 @@ PyObject *py_verify(PyObject *, PyObject *const *a, Py_ssize_t n)
         const SpecOut out = {(int32_t *)p[0], (int32_t *)p[1], (int32_t *)p[2], (int32_t *)p[3], (int32_t *)p[4],
                              (float *)p[5], (float *)p[6], (float *)p[7], (float *)p[8], (float *)p[9]};
         void *st = stream_of(a[13]);
-        if (code == 0) check(lib.specinfer(&in, &out, ws.ptr, ws.bytes, st), "spec_verify_specinfer");
-        else if (code == 1) check(lib.traversal(&in, &out, ws.ptr, ws.bytes, st), "spec_verify_traversal");
-        else check(lib.otlp(&in, &out, code - 2, ws.ptr, ws.bytes, st), "spec_verify_otlp");
+        const int rc = unlocked([&] {
+            return code == 0   ? lib.specinfer(&in, &out, ws.ptr, ws.bytes, st)
+                   : code == 1 ? lib.traversal(&in, &out, ws.ptr, ws.bytes, st)
+                               : lib.otlp(&in, &out, code - 2, ws.ptr, ws.bytes, st);
+        });
+        check(rc, code == 0 ? "spec_verify_specinfer" : code == 1 ? "spec_verify_traversal" : "spec_verify_otlp");
         return given == Py_None ? result(verify_outputs_class, t, 10) : Py_NewRef(given);
     });
 }
@@ -259,7 +273,8 @@ PyObject *py_analysis(PyObject *, PyObject *const *a, Py_ssize_t n)
         const Scratch ws = scratch_of(a[10], bytes);
         const SpecAnalysisOut out = {(float *)t[0].data_ptr(), (float *)t[1].data_ptr(), (float *)t[2].data_ptr(),
                                      (float *)t[3].data_ptr(), (float *)t[4].data_ptr()};
-        check(lib.analysis(&in, &out, ws.ptr, ws.bytes, stream_of(a[11])), "spec_tree_analysis");
+        void *st = stream_of(a[11]);
+        check(unlocked([&] { return lib.analysis(&in, &out, ws.ptr, ws.bytes, st); }), "spec_tree_analysis");
         return result(analysis_outputs_class, t, 5);
     });
 }
@@ -287,8 +302,10 @@ PyObject *py_probs(PyObject *, PyObject *const *a, Py_ssize_t n)
         int64_t bytes = 0;
         check(lib.workspace_bytes(&in, &bytes), "spec_workspace_bytes");
         const Scratch ws = scratch_of(a[8], bytes);        // holds the row cuts when truncating
-        check(lib.probs(&in, truncated(a[1]), probs.defined() ? (float *)probs.data_ptr() : nullptr,
-                        stats.defined() ? (float *)stats.data_ptr() : nullptr, ws.ptr, ws.bytes, stream_of(a[9])), "spec_tree_probs");
+        const int which = truncated(a[1]);
+        float *pr = probs.defined() ? (float *)probs.data_ptr() : nullptr, *st = stats.defined() ? (float *)stats.data_ptr() : nullptr;
+        void *stream = stream_of(a[9]);
+        check(unlocked([&] { return lib.probs(&in, which, pr, st, ws.ptr, ws.bytes, stream); }), "spec_tree_probs");
         PyObject *p = probs.defined() ? THPVariable_Wrap(probs) : Py_NewRef(Py_None);
         PyObject *s = stats.defined() ? THPVariable_Wrap(stats) : Py_NewRef(Py_None);
         PyObject *r = p && s ? PyTuple_Pack(2, p, s) : nullptr;
@@ -310,9 +327,12 @@ PyObject *py_bonus(PyObject *, PyObject *const *a, Py_ssize_t n)
         const bool want = PyObject_IsTrue(a[2]);
         at::Tensor token = empty({w.size(0)}, at::kInt, w.device()), margin;
         if (want) margin = empty({w.size(0)}, at::kFloat, w.device());
-        check(lib.bonus((const float *)w.data_ptr(), (int32_t)w.size(0), (int32_t)w.size(1), (const float *)u.data_ptr(),
-                        (int32_t *)token.data_ptr(), want ? (float *)margin.data_ptr() : nullptr, nullptr, 0, stream_of(a[3])),
-              "spec_sample_bonus");
+        const float *wp = (const float *)w.data_ptr(), *up = (const float *)u.data_ptr();
+        const int32_t R = (int32_t)w.size(0), V = (int32_t)w.size(1);
+        int32_t *tp = (int32_t *)token.data_ptr();
+        float *mp = want ? (float *)margin.data_ptr() : nullptr;
+        void *st = stream_of(a[3]);
+        check(unlocked([&] { return lib.bonus(wp, R, V, up, tp, mp, nullptr, 0, st); }), "spec_sample_bonus");
         PyObject *t = THPVariable_Wrap(token);
         if (!want || !t) return t;
         PyObject *m = THPVariable_Wrap(margin), *r = m ? PyTuple_Pack(2, t, m) : nullptr;
@@ -330,7 +350,11 @@ PyObject *py_launch(PyObject *, PyObject *const *a, Py_ssize_t n)
     return guarded([&]() -> PyObject * {
         const auto at_ = [&](int i) { return (void *)(intptr_t)integer(a[i]); };
         const bool traversal = integer(a[0]) != 0;
-        check((traversal ? lib.traversal : lib.specinfer)((const SpecIn *)at_(1), (const SpecOut *)at_(2), at_(3), integer(a[4]), stream_of(a[5])),
+        const SpecIn *in = (const SpecIn *)at_(1);
+        const SpecOut *out = (const SpecOut *)at_(2);
+        void *ws = at_(3), *st = stream_of(a[5]);
+        const int64_t bytes = integer(a[4]);
+        check(unlocked([&] { return (traversal ? lib.traversal : lib.specinfer)(in, out, ws, bytes, st); }),
               traversal ? "spec_verify_traversal" : "spec_verify_specinfer");
         Py_RETURN_NONE;
     });

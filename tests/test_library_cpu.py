@@ -3,6 +3,8 @@ rejects bad arguments on the host before touching a device.  No kernel is launch
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -117,3 +119,31 @@ def test_binding_refuses_to_run_without_a_gpu():
         binding.tree_probs(z)
     with pytest.raises(RuntimeError):
         binding.sample_bonus(torch.zeros((1, 8)), torch.zeros(1))
+
+
+def test_a_launch_releases_the_interpreter_lock(tmp_path):
+    """Other Python threads run while a call into the library waits (a stand-in library whose call sleeps)."""
+    names = ("spec_workspace_bytes", "spec_analysis_workspace_bytes", "spec_verify_traversal", "spec_verify_otlp", "spec_tree_analysis",
+             "spec_tree_probs", "spec_sample_bonus")
+    src, lib = tmp_path / "slow.c", tmp_path / "slow.so"
+    src.write_text("#include <unistd.h>\nint spec_verify_specinfer(void) { usleep(400000); return 0; }\n" +
+                   "".join(f"int {n}(void) {{ return 0; }}\n" for n in names))
+    subprocess.check_call(["gcc", "-shared", "-fPIC", "-o", str(lib), str(src)])
+    code = f"""
+import threading, time, torch
+from paper_2602_16994_b200 import _torch_calls as c
+class Stream: cuda_stream = 0
+c.init({str(lib)!r}, object, object)
+gaps, going = [0.0], True
+def tick():
+    last = time.monotonic()
+    while going:
+        time.sleep(0.005)
+        now = time.monotonic(); gaps.append(now - last); last = now
+t = threading.Thread(target=tick); t.start()
+time.sleep(0.05)
+c.launch(0, 1, 1, 1, 0, Stream)
+going = False; t.join()
+assert max(gaps) < 0.2, max(gaps)
+"""
+    subprocess.check_call([sys.executable, "-c", code], cwd=ROOT)
