@@ -7,7 +7,6 @@
 // arguments, chooses the launch plan and enqueues; it never allocates and, except for the
 // host-buffer entry point, never synchronises.
 #include <algorithm>
-#include <vector>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -604,22 +603,32 @@ HostLayout host_layout(const SpecIn *in)
 
 // The draft rows to the device: those of childless nodes stay behind (a tree of 4 branches: 1 row in 5; B = 8, V = 128256: 1.51 ->
 // 1.38 ms a call, which is bound by the PCIe copies).  A gap is left out where its bytes take longer than the
-// copy that it makes necessary (a few us, 256 KB).  A stream that still has work may yet write the tree: then, all rows.
+// copy that it makes necessary (a few us, 256 KB).  Work that the stream still has may yet write the tree: it is waited for
+// before the tree is read (the copies would have waited for it as well, and the call ends with a wait).
 constexpr int64_t GAP_BYTES = 256 << 10, GAP_ROW_BYTES = 64 << 10;
+cudaError_t wait_for_earlier_work(cudaStream_t st)
+{
+    cudaEvent_t e;                    // (an event, so that the default stream's order with other streams counts)
+    cudaError_t rc = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
+    if (rc != cudaSuccess) return rc;
+    rc = cudaEventRecord(e, st);
+    if (rc == cudaSuccess) rc = cudaEventSynchronize(e);
+    cudaEventDestroy(e);
+    return rc;
+}
 cudaError_t copy_draft_rows(const SpecIn *in, const HostLayout &L, unsigned char *dst, cudaStream_t st)
 {
     const unsigned char *src = (const unsigned char *)in->draft_logits;
     const int64_t row = L.logit_bytes / ((int64_t)in->B * in->N), seq = row * in->N;
-    if (row < GAP_ROW_BYTES || cudaStreamQuery(st) != cudaSuccess) {
-        cudaGetLastError();
-        return cudaMemcpyAsync(dst, src, (size_t)L.logit_bytes, cudaMemcpyHostToDevice, st);
-    }
+    if (row < GAP_ROW_BYTES) return cudaMemcpyAsync(dst, src, (size_t)L.logit_bytes, cudaMemcpyHostToDevice, st);
+    const cudaError_t waited = wait_for_earlier_work(st);
+    if (waited != cudaSuccess) return waited;
     // one tree for all: a strided copy per run of nodes; a tree per sequence: copies per sequence
     const int trees = in->topo_seq_stride ? in->B : 1, N = in->N;
     const int64_t height = in->topo_seq_stride ? 1 : in->B;
-    std::vector<char> inner(N);
+    char inner[SPEC_MAX_NODES];
     for (int t = 0; t < trees; ++t) {
-        std::fill(inner.begin(), inner.end(), 0);
+        std::fill(inner, inner + N, 0);
         for (int c = 0; c < N; ++c) {
             const int pa = in->parent[(int64_t)t * in->topo_seq_stride + c];
             if (pa >= 0 && pa < N) inner[pa] = 1;

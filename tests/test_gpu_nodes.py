@@ -47,9 +47,11 @@ def test_rows_at_any_alignment(shift):
             assert np.array_equal(getattr(want, f).cpu().numpy(), getattr(got, f).cpu().numpy()), f
 
 
+@pytest.mark.parametrize("busy", [False, True])
 @pytest.mark.parametrize("per_seq", [False, True])
-def test_host_call_leaves_childless_rows_behind(per_seq):
-    """Rows long enough that the host-buffer call skips the draft rows of childless nodes; the same decisions."""
+def test_host_call_leaves_childless_rows_behind(per_seq, busy):
+    """Rows long enough that the host-buffer call skips the draft rows of childless nodes, also on a stream that still has
+    work to do; the same decisions."""
     w = Workload("host", 3, 40000, "bf16", 3, 1, 2, 0.7)
     d = make_batch(w, seed=2, device="cuda")
     several = lambda t: t.reshape(1, -1).repeat(w.B, 1).contiguous() if per_seq else t
@@ -57,7 +59,16 @@ def test_host_call_leaves_childless_rows_behind(per_seq):
         want = call(d.target_logits, d.draft_logits, several(d.parent), d.token, d.u_accept, d.u_bonus)
         hv = binding.HostVerifier(w.B, w.N, w.V, torch.bfloat16, algorithm=algo, per_sequence_topology=per_seq)
         host = [t.cpu().pin_memory() for t in (d.target_logits, d.draft_logits, several(d.parent), d.token, d.u_accept, d.u_bonus)]
+        hv.staging.fill_(0xA5)
+        torch.cuda.synchronize()
+        if busy:
+            with torch.cuda.stream(hv.stream):
+                torch.cuda._sleep(20_000_000)                  # about 10 ms
         got = hv.run(*host)
+        off = -hv.staging.data_ptr() % 256 + (w.B * w.N * w.V * 2 + 255) // 256 * 256        # the staged draft rows
+        rows = hv.staging[off:off + w.B * w.N * w.V * 2].view(w.B, w.N, w.V * 2)
+        left = int((rows == 0xA5).all(-1).sum())
+        assert left * w.V * 2 == hv.h2d_bytes() - hv.h2d_bytes(host[2])
         for f in ("accepted_node", "accept_len", "out_tokens", "bonus_token", "status"):
             assert np.array_equal(getattr(want, f).cpu().numpy(), got[f].numpy()), (algo, f)
         assert hv.h2d_bytes(host[2]) < hv.h2d_bytes()
