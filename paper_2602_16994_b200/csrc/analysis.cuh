@@ -83,16 +83,19 @@ struct FnSpecTrRes {    // sum d, sum d (1 - (1-r)^k), d = (p - min(p/rho, q) ga
 // SpecTr's division factor: the root of f(rho) = 1 - (1 - beta)^k - rho beta on [1, k] (Appendix B), f(1) >= 0 >= f(k).
 // Regula falsi with the Illinois rule (the value at an end that stays is halved), and the middle whenever two steps
 // have not halved the bracket -- so never more than about twice the steps of a bisection, and about ten where f is
-// smooth (a bisection to the same 1e-9 takes 31, each a sweep over the node and a sum over the cluster).
+// smooth (40 halvings of [1, k], the accuracy that is asked for here, are 40 sweeps over the node and sums over the cluster).
+// (on the host too, for its test)
+#pragma nv_exec_check_disable
 template <typename F>
-__device__ __forceinline__ double spectr_root(double k, F beta)
+__host__ __device__ __forceinline__ double spectr_root(double k, F beta)
 {
     const auto f = [&](double r) { const double b = beta(r); return (1.0 - pow(1.0 - b, k)) - r * b; };
     double lo = 1.0, hi = k, flo = f(lo), fhi = f(hi);
     if (!(flo > 0.0)) return 1.0;
+    const double close = (k - 1.0) * 9.094947017729282e-13;       // 2^-40
     double was = hi - lo;
     int side = 0;
-    for (int it = 0; it < 64 && hi - lo > 1.0e-9; ++it) {
+    for (int it = 0; it < 96 && hi - lo > close; ++it) {
         double x = fhi < 0.0 ? (lo * fhi - hi * flo) / (fhi - flo) : hi;
         if ((it & 1) && hi - lo > 0.5 * was) x = 0.5 * (lo + hi);
         if (it & 1) was = hi - lo;
