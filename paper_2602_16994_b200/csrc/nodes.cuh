@@ -211,7 +211,7 @@ __device__ __noinline__ void node_sums(const Slice &sl, const NodeRows &nr, doub
     const bool vec = sl.vec;
     const float s_hi = nr.s_hi, s_lo = nr.s_lo, O_p = (float)nr.O_p, O_q = (float)nr.O_q, cut_p = nr.cut_p, cut_q = nr.cut_q;
     const float thr_p = nr.thrB_p, thr_q = nr.thrB_q;
-    float g_hi, g_lo, dsx = 0.f, ap = 0.f, aq = 0.f;
+    float g_hi, g_lo, dsx = 0.f;
     split_float(g, g_hi, g_lo);
     double o0 = 0.0, o1 = 0.0;
     int n = 0;                             // entries of the warp's list (below 32 between chunks)
@@ -278,8 +278,9 @@ __device__ __noinline__ void node_sums(const Slice &sl, const NodeRows &nr, doub
                 }
             }
         }
-        if (KIND == SUM_NORM) { ap += sum_chunk(ep); aq += sum_chunk(eq); }
-        else ap += step_chunk(ep, eq, g_hi, g_lo);
+        // (a thread's sums over its chunks in fp64: in fp32 each of up to hundreds of additions would round)
+        if (KIND == SUM_NORM) { o0 += (double)sum_chunk(ep); o1 += (double)sum_chunk(eq); }
+        else o0 += (double)step_chunk(ep, eq, g_hi, g_lo);
     }
     stream::cp_async_wait<0>();
     if (HEAVY && lane < n) {
@@ -288,8 +289,8 @@ __device__ __noinline__ void node_sums(const Slice &sl, const NodeRows &nr, doub
         o1 += x.y;
     }
     __syncwarp();
-    o[0] = o0 + (double)ap;
-    o[1] = o1 + (double)aq;
+    o[0] = o0;
+    o[1] = o1;
 }
 
 // What a node hands its first child depends on: that child, its logits in the node's rows, and whether anything is wrong with
