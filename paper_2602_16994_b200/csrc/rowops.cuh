@@ -242,13 +242,11 @@ __device__ __forceinline__ void widen_exp(float *region, int SL, int dtype, int 
     kept = nk;
 }
 
-// Inverse CDF inside one slice.  Weights w_t = (ep[t] - gamma eq[t])+ (eq may be NULL: w = ep).
-// Each thread owns a contiguous run of float4 groups (an odd count, so that the 128-bit shared loads
-// of a warp fall in distinct bank groups), sums it in fp64, a block scan finds the owning thread,
+// Inverse CDF inside one slice of weights.  Each thread owns a contiguous run of float4 groups (an odd count, so that
+// the 128-bit shared loads of a warp fall in distinct bank groups), sums it in fp64, a block scan finds the owning thread,
 // which walks its run again.  Returns the local token index (block-uniform), or the last
 // positive-weight token if tau is not below the slice total, or -1 if the slice holds no weight.
-__device__ __forceinline__ int slice_inverse_cdf(Shared &S, const float *ep, const float *eq, int SL,
-                                                 float g_hi, float g_lo, double tau, double &dist_lo,
+__device__ __forceinline__ int slice_inverse_cdf(Shared &S, const float *ep, int SL, double tau, double &dist_lo,
                                                  double &dist_hi)
 {
     const int nv = SL >> 2;
@@ -256,19 +254,12 @@ __device__ __forceinline__ int slice_inverse_cdf(Shared &S, const float *ep, con
     L4 |= 1;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int i0 = threadIdx.x * L4, i1 = min(i0 + L4, nv);
-    const float4 *a = (const float4 *)ep, *b = (const float4 *)eq;
+    const float4 *a = (const float4 *)ep;
     double seg = 0.0;
     int last_pos = -1;
     for (int i = i0; i < i1; ++i) {
         float4 p = a[i];
         float v[4] = {p.x, p.y, p.z, p.w};
-        if (eq) {
-            float4 q = b[i];
-            v[0] = fmaxf(fmaf(-g_lo, q.x, fmaf(-g_hi, q.x, p.x)), 0.f);
-            v[1] = fmaxf(fmaf(-g_lo, q.y, fmaf(-g_hi, q.y, p.y)), 0.f);
-            v[2] = fmaxf(fmaf(-g_lo, q.z, fmaf(-g_hi, q.z, p.z)), 0.f);
-            v[3] = fmaxf(fmaf(-g_lo, q.w, fmaf(-g_hi, q.w, p.w)), 0.f);
-        }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             seg += (double)v[k];
@@ -300,13 +291,6 @@ __device__ __forceinline__ int slice_inverse_cdf(Shared &S, const float *ep, con
         for (int i = i0; i < i1 && found < 0; ++i) {
             float4 p = a[i];
             float v[4] = {p.x, p.y, p.z, p.w};
-            if (eq) {
-                float4 q = b[i];
-                v[0] = fmaxf(fmaf(-g_lo, q.x, fmaf(-g_hi, q.x, p.x)), 0.f);
-                v[1] = fmaxf(fmaf(-g_lo, q.y, fmaf(-g_hi, q.y, p.y)), 0.f);
-                v[2] = fmaxf(fmaf(-g_lo, q.z, fmaf(-g_hi, q.z, p.z)), 0.f);
-                v[3] = fmaxf(fmaf(-g_lo, q.w, fmaf(-g_hi, q.w, p.w)), 0.f);
-            }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if (found < 0) {
@@ -496,7 +480,7 @@ __global__ void __launch_bounds__(NT, 1) spec_bonus_kernel(const BParams P)
     }
     if (owner == rank) {
         double dlo = 0.0, dhi = 0.0;
-        int t = slice_inverse_cdf(S, ep, nullptr, SL, 0.f, 0.f, tau, dlo, dhi);
+        int t = slice_inverse_cdf(S, ep, SL, tau, dlo, dhi);
         if (tid == 0) {
             P.token[r_id] = t >= 0 ? (int)(tok0 + t) : -1;
             if (P.margin) P.margin[r_id] = (float)(fmin(dlo, dhi) / tot);

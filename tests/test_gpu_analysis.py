@@ -21,6 +21,8 @@ SHAPES = [
     Workload("an_tinyV_dups", 16, 6, "f32", 3, 1, 2, 1.0),
     Workload("an_v4099_topk", 3, 4099, "bf16", 3, 1, 2, 1.0, temperature=0.7, top_k=40),
     Workload("an_v262144", 1, 262144, "bf16", 4, 1, 2, 0.75),
+    Workload("an_v450001", 1, 450001, "bf16", 3, 1, 2, 0.75),          # part of a node in registers
+    Workload("an_v620003_f32", 1, 620003, "f32", 2, 1, 2, 0.75),
 ]
 
 

@@ -29,6 +29,18 @@ def test_nodes(w, algo):
     check_batch(make_batch(w, seed=3, device="cuda"), algo, full=False)
 
 
+@pytest.mark.parametrize("algo", ["specinfer", "traversal"])
+@pytest.mark.parametrize("w", [
+    Workload("v420001", 2, 420001, "bf16", 3, 1, 2, 0.7),                          # registers in the recursion, none in the draw
+    Workload("v450001", 2, 450001, "bf16", 3, 2, 2, 0.6, temperature=0.5),
+    Workload("v620003", 1, 620003, "f32", 3, 1, 2, 0.7),                           # close to the largest V
+], ids=lambda w: w.name)
+def test_vocabularies_beyond_shared_memory(w, algo):
+    """Above about 400000 tokens a node's e no longer fit in the shared memory of 16 CTAs: eight chunks per thread stay in
+    registers, in every cluster kernel (the plain SpecInfer call is the walk, the others go node by node)."""
+    check_batch(make_batch(w, seed=4, device="cuda"), algo)
+
+
 @pytest.mark.parametrize("shift", [(1, 1), (1, 2), (0, 3)])
 def test_rows_at_any_alignment(shift):
     """Target and draft tensors that start at their own odd offsets: the same results as aligned ones."""

@@ -22,6 +22,7 @@ SHAPES = [
     Workload("ot_v32000_k2_T07", 4, 32000, "bf16", 2, 1, 3, 0.8, temperature=0.7),
     Workload("ot_v128256_k4", 3, 128256, "bf16", 4, 1, 2, 0.5),
     Workload("ot_v4099_topk", 6, 4099, "bf16", 3, 1, 2, 0.7, temperature=0.8, top_k=40),
+    Workload("ot_v450001_k3_T04", 3, 450001, "bf16", 3, 1, 2, 0.3, temperature=0.4),      # part of a node in registers
     Workload("ot_v1000_path", 6, 1000, "f32", 1, 0, 5, 0.5),
 ]
 
