@@ -269,9 +269,8 @@ def test_traversal_weight_one_with_a_vanishing_residual():
 
 
 def test_traversal_skipping_does_not_change_the_outcome():
-    """Without per-node diagnostics the Traversal call skips subtrees that come wholly after a node already
-    known to be accepted, and nodes below a weight of 0.  Outcome and residual must be those of the call
-    that evaluates every node (diagnostics on), on trees wide and deep enough for both kinds of skipping."""
+    """Without per-node diagnostics the Traversal call reads no rows of nodes of weight 0.  Outcome and residual
+    must be those of the call that evaluates every node (diagnostics on), on trees wide and deep enough."""
     skipped_something = 0
     for seed in range(10):
         w = small("skip", 6000, "bf16", 4, 2, 4, 6, sigma=0.6)
@@ -281,9 +280,10 @@ def test_traversal_skipping_does_not_change_the_outcome():
         for name in ("accepted_node", "accept_len", "bonus_token", "out_tokens", "status"):
             assert torch.equal(getattr(plain, name), getattr(full, name)), (seed, name)
         assert torch.equal(plain.residual, full.residual), seed
-        # the accepted node is rarely the last one in traversal order: then there was something to skip
         N = w.N
-        skipped_something += int((full.accepted_node != 0).sum().item())
+        inner = torch.zeros(N, dtype=torch.bool, device="cuda")
+        inner[batch.parent.reshape(-1, N)[0, 1:].long()] = True
+        skipped_something += int((full.node_w_in[:, inner] == 0).sum().item())
         assert (full.node_thr[:, 0] == 1.0).all() and full.node_thr.shape == (w.B, N)
     assert skipped_something > 0
 
@@ -291,15 +291,15 @@ def test_traversal_skipping_does_not_change_the_outcome():
 TREE_SHAPES = [
     Workload("s_k8_root", 6, 3000, "bf16", 8, 0, 3, 0.6),        # N = 25: a wide root
     Workload("s_k2_deep", 6, 2000, "f32", 2, 3, 6, 0.4),          # N = 16: deep branches
-    Workload("s_k5_d1", 6, 5000, "bf16", 5, 1, 6, 0.5),           # N = 32: the largest tree with a post-order table
-    Workload("s_k6_d1", 4, 4000, "bf16", 6, 1, 6, 0.5),           # N = 38: no table, nothing skipped by rank
+    Workload("s_k5_d1", 6, 5000, "bf16", 5, 1, 6, 0.5),           # N = 32: the largest tree selected by a warp in parallel
+    Workload("s_k6_d1", 4, 4000, "bf16", 6, 1, 6, 0.5),           # N = 38: selected serially
 ]
 
 
 @pytest.mark.parametrize("w", TREE_SHAPES, ids=lambda w: w.name)
 def test_traversal_on_wide_and_deep_trees(w):
-    """Traversal's hand-out hints (weight 0 at an ancestor, subtree after a known acceptance) on trees of other
-    shapes than the configs', at and beyond the size limit of the post-order table."""
+    """Traversal (weight 0 at an ancestor among its nodes) on trees of other shapes than the configs', at and beyond the
+    size limit of the warp-parallel selection."""
     total = Tally()
     for seed in range(100, 108):
         total.add(check_batch(make_batch(w, seed=seed, device="cuda"), "traversal", full=(seed % 4 == 0)))

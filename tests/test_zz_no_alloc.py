@@ -5,7 +5,7 @@ plugin inside a server that owns the memory pool, a decoding loop in which an al
 stall): its scratch is an array inside the library instead of a caller-supplied workspace.  It must
 give what ``spec_verify_specinfer`` gives.  Calls come in pairs and the second shape is smaller than
 the first, because the second call finds the first one's records, published weights, arrival counters
-and row lists still in the array: the every-node path (diagnostic outputs) and the top-k / top-p path
+and statistics still in the array: the every-node path (diagnostic outputs) and the top-k / top-p path
 are the ones that depend on the call clearing what must start empty.  This file sorts last on
 purpose, so that a run that stops at the first failure has already run every other test; it also
 passes on its own in a fresh process.
@@ -50,7 +50,7 @@ def test_static_scratch_matches_workspace_entry_point_twice():
 
 @pytest.mark.parametrize("trunc", [dict(), dict(top_k=40), dict(top_p=0.9)], ids=["plain", "top_k", "top_p"])
 def test_static_scratch_every_node_path_twice_and_allocates_nothing(trunc):
-    """Diagnostic outputs send the call through the every-node kernel, whose published-weight slots and
+    """Diagnostic outputs send the call through the node kernels, whose published-weight slots and
     arrival counters live in the shared array; the second, smaller call must not see the first one's."""
     shapes = [Workload("nb1", 8, 32000, "bf16", 4, 1, 3, 1.0, temperature=0.7, **trunc),
               Workload("nb2", 3, 8192, "bf16", 2, 1, 2, 0.8, temperature=0.7, **trunc)]
