@@ -36,12 +36,12 @@ ROTATE_BYTES = 4 * L2_BYTES          # bytes touched before an input copy is rea
 # (every logit once), and both verifiers start with it.
 STAT_KERNEL = {False: "stream::spec_row_partial_kernel (row statistics: the one pass over the logits in HBM)",
                True: "trunc::spec_row_trunc_kernel (row statistics and cuts: the one pass over the logits in HBM)"}
-# dram__bytes_read.sum + dram__bytes_write.sum per launch of that kernel from the ncu captures summarised
-# under profiles/ (cold L2).  Workloads without a capture: null.
-TRAFFIC_BYTES = {"cfg2_llama3_b8": 69_799_168 + 626_432}
+# dram__bytes_read.sum + dram__bytes_write.sum per launch of that kernel, launched in a row, from the ncu
+# captures summarised under profiles/.  Workloads without a capture: null.
+TRAFFIC_BYTES = {"cfg2_llama3_b8": 69_770_000 + 100_000}
 # the same counters summed over the kernels of a whole call, captured in one pass without cache flushes between
-# the kernels (profiles/per_config.md): the second kernel of a call finds most of its rows in L2
-TRAFFIC_CALL_BYTES = {"cfg2_llama3_b8": {"specinfer": 70_810_000 + 90_000, "traversal": 70_810_000 + 9_200_000}}
+# the kernels (profiles/per_config.md): the later kernels of a call find most of their rows in L2
+TRAFFIC_CALL_BYTES = {"cfg2_llama3_b8": {"specinfer": 69_790_000 + 1_600_000, "traversal": 84_100_000 + 28_300_000}}
 
 
 def parse_args():
