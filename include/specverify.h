@@ -148,7 +148,7 @@ int32_t spec_verify_specinfer(const SpecIn *in, const SpecOut *out, void *ws, in
  * first child, in list order, that carries it, and stops when no child does -- that token is the
  * correction token).  solver: 0 = NSS (Algorithm 1: the token is drawn from p, the drafts are ignored),
  * 1 = NaiveTree (Algorithm 2: the first child is tested with min(1, p/q), otherwise a draw from
- * norm((p - q)+)), 2 = SpecTr K-SEQ (Algorithm 3: division factor rho* by bisection, every child
+ * norm((p - q)+)), 2 = SpecTr K-SEQ (Algorithm 3: division factor rho* by root search, every child
  * tested with min(1, p / (rho q)), otherwise a draw from its residual).  A child's test uses its entry
  * of u_accept, a draw at node a the entry u_bonus[a].  Same inputs, workspace, stream and status rules
  * as spec_verify_specinfer; of SpecOut only accepted_node, accept_len, out_tokens, bonus_token and
@@ -212,7 +212,7 @@ int32_t spec_verify_traversal(const SpecIn *in, const SpecOut *out, void *ws, in
  *               equation (3) (average it over sampled trees for the paper's estimator).
  * Rows of childless nodes are NaN in acceptance / divergence.  All outputs are device pointers, all
  * required.  `ws`: spec_analysis_workspace_bytes() bytes.  u_accept / u_bonus of `in` must be valid
- * but do not influence the outputs.  SpecTr's rho* is found by 40 bisection steps on [1, k].
+ * but do not influence the outputs.  SpecTr's rho* is found to (k - 1) 2^-40 on [1, k].
  */
 typedef struct {
     float *acceptance;
@@ -272,7 +272,7 @@ int64_t spec_kernel_launches(void);
  * is bounded (Section "General rules": a wait that runs out is reported as SPEC_DEV_TIMEOUT, nothing
  * hangs); these two settings let a test watch that happen.  wait_cycles: the limit of every on-device
  * wait in clock cycles (<= 0: the default, about 2 s).  hold_slot: index b * N + node of one node whose
- * Traversal weight the every-node kernel then never publishes, so that the node's own wait runs out
+ * Traversal weight the node kernels then never publish, so that the node's own wait runs out
  * (-1: none).  Synchronous (copies to constant memory of the current device); call it between
  * verification calls, never while one is in flight.
  */

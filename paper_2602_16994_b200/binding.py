@@ -1,10 +1,10 @@
-"""Thin binding of libspecverify.so: argument marshalling only.
+"""Binding of libspecverify.so: argument marshalling only.
 
 Every step of the verification path runs inside the CUDA library; this module turns torch tensors
 into the plain pointers of the C ABI (``include/specverify.h``), owns the scratch workspace and
 allocates output tensors.  The calls of a decoding loop do that in native code (``csrc/torch_calls.cpp``);
-the host-buffer call, the plan queries and the caller-allocated entry point go through ctypes.  There is no CPU fallback: a missing library or a missing CUDA device
-raises ``RuntimeError``.
+prepared calls, the host-buffer call, the plan queries and the entry point without a workspace go through ctypes.
+There is no CPU fallback: a missing library or a missing CUDA device raises ``RuntimeError``.
 
 Device-resident API (inputs already in HBM, nothing is synchronised):
     verify_specinfer / verify_traversal / tree_probs / sample_bonus

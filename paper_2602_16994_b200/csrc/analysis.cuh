@@ -1,10 +1,10 @@
-// Offline analysis of a draft tree on the resident node data of the every-node kernel (nodes.cuh in its
+// Offline analysis of a draft tree on the resident node data of the recursion kernel (nodes.cuh in its
 // analysis instantiation): acceptance rates (Definition 5.1, Algorithms 6-9), the divergences between
 // target and draft (Section 5's L1, the selector's KL features of Section 6), branching probabilities
 // (Definition 5.3, Algorithms 11-14) and the block-efficiency sum of equation (3); and the forward-time
 // model of equation (8).
 //
-// Division of work.  The every-node kernel holds a node's e_p, e_q on chip with its dominant tokens
+// Division of work.  The recursion kernel holds a node's e_p, e_q on chip with its dominant tokens
 // exact; in analysis mode it runs, before the SpecInfer recursion, read-only sweeps for the vocabulary-wide
 // sums (the functors below) and the search for SpecTr's rho*, and dumps per node the scalars everything
 // else follows from (AnRec).  spec_branch_kernel (one warp per node) turns them into branching
@@ -21,7 +21,7 @@ namespace specv {
 
 constexpr int AN_KDP = 10;            // uniform-order SpecInfer: the DP covers up to 2^AN_KDP sets of children
 
-// per node, dumped by the every-node kernel in analysis mode
+// per node, dumped by the recursion kernel in analysis mode
 struct __align__(16) AnRec {
     double A[KMAX + 1][KMAX];   // A[i][t] = min(1, p_i(x_t) / q(x_t)) for round i < k; row k: p_k(x_t)
     double S[KMAX];             // residual mass of round i (0 once the state equals q)

@@ -14,7 +14,7 @@ constexpr int KMAX = SPEC_MAX_CHILDREN;
 // that a test can shorten it (spec_test_hooks) and watch a wait run out without waiting for seconds.
 constexpr long long WAIT_CYCLES_DEFAULT = 4000000000ll;
 __constant__ long long c_wait_cycles = WAIT_CYCLES_DEFAULT;
-// Test hook: index b * N + node of a published-weight slot that the every-node kernel leaves pending (-1: none)
+// Test hook: index b * N + node of a published-weight slot that the node kernels leave pending (-1: none)
 __constant__ int c_hold_slot = -1;
 #define WAIT_CYCLES c_wait_cycles
 constexpr unsigned long long W_PENDING = 0xFFFFFFFFFFFFFFFFull;

@@ -50,9 +50,10 @@ struct NParams {
     float *an_div;            // [B,N,3] L1, KL(p||q), KL(q||p)
 };
 
-// A sum of fp32 exponentials is good to 2.4e-7 of the mass where one token may hold most of it, and to less than half of that
-// where none holds more than a quarter (LIST_FLAT_Z); a node's weight S / (S + 1 - w) to that over S + 1 - w.  So
-// fp32 sums are used on flat rows only, and only while S + 1 - w is above this.
+// A sum of fp32 exponentials, fp64 above a thread's chunk of 8, is off by at most 2^-22 + 3 2^-24 = 4.2e-7 of the mass.  Measured
+// against fp64 (V = 6080 to 262144): 2.9e-7 where one token may hold most of it, 8.6e-8 where none holds more than a
+// quarter (LIST_FLAT_Z).  A node's weight S / (S + 1 - w) is off by that over S + 1 - w.  So fp32 sums are used on
+// flat rows only, and only while S + 1 - w is above this (bound 8.4e-6 in the weight).
 constexpr double SMALL_STEP = 0.05;
 __device__ __forceinline__ bool flat_rows(double Z_p, double Z_q) { return Z_p > LIST_FLAT_Z && Z_q > LIST_FLAT_Z; }
 constexpr int FEW_SEQS = 2048;        // nodes whose child counts a cluster looks at in one go
@@ -175,13 +176,14 @@ __device__ __noinline__ void leaf_record(const VParams &P, const RowPart *part, 
 // ------------------------------------------------------------------------------------------------
 // nodes with one child
 // ------------------------------------------------------------------------------------------------
-// Sums of NT threads (a CTA, or a warp) over their share of a node's two rows, which come through a ring in shared memory: every thread copies and reads
-// its own chunks, NS - 1 of them ahead (one chunk ahead in registers, a pass of one CTA over V = 128256 took 33 us, nearly all of
-// it the latency of L2).
+// Sums of NT threads (a CTA, or a warp) over their share of a node's two rows, which come through a ring in shared memory:
+// every thread copies and reads its own chunks, NS - 1 of them ahead (one chunk ahead in registers, a pass of one CTA over
+// V = 128256 took 33 us, nearly all of it the latency of L2).
 // Kinds of sums: SUM_STEP o[0] = sum (g e_p - e_q)+ in fp32; SUM_STEP_HEAVY the same and SUM_NORM the rows' normalisers (o[0],
 // o[1]) with the tokens above 2^-DOM_S of a row's mass (at most 1024 per row, about 120 on the synthetic logits) in fp64
-// and the others in fp32, whose share of the error is then below 1e-8 of the mass.  They are collected per warp and
-// evaluated 32 at a time.
+// and the others in fp32.  Each of those is good to 2^-22 of itself, so their sum to 2.4e-7 of their share of the mass; they are at
+// least as many as 1024 times that share and round by themselves, so 2^-22 / 32 = 7e-9 is its usual size.  The heavy ones
+// are collected per warp and evaluated 32 at a time.
 enum SumKind { SUM_STEP, SUM_STEP_HEAVY, SUM_NORM };
 constexpr int DOM_S = 10;
 template <int DT> constexpr int NS = DT == SPEC_BF16 ? 4 : 3;                                  // stages of the ring

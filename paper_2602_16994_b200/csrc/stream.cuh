@@ -4,9 +4,9 @@
 // the asynchronous copies of the next slices in flight while the current one is exponentiated.
 //
 // A thread turns its logits into e = 2^(z s - o) (s = log2(e)/T, o = ceil of its own largest z s, an
-// integer, so partial sums combine by exact powers of two) and the CTA writes, for its slice,
+// integer, so partial sums combine by exact powers of two) and the CTA writes, for its row or part of one,
 //     O = largest o, S = sum e 2^(o - O), X = sum e x 2^(o - O) with x = z s - O, the largest exponent.
-// The walk kernel merges the slices of a row when it needs the row's normaliser.
+// Rows in parts (batches with fewer rows than half the places) are merged by spec_row_merge_kernel.
 #pragma once
 #include "common.cuh"
 

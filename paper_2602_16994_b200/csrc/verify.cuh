@@ -12,10 +12,10 @@
 // in registers, the others in shared memory; nothing is written back to HBM.
 //
 // A node on chip is a chain of short dependent phases (load, exponentials, a few sweeps, each ended by a sum over the
-// cluster), so it is bound by latency, not by bandwidth or arithmetic.  Hence: every consumer thread loads its own
-// logits, all of them at once (a ring filled by a producer warp kept 3 of 9 tiles in flight and cost a wait and a
-// hand-back per tile: 5 us for the first pass at V = 128256, 2 us now); 16 consumer warps where one CTA has an SM to
-// itself (a sweep is 32 logits per thread), 8 where two share it.
+// cluster), so it is bound by latency, not by bandwidth or arithmetic.  Hence every consumer thread loads its own
+// logits, three chunks ahead of the one it works on (a ring filled by a producer warp kept 3 of 9 tiles in flight and cost a
+// wait and a hand-back per tile: 5 us for the first pass at V = 128256, 2 us now).  All kernels have 8 warps: 8 consumers, or
+// 7 and a helper warp (spec_recursion_kernel).
 //
 // The recursion is the paper's own, step by step.  A node's state after j rejected children is the
 // residual law P_j with P_0 = p, held as u_j(t) = kappa_j P_j(t) in place of the resident e_p:
