@@ -6,22 +6,29 @@
 // the cut is set aside as a CANDIDATE:
 //   top-k        bound = the k-th largest of the units' maxima in the first slice (each is a logit of the row, so
 //                at least k logits lie at or above it), tightened to the k-th largest candidate so far a few times;
-//   top-p alone  the mass of the whole row, which fixes the target, is summed in the same pass; bf16: bound = the cut
-//                that the first slice alone would have at a larger top-p (a guess: the end of the row tells whether
-//                the nucleus stayed above it); fp32: WINDOW_OCTAVES below the row's running maximum.
-// One packed maximum per 16-byte unit finds the units that hold a candidate; a warp lists those of its share of a
-// slice and then looks at their logits, a logit per lane, in the ring.  bf16 candidates become counts in a histogram over logit VALUES (a bf16 logit has 16 bits: 20 octaves of
+//   top-p alone  the mass of the whole row, which fixes the target, is summed in the same pass; bf16: bound = the cut that the first
+//                slices alone would have at a larger top-p, after 1, 4 and 16 of them (a guess: the end of the row tells
+//                whether the nucleus stayed above it); fp32: WINDOW_OCTAVES below the row's running maximum.
+// bf16 candidates become counts in a histogram over logit VALUES (a bf16 logit has 16 bits: 20 octaves of
 // magnitude, both signs, are 5120 bins), from which both cuts and all kept sums follow: the mass of a bin is
 // its count times the mass of its value, and no number of candidates overflows it.  fp32 candidates become a
-// list of keys (4096 entries) for a radix selection.  Where the first slice says that more than DENSE of the row are
-// candidates (T near 1 with top-p near 1: a quarter of it) every logit is compared and counted on the spot.
+// list of keys (4096 entries) for a radix selection.
+// How candidates are found: top-k (a few hundred per row) and fp32: one packed maximum per 16-byte unit finds the units that hold one;
+// a warp lists those of its share of a slice and then looks at their logits, a logit per lane, in the ring.  bf16 top-p, with a
+// few per cent of candidates or (T near 1 with top-p near 1) a quarter of the row: all logits of a unit that holds
+// one anywhere in the warp are counted, without a branch (count_unit).
 // A bf16 nucleus that reaches below the bound is counted again from L2, down to one that the row's mass guarantees.
 // What is left over (fp32 nuclei beyond the list, k above 1024 (fp32: 256), values outside the 20 octaves) runs an adaptive
 // radix selection over the row in L2, in the same CTA.
 //
-// Bound by HBM for large batches.  The ring runs ahead across rows, so the copies of the next row are in flight
-// while the selection of the current one (a few microseconds of block-wide scans) runs.
+// top-k is bound by HBM for large batches; the ring runs ahead across rows, so the copies of the next row are in flight
+// while the selection of the current one (a few microseconds of scans) runs.  top-p is bound by instructions: per logit 4.4 for its mass,
+// 2.5 where it is counted, about 5 for ring, maxima and tests.  Row statistics of 2368 rows of 151936 (T 0.6, top-p 0.95): 341 -> 286 us;
+// 272 rows of 128256 (T 1, top-p 0.99, nuclei of 30000): 97 -> 51 us, since every logit of a slice is counted by
+// multiply-adds and not by branches, and the bound rises as the row goes by.
 #pragma once
+#include <cuda_bf16.h>
+
 #include "common.cuh"
 #include "cut.cuh"
 #include "stream.cuh"
@@ -34,12 +41,11 @@ constexpr int NW = NT / 32;
 constexpr int UN = 4;                // 16-byte units per thread and slice
 constexpr int DEPTH = 3;             // stages of the ring, one slice each
 constexpr int NB = cut::NB;          // bins of a radix level
-constexpr int PER = NB / NT;
 constexpr int CAP = 4096;            // fp32: candidate keys per row
 constexpr float WINDOW_OCTAVES = 14.f;
 constexpr float SAMPLE_OCTAVES = 24.f;   // bf16 top-p: how far below its maximum the first slice is counted
-constexpr float SAMPLE_REST = 0.7f;      // safety factor of the bound it gives (mass_bound)
-constexpr float DENSE = 0.008f;           // share of candidates above which a list of units costs more than counting all
+constexpr float SAMPLE_REST = 0.7f;      // safety factor of the bounds from a part of the row (mass_bound)
+constexpr float UNSET = -2.0e9f;
 constexpr float LOWEST = -3.3e38f;   // a bound that every finite logit passes and -inf does not
 template <int DT> constexpr int K_FAST = DT == SPEC_BF16 ? UN * NT : NT;      // largest top-k the first slice can bound
 
@@ -48,6 +54,7 @@ template <int DT> constexpr int K_FAST = DT == SPEC_BF16 ? UN * NT : NT;      //
 constexpr int TB = 20 * 128;
 constexpr int M0 = (127 - 11) << 7;
 constexpr float HIGH = 508.f;                 // below the outermost bin's value
+constexpr int PLAIN_KEY = M0 + 33;            // the smallest value that has 32 values with bins of their own below it, as bits
 constexpr int ODD_LOW = 1, ODD_HIGH = 2;      // a candidate in such a shared bin (other than 0) was seen
 
 struct RParams {
@@ -72,9 +79,9 @@ struct __align__(16) Shared {
     Scale sc;
     unsigned long long warp_tot[NW];
     double red[NW][2];
-    int verdict;               // bf16: what the selecting warp found (below)
-    float bound;               // top-k: the bound it set
-    double total;              // mass of the row in units of its largest e
+    int verdict;               // bf16: what a selecting warp found, or see mass_bound
+    float bound;               // fp32 top-p: the block's bound
+    unsigned inner[SPEC_MAX_NODES / 32];       // one tree for all: its nodes with children
     uint32_t runmax;           // key of the largest logit seen by the row so far
     int count;                 // fp32: candidates appended (may exceed CAP: overflow)
     int odd;
@@ -83,14 +90,15 @@ struct __align__(16) Shared {
 };
 template <int DT> struct Layout {
     static constexpr int RING = DEPTH * UN * NT * 16;
-    static constexpr int HITS = NW * UN * 32;            // a byte per unit of a warp's share of a slice
+    // a byte per unit of a warp's share of a slice; bf16 top-p: a word per lane (count_unit)
+    static constexpr int HITS = NW * UN * 32;
     // bf16: counts of 2 TB values; fp32: a radix histogram (64-bit bins as two words) and the candidate keys
     static constexpr int BINS = DT == SPEC_BF16 ? 2 * TB * 4 : NB * 8 + CAP * 4;
     static constexpr int BYTES = RING + HITS + BINS + (int)sizeof(Shared);
 };
 static_assert(2 * TB * 4 >= NB * 8, "the radix histogram of the slow path fits in the value bins");
 template <int DT> constexpr int CTAS = DT == SPEC_BF16 ? 3 : 2;       // per SM
-static_assert(Layout<SPEC_BF16>::BYTES <= (227 * 1024) / 3 - 1024 && Layout<SPEC_F32>::BYTES <= 113 * 1024, "CTAs per SM");
+static_assert(Layout<SPEC_BF16>::BYTES <= (228 * 1024) / 3 - 1024 && Layout<SPEC_F32>::BYTES <= 113 * 1024, "CTAs per SM");
 
 // e 2^44 truncated to an integer, for e = 2^x in [0, 2): integer arithmetic on the bits of the float
 // (the same value as casting the exact product (double)e * 2^44 to an unsigned integer)
@@ -128,36 +136,67 @@ __device__ __forceinline__ int last_bin_above(float bound)
     if (b == TB || b == TB - 1) return bound <= 0.f ? b : b - 1;
     return (bound > 0.f && value_of_bin(b) < bound) ? b - 1 : b;
 }
+// bf16 values as integers in their order, -0 and +0 alike: the smallest that is at or above `bound` (one above -inf)
+__device__ __forceinline__ int bound_key(float bound)
+{
+    const uint32_t u = __float_as_uint(bound);
+    const int mag = (int)(u >> 16) & 0x7FFF;
+    if (!(u >> 31)) return mag + ((u & 0xFFFFu) ? 1 : 0);
+    return mag ? -1 - mag : 0;
+}
+// What the counting of bf16 logits needs to know about a bound.
+struct Counter {
+    int kb;                    // the bound as a key
+    // the bound and the 32 keys below it are positive values with bins of their own
+    __device__ __forceinline__ bool plain() const { return kb >= PLAIN_KEY; }
+    // whether a unit with these maxima holds a candidate
+    __device__ __forceinline__ bool reaches(uint32_t max_pair) const
+    {
+        const uint32_t pair = (uint32_t)(kb >= 0 ? kb : 0x8000 | (-1 - kb)) * 0x10001u;
+        return __hge2_mask(reinterpret_cast<const __nv_bfloat162 &>(max_pair), reinterpret_cast<const __nv_bfloat162 &>(pair)) != 0u;
+    }
+};
+// Counts the 8 logits of a bf16 unit that are at or above the bound.  Every lane adds to some word for each of its logits: an
+// addition under a predicate is a branch to the compiler, and a slice of 8192 logits then takes 1310 cycles with no candidate
+// and 2150 with 9 to 49 % of them (one CTA of 8 warps on an SM); without, 675 and 760 to 900.
+// plain, and no logit of the unit reaches HIGH: positive values order like their bits, so a logit below the bound is raised to one of
+// the 32 keys below it, whose bins nobody reads any more (bounds only rise), and a pair of logits takes one maximum,
+// two multiply-adds and the two additions.
+__device__ __forceinline__ void count_unit(const Counter &C, uint32_t bins, uint32_t dump, int *odd, const uint4 &r, bool plain)
+{
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+    if (plain) {
+        const int base = (int)bins + (TB - 1 + M0) * 4;
+        const uint32_t floor = (uint32_t)(C.kb - 1 - (int)(threadIdx.x & 31)) * 0x10001u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            uint32_t v;
+            asm("max.s16x2 %0, %1, %2;" : "=r"(v) : "r"(w[k]), "r"(floor));
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(__dp2a_lo((int)v, 0x00FC, base)));        // base - 4 low half
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(__dp2a_lo((int)v, 0xFC00, base)));        // base - 4 high half
+        }
+    } else {
+        int seen = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int v = (k & 1) ? (int)w[k >> 1] >> 16 : (int)(short)w[k >> 1];
+            int key = v ^ ((v >> 31) & 0x7FFF);
+            key += key == -1 ? 1 : 0;
+            const int mag = key < 0 ? -1 - key : key;
+            const int b = key >= 0 ? max(min(TB - 1 + M0 - key, TB - 1), 0) : min(max(TB - M0 + mag, TB), 2 * TB - 1);
+            if (key >= C.kb) seen |= (mag - 1 < M0 && mag > 0 ? ODD_LOW : 0) | (mag >= M0 + TB - 1 ? ODD_HIGH : 0);
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(key >= C.kb ? bins + 4u * (uint32_t)b : dump));
+        }
+        if (seen) atomicOr(odd, seen);
+    }
+}
+
 __device__ __forceinline__ void count_value(uint32_t *cnt, int *odd, uint32_t u16)
 {
     int t;
     const int b = bin_of(u16, t);
     if ((unsigned)(t - 1) >= (unsigned)(TB - 2) && (u16 & 0x7FFFu)) atomicOr(odd, t ? ODD_HIGH : ODD_LOW);
     atomicAdd(&cnt[b], 1u);
-}
-// The 8 logits of a bf16 unit that are at or above the bound.  zmax: none is larger.
-__device__ __forceinline__ void count_unit(uint32_t *cnt, int *odd, const uint4 &r, float bound, float zmax)
-{
-    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-    const int b16 = (int)(__float_as_uint(bound) >> 16) + ((__float_as_uint(bound) & 0xFFFFu) ? 1 : 0);
-    if (bound > 0.f && b16 >= M0 && zmax < HIGH) {
-        // Positive values order like their bits and none of these falls into a shared bin: four instructions a logit
-        // (written out: the compiler makes a branch of the predicated addition, twice as many).
-        const uint32_t base = smem_u32(cnt) + (uint32_t)(TB - 1 + M0) * 4u;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int v = (k & 1) ? (int)w[k >> 1] >> 16 : (int)(short)w[k >> 1];
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.ge.s32 p, %0, %1;\n\t@p red.shared.add.u32 [%2], 1;\n\t}" ::"r"(v), "r"(b16),
-                         "r"(base - 4u * (uint32_t)v)
-                         : "memory");
-        }
-    } else {
-        float z[8];
-        stream::unpack_unit<SPEC_BF16>(r, z);
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (z[k] >= bound) count_value(cnt, odd, __float_as_uint(z[k]) >> 16);
-    }
 }
 
 // The first of the bins b0 .. b1 at which the running sum of weight(bin) reaches `target`, by one warp, 128 bins per
@@ -198,47 +237,39 @@ __device__ __forceinline__ int warp_find(int b0, int b1, double target, F weight
 }
 
 // The first of the bins b0 .. b1 at which the running sum of weight(bin) reaches `target`; -1 when the total
-// stays below.  before: the sum of the bins ahead of it.  All threads of the block call it and get the answer.
-template <typename F>
-__device__ __forceinline__ int find_bin(Shared &S, int b0, int b1, double target, unsigned long long &before, F weight)
+// stays below.  before: the sum of the bins ahead of it.  All threads of the block call it and get the answer.  Every thread takes a run
+// of an odd number of bins (consecutive lanes then read different banks) and goes through it a second time where the target lies in it.
+template <typename T, typename F>
+__device__ __forceinline__ int find_bin(Shared &S, int b0, int b1, double target, T &before, F weight)
 {
+    static_assert(sizeof(T) <= 8, "fits the slot");
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    unsigned long long carry = 0;
-    int found = -1;
-    before = 0;
-    for (int base = b0; base <= b1 && found < 0; base += NT * PER) {
-        unsigned long long loc[PER], lsum = 0;
+    const int per = ((b1 - b0) / NT + 1) | 1, i0 = b0 + tid * per, i1 = min(i0 + per - 1, b1);
+    T sum = 0;
+    for (int i = i0; i <= i1; ++i) sum += weight(i);
+    T incl = sum;
 #pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            const int b = base + tid * PER + k;
-            loc[k] = b <= b1 ? weight(b) : 0ull;
-            lsum += loc[k];
-        }
-        unsigned long long incl = lsum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        __syncthreads();
-        if (lane == 31) S.warp_tot[w] = incl;
-        if (tid == 0) S.sel_bin = -1;
-        __syncthreads();
-        unsigned long long ahead = carry;
-        for (int k = 0; k < NW; ++k) { const unsigned long long t = S.warp_tot[k]; carry += t; if (k < w) ahead += t; }
-        unsigned long long run = ahead + incl - lsum;
-        if ((double)run < target && (double)(run + lsum) >= target) {
-#pragma unroll
-            for (int k = 0; k < PER; ++k) {
-                if ((double)run < target && (double)(run + loc[k]) >= target) { S.sel_bin = base + tid * PER + k; S.sel_before = run; }
-                run += loc[k];
-            }
-        }
-        __syncthreads();
-        found = S.sel_bin;
-        before = S.sel_before;
+    for (int o = 1; o < 32; o <<= 1) {
+        const T t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
     }
-    return found;
+    T *tot = reinterpret_cast<T *>(S.warp_tot), *sel = reinterpret_cast<T *>(&S.sel_before);
+    __syncthreads();
+    if (lane == 31) tot[w] = incl;
+    if (tid == 0) { S.sel_bin = -1; *sel = 0; }
+    __syncthreads();
+    T run = incl - sum;
+    for (int k = 0; k < w; ++k) run += tot[k];
+    if ((double)run < target && (double)(run + sum) >= target) {
+        for (int i = i0; i <= i1; ++i) {
+            const T x = weight(i);
+            if ((double)(run + x) >= target) { S.sel_bin = i; *sel = run; break; }
+            run += x;
+        }
+    }
+    __syncthreads();
+    before = *sel;
+    return S.sel_bin;
 }
 
 __device__ __forceinline__ unsigned long long block_sum(Shared &S, unsigned long long v)
@@ -284,8 +315,8 @@ __device__ __forceinline__ bool radix_select(Shared &S, uint32_t *lo, uint32_t *
         });
         __syncthreads();
         unsigned long long before;
-        const int bin = find_bin(S, 0, (int)(range >> sh), need - above, before,
-                                 [&](int b) { return ((unsigned long long)hi[b] << 32) | lo[b]; });
+        const int bin = find_bin<unsigned long long>(S, 0, (int)(range >> sh), need - above, before,
+                                                     [&](int b) { return ((unsigned long long)hi[b] << 32) | lo[b]; });
         if (bin < 0) return false;
         above += (double)before;
         khi -= (uint32_t)bin << sh;
@@ -395,27 +426,43 @@ template <int DT> struct Smem {
     uint32_t *bins, *keys;       // keys: fp32 only
     Shared &S;
     __device__ __forceinline__ Smem()
-        : ring(reinterpret_cast<uint4 *>(dyn_smem)), hits(dyn_smem + Layout<DT>::RING + (threadIdx.x >> 5) * UN * 32),
+        : ring(reinterpret_cast<uint4 *>(dyn_smem)),
+          hits(dyn_smem + Layout<DT>::RING + (threadIdx.x >> 5) * UN * 32),
           bins(reinterpret_cast<uint32_t *>(dyn_smem + Layout<DT>::RING + Layout<DT>::HITS)), keys(bins + 2 * NB),
           S(*reinterpret_cast<Shared *>(dyn_smem + Layout<DT>::RING + Layout<DT>::HITS + Layout<DT>::BINS)) {}
+    __device__ __forceinline__ void count(const Counter &c, const uint4 &r, bool plain) const { count_unit(c, smem_u32(bins), smem_u32(hits) + (threadIdx.x & 31) * 4, &S.odd, r, plain); }
 };
 
+// row / N and row % N for row < 2^24
+struct Split {
+    int b, a;
+    __device__ __forceinline__ Split(int row, int N, float inv)
+    {
+        b = (int)((float)row * inv);                 // (off by one at most)
+        a = row - b * N;
+        if (a < 0) { --b; a += N; }
+        if (a >= N) { ++b; a -= N; }
+    }
+};
 // The first item from `id` on, in steps of the grid, whose row is read: every target row, the draft rows of nodes with
-// children (every warp finds out by itself).
-__device__ __noinline__ int next_read(const RParams &P, int id, int items)
+// children (one tree for all: from the block's list; else every warp finds out by itself).
+__device__ __noinline__ int next_read(const RParams &P, int id, int items, const unsigned *inner)
 {
+    const float inv = 1.f / (float)P.N;
     for (; id < items; id += gridDim.x) {
         if ((id & 1) == 0) break;
-        const int row = id >> 1;
-        if (P.parent && stream::has_children(P.parent + (row / P.N) * P.topo_stride, P.N, row % P.N, threadIdx.x & 31)) break;
+        if (!P.parent) continue;
+        const Split r(id >> 1, P.N, inv);
+        if (P.topo_stride == 0 ? (inner[r.a >> 5] >> (r.a & 31)) & 1u
+                               : stream::has_children(P.parent + r.b * P.topo_stride, P.N, r.a, threadIdx.x & 31)) break;
     }
     return id;
 }
 template <int DT>
 __device__ __forceinline__ stream::RowSpan span_of(const RParams &P, int id)
 {
-    const int row = id >> 1;
-    return stream::row_span<DT>((id & 1) ? P.zq : P.zp, (row / P.N) * P.seq_stride + (row % P.N) * P.node_stride, P.V);
+    const Split r(id >> 1, P.N, 1.f / (float)P.N);
+    return stream::row_span<DT>((id & 1) ? P.zq : P.zp, r.b * P.seq_stride + r.a * P.node_stride, P.V);
 }
 
 // top-k: a bound from the first slice (the k-th largest of its units' maxima mu; fp32: of the threads' maxima), or
@@ -499,78 +546,128 @@ __device__ __noinline__ float tighter_bound(int top_k, float bound)
     return bound;
 }
 
-// bf16 top-p: a bound from the n logits seen so far, whose candidates are in the bins down to `loose` (all threads
-// have put theirs there): the cut these alone would have at a larger top-p.  m: their maximum; set / of / Sd: the
-// thread's reference and sum of e.  Returns the bound; S.verdict: whether to count densely from it.
-__device__ __noinline__ float mass_bound(float m, float loose, bool set, float of_t, double Sd, float top_p, float sf, double s_d, int n, int V)
+// bf16 top-p: a bound from the n logits seen so far, whose candidates are in the bins down to `bound`: where the tokens below it, taken
+// for the whole row, would together fall short of 1 - top_p of the mass seen so far (SAMPLE_REST of it).  That mass only
+// grows, so the guess fails only where the first part of a row holds fewer of its light tokens than the rest; it
+// gets better as V / n goes to 1, hence it is made again after 4 and 16 slices.  All threads of the block; tmax, of, Sd: what the
+// thread has seen (Pass).  S.verdict = 1: the bins hold so little of the mass seen so far that the cut can't be expected above `bound`.
+__device__ __noinline__ float mass_bound(float tmax, float bound, float of, double Sd, float top_p, int n, int V)
 {
     const Smem<SPEC_BF16> M;
     Shared &S = M.S;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int o_t = set ? (int)of_t : ROWPART_EMPTY;
+    const float sf = S.sc.sf;
+    const int o_t = of > UNSET ? (int)of : ROWPART_EMPTY;
     const int O_w = __reduce_max_sync(0xffffffffu, o_t);
     const double Sw = warp_sum(Sd * (double)pow2i(max(o_t - O_w, -127)));
-    if (lane == 0) { S.red[w][0] = Sw; S.red[w][1] = (double)O_w; }
-    __syncthreads();
-    if (w == 0) {
-        const int Ok = lane < NW ? (int)S.red[lane][1] : ROWPART_EMPTY;
-        const int Om = __reduce_max_sync(0xffffffffu, Ok);
-        double total = warp_sum(lane < NW ? S.red[lane][0] * (double)pow2i(max(Ok - Om, -127)) : 0.0);
-        total *= (double)exp2f((float)((double)Om - (double)m * s_d));
-        const int b_max = bin_of(m), b_lo = last_bin_above(loose);
-        const int kb = warp_find<unsigned long long>(b_max, b_lo, (1.0 - (double)(SAMPLE_REST * (float)n / (float)V) * (1.0 - (double)top_p)) * total * cut::FIX, [&](int i) {
-            const unsigned long long c = M.bins[i];
-            return c ? c * fix44(ex2_approx((value_of_bin(i) - m) * sf)) : 0ull;
-        });
-        uint32_t c = 0;
-        for (int i = b_max + lane; i <= (kb >= 0 ? kb : b_lo); i += 32) c += M.bins[i];
-        c = __reduce_add_sync(0xffffffffu, c);
-        if (lane == 0) {
-            S.bound = kb >= 0 && kb != TB && kb != TB - 1 ? value_of_bin(kb) : loose;
-            S.verdict = (float)c > DENSE * (float)n ? 1 : 0;
-        }
-    }
-    __syncthreads();
-    return S.bound;
-}
-// the maximum of the block's logits so far, from the threads' maxima
-__device__ __forceinline__ float block_max(Shared &S, float ms)
-{
-    const uint32_t km = __reduce_max_sync(0xffffffffu, cut::key_of(ms));
-    if ((threadIdx.x & 31) == 0) atomicMax(&S.runmax, km);
-    __syncthreads();
-    return cut::value_of(S.runmax);
-}
-// the first slice (r0 .. r3, beyond the row: -inf) into the bins, and the first bound from it
-__device__ __noinline__ float sample_bound(const uint4 r0, const uint4 r1, const uint4 r2, const uint4 r3, float ms, bool set,
-                                           float of_t, double Sd, float top_p, int n, int V)
-{
-    const Smem<SPEC_BF16> M;
-    Shared &S = M.S;
-    const float m = block_max(S, ms);
-    const float sf = S.sc.sf;
-    const double s_d = S.sc.s_d;
+    const uint32_t km = __reduce_max_sync(0xffffffffu, cut::key_of(tmax));
+    if (lane == 0) { S.red[w][0] = Sw; S.red[w][1] = __hiloint2double((int)km, O_w); }
+    __syncthreads();                                  // all candidates so far are in
+    const double part = S.red[lane & (NW - 1)][1];
+    const float m = cut::value_of(__reduce_max_sync(0xffffffffu, (uint32_t)__double2hiint(part)));
     if (!(m > -CUDART_INF_F && m < CUDART_INF_F)) {       // nothing finite so far, or a row that will be reported
+        __syncthreads();                              // (the partials may be written again)
         if (threadIdx.x == 0) S.verdict = 1;
         __syncthreads();
-        return LOWEST;
+        return bound;
     }
-    const float loose = fmaxf(m - SAMPLE_OCTAVES / sf, LOWEST);
-    count_unit(M.bins, &S.odd, r0, loose, ms);
-    count_unit(M.bins, &S.odd, r1, loose, ms);
-    count_unit(M.bins, &S.odd, r2, loose, ms);
-    count_unit(M.bins, &S.odd, r3, loose, ms);
-    return mass_bound(m, loose, set, of_t, Sd, top_p, sf, s_d, n, V);
+    const int Ok = __double2loint(part), Om = __reduce_max_sync(0xffffffffu, Ok);
+    double total = lane < NW ? S.red[lane][0] * (double)pow2i(max(Ok - Om, -127)) : 0.0;
+    total = warp_sum(total) * (double)exp2f((float)((double)Om - (double)m * S.sc.s_d));
+    const double need = (1.0 - (double)(SAMPLE_REST * (float)n / (float)V) * (1.0 - (double)top_p)) * total;
+    const auto mass = [&](int i) {
+        const uint32_t c = M.bins[i];
+        return c ? (double)((float)c * ex2_approx((value_of_bin(i) - m) * sf)) : 0.0;
+    };
+    double before;
+    const int b1 = last_bin_above(bound);
+    const int kb = find_bin<double>(S, bin_of(m), b1, need, before, mass);
+    if (kb < 0) {
+        const int enough = find_bin<double>(S, bin_of(m), b1, (1.0 - 0.5 * (1.0 - (double)top_p)) * total, before, mass);
+        if (threadIdx.x == 0) S.verdict = enough < 0 ? 1 : 0;
+        __syncthreads();
+    }
+    return kb > 0 && kb < 2 * TB - 1 && kb != TB && kb != TB - 1 ? fmaxf(bound, value_of_bin(kb)) : bound;
+}
+// How far down the first slice matters; ms: the thread's maximum.
+__device__ __forceinline__ float sample_floor()
+{
+    const Smem<SPEC_BF16> M;
+    const float m = cut::value_of(M.S.runmax);
+    return m > -CUDART_INF_F && m < CUDART_INF_F ? fmaxf(m - SAMPLE_OCTAVES / M.S.sc.sf, LOWEST) : LOWEST;
+}
+__device__ __noinline__ float sample_bound(float ms)
+{
+    const Smem<SPEC_BF16> M;
+    const uint32_t km = __reduce_max_sync(0xffffffffu, cut::key_of(ms));
+    if ((threadIdx.x & 31) == 0) atomicMax(&M.S.runmax, km);
+    if (threadIdx.x == 0) M.S.verdict = 0;
+    __syncthreads();
+    return sample_floor();
+}
+// The first bound, from the first slice alone.  Of a row of several slices only positive logits have been counted: a cut below zero
+// keeps more than half of a row of logits around zero.  Where they hold too little of the mass, the slice is counted again, from the
+// ring (stage: the warp's share), all of it that matters.
+__device__ __noinline__ float first_mass_bound(float tmax, float bound, float of, double Sd, float top_p, int n, int V, const uint4 *stage)
+{
+    const Smem<SPEC_BF16> M;
+    const float b = mass_bound(tmax, bound, of, Sd, top_p, n, V);
+    if (!M.S.verdict) return b;
+    const float loose = sample_floor();
+    const Counter cnt{bound_key(loose)};
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * TB / 4; i += NT) reinterpret_cast<uint4 *>(M.bins)[i] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    for (int c = 0; c < UN; ++c) M.count(cnt, stage[c * NT + (threadIdx.x & 31)], false);
+    return mass_bound(tmax, loose, of, Sd, top_p, n, V);
 }
 
-// what the pass over a row leaves in a thread
+// units of which some logits may be negative, or reach HIGH
+__device__ __noinline__ void count_pair(const Counter cnt, const uint4 r0, const uint4 r1)
+{
+    const Smem<SPEC_BF16> M;
+    M.count(cnt, r0, false);
+    M.count(cnt, r1, false);
+}
+
+// what the pass over a row leaves in a thread (UNSET: no reference yet)
 struct Pass {
     float tmax;                // the thread's maximum (NaN if it saw one)
     float of;                  // its integer reference, and its sum of e in units of 2^of (TOTAL)
     double Sd;
-    bool set;
     float bound;               // the row is complete from it upwards (fp32 top-p: from the window upwards)
 };
+
+// Adds n units to the row's mass, as in the streaming statistics kernel: a running integer reference per thread, fp32 sums (a chain of
+// additions per unit), fp64 above.  ms: the units' maximum.
+template <int DT, int NU>
+__device__ __forceinline__ void add_mass(const uint4 (&raw)[NU], float ms, float s_hi, float s_lo, Pass &ps)
+{
+    constexpr int E = DT == SPEC_BF16 ? 8 : 4;
+    if (!(ms > -CUDART_INF_F && ms < CUDART_INF_F)) return;
+    const float onew = fminf(fmaxf(ceilf(ms * s_hi), -1.0e9f), 1.0e9f);
+    if (onew > ps.of) { ps.Sd *= (double)pow2i((int)fmaxf(ps.of - onew, -127.f)); ps.of = onew; }
+    const unsigned long long sh2 = pack_f32x2(s_hi, s_hi), sl2 = pack_f32x2(s_lo, s_lo), no2 = pack_f32x2(-ps.of, -ps.of);
+    unsigned long long sum = 0ull;
+#pragma unroll
+    for (int c = 0; c < NU; ++c) {
+        float z[E];
+        stream::unpack_unit<DT>(raw[c], z);
+        unsigned long long acc = 0ull;
+#pragma unroll
+        for (int k = 0; k < E; k += 2) {
+            const unsigned long long z2 = pack_f32x2(z[k], z[k + 1]);
+            float x0, x1;
+            unpack_f32x2(fma_f32x2(z2, sl2, fma_f32x2(z2, sh2, no2)), x0, x1);
+            const unsigned long long e2 = pack_f32x2(ex2_approx(x0), ex2_approx(x1));
+            acc = k == 0 ? e2 : add_f32x2(acc, e2);
+        }
+        sum = c == 0 ? acc : add_f32x2(sum, acc);
+    }
+    float a0, a1;
+    unpack_f32x2(sum, a0, a1);
+    ps.Sd += (double)(a0 + a1);
+}
 
 // The row's statistics from what the pass has set aside; leaves bins and counters as the next row wants them.
 template <int DT, bool TOTAL>
@@ -600,7 +697,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
         int O_w = 0;
         double Sw = 0.0;
         if (TOTAL) {
-            const int o_t = ps.set ? (int)ps.of : ROWPART_EMPTY;
+            const int o_t = ps.of > UNSET ? (int)ps.of : ROWPART_EMPTY;
             O_w = __reduce_max_sync(0xffffffffu, o_t);
             Sw = warp_sum(ps.Sd * (double)pow2i(max(o_t - O_w, -127)));
         }
@@ -626,13 +723,12 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             __syncthreads();
             return;
         }
-        if (TOTAL && (DT == SPEC_F32 || w == 0)) {
+        if (TOTAL) {
             const int Om = __reduce_max_sync(0xffffffffu, Ok);
             total = warp_sum(lane < NW ? S.red[lane][0] * pow2d(max(Ok - Om, -1000)) : 0.0);
             // from units of 2^Om to units of the row maximum: 2^(Om - m s), Om - m s in [0, 1]
             const double d = (double)Om - (double)m * s_d;
             total *= 1.4142135623730951 * exp2_frac(fmin(fmax(d, 0.0), 1.0) - 0.5);
-            if (lane == 0) S.total = total;
         }
     }
     const double Od = ceil((double)m * s_d);
@@ -648,32 +744,18 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
     bool settled = false;
     if (DT == SPEC_BF16) {
         const int b_max = bin_of(m);
-        // selection, kept sums and record by one warp, from bins that are complete down to b_lo; says whether it
-        // could settle the row
-        auto select = [&](int b_lo) {
-            auto count = [&](int i) { return bins[i]; };
-            auto mass = [&](int i) {
-                const unsigned long long c = bins[i];
-                return c ? c * fix44(ex2_approx((value_of_bin(i) - m) * sf)) : 0ull;
-            };
-            int b_cut = -1;
-            if (TOTAL) {
-                b_cut = warp_find<unsigned long long>(b_max, b_lo, (double)P.top_p * total * cut::FIX, mass);
-            } else if (P.top_k <= K_FAST<DT>) {
-                b_cut = warp_find<uint32_t>(b_max, b_lo, (double)P.top_k, count);
-                if (use_p && b_cut >= 0) {
-                    // the set's mass, exactly: its tokens are all in the bins
-                    unsigned long long part = 0;
-                    for (int i = b_max + lane; i <= b_cut; i += 32) part += mass(i);
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-                    const int b_p = warp_find<unsigned long long>(b_max, b_cut, (double)P.top_p * (double)part, mass);
-                    if (b_p >= 0) b_cut = b_p;       // (else the set itself stays below the target: rounding)
-                }
-            }
-            if (b_cut < 0) return false;
-            // (a shared bin among the kept ones holds values that the bins cannot tell apart)
-            if (fabsf(m) >= HIGH || (S.odd & ODD_HIGH) || ((S.odd & ODD_LOW) && b_cut >= TB - 1)) return false;
+        // Selection, kept sums and record from bins that are complete down to b_lo; says whether that settles the row.  By one warp: the
+        // other CTAs of the SM make better use of the issue slots (by the block: 165 against 151 us on 3008 rows of top-k at V = 128256,
+        // and within 1 us on few rows with wide nuclei).
+        auto mass = [&](int i) {
+            const unsigned long long c = bins[i];
+            return c ? c * fix44(ex2_approx((value_of_bin(i) - m) * sf)) : 0ull;
+        };
+        // (a shared bin among the kept ones holds values that the bins cannot tell apart)
+        auto sound = [&](int b_cut) {
+            return b_cut >= 0 && !(fabsf(m) >= HIGH || (S.odd & ODD_HIGH) || ((S.odd & ODD_LOW) && b_cut >= TB - 1));
+        };
+        auto keep = [&](int b_cut) {
             double Z = 0.0, X = 0.0;
             for (int i = b_max + lane; i <= b_cut; i += 32) {
                 const uint32_t c = bins[i];
@@ -688,31 +770,47 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             Z = warp_sum(Z);
             X = warp_sum(X);
             if (lane == 0) write(Z, X, value_of_bin(b_cut));
-            return true;
         };
-        if (w == 0) {
-            const bool ok = select(last_bin_above(ps.bound));
-            if (lane == 0) S.verdict = ok ? 1 : 0;
-        }
-        __syncthreads();
-        settled = S.verdict != 0;
+        auto select = [&](int b_lo) {
+            __syncthreads();
+            if (w == 0) {
+                int b_cut = -1;
+                if (TOTAL) {
+                    b_cut = warp_find<unsigned long long>(b_max, b_lo, (double)P.top_p * total * cut::FIX, mass);
+                } else if (P.top_k <= K_FAST<DT>) {
+                    b_cut = warp_find<uint32_t>(b_max, b_lo, (double)P.top_k, [&](int i) { return bins[i]; });
+                    if (use_p && b_cut >= 0) {
+                        // the set's mass, exactly: its tokens are all in the bins
+                        unsigned long long part = 0;
+                        for (int i = b_max + lane; i <= b_cut; i += 32) part += mass(i);
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+                        const int b_p = warp_find<unsigned long long>(b_max, b_cut, (double)P.top_p * (double)part, mass);
+                        if (b_p >= 0) b_cut = b_p;       // (else the set itself stays below the target: rounding)
+                    }
+                }
+                const bool ok = sound(b_cut);
+                if (ok) keep(b_cut);
+                if (lane == 0) S.verdict = ok ? 1 : 0;
+            }
+            __syncthreads();
+            return S.verdict != 0;
+        };
+        settled = select(last_bin_above(ps.bound));
         if (TOTAL && !settled) {
-            total = S.total;
             // The nucleus reaches below the bound.  All tokens more than log2(V / ((1 - top_p) total)) octaves
             // below the maximum together have no more than 1 - top_p of the mass: counted again, from L2, down
             // to there.
             const float wide = log2f((float)P.V / ((1.f - P.top_p) * (float)total)) + 0.01f;
             const float bound2 = fmaxf(m - wide / sf, LOWEST);
+            const Counter C{bound_key(bound2)};
+            const bool plain = C.plain() && m < HIGH;
+            __syncthreads();
             clear();
             __syncthreads();
-            visit_units<DT>(span_of<DT>(P, id), [&](const uint4 &r) { count_unit(bins, &S.odd, r, bound2, m); });
+            visit_units<DT>(span_of<DT>(P, id), [&](const uint4 &r) { M.count(C, r, plain); });
             __syncthreads();
-            if (w == 0) {
-                const bool ok = select(last_bin_above(bound2));
-                if (lane == 0) S.verdict = ok ? 1 : 0;
-            }
-            __syncthreads();
-            settled = S.verdict != 0;
+            settled = select(last_bin_above(bound2));
         }
     } else {
         // ---- fp32: radix selection on the list of candidates --------------------------------------------------
@@ -764,9 +862,11 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
         }
     }
     if (!settled) {
+        __syncthreads();
         const Kept kp = settle_from_row<DT>(S, bins, span_of<DT>(P, id), P.V, P.top_k, P.top_p, m, sf, s_hi, s_lo, of, total);
         if (tid == 0) write(kp.Z, kp.X, kp.key ? cut::value_of(kp.key) : -CUDART_INF_F);
     }
+    if (DT == SPEC_BF16) __syncthreads();                // the bins have been read
     clear();
     if (tid == 0) { S.runmax = 0u; S.count = 0; S.odd = 0; }
     __syncthreads();             // the bins, counters and partials are free for the next row
@@ -787,6 +887,14 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
 
     if (DT == SPEC_BF16) for (int i = tid; i < 2 * TB; i += NT) M.bins[i] = 0;
     if (tid == 0) { S.runmax = 0u; S.count = 0; S.odd = 0; }
+    if (P.parent && P.topo_stride == 0) {
+        for (int i = tid; i < (P.N + 31) / 32; i += NT) S.inner[i] = 0u;
+        __syncthreads();
+        for (int c = 1 + tid; c < P.N; c += NT) {
+            const int pa = __ldg(P.parent + c);
+            if (pa >= 0 && pa < c) atomicOr(&S.inner[pa >> 5], 1u << (pa & 31));
+        }
+    }
     __syncthreads();
 
     // ---- the copying side of the ring: DEPTH - 1 slices ahead, across rows ----------------------------------
@@ -796,7 +904,7 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
     bool i_more = true;
     auto issue = [&]() {
         if (i_more && i_left + tid <= 0) {
-            i_id = next_read(P, i_id + gridDim.x, items);
+            i_id = next_read(P, i_id + gridDim.x, items, S.inner);
             i_more = i_id < items;
             if (i_more) {
                 const stream::RowSpan r = span_of<DT>(P, i_id);
@@ -818,14 +926,14 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
     for (int k = 0; k < DEPTH - 1; ++k) issue();
 
     int c_stage = 0;
-    float T_now = 0.f, s_hi = 0.f, s_lo = 0.f, window = 0.f;      // of the current temperature
+    float T_now = 0.f, s_hi = 0.f, s_lo = 0.f;      // of the current temperature
     for (int id = blockIdx.x; id < items; id += gridDim.x) {
         // ---- rows that are not read, up to the next one that is --------------------------------------------------
-        const int to = next_read(P, id, items);
+        const int to = next_read(P, id, items, S.inner);
         for (; id < min(to + 1, items); id += gridDim.x) {
             if (tid == 0) {
                 const int node = id >> 1;
-                if ((id & 1) == 0) P.init.set(node, node / P.N, node % P.N);
+                if ((id & 1) == 0) { const Split r(node, P.N, 1.f / (float)P.N); P.init.set(node, r.b, r.a); }
                 if (id < to) {
                     RowPart r = {};
                     r.cut = -CUDART_INF_F; r.O = ROWPART_EMPTY; r.bad = -1;
@@ -837,7 +945,7 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
         }
         if (id >= items) break;
         const stream::RowSpan row = span_of<DT>(P, id);
-        const float T = P.T_seq ? __ldg(P.T_seq + (id >> 1) / P.N) : P.T;
+        const float T = P.T_seq ? __ldg(P.T_seq + Split(id >> 1, P.N, 1.f / (float)P.N).b) : P.T;
         if (T != T_now) {                      // (the block agrees; the scale factors are next read after a barrier)
             T_now = T;
             const double s_d = 1.4426950408889634 / (double)T;
@@ -846,70 +954,83 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
                 const float sf = 1.4426950408889634f / T;
                 S.sc = Scale{T, sf, s_hi, s_lo, WINDOW_OCTAVES / sf, s_d};
             }
-            window = WINDOW_OCTAVES / (1.4426950408889634f / T);
         }
         // ---- the pass ------------------------------------------------------------------------------------------
-        Pass ps = {-CUDART_INF_F, 0.f, 0.0, false, LOWEST};
-        bool dense = false;                // bf16 top-p: count every logit on the spot
+        Pass ps = {-CUDART_INF_F, UNSET, 0.0, LOWEST};
+        Counter cnt{0};
+        int sure = 0;                      // slices for which the warp takes all its units to hold candidates
         const int nsl = (row.units + NT * UN - 1) / (NT * UN);
         for (int sl = 0; sl < nsl; ++sl) {
-            if (!(DT == SPEC_BF16 && TOTAL) && nsl > sl + 2 && (sl == 2 || sl == 6 || (DT == SPEC_F32 && sl == 16))) {
-                // a better bound, from the slices so far
+            // a better bound, from the slices so far
+            if (DT == SPEC_BF16 && TOTAL) {
+                if ((sl == 4 || sl == 16) && nsl > sl + 2) {
+                    ps.bound = mass_bound(ps.tmax, ps.bound, ps.of, ps.Sd, P.top_p, min(P.V, sl * UN * NT * E), P.V);
+                    cnt.kb = bound_key(ps.bound);
+                    sure = 0;
+                }
+            } else if (nsl > sl + 2 && (sl == 2 || sl == 6 || (DT == SPEC_F32 && sl == 16))) {
                 ps.bound = tighter_bound<DT, TOTAL>(P.top_k, ps.bound);
             }
             stream::cp_async_wait<DEPTH - 2>();
             issue();                                    // into the stage of the previous iteration
             uint4 *const stage = M.ring + c_stage * UN * NT + (tid & ~31);      // the warp's share of the slice
             c_stage = c_stage + 1 == DEPTH ? 0 : c_stage + 1;
-            uint4 raw[UN];
-#pragma unroll
-            for (int c = 0; c < UN; ++c) raw[c] = stage[c * NT + lane];
             if (sl == 0 || sl == nsl - 1) {
 #pragma unroll
                 for (int c = 0; c < UN; ++c) {
-                    stream::mask_unit<DT>(raw[c], (sl * UN + c) * NT + tid, row);
-                    stage[c * NT + lane] = raw[c];
+                    uint4 r = stage[c * NT + lane];
+                    stream::mask_unit<DT>(r, (sl * UN + c) * NT + tid, row);
+                    stage[c * NT + lane] = r;
                 }
             }
-            // the units' maxima (bf16: still as pairs) and the thread's maximum of the slice; a NaN stays
-            uint32_t mu[UN];
-#pragma unroll
-            for (int c = 0; c < UN; ++c) mu[c] = stream::unit_max_raw<DT>(raw[c]);
-            const float ms = stream::fold_max<DT>(stream::max_raw<DT>(stream::max_raw<DT>(mu[0], mu[1]), stream::max_raw<DT>(mu[2], mu[3])));
-            static_assert(UN == 4, "slice maximum of four units");
-            if (TOTAL && ms > -CUDART_INF_F && ms < CUDART_INF_F) {
-                // the row's mass, as in the streaming statistics kernel: a running integer reference per
-                // thread, fp32 sums of a slice's logits, fp64 above
-                const float onew = fminf(fmaxf(ceilf(ms * s_hi), -1.0e9f), 1.0e9f);
-                if (!ps.set) { ps.of = onew; ps.set = true; }
-                else if (onew > ps.of) { ps.Sd *= (double)pow2i((int)fmaxf(ps.of - onew, -127.f)); ps.of = onew; }
-                unsigned long long acc[2] = {0ull, 0ull};
-                const unsigned long long sh2 = pack_f32x2(s_hi, s_hi), sl2 = pack_f32x2(s_lo, s_lo), no2 = pack_f32x2(-ps.of, -ps.of);
-#pragma unroll
-                for (int c = 0; c < UN; ++c) {
-                    float z[E];
-                    stream::unpack_unit<DT>(raw[c], z);
-#pragma unroll
-                    for (int k = 0; k < E; k += 2) {
-                        const unsigned long long z2 = pack_f32x2(z[k], z[k + 1]);
-                        float x0, x1;
-                        unpack_f32x2(fma_f32x2(z2, sl2, fma_f32x2(z2, sh2, no2)), x0, x1);
-                        acc[c & 1] = add_f32x2(acc[c & 1], pack_f32x2(ex2_approx(x0), ex2_approx(x1)));
-                    }
-                }
-                float a0, a1;
-                unpack_f32x2(add_f32x2(acc[0], acc[1]), a0, a1);
-                ps.Sd += (double)(a0 + a1);
-            }
-            // ---- the running maximum and the bound ----------------------------------------------------------------
             if (DT == SPEC_BF16 && TOTAL) {
                 if (sl == 0) {
-                    ps.tmax = ms;
-                    ps.bound = sample_bound(raw[0], raw[1], raw[2], raw[3], ms, ps.set, ps.of, ps.Sd, P.top_p, min(P.V, UN * NT * E), P.V);
-                    dense = S.verdict != 0;
-                    continue;                           // (the first slice is in the bins)
+                    uint32_t m = 0xFF80FF80u;
+#pragma unroll
+                    for (int c = 0; c < UN; ++c) m = stream::max_raw<DT>(m, stream::unit_max_raw<DT>(stage[c * NT + lane]));
+                    ps.bound = sample_bound(stream::fold_max<DT>(m));
+                    if (nsl > 1) ps.bound = fmaxf(ps.bound, __uint_as_float((uint32_t)PLAIN_KEY << 16));
+                    cnt.kb = bound_key(ps.bound);
+                }
+                // two units at a time: what a step needs fits the registers
+                bool all = true;
+#pragma unroll 1
+                for (int c = 0; c < UN; c += 2) {
+                    uint4 raw[2] = {stage[c * NT + lane], stage[(c + 1) * NT + lane]};
+                    const uint32_t mu[2] = {stream::unit_max_raw<DT>(raw[0]), stream::unit_max_raw<DT>(raw[1])};
+                    const float ms = stream::fold_max<DT>(stream::max_raw<DT>(mu[0], mu[1]));      // (a NaN stays)
+                    ps.tmax = stream::max_nan(ps.tmax, ms);
+                    add_mass<DT, 2>(raw, ms, s_hi, s_lo, ps);
+                    // A unit that holds a candidate anywhere in the warp is counted by all lanes.  Where all units of a slice did, those
+                    // of the next three are not asked.
+                    if (!cnt.plain() || __any_sync(0xffffffffu, !(ms < HIGH))) {
+                        if (__any_sync(0xffffffffu, ms >= ps.bound)) count_pair(cnt, raw[0], raw[1]);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            if (sure > 0 || __any_sync(0xffffffffu, cnt.reaches(mu[k]))) M.count(cnt, raw[k], true);
+                            else all = false;
+                        }
+                    }
+                }
+                sure = sure > 0 ? sure - 1 : all ? 3 : 0;
+                if (sl == 0 && nsl > 1) {
+                    ps.bound = first_mass_bound(ps.tmax, ps.bound, ps.of, ps.Sd, P.top_p, min(P.V, UN * NT * E), P.V, stage);
+                    cnt.kb = bound_key(ps.bound);
+                    sure = 0;
                 }
             } else {
+                uint4 raw[UN];
+#pragma unroll
+                for (int c = 0; c < UN; ++c) raw[c] = stage[c * NT + lane];
+                // the units' maxima (bf16: still as pairs) and the thread's maximum of the slice; a NaN stays
+                uint32_t mu[UN];
+#pragma unroll
+                for (int c = 0; c < UN; ++c) mu[c] = stream::unit_max_raw<DT>(raw[c]);
+                const float ms = stream::fold_max<DT>(stream::max_raw<DT>(stream::max_raw<DT>(mu[0], mu[1]), stream::max_raw<DT>(mu[2], mu[3])));
+                static_assert(UN == 4, "slice maximum of four units");
+                if (TOTAL) add_mass<DT, UN>(raw, ms, s_hi, s_lo, ps);
+                // ---- the running maximum and the bound ----------------------------------------------------------------
                 if (sl == 0) {
                     const uint32_t km = __reduce_max_sync(0xffffffffu, cut::key_of(ms));
                     if (lane == 0) atomicMax(&S.runmax, km);
@@ -918,43 +1039,40 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
                 } else if (ms > ps.tmax && ms > cut::value_of(*(volatile uint32_t *)&S.runmax)) {
                     atomicMax(&S.runmax, cut::key_of(ms));
                 }
-                if (TOTAL) ps.bound = fmaxf(cut::value_of(*(volatile uint32_t *)&S.runmax) - window, LOWEST);
-            }
-            ps.tmax = stream::max_nan(ps.tmax, ms);
-            // ---- candidates ----------------------------------------------------------------------------------
-            if (DT == SPEC_BF16 && TOTAL && dense) {
+                if (TOTAL) ps.bound = fmaxf(cut::value_of(*(volatile uint32_t *)&S.runmax) - S.sc.window, LOWEST);
+                ps.tmax = stream::max_nan(ps.tmax, ms);
+                // ---- candidates ----------------------------------------------------------------------------------
+                if (__any_sync(0xffffffffu, ms >= ps.bound)) {
+                    int n = 0;
 #pragma unroll
-                for (int c = 0; c < UN; ++c) count_unit(M.bins, &S.odd, raw[c], ps.bound, ms);
-            } else if (__any_sync(0xffffffffu, ms >= ps.bound)) {
-                int n = 0;
-#pragma unroll
-                for (int c = 0; c < UN; ++c) {
-                    const bool in = stream::fold_max<DT>(mu[c]) >= ps.bound;
-                    const unsigned bal = __ballot_sync(0xffffffffu, in);
-                    if (in) M.hits[n + __popc(bal & lt)] = (unsigned char)(c * 32 + lane);
-                    n += __popc(bal);
-                }
-                __syncwarp();
-                for (int i0 = 0; i0 < n * E; i0 += 32) {          // a logit per lane
-                    const int i = i0 + lane;
-                    const bool on = i < n * E;
-                    const int u = on ? M.hits[i / E] : 0;
-                    const uint4 *unit = stage + (u >> 5) * NT + (u & 31);
-                    if (DT == SPEC_BF16) {
-                        const uint32_t u16 = on ? reinterpret_cast<const unsigned short *>(unit)[i % E] : 0xFF80u;
-                        if (__uint_as_float(u16 << 16) >= ps.bound) count_value(M.bins, &S.odd, u16);
-                    } else {
-                        const float z = on ? reinterpret_cast<const float *>(unit)[i % E] : -CUDART_INF_F;
-                        const bool in = z >= ps.bound;
+                    for (int c = 0; c < UN; ++c) {
+                        const bool in = stream::fold_max<DT>(mu[c]) >= ps.bound;
                         const unsigned bal = __ballot_sync(0xffffffffu, in);
-                        if (!bal) continue;
-                        int base = 0;
-                        if (lane == 0) base = atomicAdd(&S.count, __popc(bal));
-                        const int pos = __shfl_sync(0xffffffffu, base, 0) + __popc(bal & lt);
-                        if (in && pos < CAP) M.keys[pos] = cut::key_of(z);
+                        if (in) M.hits[n + __popc(bal & lt)] = (unsigned char)(c * 32 + lane);
+                        n += __popc(bal);
                     }
+                    __syncwarp();
+                    for (int i0 = 0; i0 < n * E; i0 += 32) {          // a logit per lane
+                        const int i = i0 + lane;
+                        const bool on = i < n * E;
+                        const int u = on ? M.hits[i / E] : 0;
+                        const uint4 *unit = stage + (u >> 5) * NT + (u & 31);
+                        if (DT == SPEC_BF16) {
+                            const uint32_t u16 = on ? reinterpret_cast<const unsigned short *>(unit)[i % E] : 0xFF80u;
+                            if (__uint_as_float(u16 << 16) >= ps.bound) count_value(M.bins, &S.odd, u16);
+                        } else {
+                            const float z = on ? reinterpret_cast<const float *>(unit)[i % E] : -CUDART_INF_F;
+                            const bool in = z >= ps.bound;
+                            const unsigned bal = __ballot_sync(0xffffffffu, in);
+                            if (!bal) continue;
+                            int base = 0;
+                            if (lane == 0) base = atomicAdd(&S.count, __popc(bal));
+                            const int pos = __shfl_sync(0xffffffffu, base, 0) + __popc(bal & lt);
+                            if (in && pos < CAP) M.keys[pos] = cut::key_of(z);
+                        }
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
             }
         }
         finish_row<DT, TOTAL>(P, id, ps);

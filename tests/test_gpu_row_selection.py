@@ -68,3 +68,22 @@ def test_first_slice_unlike_the_rest(dtype, trunc, order):
     else:
         z = torch.sort(z.float(), dim=-1, descending=order == "descending").values.to(dtype)
     check(z, trunc, T=0.7)
+
+
+@pytest.mark.parametrize("V", [20000, 150001], ids=["3_slices", "19_slices"])
+@pytest.mark.parametrize("shift,scale,p", [(-40.0, 3.0, 0.95),      # no positive logit: the first slice is counted again
+                                           (0.0, 0.5, 0.99),        # a nucleus that reaches far below zero
+                                           (1.5, 1.0, 0.9),         # a cut next to the bins that share values
+                                           (12.0, 3.0, 0.99), (12.0, 3.0, 0.5)])
+def test_bounds_from_the_first_slices(V, shift, scale, p):
+    g = torch.Generator(device="cuda").manual_seed(5)
+    z = (torch.randn((1, 3, V), generator=g, device="cuda") * scale + shift).to(BF)
+    z[0, 1, 8192:] -= 6.0                          # all the mass in the first slice
+    z[0, 2, :8192] -= 6.0                          # ... and next to none
+    check(z, dict(top_p=p))
+
+
+def test_a_value_beyond_the_bins_late_in_the_row():
+    z = rows(40000, BF)
+    z[0, 0, 30000], z[1, 2, 39999], z[1, 0, 100] = 600.0, 511.0, -700.0
+    check(z, dict(top_p=0.95), T=200.0)
