@@ -157,6 +157,29 @@ __device__ __forceinline__ double exp2_frac(double f)
     const double q0 = fma(t2, p1, p0), q1 = fma(t2, p3, p2), q2 = fma(t2, p5, p4);
     return fma(t8, fma(t4, p6, q2), fma(t4, q1, q0));
 }
+// 2^(z s - O) in fp64 (about 1e-15 relative); 0 for -inf and for exponents below the double range
+__device__ __forceinline__ double exp2_exact(float z, double s_d, int O)
+{
+    const double xd = (double)z * s_d - (double)O;
+    if (!(xd > -1000.0)) return 0.0;
+    const double nd = rint(xd);
+    return exp2_frac(xd - nd) * pow2d((int)nd);
+}
+// 2^(z s - O) in fp32 to about half a unit in the last place, s = s_hi + s_lo (Taylor series of 2^f, |f| <= 0.5, to degree 7): unlike those of
+// ex2.approx, whose mean is -3e-8 to -5e-8, its errors average out.  0 below 2^-126 and for -inf.
+__device__ __forceinline__ float exp2_fine(float z, float s_hi, float s_lo, int O)
+{
+    const float n = rintf(z * s_hi), f = fmaf(z, s_lo, fmaf(z, s_hi, -n));
+    float p = 1.5252734e-5f;
+    p = fmaf(p, f, 1.5403530e-4f);
+    p = fmaf(p, f, 1.3333558e-3f);
+    p = fmaf(p, f, 9.6181291e-3f);
+    p = fmaf(p, f, 5.5504109e-2f);
+    p = fmaf(p, f, 2.4022651e-1f);
+    p = fmaf(p, f, 6.9314718e-1f);
+    p = fmaf(p, f, 1.0f);
+    return z > -CUDART_INF_F ? p * pow2i((int)n - O) : 0.f;
+}
 // fp32 pairs in one 64-bit register: packed fused multiply-add and add (sm_100)
 __device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi)
 {

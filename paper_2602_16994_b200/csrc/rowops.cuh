@@ -1,11 +1,16 @@
 // Row kernels of libspecverify: materialised sampling distributions (spec_tree_probs) and the
-// stand-alone inverse-CDF draw (spec_sample_bonus).  One cluster per row; each CTA stages its
-// vocabulary slice with bulk asynchronous copies and the CTAs combine through distributed shared
-// memory.  These are utility entry points; the verification path proper is verify.cuh.
+// stand-alone inverse-CDF draw (spec_sample_bonus).  These are utility entry points; the verification path proper is
+// verify.cuh.
+//   distributions  without truncation: one cluster per row, each CTA stages its vocabulary slice with bulk asynchronous copies and the
+//                  CTAs combine through distributed shared memory (spec_probs_kernel); with top-k / top-p: the selection kernel of
+//                  trunc.cuh, then one pass that writes (spec_probs_kept_kernel);
+//   draw           a cluster per row, nothing staged (spec_bonus_kernel).
 #pragma once
 #include <cooperative_groups.h>
+#include <type_traits>
 
 #include "common.cuh"
+#include "stream.cuh"
 
 namespace specv {
 namespace rowops {
@@ -242,79 +247,6 @@ __device__ __forceinline__ void widen_exp(float *region, int SL, int dtype, int 
     kept = nk;
 }
 
-// Inverse CDF inside one slice of weights.  Each thread owns a contiguous run of float4 groups (an odd count, so that
-// the 128-bit shared loads of a warp fall in distinct bank groups), sums it in fp64, a block scan finds the owning thread,
-// which walks its run again.  Returns the local token index (block-uniform), or the last
-// positive-weight token if tau is not below the slice total, or -1 if the slice holds no weight.
-__device__ __forceinline__ int slice_inverse_cdf(Shared &S, const float *ep, int SL, double tau, double &dist_lo,
-                                                 double &dist_hi)
-{
-    const int nv = SL >> 2;
-    int L4 = (nv + NT - 1) / NT;
-    L4 |= 1;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int i0 = threadIdx.x * L4, i1 = min(i0 + L4, nv);
-    const float4 *a = (const float4 *)ep;
-    double seg = 0.0;
-    int last_pos = -1;
-    for (int i = i0; i < i1; ++i) {
-        float4 p = a[i];
-        float v[4] = {p.x, p.y, p.z, p.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            seg += (double)v[k];
-            if (v[k] > 0.f) last_pos = i * 4 + k;
-        }
-    }
-    // block-wide exclusive scan of seg
-    double inc = seg;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        double t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-    }
-    __syncthreads();                    // warp_part / ctl may still be read from the previous phase
-    if (lane == 31) S.warp_part[w][0] = inc;
-    if (threadIdx.x == 0) { S.ctl_i[2] = -1; S.ctl_i[3] = -1; }
-    __syncthreads();
-    double base = 0.0, total = 0.0;
-    for (int k = 0; k < NWARP; ++k) {
-        double t = S.warp_part[k][0];
-        if (k < w) base += t;
-        total += t;
-    }
-    double excl = base + inc - seg, incl = base + inc;
-    if (seg > 0.0 && excl <= tau && tau < incl) {
-        double run = excl;
-        int found = -1;
-        double before = excl;
-        for (int i = i0; i < i1 && found < 0; ++i) {
-            float4 p = a[i];
-            float v[4] = {p.x, p.y, p.z, p.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (found < 0) {
-                    before = run;
-                    run += (double)v[k];
-                    if (run > tau) found = i * 4 + k;
-                }
-            }
-        }
-        if (found < 0) found = last_pos;   // cannot happen: incl is this very sum
-        S.ctl_i[2] = found;
-        S.ctl_d[2] = tau - before;
-        S.ctl_d[3] = run - tau;
-    }
-    // fallback: last positive-weight token of the slice
-    if (last_pos >= 0) atomicMax(&S.ctl_i[3], last_pos);
-    __syncthreads();
-    int tok = S.ctl_i[2];
-    if (tok >= 0) { dist_lo = S.ctl_d[2]; dist_hi = S.ctl_d[3]; }
-    else { tok = S.ctl_i[3]; dist_lo = 0.0; dist_hi = 0.0; }
-    (void)total;
-    return tok;
-}
-
 // ------------------------------------------------------------------------------------------------
 // spec_tree_probs: materialise the sampling distribution of every row
 // ------------------------------------------------------------------------------------------------
@@ -325,11 +257,9 @@ struct TParams {
     float T;
     const float *T_seq;
     float *probs, *stats;
-    const float *cut;        // optional [rows*2] smallest kept logit (target, draft) of every row
-    int which;
 };
 
-__global__ void __launch_bounds__(NT, 1) spec_probs_kernel(const TParams P)
+__global__ void __launch_bounds__(NT, 2) spec_probs_kernel(const TParams P)
 {
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
@@ -368,9 +298,8 @@ __global__ void __launch_bounds__(NT, 1) spec_probs_kernel(const TParams P)
     double v[NX];
 #pragma unroll
     for (int i = 0; i < NX; ++i) v[i] = 0.0;
-    const float cutv = P.cut ? __ldg(P.cut + (long long)row_id * 2 + P.which) : -CUDART_INF_F;
     int kept = 0;
-    widen_exp(ep, SL, P.dtype, n, ref, cutv, s_hi, s_lo, v[1], v[2], kept);
+    widen_exp(ep, SL, P.dtype, n, ref, -CUDART_INF_F, s_hi, s_lo, v[1], v[2], kept);
     {
         double red[3] = {v[1], v[2], (double)kept};
         block_sum<3>(S, red);
@@ -409,7 +338,99 @@ __global__ void __launch_bounds__(NT, 1) spec_probs_kernel(const TParams P)
             double nkept = 0.0;
             for (int r = 0; r < C; ++r) nkept += X[r][3];
             st[0] = (float)(mg / T); st[1] = (float)Z; st[2] = (float)nkept;
-            st[3] = (float)h; st[4] = (float)(1.0 / Z); st[5] = cutv;
+            st[3] = (float)h; st[4] = (float)(1.0 / Z); st[5] = -CUDART_INF_F;
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// spec_tree_probs under top-k / top-p: the kept tokens of a row are known by value (its record), so that its distribution is written
+// in one pass without shared memory or barriers
+// ------------------------------------------------------------------------------------------------
+// A CTA writes parts of KEPT_PART tokens, four consecutive tokens per thread and step; all its loads are issued first.  Bound by
+// the writes.
+// 76 rows of 128256, bf16 (58 MB): 37 us with the row staged in shared memory and widened there, 14 now.
+constexpr int KEPT_NT = 256, KEPT_STEPS = 4, KEPT_PART = KEPT_NT * 4 * KEPT_STEPS;
+struct KParams {
+    int N, V, parts;
+    long long items;         // rows * parts
+    const void *z;
+    long long seq_stride, node_stride;
+    float T;
+    const float *T_seq;
+    const RowPart *part;     // [rows][2], the first of each pair
+    const int *kept;         // [rows][2]
+    float *probs, *stats;
+};
+// of a token that is no less than 2^-4 of the unit of the row's sum
+__device__ __noinline__ float heavy_prob(float z, double s_d, int O, double S) { return (float)(exp2_exact(z, s_d, O) / S); }
+
+template <int DT>
+__global__ void __launch_bounds__(KEPT_NT, 4) spec_probs_kept_kernel(const KParams P)
+{
+    constexpr int ESZ = DT == SPEC_BF16 ? 2 : 4;
+    const int tid = threadIdx.x;
+    grid_dependency_wait();
+    for (long long it = blockIdx.x; it < P.items; it += gridDim.x) {
+        const int row = (int)(it / P.parts), part = (int)(it % P.parts), b = row / P.N;
+        const RowPart *rp = P.part + 2ll * row;
+        const double S = rp->S, s_d = 1.4426950408889634 / (double)(P.T_seq ? __ldg(P.T_seq + b) : P.T);
+        const int O = rp->O, bad = rp->bad;
+        const float cut = rp->cut;
+        if (P.stats && part == 0 && tid == 0) {
+            float *st = P.stats + 6ll * row;
+            if (bad) {
+                for (int i = 0; i < 6; ++i) st[i] = CUDART_NAN_F;
+            } else {
+                // in units of the largest e, 2^xmax
+                const double x = (double)rp->xmax, Z = S * exp2(-x);
+                st[0] = (float)(((double)O + x) * 0.6931471805599453); st[1] = (float)Z; st[2] = (float)P.kept[2ll * row];
+                st[3] = (float)(log(S) - 0.6931471805599453 * rp->X / S); st[4] = (float)(1.0 / Z); st[5] = cut;
+            }
+        }
+        if (!P.probs) continue;
+        float s_hi, s_lo, inv_hi, inv_lo;
+        stream::split_scale(s_d, s_hi, s_lo);
+        split_float(bad ? 0.0 : 1.0 / S, inv_hi, inv_lo);
+        const unsigned char *z = (const unsigned char *)P.z + ((long long)b * P.seq_stride + (long long)(row % P.N) * P.node_stride) * ESZ;
+        float *out = P.probs + (long long)row * P.V;
+        const int t0 = part * KEPT_PART, t1 = min(P.V, t0 + KEPT_PART);
+        const float near = (float)(((double)O - 4.0) / s_d);
+        const auto prob = [&](float v) {
+            if (!(v >= cut) || bad) return 0.f;
+            if (v >= near) return heavy_prob(v, s_d, O, S);
+            const float e = exp2_fine(v, s_hi, s_lo, O);
+            return fmaf(e, inv_lo, e * inv_hi);
+        };
+        // (t0 is a multiple of 4; a row whose logits or probabilities start elsewhere goes token by token)
+        if (((uintptr_t)z & (4 * ESZ - 1)) == 0 && ((uintptr_t)out & 15) == 0) {
+            using Four = std::conditional_t<DT == SPEC_BF16, uint2, uint4>;
+            Four raw[KEPT_STEPS];
+#pragma unroll
+            for (int k = 0; k < KEPT_STEPS; ++k) {
+                const int t = t0 + (k * KEPT_NT + tid) * 4;
+                if (t + 3 < t1) raw[k] = __ldg(reinterpret_cast<const Four *>(z + (size_t)t * ESZ));
+            }
+#pragma unroll
+            for (int k = 0; k < KEPT_STEPS; ++k) {
+                const int t = t0 + (k * KEPT_NT + tid) * 4;
+                if (t + 3 < t1) {
+                    float v[4];
+                    if constexpr (DT == SPEC_BF16) {
+                        v[0] = bf16_lo(raw[k].x); v[1] = bf16_hi(raw[k].x); v[2] = bf16_lo(raw[k].y); v[3] = bf16_hi(raw[k].y);
+                    } else {
+                        v[0] = __uint_as_float(raw[k].x); v[1] = __uint_as_float(raw[k].y); v[2] = __uint_as_float(raw[k].z); v[3] = __uint_as_float(raw[k].w);
+                    }
+                    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])) >= cut) o = make_float4(prob(v[0]), prob(v[1]), prob(v[2]), prob(v[3]));
+                    *reinterpret_cast<float4 *>(out + t) = o;
+                } else {
+                    for (int i = t; i < t1; ++i) out[i] = prob(load_logit(z, DT, i));
+                }
+            }
+        } else {
+#pragma unroll 4
+            for (int t = t0 + tid; t < t1; t += KEPT_NT) out[t] = prob(load_logit(z, DT, t));
         }
     }
 }
@@ -417,77 +438,130 @@ __global__ void __launch_bounds__(NT, 1) spec_probs_kernel(const TParams P)
 // ------------------------------------------------------------------------------------------------
 // spec_sample_bonus: inverse CDF over rows of fp32 weights
 // ------------------------------------------------------------------------------------------------
+// A cluster per row, a slice per CTA, a tile of 128 weights per warp and step.  The sums of the tiles stay in shared memory; the cluster
+// exchanges the slices' sums, and the CTA that owns the target finds the tile by one scan and reads that tile once more.  Nothing else is
+// kept, so an SM holds eight CTAs with four tiles per warp in flight.  76 rows of 128256 (39 MB, written just before): 20 us with
+// the slices staged in shared memory, one CTA per SM; 12 now.
+constexpr int BN_NT = 256, BN_TILE = 128, BN_TILES = 1024;      // tiles of a slice at most
+constexpr int BN_CMAX = 8;
 struct BParams {
-    int R, V, SL;
+    int R, V, SL;            // SL: weights of a slice, a multiple of BN_TILE
     const float *w, *u;
     int *token;
     float *margin;
 };
+// first lane with running sum > tau (and weight); else the last with weight and rest = inf; -1 where there is none
+__device__ __forceinline__ int first_above(double v, double tau, double &rest)
+{
+    const int lane = threadIdx.x & 31;
+    double incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const unsigned hit = __ballot_sync(0xffffffffu, v > 0.0 && incl > tau), pos = __ballot_sync(0xffffffffu, v > 0.0);
+    const int at = hit ? __ffs(hit) - 1 : 31 - __clz(pos);
+    const double before = __shfl_sync(0xffffffffu, incl - v, at < 0 ? 0 : at);
+    rest = hit ? tau - before : CUDART_INF;
+    return pos ? at : -1;
+}
+// the lane's four consecutive weights of a tile; beyond the slice: 0
+__device__ __forceinline__ float4 tile_weights(const float *row, int t, int end, bool vec)
+{
+    if (vec && t + 3 < end) return __ldg(reinterpret_cast<const float4 *>(row + t));
+    return make_float4(t < end ? __ldg(row + t) : 0.f, t + 1 < end ? __ldg(row + t + 1) : 0.f, t + 2 < end ? __ldg(row + t + 2) : 0.f,
+                       t + 3 < end ? __ldg(row + t + 3) : 0.f);
+}
 
-__global__ void __launch_bounds__(NT, 1) spec_bonus_kernel(const BParams P)
+__global__ void __launch_bounds__(BN_NT) spec_bonus_kernel(const BParams P)
 {
     cg::cluster_group cluster = cg::this_cluster();
-    const int C = (int)cluster.num_blocks();
-    const int rank = (int)cluster.block_rank();
-    const int r_id = blockIdx.x / C;
-    const int tid = threadIdx.x;
-    const int SL = P.SL;
-    __shared__ Shared S;
-    float *ep = (float *)dyn_smem;
-    const long long tok0 = (long long)rank * SL;
-    const int n = (int)max(0ll, min((long long)SL, (long long)P.V - tok0));
-    if (tid == 0) { mbar_init(&S.mbar, 1); mbar_fence_init(); }
-    __syncthreads();
+    const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int r_id = blockIdx.x / C, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ double tile[BN_TILES], total[BN_CMAX];
+    grid_dependency_wait();
     const float *row = P.w + (long long)r_id * P.V;
-    uint32_t tx = stage_row(ep, SL, SPEC_F32, row, tok0, n, &S.mbar, true);
-    if (tid == 0 && tx) mbar_expect_tx(&S.mbar, tx);
-    stage_row(ep, SL, SPEC_F32, row, tok0, n, &S.mbar, false);
-    int gave_up = 0;
-    if (tx) gave_up = mbar_wait(&S.mbar, 0) ? 0 : 1;
-    for (int i = n + tid; i < SL; i += NT) ep[i] = 0.f;     // padding carries no weight
-    // a copy that was given up on: the slice counts as empty (its bytes may still be on their way)
-    if (__syncthreads_or(gave_up))
-        for (int i = tid; i < SL; i += NT) ep[i] = 0.f;
-    __syncthreads();
-    // slice total in the same order the search will use is not required: the search rescans
-    double acc = 0.0;
-    {
-        const float4 *a4 = (const float4 *)ep;
-        for (int i = tid; i < (SL >> 2); i += NT) {
-            float4 p = a4[i];
-            acc += (double)((p.x + p.y) + (p.z + p.w));
+    const bool vec = ((uintptr_t)row & 15) == 0;
+    const int t0 = rank * P.SL, end = min(P.V, t0 + P.SL), tiles = max(0, (end - t0 + BN_TILE - 1) / BN_TILE);
+    constexpr int AHEAD = 4, WARPS = BN_NT / 32;
+    for (int i0 = warp; i0 < tiles; i0 += WARPS * AHEAD) {
+        float4 x[AHEAD];
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) x[k] = tile_weights(row, t0 + (i0 + k * WARPS) * BN_TILE + lane * 4, end, vec);
+        double s[AHEAD];
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) s[k] = ((double)x[k].x + (double)x[k].y) + ((double)x[k].z + (double)x[k].w);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+            for (int k = 0; k < AHEAD; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+        }
+        if (lane < AHEAD) {
+            const int i = i0 + lane * WARPS;
+            const double mine = lane == 0 ? s[0] : lane == 1 ? s[1] : lane == 2 ? s[2] : s[3];
+            if (i < tiles) tile[i] = mine;
         }
     }
-    double red[1] = {acc};
-    block_sum<1>(S, red);
-    cluster.sync();                      // peers must be running before their shared memory is written
-    cluster_allgather(cluster, S, 0, red, 1);
-    double (*X)[NX] = S.xchg[0];
-    double tot = 0.0;
-    for (int r = 0; r < C; ++r) tot += X[r][0];
-    const double target = (double)__ldg(P.u + r_id) * tot;
-    int owner = -1, last_pos = -1;
-    double pre = 0.0, tau = 0.0;
-    for (int r = 0; r < C; ++r) {
-        if (X[r][0] > 0.0) last_pos = r;
-        if (owner < 0 && pre + X[r][0] > target) { owner = r; tau = target - pre; }
-        if (owner < 0) pre += X[r][0];
+    __syncthreads();
+    // a run of tiles per lane (of every warp alike: the slice's sum is needed by all)
+    const int per = ((tiles + 31) / 32) | 1, i0 = lane * per, i1 = min(tiles, i0 + per);
+    double mine = 0.0;
+    for (int i = i0; i < i1; ++i) mine += tile[i];
+    const double slice = warp_sum(mine);
+    if (C > 1) {
+        cluster.sync();                  // peers must be running before their shared memory is written
+        if (tid < C) *cluster.map_shared_rank(&total[rank], tid) = slice;
+        cluster.sync();
+    } else {
+        if (tid == 0) total[0] = slice;
+        __syncthreads();
     }
-    if (owner < 0) { owner = last_pos; tau = CUDART_INF; }
+    const double share = lane < C ? total[lane] : 0.0;
+    double all = 0.0;
+    for (int r = 0; r < C; ++r) all += total[r];
+    double tau, tau2, tau3;
+    const int owner = first_above(share, (double)__ldg(P.u + r_id) * all, tau);
     if (owner < 0) {
         if (rank == 0 && tid == 0) { P.token[r_id] = -1; if (P.margin) P.margin[r_id] = 0.f; }
         return;
     }
-    if (owner == rank) {
-        double dlo = 0.0, dhi = 0.0;
-        int t = slice_inverse_cdf(S, ep, SL, tau, dlo, dhi);
-        if (tid == 0) {
-            P.token[r_id] = t >= 0 ? (int)(tok0 + t) : -1;
-            if (P.margin) P.margin[r_id] = (float)(fmin(dlo, dhi) / tot);
+    if (owner != rank || warp != 0) return;
+    const int l = first_above(mine, tau, tau2);
+    // the tile inside the lane's run, by that lane
+    int ti = -1;
+    double rest = tau2;
+    if (lane == l) {
+        int last = -1;
+        double run = 0.0, upto = 0.0;
+        for (int i = i0; i < i1; ++i) {
+            const double x = tile[i];
+            if (x > 0.0) last = i;
+            if (x > 0.0 && run + x > tau2) { ti = i; upto = run; break; }
+            run += x;
         }
+        if (ti >= 0) rest = tau2 - upto;
+        else { ti = last; rest = CUDART_INF; }
     }
+    ti = __shfl_sync(0xffffffffu, ti, l < 0 ? 0 : l);
+    rest = __shfl_sync(0xffffffffu, rest, l < 0 ? 0 : l);
+    const int at = t0 + ti * BN_TILE + lane * 4;
+    const float4 x = tile_weights(row, at, end, vec);
+    const float v[4] = {x.x, x.y, x.z, x.w};
+    const int who = first_above(((double)v[0] + (double)v[1]) + ((double)v[2] + (double)v[3]), rest, tau3);
+    if (lane != who) return;
+    int found = -1, last = -1;
+    double run = 0.0, lo = 0.0, hi = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double before = run;
+        run += (double)v[k];
+        if (v[k] > 0.f) last = k;
+        if (found < 0 && run > tau3) { found = k; lo = tau3 - before; hi = run - tau3; }
+    }
+    P.token[r_id] = at + (found >= 0 ? found : last);
+    if (P.margin) P.margin[r_id] = found >= 0 ? (float)(fmin(lo, hi) / all) : 0.f;
 }
-
 
 }  // namespace rowops
 }  // namespace specv

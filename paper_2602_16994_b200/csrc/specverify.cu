@@ -124,17 +124,19 @@ struct RowPlan {
 };
 constexpr int ROW_SMEM_BUDGET = 227 * 1024 - (int)sizeof(rowops::Shared) - 1024;
 
+// a row in the shared memory of a cluster: two CTAs per SM where eight CTAs are enough for that
 bool make_row_plan(int V, int bytes_per_token, RowPlan *p)
 {
-    for (int C = 1; C <= rowops::CMAX; C <<= 1) {
-        long long sl = ((long long)V + C - 1) / C;
-        sl = (sl + 63) / 64 * 64;
-        long long need = sl * bytes_per_token;
-        if (need <= ROW_SMEM_BUDGET) {
-            p->C = C; p->SL = (int)sl; p->smem = (int)need;
-            return true;
+    for (const int budget : {ROW_SMEM_BUDGET / 2 - 4096, ROW_SMEM_BUDGET})
+        for (int C = 1; C <= (budget == ROW_SMEM_BUDGET ? rowops::CMAX : 8); C <<= 1) {
+            long long sl = ((long long)V + C - 1) / C;
+            sl = (sl + 63) / 64 * 64;
+            long long need = sl * bytes_per_token;
+            if (need <= budget) {
+                p->C = C; p->SL = (int)sl; p->smem = (int)need;
+                return true;
+            }
         }
-    }
     return false;
 }
 
@@ -159,9 +161,9 @@ int check_in(const SpecIn *in, bool need_tree)
 
 inline int64_t up256(int64_t x) { return (x + 255) / 256 * 256; }
 
-// workspace layout: node records | published weights + arrival counters (cleared per call) | row cuts
+// workspace layout: node records | published weights + arrival counters (cleared per call) | kept counts
 struct WsLayout {
-    int64_t rec, pub, fin, done, ticket, chain, cut, stat, gseq, total;
+    int64_t rec, pub, fin, done, ticket, chain, kept, stat, gseq, total;
 };
 constexpr int MAX_PARTS = 4;      // parts a row may be split into by the streaming statistics kernel
 WsLayout ws_layout(const SpecIn *in, int slices = MAX_PARTS)   // slices = 0: one record per row only
@@ -177,7 +179,7 @@ WsLayout ws_layout(const SpecIn *in, int slices = MAX_PARTS)   // slices = 0: on
     L.ticket = o; o += 4;
     o = up256(o);
     L.chain = o; o += up256(nodes * (int64_t)sizeof(ChainRec));
-    L.cut = o; o += up256(nodes * 8);
+    L.kept = o; o += up256(nodes * 8);
     L.stat = o; o += up256(nodes * 2 * (slices + 1) * (int64_t)sizeof(RowPart));      // one record per row, then the parts
     L.gseq = o; o += up256(nodes * KMAX * 8);       // step coefficients of every node
     L.total = o;
@@ -331,7 +333,8 @@ int launch_trunc(const SpecIn *in, const void *zp, const void *zq, const int *pa
     rp.B = in->B; rp.N = in->N; rp.V = in->V; rp.top_k = in->top_k; rp.top_p = in->top_p;
     rp.zp = zp; rp.zq = zq; rp.seq_stride = in->seq_stride; rp.node_stride = in->node_stride;
     rp.topo_stride = in->topo_seq_stride; rp.parent = parent; rp.T = in->temperature; rp.T_seq = in->temperature_per_seq;
-    rp.part = (RowPart *)(ws + L.stat); rp.cut = (float *)(ws + L.cut); rp.init = init;
+    rp.part = (RowPart *)(ws + L.stat); rp.init = init;
+    rp.kept = parent ? nullptr : (int *)(ws + L.kept);
     const bool bf = in->logits_dtype == SPEC_BF16;
     const long long items = 2ll * in->B * in->N;
     const long long want = (long long)sm_count() * (bf ? trunc::CTAS<SPEC_BF16> : trunc::CTAS<SPEC_F32>);
@@ -858,22 +861,29 @@ int32_t spec_tree_probs(const SpecIn *in, int32_t which, float *probs, float *ro
     const void *z = which ? in->draft_logits : in->target_logits;
     if (!z || (!probs && !row_stats)) return SPEC_ERR_NULL;
     const bool trunc = (in->top_k > 0 && in->top_k < in->V) || in->top_p < 1.f;
-    const float *cutp = nullptr;
+    RowPlan pl;
+    if (!make_row_plan(in->V, 4, &pl)) return SPEC_ERR_UNSUPPORTED;
     if (trunc) {
-        // the cuts of every row of the chosen side go to slot 0 of every pair in the workspace
+        // the record of every row of the chosen side goes to the first of its pair in the workspace
         const WsLayout L = ws_layout(in);
         if (!ws || ((uintptr_t)ws & 255) || ws_bytes < L.total) return SPEC_ERR_WORKSPACE;
         rc = launch_trunc(in, z, z, nullptr, (unsigned char *)ws, L, stream::NodeInit{}, (cudaStream_t)stream);
         if (rc) return rc;
-        cutp = (const float *)((unsigned char *)ws + L.cut);
+        rowops::KParams kp = {};
+        kp.N = in->N; kp.V = in->V; kp.z = z; kp.seq_stride = in->seq_stride; kp.node_stride = in->node_stride;
+        kp.T = in->temperature; kp.T_seq = in->temperature_per_seq;
+        kp.part = (const RowPart *)((unsigned char *)ws + L.stat); kp.kept = (const int *)((unsigned char *)ws + L.kept);
+        kp.probs = probs; kp.stats = row_stats;
+        kp.parts = probs ? (in->V + rowops::KEPT_PART - 1) / rowops::KEPT_PART : 1;
+        kp.items = (long long)in->B * in->N * kp.parts;
+        const int grid = (int)std::min(kp.items, 1ll << 20);
+        const auto go = [&](auto kernel) { return launch_clustered(kernel, grid, 1, rowops::KEPT_NT, 0, (cudaStream_t)stream, &kp, true); };
+        return in->logits_dtype == SPEC_BF16 ? go(rowops::spec_probs_kept_kernel<SPEC_BF16>) : go(rowops::spec_probs_kept_kernel<SPEC_F32>);
     }
-    RowPlan pl;
-    if (!make_row_plan(in->V, 4, &pl)) return SPEC_ERR_UNSUPPORTED;
     rowops::TParams tp = {};
     tp.rows = in->B * in->N; tp.N = in->N; tp.V = in->V; tp.dtype = in->logits_dtype; tp.SL = pl.SL;
     tp.z = z; tp.seq_stride = in->seq_stride; tp.node_stride = in->node_stride;
     tp.T = in->temperature; tp.T_seq = in->temperature_per_seq; tp.probs = probs; tp.stats = row_stats;
-    tp.cut = cutp; tp.which = 0;
     rc = prepare_kernel(rowops::spec_probs_kernel, pl.C, pl.smem);
     if (rc) return rc;
     return launch_clustered(rowops::spec_probs_kernel, tp.rows * pl.C, pl.C, rowops::NT, pl.smem, (cudaStream_t)stream, &tp);
@@ -887,10 +897,11 @@ int32_t spec_sample_bonus(const float *weights, int32_t R, int32_t V, const floa
     if (R <= 0 || V <= 0) return SPEC_ERR_SHAPE;
     RowPlan pl;
     if (!make_row_plan(V, 4, &pl)) return SPEC_ERR_UNSUPPORTED;
-    rowops::BParams bp = {R, V, pl.SL, weights, u, token, margin};
-    int rc = prepare_kernel(rowops::spec_bonus_kernel, pl.C, pl.smem);
-    if (rc) return rc;
-    return launch_clustered(rowops::spec_bonus_kernel, R * pl.C, pl.C, rowops::NT, pl.smem, (cudaStream_t)stream, &bp);
+    // CTAs for about four per SM, a slice of at least 4096 weights each, as many as the tiles' sums of a slice ask for
+    int C = 1;
+    while (C < rowops::BN_CMAX && (((long long)R * C < 4ll * sm_count() && V >= C * 8192) || (V + C - 1) / C > (rowops::BN_TILES - 1) * rowops::BN_TILE)) C <<= 1;
+    rowops::BParams bp = {R, V, up((V + C - 1) / C, rowops::BN_TILE), weights, u, token, margin};
+    return launch_clustered(rowops::spec_bonus_kernel, R * C, C, rowops::BN_NT, 0, (cudaStream_t)stream, &bp, true);
 }
 
 int32_t spec_host_staging_bytes(const SpecIn *in, int64_t *bytes)

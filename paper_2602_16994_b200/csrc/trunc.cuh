@@ -66,7 +66,7 @@ struct RParams {
     float T;
     const float *T_seq;
     RowPart *part;             // [B*N*2] the rows' statistics
-    float *cut;                // [B*N*2] smallest kept logit of every row (for spec_tree_probs)
+    int *kept;                 // [B*N*2] kept tokens of every row (spec_tree_probs; NULL: not wanted)
     stream::NodeInit init;     // per-call words of the workspace to set (every-node verification)
 };
 
@@ -362,22 +362,30 @@ __device__ __forceinline__ void visit_row(const stream::RowSpan &row, F f)
     }
 }
 
+// adds c tokens of logit z to a row's kept sums, in fp64: the sums are shared by all that is made of the row
+__device__ __forceinline__ void add_kept(float z, double c, double s_d, double O, double &Z, double &X)
+{
+    const double x = fmax((double)z * s_d - O, -200.0), n = rint(x), e = c * exp2_frac_once(x - n) * pow2d((int)n);
+    Z += e;
+    X += e * x;
+}
 struct Kept {
     uint32_t key;      // key of the cut (0: nothing is cut)
     double Z, X;       // sum over the kept tokens of e and e x
+    int n;             // their number
 };
 
 // Selection and kept sums of a row the one pass could not settle: radix levels over the row in L2.  total: mass
 // of the row in units of its largest e (top-p alone; it only narrows the first range).  Out of line: rare.
 template <int DT>
 __device__ __noinline__ Kept settle_from_row(Shared &S, uint32_t *bins, const stream::RowSpan row, int V, int top_k,
-                                             float top_p, float m, float sf, float s_hi, float s_lo, float of, double total)
+                                             float top_p, float m, float sf, float s_hi, float s_lo, double s_d, float of, double total)
 {
     uint32_t *lo = bins, *hi = bins + NB;
     const bool use_k = top_k > 0 && top_k < V, use_p = top_p < 1.f;
     const uint32_t key_m = cut::key_of(m);
     const auto visit = [&](auto g) { visit_row<DT>(row, [&](float z) { g(cut::key_of(z)); }); };
-    Kept r = {0u, 0.0, 0.0};
+    Kept r = {0u, 0.0, 0.0, 0};
     if (use_k && !radix_select<false>(S, lo, hi, (double)top_k, 0u, key_m, m, sf, r.key, visit)) r.key = 0u;
     if (use_p) {
         const uint32_t key_k = r.key;
@@ -397,14 +405,21 @@ __device__ __noinline__ Kept settle_from_row(Shared &S, uint32_t *bins, const st
     }
     const float cutv = r.key == 0u ? -CUDART_INF_F : cut::value_of(r.key);
     double Z = 0.0, X = 0.0;
+    int n = 0;
     visit_row<DT>(row, [&](float z) {
         if (z >= cutv) {
             const float x = fmaxf(fmaf(z, s_lo, fmaf(z, s_hi, -of)), -200.f);
-            const float e = ex2_approx(x);
-            Z += (double)e;
-            X += (double)e * (double)x;
+            ++n;
+            if (x > -4.f) {                            // (there may be as many tokens as the row has: only the largest in fp64)
+                add_kept(z, 1.0, s_d, (double)of, Z, X);
+            } else {
+                const float e = exp2_fine(z, s_hi, s_lo, (int)of);
+                Z += (double)e;
+                X += (double)e * (double)x;
+            }
         }
     });
+    r.n = (int)block_sum(S, (unsigned long long)n);
     Z = warp_sum(Z);
     X = warp_sum(X);
     __syncthreads();
@@ -715,7 +730,6 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
                 RowPart r = {};
                 r.cut = -CUDART_INF_F; r.O = ROWPART_EMPTY; r.bad = 1;
                 *out = r;
-                P.cut[id] = -CUDART_INF_F;
             }
             __syncthreads();
             clear();
@@ -731,15 +745,15 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             total *= 1.4142135623730951 * exp2_frac(fmin(fmax(d, 0.0), 1.0) - 0.5);
         }
     }
-    const double Od = ceil((double)m * s_d);
-    const float of = (float)fmin(fmax(Od, -1.0e9), 1.0e9);
-    auto write = [&](double Z, double X, float cutv) {
+    const double Od = fmin(fmax(ceil((double)m * s_d), -1.0e9), 1.0e9);
+    const float of = (float)Od;
+    auto write = [&](double Z, double X, float cutv, int kept) {
         RowPart r;
-        r.S = Z; r.X = X; r.O = (int)of; r.cut = cutv;
+        r.S = Z; r.X = X; r.O = (int)Od; r.cut = cutv;
         r.xmax = (float)((double)m * s_d - (double)of);
         r.bad = 0;
         *out = r;
-        P.cut[id] = cutv;
+        if (P.kept) P.kept[id] = kept;
     };
     bool settled = false;
     if (DT == SPEC_BF16) {
@@ -757,19 +771,16 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
         };
         auto keep = [&](int b_cut) {
             double Z = 0.0, X = 0.0;
+            int n = 0;
             for (int i = b_max + lane; i <= b_cut; i += 32) {
                 const uint32_t c = bins[i];
-                if (c) {
-                    const float z = value_of_bin(i);
-                    const float x = fmaxf(fmaf(z, s_lo, fmaf(z, s_hi, -of)), -200.f);
-                    const double e = (double)ex2_approx(x) * (double)c;
-                    Z += e;
-                    X += e * (double)x;
-                }
+                if (c) add_kept(value_of_bin(i), (double)c, s_d, Od, Z, X);
+                n += (int)c;
             }
             Z = warp_sum(Z);
             X = warp_sum(X);
-            if (lane == 0) write(Z, X, value_of_bin(b_cut));
+            n = __reduce_add_sync(0xffffffffu, n);
+            if (lane == 0) write(Z, X, value_of_bin(b_cut), n);
         };
         auto select = [&](int b_lo) {
             __syncthreads();
@@ -819,6 +830,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
         uint32_t key = 0u;
         float cutv = -CUDART_INF_F;
         double Z = 0.0, X = 0.0;
+        int kept = 0;
         settled = n <= CAP && (TOTAL || P.top_k <= K_FAST<DT>);
         // (at least k logits lie at or above the bound, so the k-th largest is in the list)
         if (settled && use_k) settled = radix_select<false>(S, bins, bins + NB, (double)P.top_k, 0u, cut::key_of(m), m, sf, key, visit);
@@ -840,14 +852,9 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
         if (settled) {
             cutv = cut::value_of(key);
             for (int i = tid; i < n; i += NT)
-                if (keys[i] >= key) {
-                    const float z = cut::value_of(keys[i]);
-                    const float x = fmaxf(fmaf(z, s_lo, fmaf(z, s_hi, -of)), -200.f);
-                    const double e = (double)ex2_approx(x);
-                    Z += e;
-                    X += e * (double)x;
-                }
+                if (keys[i] >= key) { add_kept(cut::value_of(keys[i]), 1.0, s_d, Od, Z, X); ++kept; }
         }
+        if (P.kept) kept = (int)block_sum(S, (unsigned long long)kept);
         if (settled) {
             Z = warp_sum(Z);
             X = warp_sum(X);
@@ -857,14 +864,14 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             Z = X = 0.0;
             if (tid == 0) {
                 for (int k = 0; k < NW; ++k) { Z += S.red[k][0]; X += S.red[k][1]; }
-                write(Z, X, cutv);
+                write(Z, X, cutv, kept);
             }
         }
     }
     if (!settled) {
         __syncthreads();
-        const Kept kp = settle_from_row<DT>(S, bins, span_of<DT>(P, id), P.V, P.top_k, P.top_p, m, sf, s_hi, s_lo, of, total);
-        if (tid == 0) write(kp.Z, kp.X, kp.key ? cut::value_of(kp.key) : -CUDART_INF_F);
+        const Kept kp = settle_from_row<DT>(S, bins, span_of<DT>(P, id), P.V, P.top_k, P.top_p, m, sf, s_hi, s_lo, s_d, of, total);
+        if (tid == 0) write(kp.Z, kp.X, kp.key ? cut::value_of(kp.key) : -CUDART_INF_F, kp.n);
     }
     if (DT == SPEC_BF16) __syncthreads();                // the bins have been read
     clear();
@@ -938,8 +945,7 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
                     RowPart r = {};
                     r.cut = -CUDART_INF_F; r.O = ROWPART_EMPTY; r.bad = -1;
                     P.part[id] = r;
-                    P.cut[id] = -CUDART_INF_F;
-                }
+                    }
             }
             if (id == to) break;
         }

@@ -277,15 +277,6 @@ __device__ __noinline__ int pick_lane(double v, double tau, double &tau_res)
     return pos ? 31 - __clz(pos) : -1;
 }
 
-// 2^(z s - O) in fp64 (about 1e-15 relative); 0 for -inf and for exponents below the double range
-__device__ __forceinline__ double exp2_exact(float z, double s_d, int O)
-{
-    const double xd = (double)z * s_d - (double)O;
-    if (!(xd > -1000.0)) return 0.0;
-    const double nd = rint(xd);
-    return exp2_frac(xd - nd) * pow2d((int)nd);
-}
-
 // ------------------------------------------------------------------------------------------------
 // pass 1: a node's rows into resident e, its dominant tokens into the warp's exact list
 // ------------------------------------------------------------------------------------------------

@@ -161,10 +161,10 @@ def test_tree_probs(V, dtype):
         np.testing.assert_allclose(st[..., 4], rs[..., 4], atol=PROB_TOL)
 
 
-@pytest.mark.parametrize("V", [7, 1000, 50001, 128256, 300000])
-def test_sample_bonus(V):
+@pytest.mark.parametrize("V,R", [(7, 64), (1000, 64), (50001, 64), (128256, 64), (300000, 64),
+                                 (127, 6), (8192, 6), (16385, 700), (4096, 300)])        # slices and tiles: their edges, one CTA a row
+def test_sample_bonus(V, R):
     g = torch.Generator(device="cuda").manual_seed(8)
-    R = 64
     w = torch.rand((R, V), generator=g, device="cuda")
     w = torch.where(torch.rand((R, V), generator=g, device="cuda") < 0.4, torch.zeros_like(w), w)
     w[3] = 0.0                                   # an all-zero row
