@@ -135,6 +135,7 @@ __device__ __forceinline__ double ratio(double P, double Q) { return !(P > 0.0) 
 __global__ void __launch_bounds__(128) spec_branch_kernel(const BParams P)
 {
     __shared__ double dp[4][1 << AN_KDP];
+    grid_dependency_wait();
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long node = (long long)blockIdx.x * 4 + wib;
     if (node >= (long long)P.B * P.N) return;
@@ -273,6 +274,7 @@ struct RParams {
 // one thread per (solver, sequence): parents come before their children
 __global__ void spec_reach_kernel(const RParams P)
 {
+    grid_dependency_wait();
     const int id = blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= NSOLVER * P.B) return;
     const int s = id / P.B, b = id % P.B;

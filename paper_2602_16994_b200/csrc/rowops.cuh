@@ -262,6 +262,7 @@ struct TParams {
 __global__ void __launch_bounds__(NT, 2) spec_probs_kernel(const TParams P)
 {
     cg::cluster_group cluster = cg::this_cluster();
+    grid_dependency_wait();
     const int C = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
     const int row_id = blockIdx.x / C;

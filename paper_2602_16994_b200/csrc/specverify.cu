@@ -46,6 +46,7 @@ struct RParams {
 // node's recorded coefficients, u <- (g_j u - e_q)+ from u = e_p, divided by the recorded total.
 __global__ void spec_residual_kernel(const RParams P)
 {
+    grid_dependency_wait();
     const int b = blockIdx.y;
     const int acc = P.accepted[b];
     float *out = P.residual + (long long)b * P.V;
@@ -165,8 +166,7 @@ inline int64_t up256(int64_t x) { return (x + 255) / 256 * 256; }
 struct WsLayout {
     int64_t rec, pub, fin, done, ticket, chain, kept, stat, gseq, total;
 };
-constexpr int MAX_PARTS = 4;      // parts a row may be split into by the streaming statistics kernel
-WsLayout ws_layout(const SpecIn *in, int slices = MAX_PARTS)   // slices = 0: one record per row only
+WsLayout ws_layout(const SpecIn *in)
 {
     WsLayout L;
     const int64_t nodes = (int64_t)in->B * in->N;
@@ -180,7 +180,7 @@ WsLayout ws_layout(const SpecIn *in, int slices = MAX_PARTS)   // slices = 0: on
     o = up256(o);
     L.chain = o; o += up256(nodes * (int64_t)sizeof(ChainRec));
     L.kept = o; o += up256(nodes * 8);
-    L.stat = o; o += up256(nodes * 2 * (slices + 1) * (int64_t)sizeof(RowPart));      // one record per row, then the parts
+    L.stat = o; o += up256(nodes * 2 * (int64_t)sizeof(RowPart));
     L.gseq = o; o += up256(nodes * KMAX * 8);       // step coefficients of every node
     L.total = o;
     return L;
@@ -198,20 +198,47 @@ int launch_clustered(K kernel, int ctas, int C, int threads, int smem, cudaStrea
     cfg.blockDim = dim3((unsigned)threads, 1, 1);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = st;
+    // (C = 0: a kernel that knows no clusters; the recursion kernel uses cluster instructions in a cluster of one as well)
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    unsigned n = 0;
+    if (C > 0) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = C;
+        attr[n].val.clusterDim.y = 1;
+        attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
     // dependent: the kernel waits by itself (grid_dependency_wait) for the kernel before it in the stream, so
     // its CTAs may be placed, and run their set-up, while that kernel's last CTAs still work
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    if (dependent) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = dependent ? 2 : 1;
+    cfg.numAttrs = n;
     void *args[1] = {params_ptr};
     cudaError_t e = cudaLaunchKernelExC(&cfg, (const void *)kernel, args);
     if (e != cudaSuccess) { cudaGetLastError(); return SPEC_ERR_CUDA; }
+    g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
+    return SPEC_OK;
+}
+
+// a kernel without clusters or dynamic shared memory that waits by itself for the kernel before it
+template <typename K, typename A>
+int launch_after(K kernel, dim3 grid, int threads, cudaStream_t st, A *params)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void *args[1] = {params};
+    if (cudaLaunchKernelExC(&cfg, (const void *)kernel, args) != cudaSuccess) { cudaGetLastError(); return SPEC_ERR_CUDA; }
     g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
     return SPEC_OK;
 }
@@ -343,9 +370,7 @@ int launch_trunc(const SpecIn *in, const void *zp, const void *zq, const int *pa
     auto go = [&](auto kernel, int smem) {
         const int rc = prepare_kernel(kernel, 1, smem);
         if (rc) return rc;
-        kernel<<<grid, trunc::NT, smem, st>>>(rp);
-        g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
-        return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_ERR_CUDA;
+        return launch_clustered(kernel, (int)grid, 0, trunc::NT, smem, st, &rp, true);
     };
     if (bf)
         return total ? go(trunc::spec_row_trunc_kernel<SPEC_BF16, true>, trunc::Layout<SPEC_BF16>::BYTES)
@@ -368,73 +393,52 @@ int launch_walk(const VPlan &pl, WParams &wp, cudaStream_t st)
     return launch_clustered(kernel, nc * pl.C, pl.C, threads, pl.smem, st, &wp, true);
 }
 
-// Statistics of every row the verifiers read (reference, normaliser, cut; one record per row at the
-// start of the statistics region), and the entropy features when asked for.  `parts`: the streaming
-// kernel may split rows into parts (needs the parts region of the workspace).
-int row_statistics(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, bool trunc, bool parts,
-                   cudaStream_t st, bool init_nodes = false)
+// Statistics of every row the verifiers read (reference, normaliser, cut), and the entropy features when asked for.
+int row_statistics(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, bool trunc, cudaStream_t st,
+                   bool init_nodes = false)
 {
-    int rc;
-    int NSL = 1;
-    RowPart *part = (RowPart *)(w + L.stat);
     stream::NodeInit init = {};
     if (init_nodes)
         init = {(unsigned long long *)(w + L.pub), (unsigned int *)(w + L.done), (int *)(w + L.fin),
                 (unsigned int *)(w + L.ticket), (ulonglong2 *)(w + L.chain)};
+    const bool feat = out->node_features != nullptr;
+    const auto features = [&]() {
+        if (!feat) return (int)SPEC_OK;
+        stream::FParams fp = {2ll * in->B * in->N, (const RowPart *)(w + L.stat), out->node_features};
+        return launch_after(stream::spec_features_kernel, dim3((unsigned)((fp.rows + 127) / 128)), 128, st, &fp);
+    };
     if (trunc) {
-        rc = launch_trunc(in, in->target_logits, in->draft_logits, in->parent, w, L, init, st);
-        if (rc) return rc;
-    } else {
-        // rows are split into parts only when there are fewer rows than resident CTAs
-        const long long rows2 = 2ll * in->B * in->N;
-        const int slices_row = (in->V + stream::SLICE - 1) / stream::SLICE;
-        NSL = 1;
-        while (parts && NSL < MAX_PARTS && NSL < slices_row && rows2 * NSL < 2 * sm_count()) NSL *= 2;
-        stream::SParams sp = {};
-        sp.B = in->B; sp.N = in->N; sp.V = in->V; sp.NSL = NSL;
-        sp.zp = in->target_logits; sp.zq = in->draft_logits;
-        sp.seq_stride = in->seq_stride; sp.node_stride = in->node_stride; sp.topo_stride = in->topo_seq_stride;
-        sp.parent = in->parent; sp.T = in->temperature; sp.T_seq = in->temperature_per_seq; sp.part = part;
-        // parts go to the second half of the statistics region, the merged rows to its start; a row
-        // in one part is final as written.  One CTA per item: those of unread rows retire at once.
-        RowPart *parts = part + 2ll * in->B * in->N;
-        sp.part = NSL > 1 ? parts : part;
-        sp.init = init;
-        const long long items = 2ll * in->B * in->N * NSL;
-        const unsigned grid = (unsigned)(items < (1ll << 20) ? items : (1ll << 20));
-        int prc;
-        const bool feat = out->node_features != nullptr;
-#define SPECV_STREAM(DTV, FT)                                                                                     \
-    do {                                                                                                          \
-        if ((prc = prepare_kernel(stream::spec_row_partial_kernel<DTV, FT>, 1, stream::Ring<DTV>::BYTES))) return prc; \
-        stream::spec_row_partial_kernel<DTV, FT><<<grid, stream::NT, stream::Ring<DTV>::BYTES, st>>>(sp);         \
-        g_kernel_launches.fetch_add(1, std::memory_order_relaxed);                                               \
-    } while (0)
-        if (in->logits_dtype == SPEC_BF16) { if (feat) SPECV_STREAM(SPEC_BF16, true); else SPECV_STREAM(SPEC_BF16, false); }
-        else { if (feat) SPECV_STREAM(SPEC_F32, true); else SPECV_STREAM(SPEC_F32, false); }
-#undef SPECV_STREAM
-        if (cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
-        if (NSL > 1) {
-            stream::MParams mp = {2ll * in->B * in->N, NSL, parts, part};
-            stream::spec_row_merge_kernel<<<(unsigned)((mp.rows2 * 32 + 255) / 256), 256, 0, st>>>(mp);
-            g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
-            if (cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
-        }
-        NSL = 1;
+        const int rc = launch_trunc(in, in->target_logits, in->draft_logits, in->parent, w, L, init, st);
+        return rc ? rc : features();
     }
-    if (out->node_features) {
-        stream::FParams fp = {(long long)in->B * in->N, NSL, part, out->node_features};
-        const unsigned grid = (unsigned)(((long long)in->B * in->N * 32 + 255) / 256);
-        stream::spec_features_kernel<<<grid, 256, 0, st>>>(fp);
-        g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
-        if (cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
-    }
-    return SPEC_OK;
+    // rows are split into parts only when there are fewer rows than resident CTAs
+    const long long rows2 = 2ll * in->B * in->N;
+    const int slices_row = (in->V + stream::SLICE - 1) / stream::SLICE;
+    int NSL = 1;
+    while (NSL < stream::MAX_PARTS && NSL < slices_row && rows2 * NSL < 2 * sm_count()) NSL *= 2;
+    stream::SParams sp = {};
+    sp.B = in->B; sp.N = in->N; sp.V = in->V; sp.NSL = NSL;
+    sp.zp = in->target_logits; sp.zq = in->draft_logits;
+    sp.seq_stride = in->seq_stride; sp.node_stride = in->node_stride; sp.topo_stride = in->topo_seq_stride;
+    sp.parent = in->parent; sp.T = in->temperature; sp.T_seq = in->temperature_per_seq;
+    sp.part = (RowPart *)(w + L.stat); sp.init = init;
+    // one CTA per item: those of unread rows retire at once
+    const long long items = rows2 * NSL;
+    const int grid = (int)(items < (1ll << 20) ? items : (1ll << 20));
+    const auto go = [&](auto kernel, int smem) {
+        int rc = prepare_kernel(kernel, 1, smem);
+        if (!rc) rc = launch_clustered(kernel, grid, NSL > 1 ? NSL : 0, stream::NT, smem, st, &sp, true);
+        return rc ? rc : features();
+    };
+    if (in->logits_dtype == SPEC_BF16)
+        return feat ? go(stream::spec_row_partial_kernel<SPEC_BF16, true>, stream::Ring<SPEC_BF16>::BYTES)
+                    : go(stream::spec_row_partial_kernel<SPEC_BF16, false>, stream::Ring<SPEC_BF16>::BYTES);
+    return feat ? go(stream::spec_row_partial_kernel<SPEC_F32, true>, stream::Ring<SPEC_F32>::BYTES)
+                : go(stream::spec_row_partial_kernel<SPEC_F32, false>, stream::Ring<SPEC_F32>::BYTES);
 }
 
 // solver: -1 SpecInfer, otherwise the OTLP solver of spec_verify_otlp
-int verify_walk(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, bool trunc, bool parts,
-                cudaStream_t st, int solver = -1)
+int verify_walk(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, bool trunc, cudaStream_t st, int solver = -1)
 {
     // The walk keeps one cluster per sequence busy.  While all of them fit on the chip with one CTA per SM, a CTA may use
     // all of an SM's registers; larger batches share the SMs.
@@ -444,7 +448,7 @@ int verify_walk(const SpecIn *in, const SpecOut *out, unsigned char *w, const Ws
     const bool whole = fits && ((long long)in->B * one.C <= sm_count() || !two_cta_plan(in->V, (int)sizeof(WHdr), &pl));
     if (whole) pl = one;
     else if (!fits) return SPEC_ERR_UNSUPPORTED;
-    int rc = row_statistics(in, out, w, L, trunc, parts, st);
+    int rc = row_statistics(in, out, w, L, trunc, st);
     if (rc) return rc;
     WParams wp = {};
     wp.B = in->B; wp.N = in->N; wp.V = in->V; wp.C = pl.C; wp.off_es = pl.off_es;
@@ -529,15 +533,14 @@ int launch_nodes(const SpecIn *in, NParams &np, bool analysis, cudaStream_t st)
     return bf ? launch_finish<SPEC_BF16, 0>(fi, np, st) : launch_finish<SPEC_F32, 0>(fi, np, st);
 }
 
-int verify_common(const SpecIn *in, const SpecOut *out, void *ws, int64_t ws_bytes, void *stream, int mode,
-                  bool parts = true)
+int verify_common(const SpecIn *in, const SpecOut *out, void *ws, int64_t ws_bytes, void *stream, int mode)
 {
     int rc = check_in(in, true);
     if (rc) return rc;
     if (!out || !out->accepted_node || !out->accept_len || !out->out_tokens || !out->bonus_token || !out->status)
         return SPEC_ERR_NULL;
     const bool trunc = (in->top_k > 0 && in->top_k < in->V) || in->top_p < 1.f;
-    const WsLayout L = ws_layout(in, parts ? MAX_PARTS : 0);
+    const WsLayout L = ws_layout(in);
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < L.total) return SPEC_ERR_WORKSPACE;
     VPlan pl;
     bool big;
@@ -545,10 +548,10 @@ int verify_common(const SpecIn *in, const SpecOut *out, void *ws, int64_t ws_byt
     cudaStream_t st = (cudaStream_t)stream;
     unsigned char *w = (unsigned char *)ws;
     const bool diagnostics = out->residual || out->node_thr || out->node_w_in || out->margin;
-    if (mode == MODE_SPECINFER && !diagnostics && in->N <= NWALK) return verify_walk(in, out, w, L, trunc, parts, st);
+    if (mode == MODE_SPECINFER && !diagnostics && in->N <= NWALK) return verify_walk(in, out, w, L, trunc, st);
     // every node of every sequence on chip once, on top of the row statistics (which also set the
     // published-weight slots to pending and the arrival counters to zero)
-    rc = row_statistics(in, out, w, L, trunc, parts, st, true);
+    rc = row_statistics(in, out, w, L, trunc, st, true);
     if (rc) return rc;
     NParams tp = {};
     fill_params(in, out, w, L, mode, tp);
@@ -564,9 +567,8 @@ int verify_common(const SpecIn *in, const SpecOut *out, void *ws, int64_t ws_byt
         rp.rec = vp.rec; rp.gseq = tp.gseq; rp.accepted = out->accepted_node; rp.residual = out->residual;
         int gx = (in->V + 255) / 256;
         if (gx > 296) gx = 296;
-        spec_residual_kernel<<<dim3(gx, in->B), 256, 0, st>>>(rp);
-        g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
-        if (cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
+        rc = launch_after(spec_residual_kernel, dim3(gx, in->B), 256, st, &rp);
+        if (rc) return rc;
     }
     return SPEC_OK;
 }
@@ -729,7 +731,7 @@ int32_t spec_row_statistics(const SpecIn *in, void *ws, int64_t ws_bytes, void *
     const WsLayout L = ws_layout(in);
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < L.total) return SPEC_ERR_WORKSPACE;
     SpecOut none = {};
-    return row_statistics(in, &none, (unsigned char *)ws, L, trunc, true, (cudaStream_t)stream, true);
+    return row_statistics(in, &none, (unsigned char *)ws, L, trunc, (cudaStream_t)stream, true);
 }
 
 int32_t spec_verify_specinfer(const SpecIn *in, const SpecOut *out, void *ws, int64_t ws_bytes, void *stream)
@@ -754,18 +756,18 @@ int32_t spec_verify_otlp(const SpecIn *in, const SpecOut *out, int32_t solver, v
     const bool trunc = (in->top_k > 0 && in->top_k < in->V) || in->top_p < 1.f;
     const WsLayout L = ws_layout(in);
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < L.total) return SPEC_ERR_WORKSPACE;
-    return verify_walk(in, out, (unsigned char *)ws, L, trunc, true, (cudaStream_t)stream, solver);
+    return verify_walk(in, out, (unsigned char *)ws, L, trunc, (cudaStream_t)stream, solver);
 }
 
 int32_t spec_verify_specinfer_static(const SpecIn *in, const SpecOut *out, void *stream)
 {
     int rc = check_in(in, true);
     if (rc) return rc;
-    if ((int64_t)in->B * in->N > SPEC_STATIC_MAX_NODES || ws_layout(in, 0).total > STATIC_WS_BYTES) return SPEC_ERR_WORKSPACE;
+    if ((int64_t)in->B * in->N > SPEC_STATIC_MAX_NODES || ws_layout(in).total > STATIC_WS_BYTES) return SPEC_ERR_WORKSPACE;
     void *ws = nullptr;
     rc = static_ws_address(&ws);
     if (rc) return rc;
-    return verify_common(in, out, ws, STATIC_WS_BYTES, stream, MODE_SPECINFER, false);
+    return verify_common(in, out, ws, STATIC_WS_BYTES, stream, MODE_SPECINFER);
 }
 
 // analysis workspace: the verifiers' layout | per-node scalars | scratch for the decision outputs nobody reads
@@ -822,7 +824,7 @@ int32_t spec_tree_analysis(const SpecIn *in, const SpecAnalysisOut *out, void *w
     so.accepted_node = (int32_t *)(w + A.acc); so.accept_len = (int32_t *)(w + A.len);
     so.out_tokens = (int32_t *)(w + A.toks); so.bonus_token = (int32_t *)(w + A.bonus);
     so.status = (int32_t *)(w + A.status);
-    rc = row_statistics(in, &so, w, L, trunc, true, st, true);
+    rc = row_statistics(in, &so, w, L, trunc, st, true);
     if (rc) return rc;
     NParams tp = {};
     fill_params(in, &so, w, L, MODE_SPECINFER, tp);
@@ -831,13 +833,10 @@ int32_t spec_tree_analysis(const SpecIn *in, const SpecAnalysisOut *out, void *w
     rc = launch_nodes(in, tp, true, st);
     if (rc) return rc;
     analysis::BParams bp = {in->B, in->N, in->parent, in->token, in->topo_seq_stride, tp.an, out->acceptance, out->branch};
-    analysis::spec_branch_kernel<<<(unsigned)((nodes + 3) / 4), 128, 0, st>>>(bp);
-    g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
+    rc = launch_after(analysis::spec_branch_kernel, dim3((unsigned)((nodes + 3) / 4)), 128, st, &bp);
+    if (rc) return rc;
     analysis::RParams rp = {in->B, in->N, in->parent, in->topo_seq_stride, out->branch, out->reach, out->block_eff};
-    analysis::spec_reach_kernel<<<(unsigned)((analysis::NSOLVER * in->B + 127) / 128), 128, 0, st>>>(rp);
-    g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
-    if (cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
-    return SPEC_OK;
+    return launch_after(analysis::spec_reach_kernel, dim3((unsigned)((analysis::NSOLVER * in->B + 127) / 128)), 128, st, &rp);
 }
 
 int32_t spec_latency_model(const double *t_q, const double *t_p, int32_t n_len, int32_t ctx, const int32_t *actions,
@@ -877,7 +876,7 @@ int32_t spec_tree_probs(const SpecIn *in, int32_t which, float *probs, float *ro
         kp.parts = probs ? (in->V + rowops::KEPT_PART - 1) / rowops::KEPT_PART : 1;
         kp.items = (long long)in->B * in->N * kp.parts;
         const int grid = (int)std::min(kp.items, 1ll << 20);
-        const auto go = [&](auto kernel) { return launch_clustered(kernel, grid, 1, rowops::KEPT_NT, 0, (cudaStream_t)stream, &kp, true); };
+        const auto go = [&](auto kernel) { return launch_clustered(kernel, grid, 0, rowops::KEPT_NT, 0, (cudaStream_t)stream, &kp, true); };
         return in->logits_dtype == SPEC_BF16 ? go(rowops::spec_probs_kept_kernel<SPEC_BF16>) : go(rowops::spec_probs_kept_kernel<SPEC_F32>);
     }
     rowops::TParams tp = {};
@@ -886,7 +885,7 @@ int32_t spec_tree_probs(const SpecIn *in, int32_t which, float *probs, float *ro
     tp.T = in->temperature; tp.T_seq = in->temperature_per_seq; tp.probs = probs; tp.stats = row_stats;
     rc = prepare_kernel(rowops::spec_probs_kernel, pl.C, pl.smem);
     if (rc) return rc;
-    return launch_clustered(rowops::spec_probs_kernel, tp.rows * pl.C, pl.C, rowops::NT, pl.smem, (cudaStream_t)stream, &tp);
+    return launch_clustered(rowops::spec_probs_kernel, tp.rows * pl.C, pl.C, rowops::NT, pl.smem, (cudaStream_t)stream, &tp, true);
 }
 
 int32_t spec_sample_bonus(const float *weights, int32_t R, int32_t V, const float *u, int32_t *token,

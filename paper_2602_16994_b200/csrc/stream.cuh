@@ -6,7 +6,7 @@
 // A thread turns its logits into e = 2^(z s - o) (s = log2(e)/T, o = ceil of its own largest z s, an
 // integer, so partial sums combine by exact powers of two) and the CTA writes, for its row or part of one,
 //     O = largest o, S = sum e 2^(o - O), X = sum e x 2^(o - O) with x = z s - O, the largest exponent.
-// Rows in parts (batches with fewer rows than half the places) are merged by spec_row_merge_kernel.
+// Rows in parts (batches with fewer rows than half the places) are a cluster each, and its first CTA merges them.
 #pragma once
 #include "common.cuh"
 
@@ -25,6 +25,7 @@ constexpr int ROWPART_EMPTY = -(1 << 30);
 
 namespace stream {
 
+constexpr int MAX_PARTS = 4;             // of a row
 constexpr int NT = 256;
 constexpr int PER = 32;                  // logits per thread
 constexpr int SLICE = NT * PER;          // logits per CTA and slice
@@ -49,13 +50,13 @@ struct NodeInit {
 };
 
 struct SParams {
-    int B, N, V, NSL;        // NSL: parts a row is split into (more CTAs than rows)
+    int B, N, V, NSL;        // NSL: parts a row is split into (more CTAs than rows), a cluster of as many CTAs
     const void *zp, *zq;
     long long seq_stride, node_stride, topo_stride;
     const int *parent;
     float T;
     const float *T_seq;
-    RowPart *part;           // [B*N*2][NSL]
+    RowPart *part;           // [B*N*2]
     NodeInit init;
 };
 
@@ -184,6 +185,40 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b)
     return d;
 }
 
+// a part of a row into the same place of the cluster's first CTA
+__device__ __forceinline__ void store_part(RowPart *slot, const RowPart &r)
+{
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(at) : "r"(smem_u32(slot)));
+    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(at), "d"(r.S), "d"(r.X) : "memory");
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + 16u), "r"(r.O), "r"(__float_as_int(r.xmax)), "r"(__float_as_int(r.cut)), "r"(r.bad) : "memory");
+}
+// the parts of a row as one record, by one warp
+__device__ __forceinline__ RowPart merge_parts(const RowPart *p, int n, bool feat)
+{
+    const int lane = threadIdx.x & 31;
+    const bool has = lane < n;
+    const int Ok = has ? p[lane].O : ROWPART_EMPTY, O = __reduce_max_sync(0xffffffffu, Ok);
+    const int bad = __any_sync(0xffffffffu, has && p[lane].bad == 1);
+    double S = 0.0, X = 0.0, best = -1.0e300;
+    if (Ok > ROWPART_EMPTY) {
+        const int d = max(Ok - O, -100000);
+        const double f = pow2d(d);
+        S = p[lane].S * f;
+        X = f * (p[lane].X + (double)d * p[lane].S);
+        best = (double)Ok + (double)p[lane].xmax;
+    }
+    S = warp_sum(S);
+    X = warp_sum(X);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
+    RowPart r;
+    r.S = S; r.X = X; r.O = O; r.xmax = feat && O > ROWPART_EMPTY ? (float)(best - (double)O) : 0.f;
+    r.cut = -CUDART_INF_F;
+    r.bad = bad || !(S > 0.0) || !(S < CUDART_INF) ? 1 : 0;
+    return r;
+}
+
 // FEAT: also accumulate X (needed only by the entropy features).  Without it a NaN or +inf logit is
 // found from the sum itself (such a logit makes its e, and so the thread's sum, non-finite), which
 // keeps comparisons out of the inner loop.
@@ -193,11 +228,14 @@ __global__ void __launch_bounds__(NT, 2) spec_row_partial_kernel(const SParams P
     constexpr int NV = Ring<DT>::NV, UNITS = Ring<DT>::UNITS, DEPTH = Ring<DT>::DEPTH;
     __shared__ double sS[NT / 32], sX[NT / 32], sB[NT / 32];
     __shared__ int sO[NT / 32], sBad[NT / 32];
+    __shared__ RowPart sPart[MAX_PARTS];                          // of the cluster's row, in its first CTA
     uint4 *ring = reinterpret_cast<uint4 *>(dyn_smem);            // [DEPTH][UNITS][NT]
     const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const long long items = 2ll * P.B * P.N * P.NSL;
+    grid_dependency_wait();       // (what the call was given may come from the kernel before)
     grid_launch_dependents();     // a dependent verifier's CTAs may take the places of CTAs that have finished
+    if (P.NSL > 1) cluster_sync_all();       // the first CTA's shared memory is there to be written
 
     for (long long id = blockIdx.x; id < items; id += gridDim.x) {
         const int h = (int)(id % P.NSL);
@@ -205,11 +243,11 @@ __global__ void __launch_bounds__(NT, 2) spec_row_partial_kernel(const SParams P
         const int which = (int)(row2 & 1);
         const long long row = row2 >> 1;
         const int b = (int)(row / P.N), a = (int)(row % P.N);
-        RowPart *out = P.part + row2 * P.NSL + h;
+        RowPart *out = P.part + row2;
         if (which == 0 && h == 0 && tid == 0) P.init.set(row, b, a);
         // a draft row is read only for nodes that have children (every warp finds out by itself)
         if (which == 1 && !has_children(P.parent + (long long)b * P.topo_stride, P.N, a, lane)) {
-            if (tid == 0) { RowPart r = {}; r.O = ROWPART_EMPTY; r.cut = -CUDART_INF_F; r.bad = -1; *out = r; }
+            if (tid == 0 && h == 0) { RowPart r = {}; r.O = ROWPART_EMPTY; r.cut = -CUDART_INF_F; r.bad = -1; *out = r; }
             continue;
         }
         const RowSpan span = row_span<DT>(which ? P.zq : P.zp, (long long)b * P.seq_stride + (long long)a * P.node_stride, P.V);
@@ -381,100 +419,46 @@ __global__ void __launch_bounds__(NT, 2) spec_row_partial_kernel(const SParams P
                 RowPart r;
                 r.S = S; r.X = X; r.O = O; r.xmax = (FEAT && O > ROWPART_EMPTY) ? (float)(bst - (double)O) : 0.f;
                 r.cut = -CUDART_INF_F; r.bad = bd;
-                *out = r;
+                if (P.NSL == 1) *out = r;
+                else store_part(&sPart[h], r);
             }
         }
-    }
-}
-
-// Merge the slices of every row into one record (slice 0 of the merged array): one warp per row.
-struct MParams {
-    long long rows2;
-    int NSL;
-    const RowPart *part;     // [rows2][NSL]
-    RowPart *merged;         // [rows2]
-};
-
-__global__ void spec_row_merge_kernel(const MParams P)
-{
-    grid_launch_dependents();     // (one sequence: the ratio kernel's CTAs are in their places when the last row is merged)
-    const long long r2 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (r2 >= P.rows2) return;
-    const RowPart *p = P.part + r2 * P.NSL;
-    int O = ROWPART_EMPTY, bad = 0, unread = 0;
-    for (int j = lane; j < P.NSL; j += 32) { O = max(O, p[j].O); bad |= p[j].bad == 1; unread |= p[j].bad == -1; }
-    O = __reduce_max_sync(0xffffffffu, O);
-    bad = __any_sync(0xffffffffu, bad);
-    unread = __any_sync(0xffffffffu, unread);
-    double S = 0.0, X = 0.0, best = -1.0e300;
-    for (int j = lane; j < P.NSL; j += 32) {
-        if (p[j].O > ROWPART_EMPTY) {
-            const int d = max(p[j].O - O, -100000);
-            const double fk = pow2d(d);
-            S += p[j].S * fk;
-            X += fk * (p[j].X + (double)d * p[j].S);
-            best = fmax(best, (double)p[j].O + (double)p[j].xmax);
+        if (P.NSL > 1) {
+            cluster_sync_all();
+            if (h == 0 && w == 0) {
+                const RowPart r = merge_parts(sPart, P.NSL, FEAT);
+                if (lane == 0) *out = r;
+            }
+            cluster_sync_all();          // the parts have been read
         }
     }
-    S = warp_sum(S);
-    X = warp_sum(X);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if (lane == 0) {
-        RowPart r;
-        r.S = S; r.X = X; r.O = O; r.xmax = O > ROWPART_EMPTY ? (float)(best - (double)O) : 0.f;
-        r.cut = -CUDART_INF_F;
-        r.bad = unread ? -1 : ((bad || !(S > 0.0) || !(S < CUDART_INF)) ? 1 : 0);
-        P.merged[r2] = r;
-    }
 }
 
-// Selector features of every node from the row statistics: entropy (nats) and largest probability of
-// the target and draft sampling distributions.  One warp per node.
+// Selector features of every row from its record: entropy (nats) and largest probability, [nodes][4]: H_p, H_q, top1_p, top1_q (those of
+// a row that is not read are 0).  A thread per row.  (In the statistics kernels, by the thread that writes the record, they hold
+// up the next row of the CTA: 760 instead of 710 us for a top-k call with 12000 rows.)
 struct FParams {
-    long long nodes;
-    int NSL;
+    long long rows;          // 2 B N
     const RowPart *part;
-    float *features;         // [nodes][4]: H_p, H_q, top1_p, top1_q (q entries 0 for nodes without children)
+    float *features;
 };
 
-__global__ void spec_features_kernel(const FParams P)
+__global__ void __launch_bounds__(128) spec_features_kernel(const FParams P)
 {
-    const long long node = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (node >= P.nodes) return;
-    float f[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int which = 0; which < 2; ++which) {
-        const RowPart *p = P.part + (node * 2 + which) * P.NSL;
-        int O = ROWPART_EMPTY, bad = 0, unread = 0;
-        for (int j = lane; j < P.NSL; j += 32) { O = max(O, p[j].O); bad |= p[j].bad == 1; unread |= p[j].bad == -1; }
-        O = __reduce_max_sync(0xffffffffu, O);
-        bad = __any_sync(0xffffffffu, bad);
-        unread = __any_sync(0xffffffffu, unread);
-        double S = 0.0, X = 0.0, best = -1.0e300;
-        for (int j = lane; j < P.NSL; j += 32) {
-            if (p[j].O > ROWPART_EMPTY) {
-                const int d = max(p[j].O - O, -100000);
-                const double fk = pow2d(d);
-                S += p[j].S * fk;
-                X += fk * (p[j].X + (double)d * p[j].S);
-                best = fmax(best, (double)p[j].O + (double)p[j].xmax);
-            }
-        }
-        S = warp_sum(S);
-        X = warp_sum(X);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
-        if (unread) continue;
-        if (bad || !(S > 0.0) || !(S < CUDART_INF)) { f[which] = CUDART_NAN_F; f[2 + which] = CUDART_NAN_F; continue; }
-        f[which] = (float)(log(S) - 0.6931471805599453 * X / S);
-        f[2 + which] = (float)(exp2(best - (double)O) / S);
+    grid_dependency_wait();
+    grid_launch_dependents();
+    const long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= P.rows) return;
+    const RowPart r = P.part[row];
+    float H = 0.f, top = 0.f;
+    if (r.bad != -1) {
+        const bool ok = r.bad == 0 && r.S > 0.0 && r.S < CUDART_INF;
+        H = ok ? (float)(log(r.S) - 0.6931471805599453 * r.X / r.S) : CUDART_NAN_F;
+        top = ok ? (float)(exp2((double)r.xmax) / r.S) : CUDART_NAN_F;
     }
-    if (lane == 0) {
-        float *o = P.features + node * 4;
-        o[0] = f[0]; o[1] = f[1]; o[2] = f[2]; o[3] = f[3];
-    }
+    float *f = P.features + (row >> 1) * 4 + (row & 1);
+    f[0] = H;
+    f[2] = top;
 }
 
 }  // namespace stream

@@ -730,7 +730,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
                 RowPart r = {};
                 r.cut = -CUDART_INF_F; r.O = ROWPART_EMPTY; r.bad = 1;
                 *out = r;
-            }
+                    }
             __syncthreads();
             clear();
             if (tid == 0) { S.runmax = 0u; S.count = 0; S.odd = 0; }
@@ -890,6 +890,7 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
     const uint32_t ring_s = smem_u32(M.ring) + tid * 16u;
     const unsigned lt = (1u << lane) - 1u;
     const int items = 2 * P.B * P.N;           // (at most 2^25: the host checks B N)
+    grid_dependency_wait();       // (what the call was given may come from the kernel before)
     grid_launch_dependents();
 
     if (DT == SPEC_BF16) for (int i = tid; i < 2 * TB; i += NT) M.bins[i] = 0;
@@ -945,7 +946,7 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
                     RowPart r = {};
                     r.cut = -CUDART_INF_F; r.O = ROWPART_EMPTY; r.bad = -1;
                     P.part[id] = r;
-                    }
+                                }
             }
             if (id == to) break;
         }
