@@ -1164,6 +1164,7 @@ __global__ void __launch_bounds__(NW * 32, 1) spec_finish_kernel(const NParams N
     float4 *es = reinterpret_cast<float4 *>(dyn_smem + P.off_es);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, C = P.C;
     const unsigned rank = C > 1 ? cluster_ctarank() : 0u;
+    if (P.early) grid_launch_dependents();
     if (tid == 0) {
         common_init(S.M, NW);
         mbar_fence_init();

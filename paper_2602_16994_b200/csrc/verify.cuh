@@ -84,6 +84,7 @@ struct __align__(16) ChainRec {
 
 struct VParams {
     int B, N, V, C, mode, all_thr;
+    int early;                // let the next call's statistics take the places that are free (finish kernel)
     int off_es;               // byte offset of the resident e inside dynamic shared memory
     const void *zp, *zq;
     long long seq_stride, node_stride, topo_stride;
