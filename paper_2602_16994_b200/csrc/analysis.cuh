@@ -41,34 +41,68 @@ __device__ __forceinline__ F one_minus_power(F x, int k)
     return k > 0 ? x * s : (F)0;
 }
 struct FnFirst {        // sum |p - q|, sum min(p, q), sum p (1 - (1-q)^k)  (Algorithm 6), sum (p-q)+ (1 - (1-q)^(k-1))
-                        // (Algorithm 7), sum (p-q)+
+                        // (Algorithm 7)
     float ipf, iqf; double ip, iq; int k;
-    template <typename F> __device__ __forceinline__ void add(F p, F q, F (&a)[5]) const
+    template <typename F> __device__ __forceinline__ void add(F p, F q, F (&a)[4]) const
     {
         const F d = p - q, dp = d > (F)0 ? d : (F)0, qc = q < (F)1 ? q : (F)1;
         a[0] += d > (F)0 ? d : -d;
         a[1] += p < q ? p : q;
         a[2] += p * one_minus_power(qc, k);
         a[3] += dp * one_minus_power(qc, k - 1);
-        a[4] += dp;
     }
-    __device__ __forceinline__ void tail(float ep, float eq, float (&a)[5]) const { add(ep * ipf, eq * iqf, a); }
-    __device__ __forceinline__ void exact(double ep, double eq, double (&a)[5]) const { add(ep * ip, eq * iq, a); }
+    // (eight tokens side by side in the loop over k)
+    __device__ __forceinline__ void tail8(const float (&ep)[8], const float (&eq)[8], float (&a)[4]) const
+    {
+        float p[8], q[8], r[8], s[8], before[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) { p[t] = ep[t] * ipf; q[t] = eq[t] * iqf; r[t] = 1.f - fminf(q[t], 1.f); s[t] = 1.f; before[t] = 0.f; }
+#pragma unroll 1
+        for (int i = 1; i < k; ++i) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) { before[t] = s[t]; s[t] = fmaf(s[t], r[t], 1.f); }
+        }
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const float d = p[t] - q[t], dp = fmaxf(d, 0.f), qc = fminf(q[t], 1.f);
+            a[0] += fabsf(d);
+            a[1] += fminf(p[t], q[t]);
+            a[2] = fmaf(p[t], qc * s[t], a[2]);
+            a[3] = fmaf(dp, qc * before[t], a[3]);
+        }
+    }
+    __device__ __forceinline__ void exact(double ep, double eq, double (&a)[4]) const { add(ep * ip, eq * iq, a); }
 };
 struct FnBeta {         // beta(rho) = sum min(p / rho, q)   (Appendix B, above Algorithm 3)
     float ipf, iqf; double ip, iq;   // ip already divided by rho
-    __device__ __forceinline__ void tail(float ep, float eq, float (&a)[2]) const { a[0] += fminf(ep * ipf, eq * iqf); }
+    __device__ __forceinline__ void tail8(const float (&ep)[8], const float (&eq)[8], float (&a)[2]) const
+    {
+        float u = 0.f, v = 0.f;                 // (two chains of additions)
+#pragma unroll
+        for (int t = 0; t < 8; t += 2) { u += fminf(ep[t] * ipf, eq[t] * iqf); v += fminf(ep[t + 1] * ipf, eq[t + 1] * iqf); }
+        a[0] += u + v;
+    }
     __device__ __forceinline__ void exact(double ep, double eq, double (&a)[2]) const { a[0] += fmin(ep * ip, eq * iq); }
 };
 struct FnSpecTrRes {    // sum d, sum d (1 - (1-r)^k), d = (p - min(p/rho, q) gamma)+, r = (q - p/rho)+ / (1-beta)
     float ipf, iqf, irf, gf, ibf; double ip, iq, ir, g, ib; int k;     // ir = 1/rho, ib = 1/(1-beta) (0 when beta = 1)
-    __device__ __forceinline__ void tail(float ep, float eq, float (&a)[2]) const
+    __device__ __forceinline__ void tail8(const float (&ep)[8], const float (&eq)[8], float (&a)[2]) const
     {
-        const float p = ep * ipf, q = eq * iqf, pr = p * irf;
-        const float d = fmaxf(p - fminf(pr, q) * gf, 0.f);
-        const float r = fminf(fmaxf(q - pr, 0.f) * ibf, 1.f);
-        a[0] += d;
-        a[1] += d * one_minus_power(r, k);
+        float d[8], x[8], s[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const float p = ep[t] * ipf, q = eq[t] * iqf, pr = p * irf;
+            d[t] = fmaxf(p - fminf(pr, q) * gf, 0.f);
+            x[t] = fminf(fmaxf(q - pr, 0.f) * ibf, 1.f);
+            s[t] = 1.f;
+        }
+#pragma unroll 1
+        for (int i = 1; i < k; ++i) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) s[t] = fmaf(s[t], 1.f - x[t], 1.f);
+        }
+#pragma unroll
+        for (int t = 0; t < 8; ++t) { a[0] += d[t]; a[1] = fmaf(d[t], x[t] * s[t], a[1]); }
     }
     __device__ __forceinline__ void exact(double ep, double eq, double (&a)[2]) const
     {

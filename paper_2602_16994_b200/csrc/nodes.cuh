@@ -644,8 +644,204 @@ __global__ void __launch_bounds__(256, 3) spec_single_kernel(const NParams NP)
     if (blockIdx.x == 0) grid_dependency_wait();      // this kernel ends only after the one before it
 }
 
+// ---- the analysis of nodes with one child -----------------------------------------------------------------------------------
+// Everything Algorithms 6-9 and the divergences ask of such a node are sums over its two rows (SpecTr's division factor is 1, its
+// beta and acceptance are sum min(p, q)): two passes of the ring, nothing resident.  Tokens above 2^-DOM_S of a row's mass in fp64,
+// the others in fp32, fp64 above a chunk.
+// NORM: o = Z_p, Z_q and the cross sums of KlSums (pp, pq, qq, qp); else |p - q|, min(p, q), p min(q, 1) and (p - q)+.
+struct AnTerms {
+    double o[6];
+};
+template <bool NORM>
+__device__ __noinline__ AnTerms an_heavy(float2 z, float cut_p, float cut_q, int O_p, int O_q, double s_d, double ip, double iq)
+{
+    AnTerms t = {};
+    const double ep = z.x >= cut_p ? exp2_exact(z.x, s_d, O_p) : 0.0, eq = z.y >= cut_q ? exp2_exact(z.y, s_d, O_q) : 0.0;
+    if (NORM) {
+        const double xp = z.x >= cut_p ? (double)z.x * s_d - (double)O_p : -CUDART_INF, xq = z.y >= cut_q ? (double)z.y * s_d - (double)O_q : -CUDART_INF;
+        t.o[0] = ep; t.o[1] = eq;
+        if (ep > 0.0) { t.o[2] = ep * xp; t.o[3] = ep * xq; }
+        if (eq > 0.0) { t.o[4] = eq * xq; t.o[5] = eq * xp; }
+    } else {
+        const double p = ep * ip, q = eq * iq;
+        t.o[0] = fabs(p - q); t.o[1] = fmin(p, q); t.o[2] = p * fmin(q, 1.0); t.o[3] = fmax(p - q, 0.0);
+    }
+    return t;
+}
+template <int DT, bool NORM>
+__device__ __noinline__ AnTerms an_sums(const Slice sl, const NodeRows nr, double ip, double iq, uint4 *ring, float2 *heavy)
+{
+    constexpr int U = DT == SPEC_BF16 ? 1 : 2, NT = 256, NO = NORM ? 6 : 4;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const float s_hi = nr.s_hi, s_lo = nr.s_lo, O_p = (float)nr.O_p, O_q = (float)nr.O_q, ipf = (float)ip, iqf = (float)iq;
+    AnTerms sum = {};
+    int n = 0;                             // entries of the warp's list (below 32 between chunks)
+    ring += tid;
+    const auto take = [&](int at, bool on) {
+        const AnTerms t = an_heavy<NORM>(on ? heavy[at] : make_float2(-CUDART_INF_F, -CUDART_INF_F), nr.cut_p, nr.cut_q, nr.O_p, nr.O_q, nr.s_d, ip, iq);
+#pragma unroll
+        for (int i = 0; i < NO; ++i) sum.o[i] += on ? t.o[i] : 0.0;
+    };
+    auto issue = [&](int c) {
+        const int i = c * NT + tid;
+        if (sl.vec && i < sl.nu) {
+            const size_t u = (size_t)(sl.u0 + i) * U;
+            const uint4 *p = reinterpret_cast<const uint4 *>(sl.p) + u, *q = reinterpret_cast<const uint4 *>(sl.q) + u;
+            const uint32_t dst = smem_u32(ring + (c % NS<DT>) * 2 * U * NT);
+            stream::cp_async16(dst, p, 16);
+            stream::cp_async16(dst + U * NT * 16, q, 16);
+            if (U == 2 && (sl.u0 + i) * 8 - sl.h + 4 < sl.V) {
+                stream::cp_async16(dst + NT * 16, p + 1, 16);
+                stream::cp_async16(dst + 3 * NT * 16, q + 1, 16);
+            }
+        }
+        stream::cp_async_commit();
+    };
+#pragma unroll 1
+    for (int c = 0; c < NS<DT> - 1; ++c) issue(c);
+#pragma unroll 1
+    for (int c = 0; c * NT < sl.nu; ++c) {
+        const int i = c * NT + tid, t0 = (sl.u0 + i) * 8 - sl.h, lo = -t0, hi = i < sl.nu ? sl.V - t0 : 0;
+        RawChunk<DT> rp, rq;
+        stream::cp_async_wait<NS<DT> - 2>();
+        const uint4 *st = ring + (c % NS<DT>) * 2 * U * NT;
+        rp.a = st[0];
+        rq.a = st[U * NT];
+        if (U == 2) { rp.b = st[NT]; rq.b = st[3 * NT]; }
+        if (!sl.vec && i < sl.nu) {
+            rp = load_raw_scalar<DT>(sl.p, sl.u0 + i, sl.V);
+            rq = load_raw_scalar<DT>(sl.q, sl.u0 + i, sl.V);
+        }
+        issue(c + NS<DT> - 1);             // into the stage read in the previous iteration
+        float xp[8], xq[8], ep[8], eq[8];
+        unpack_chunk<DT>(rp, xp);
+        mask_chunk(xp, lo, hi, nr.cut_p > -CUDART_INF_F, nr.cut_p);
+        unpack_chunk<DT>(rq, xq);
+        mask_chunk(xq, lo, hi, nr.cut_q > -CUDART_INF_F, nr.cut_q);
+        unsigned m = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            xp[k] = fmaf(xp[k], s_lo, fmaf(xp[k], s_hi, -O_p));
+            xq[k] = fmaf(xq[k], s_lo, fmaf(xq[k], s_hi, -O_q));
+            ep[k] = ex2_approx(xp[k]);
+            eq[k] = ex2_approx(xq[k]);
+            if (ep[k] > nr.thrB_p || eq[k] > nr.thrB_q) { m |= 1u << k; ep[k] = eq[k] = 0.f; }
+        }
+        for (;;) {
+            const unsigned bal = __ballot_sync(0xffffffffu, m != 0);
+            if (!bal) break;
+            if (m) {
+                const int k = __ffs(m) - 1;           // (inside the row: the others' e are 0)
+                heavy[n + __popc(bal & ((1u << lane) - 1u))] = make_float2(raw_logit<DT>(rp, k), raw_logit<DT>(rq, k));
+                m &= m - 1u;
+            }
+            n += __popc(bal);
+            __syncwarp();
+            if (n >= 32) {
+                n -= 32;
+                take(n + lane, true);
+                __syncwarp();
+            }
+        }
+        float a[NO];
+#pragma unroll
+        for (int i2 = 0; i2 < NO; ++i2) a[i2] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (NORM) {
+                a[0] += ep[k];
+                a[1] += eq[k];
+                if (ep[k] > 0.f) { a[2] = fmaf(ep[k], xp[k], a[2]); a[3] = fmaf(ep[k], xq[k], a[3]); }
+                if (eq[k] > 0.f) { a[NO - 2] = fmaf(eq[k], xq[k], a[NO - 2]); a[NO - 1] = fmaf(eq[k], xp[k], a[NO - 1]); }
+            } else {
+                const float p = ep[k] * ipf, q = eq[k] * iqf, d = p - q;
+                a[0] += fabsf(d);
+                a[1] += fminf(p, q);
+                a[2] = fmaf(p, fminf(q, 1.f), a[2]);
+                a[3] += fmaxf(d, 0.f);
+            }
+        }
+#pragma unroll
+        for (int i2 = 0; i2 < NO; ++i2) sum.o[i2] += (double)a[i2];
+    }
+    stream::cp_async_wait<0>();
+    if (n > 0) take(lane, lane < n);
+    __syncwarp();
+    return sum;
+}
+
+// A cluster of P.C CTAs per node, as spec_single_kernel; nodes of other kinds leave at once.  As items of the recursion kernel, rows
+// resident, 112 such nodes at V = 128256 were 7 rounds of 26 us on its clusters; here a call takes 153 us in place of 260 (with
+// two CTAs per SM, and no spills, 162).
+template <int DT>
+__global__ void __launch_bounds__(256, 3) spec_single_analysis_kernel(const NParams NP)
+{
+    constexpr int NW = 8;
+    const VParams &P = NP.v;
+    __shared__ Common M;
+    __shared__ float2 s_heavy[NW][64];
+    __shared__ FirstChild s_f;
+    uint4 *ring = reinterpret_cast<uint4 *>(dyn_smem);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, C = P.C;
+    const unsigned rank = C > 1 ? cluster_ctarank() : 0u;
+    const int id = (int)(blockIdx.x / (unsigned)C), b = id / P.N, a = id % P.N;
+    const long long node = id;
+    grid_launch_dependents();
+    if (warp == 0) {
+        const FirstChild f = first_child<DT>(P, b, a);
+        if (lane == 0) s_f = f;
+    }
+    if (tid == 0) { common_init(M, NW); mbar_fence_init(); }
+    __syncthreads();
+    const FirstChild f = s_f;
+    const RowStat p = load_stat(NP.part + node * 2), q = load_stat(NP.part + node * 2 + 1);
+    // (what is wrong with a node is wrong for all CTAs of its cluster; its outputs stay NaN)
+    if (f.kc == 1 && !f.err && p.ok() && q.ok()) {
+        if (C > 1) cluster_sync_all();
+        Team T = {M, C, warp, lane, 0, rank, 0u};
+        NodeRows nr;
+        set_sum_rows(nr, p, q, 1.4426950408889634 / (double)(P.T_seq ? __ldg(P.T_seq + b) : P.T));
+        const Slice sl = make_slice<DT>(P.zp, P.zq, (long long)b * P.seq_stride + (long long)a * P.node_stride, P.V, C, rank);
+        double v[6], t[6], mine[6];
+        AnTerms o = an_sums<DT, true>(sl, nr, 0.0, 0.0, ring, s_heavy[warp]);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) v[i] = o.o[i];
+        cluster_sum<NW, 6>(T, v, t, mine);
+        const double Z_p = t[0], Z_q = t[1];
+        if (Z_p > 0.0 && Z_q > 0.0) {
+            const double ip = 1.0 / Z_p, iq = 1.0 / Z_q;
+            o = an_sums<DT, false>(sl, nr, ip, iq, ring, s_heavy[warp]);
+            double v4[4], t4[4], m4[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v4[i] = o.o[i];
+            cluster_sum<NW, 4>(T, v4, t4, m4);
+            if (rank == 0 && tid == 0 && !*(volatile int *)&M.poison) {
+                const double l1 = t4[0], smin = t4[1], nss = t4[2], spos = t4[3];
+                // KL(p||q) = ln 2 (sum e_p x_p - sum e_p x_q) / Z_p - ln Z_p + ln Z_q, and the mirror image
+                const double lz = log(Z_p) - log(Z_q);
+                float *ao = NP.an_acc + node * 4, *dv = NP.an_div + node * 3;
+                ao[0] = (float)nss; ao[1] = (float)smin; ao[2] = (float)smin;
+                dv[0] = (float)l1;
+                dv[1] = (float)(0.6931471805599453 * (t[2] - t[3]) * ip - lz);
+                dv[2] = (float)(0.6931471805599453 * (t[4] - t[5]) * iq + lz);
+                const double px = token_e(f.zp, p, nr.s_d) * ip, qx = token_e(f.zq, q, nr.s_d) * iq;
+                const double S = spos > RESIDUAL_FLOOR ? spos : 0.0;
+                AnRec &A = NP.an[node];
+                A.A[0][0] = fmin(1.0, token_ratio(px, qx));
+                A.A[1][0] = S > 0.0 ? fmax(px - qx, 0.0) / S : qx;            // p_1(x); S = 0: the state equals q
+                A.S[0] = S;
+                A.px[0] = px; A.qx[0] = qx;
+                A.rho = 1.0; A.beta = smin; A.pacc = smin; A.s_res = spos;
+                A.k = 1; A.valid = 1;
+            }
+        }
+        if (C > 1) cluster_sync_all();         // nobody leaves while a peer may still write to its shared memory
+    }
+    if (blockIdx.x == 0) grid_dependency_wait();      // this kernel ends only after the one before it
+}
+
 // ------------------------------------------------------------------------------------------------
-// nodes with several children (analysis: with any)
+// nodes with several children
 // ------------------------------------------------------------------------------------------------
 // what the consumers need to know about a node besides its rows
 struct __align__(16) NodeScalars {
@@ -755,11 +951,14 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) spec_recursion_kernel(const 
         const bool shared_tree = P.topo_stride == 0;
         const int G = shared_tree ? 1 : window_seqs(P), per = shared_tree ? P.B : 1;
         int b0 = 0, sidx = 0;
-        int count = list_nodes(S, P, 0, G, AN ? 1 : 2);
+        int count = list_nodes(S, P, 0, G, 2);
         long long base = 0;
         uint32_t mph[2] = {0u, 0u}, eph = 0;      // phases of the mailboxes
         int prev = -1;                       // scalars block of the item the consumers are at
         bool going = true;
+        // Analysis: where there is a cluster for every item, none draws a second one while it is at its first (50 us).
+        const int clusters = (int)(gridDim.x / (unsigned)C);
+        const bool ahead = !AN || (shared_tree ? (long long)count * per > clusters : G < P.B || count > clusters);
         // A node's record is written once its ratio is known: until then it may hold partial sums of the ratio kernel's.
         auto after_ratio = [&](int b, int a) {
             int w = 1;
@@ -809,7 +1008,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) spec_recursion_kernel(const 
             while (t >= base + (long long)count * per && !shared_tree && b0 + G < P.B) {
                 base += count;
                 b0 += G;
-                count = list_nodes(S, P, b0, min(G, P.B - b0), AN ? 1 : 2);
+                count = list_nodes(S, P, b0, min(G, P.B - b0), 2);
             }
             const int Gn = shared_tree ? 1 : min(G, P.B - b0);
             const long long k = t - base;
@@ -822,6 +1021,10 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) spec_recursion_kernel(const 
         for (int kidx = 0; going; ++kidx) {
             const int buf = kidx & 1;
             int a = 0, b = 0;
+            if (!ahead && rank == 0 && sidx > 0) {
+                if (lane == 0 && !mbar_wait(&S.sempty[(sidx - 1) & 1], (uint32_t)(((sidx - 1) >> 1) & 1))) S.M.poison = 1;
+                __syncwarp();
+            }
             // ---- the item: drawn by the first CTA's helper, passed on to the others --------------------------------
             if (rank == 0) {
                 int w = 1;
@@ -1015,25 +1218,22 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) spec_recursion_kernel(const 
                     t0 = tot[0]; t1 = tot[1];
                 };
                 // one sweep and one sum for everything that does not depend on rho
-                double v9[9], t9[9], m9[9];
+                double v6[6], t6[6], m6[6];
                 {
-                    double v5[5];
-                    reduce_sweep<NW, RC>(es, sl.nu, tid, R, L, nl, FnFirst{(float)ip, (float)iq, ip, iq, kc}, v5);
+                    double v4[4];
+                    reduce_sweep<NW, RC>(es, sl.nu, tid, R, L, nl, FnFirst{(float)ip, (float)iq, ip, iq, kc}, v4);
 #pragma unroll
-                    for (int i = 0; i < 5; ++i) v9[i] = v5[i];
-                    v9[5] = (double)kls.pp; v9[6] = (double)kls.pq; v9[7] = (double)kls.qq; v9[8] = (double)kls.qp;
-                    cluster_sum<NW, 9>(T, v9, t9, m9);
+                    for (int i = 0; i < 4; ++i) v6[i] = v4[i];
+                    v6[4] = (double)kls.pp - (double)kls.pq; v6[5] = (double)kls.qq - (double)kls.qp;
+                    cluster_sum<NW, 6>(T, v6, t6, m6);
                 }
-                const double l1 = t9[0], smin = t9[1], nss = t9[2], naive2 = t9[3], spos = t9[4];
+                const double l1 = t6[0], smin = t6[1], nss = t6[2], naive2 = t6[3];
                 // KL(p||q) = ln 2 (sum e_p x_p - sum e_p x_q) / Z_p - ln Z_p + ln Z_q, and the mirror image
                 const double lz = log(Z_p) - log(Z_q);
-                const double klpq = 0.6931471805599453 * (t9[5] - t9[6]) * ip - lz;
-                const double klqp = 0.6931471805599453 * (t9[7] - t9[8]) * iq + lz;
+                const double klpq = 0.6931471805599453 * t6[4] * ip - lz;
+                const double klqp = 0.6931471805599453 * t6[5] * iq + lz;
                 double sacc = 0.0;
-                if (kc == 1) {
-                    // one child: rho = 1, beta = sum min(p, q), and the residual (p - q)+ is where q is not above p
-                    an_beta = smin; an_pacc = smin; an_sres = spos;
-                } else {
+                {
                     double dummy;
                     const auto beta = [&](double r) {
                         const double ipr = ip / r;

@@ -521,7 +521,7 @@ int launch_nodes(const SpecIn *in, NParams &np, bool analysis, cudaStream_t st)
         return bf ? launch_branch<SPEC_BF16, 0, AN>(br, np, st) : launch_branch<SPEC_F32, 0, AN>(br, np, st);
     };
     rc = analysis ? branch(std::true_type{}) : branch(std::false_type{});
-    if (rc || analysis) return rc;
+    if (rc) return rc;
     {
         // nodes with one child: more CTAs per node while few waves hold them all (with one CTA a node its passes, not their sum, are the
         // latency: traversal, batch 8, V = 128256, 152 nodes: 131 us with 1, 109 with 2, 94 with 4)
@@ -532,6 +532,7 @@ int launch_nodes(const SpecIn *in, NParams &np, bool analysis, cudaStream_t st)
             const int e = prepare_kernel(kernel, C, smem, true);
             return e ? e : launch_clustered(kernel, (int)nodes * C, C, 256, smem, st, &np, true);
         };
+        if (analysis) return bf ? go(spec_single_analysis_kernel<SPEC_BF16>) : go(spec_single_analysis_kernel<SPEC_F32>);
         rc = bf ? go(spec_single_kernel<SPEC_BF16>) : go(spec_single_kernel<SPEC_F32>);
         if (rc) return rc;
     }

@@ -53,7 +53,7 @@ namespace specv {
 constexpr int CHMAX = 24;    // chunks per thread, in registers (RC of them) and shared memory
 constexpr int CMAX = 16;     // CTAs per cluster (above 8: non-portable size)
 constexpr int NWMAX = 8;     // consumer warps
-constexpr int NVMAX = 9;     // doubles per sum over the cluster
+constexpr int NVMAX = 6;     // doubles per sum over the cluster
 constexpr int FAST_N = 32;   // trees up to this size are finished warp-parallel
 constexpr int FIN_PENDING = -1;     // VParams::fin of a sequence whose nodes are not all done
 constexpr int FIN_FAULTY = -2;      // ... of a sequence with a device-detected fault: no bonus draw
@@ -612,7 +612,7 @@ __device__ __forceinline__ double spectr_sweep(float4 *es, int nu, int tid, Resi
     return d;
 }
 
-// A read-only sweep over the thread's share of the resident node: f.tail(e_p, e_q, a) on every fp32 token (f's running
+// A read-only sweep over the thread's share of the resident node: f.tail8(e_p, e_q, a) on every 8 fp32 tokens (f's running
 // sums), f.exact(...) in fp64 on the entry of the warp's exact list that falls to the lane.  Listed tokens are zero
 // in the fp32 arrays; every f maps (0, 0) to nothing.
 template <int NW, int RC, int NO, typename F>
@@ -629,14 +629,10 @@ __device__ __forceinline__ void reduce_sweep(const float4 *es, int nu, int tid, 
         const float4 *d = es + (size_t)((c - RC) * 4) * NCONS + tid;
         load_e8(d, NCONS, p);
         load_e8(d + 2 * NCONS, NCONS, q);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) f.tail(p[k], q[k], a);
+        f.tail8(p, q, a);
     }
 #pragma unroll
-    for (int j = 0; j < RC; ++j) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) f.tail(R.p[j][k], R.q[j][k], a);
-    }
+    for (int j = 0; j < RC; ++j) f.tail8(R.p[j], R.q[j], a);
 #pragma unroll
     for (int i = 0; i < NO; ++i) o[i] = (double)a[i];
     if ((tid & 31) < nl) f.exact(L.ep[tid & 31], L.eq[tid & 31], o);

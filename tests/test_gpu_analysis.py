@@ -23,6 +23,12 @@ SHAPES = [
     Workload("an_v262144", 1, 262144, "bf16", 4, 1, 2, 0.75),
     Workload("an_v450001", 1, 450001, "bf16", 3, 1, 2, 0.75),          # part of a node in registers
     Workload("an_v620003_f32", 1, 620003, "f32", 2, 1, 2, 0.75),
+    # nodes with one child: a chunk, a round of the ring and a CTA's share at their edges; a path only; one sequence on 8 CTAs a node
+    Workload("an_path_v7", 3, 7, "f32", 1, 0, 3, 1.0),
+    Workload("an_path_v2047", 2, 2047, "bf16", 1, 0, 3, 1.0),
+    Workload("an_path_v2049_f32", 2, 2049, "f32", 1, 0, 3, 0.5, temperature=0.5),
+    Workload("an_path_v65537", 1, 65537, "bf16", 1, 0, 4, 1.0),
+    Workload("an_path_v65536_p", 1, 65536, "bf16", 1, 0, 4, 1.0, top_p=0.9),
 ]
 
 
