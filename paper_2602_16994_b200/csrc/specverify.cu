@@ -440,14 +440,20 @@ int row_statistics(const SpecIn *in, const SpecOut *out, unsigned char *w, const
 // solver: -1 SpecInfer, otherwise the OTLP solver of spec_verify_otlp
 int verify_walk(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, bool trunc, cudaStream_t st, int solver = -1)
 {
-    // The walk keeps one cluster per sequence busy.  While all of them fit on the chip with one CTA per SM, a CTA may use
-    // all of an SM's registers; larger batches share the SMs.
+    // The walk keeps one cluster per sequence busy.  While all of them fit on the chip with one CTA per SM, a CTA has an SM to itself.
+    // Larger batches run in rounds that way, and two CTAs on an SM (half of the registers, the first chunks in them) pay only
+    // where a thread has few chunks of 16-bit logits and the clusters are no larger for it.  Calls with three nodes per path, us,
+    // two CTAs against one: V = 50257 (7 chunks) B = 40 33.5 / 36.6, V = 100352 (7) B = 80 88 / 99, 128 127 / 148; but V = 128256 (8) B = 32
+    // 57.7 / 53.0, 64 102 / 91, 128 180 / 167, V = 151936 (10) B = 32 73 / 62, V = 262144 B = 64 195 / 175, V = 65536 (cluster of 8 against
+    // 4) B = 80 73 / 64, and fp32 V = 50257 B = 90 124 / 102.  With 8 chunks also for large truncated batches (few tokens left to evaluate:
+    // top-k, V = 128256, B = 40 93 / 86, 90 156 / 162; 50 nodes, B = 128 711 / 729).
     VPlan pl, one;
     bool big;
     const bool fits = one_cta_plan(in->V, 8, (int)sizeof(WHdr), &one, &big);
-    const bool whole = fits && ((long long)in->B * one.C <= sm_count() || !two_cta_plan(in->V, (int)sizeof(WHdr), &pl));
-    if (whole) pl = one;
-    else if (!fits) return SPEC_ERR_UNSUPPORTED;
+    if (!fits) return SPEC_ERR_UNSUPPORTED;
+    const bool two = (long long)in->B * one.C > sm_count() && in->logits_dtype == SPEC_BF16 && two_cta_plan(in->V, (int)sizeof(WHdr), &pl) &&
+                     pl.C == one.C && pl.slice_len <= (trunc && (long long)in->B * one.C >= 4ll * sm_count() ? 8 : 7) * 256 * 8;
+    if (!two) pl = one;
     int rc = row_statistics(in, out, w, L, trunc, st);
     if (rc) return rc;
     WParams wp = {};
@@ -460,9 +466,9 @@ int verify_walk(const SpecIn *in, const SpecOut *out, unsigned char *w, const Ws
     const bool bf = in->logits_dtype == SPEC_BF16;
     auto go = [&](auto ot) {
         constexpr bool OT = decltype(ot)::value;
-        if (whole && big) return bf ? launch_walk<SPEC_BF16, 8, 8, 1, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 8, 1, OT>(pl, wp, st);
-        if (whole) return bf ? launch_walk<SPEC_BF16, 8, 0, 1, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 0, 1, OT>(pl, wp, st);
-        return bf ? launch_walk<SPEC_BF16, 8, 4, 2, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 4, 2, OT>(pl, wp, st);
+        if (two) return launch_walk<SPEC_BF16, 8, 4, 2, OT>(pl, wp, st);
+        if (big) return bf ? launch_walk<SPEC_BF16, 8, 8, 1, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 8, 1, OT>(pl, wp, st);
+        return bf ? launch_walk<SPEC_BF16, 8, 0, 1, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 0, 1, OT>(pl, wp, st);
     };
     return solver >= 0 ? go(std::true_type{}) : go(std::false_type{});
 }

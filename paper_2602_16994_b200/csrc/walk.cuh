@@ -68,8 +68,8 @@ struct RowSum {
     float cut;
 };
 
-// NW consumer warps (8 in all variants).  RC chunks of a thread in registers and MINB CTAs per SM: 0 and 1 while every CTA
-// has an SM to itself, 4 and 2 where two share one, 8 and 1 for vocabularies beyond the shared memory of 16 CTAs.
+// NW consumer warps (8 in all variants).  RC chunks of a thread in registers and MINB CTAs per SM: 0 and 1 where a CTA
+// has an SM to itself, 4 and 2 (bf16 only) where two share one, 8 and 1 for vocabularies beyond the shared memory of 16 CTAs.
 // OT: the walk with one of the other OTLP solvers of Appendix B instead of SpecInfer (Section 3.2: move to the
 // child whose token the solver put out, stop when the output is no child's token).  Every draw is then
 // made known to the whole cluster (one more sum), because the walk may go on from it.
