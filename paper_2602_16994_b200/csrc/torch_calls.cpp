@@ -301,7 +301,7 @@ PyObject *py_probs(PyObject *, PyObject *const *a, Py_ssize_t n)
         if (PyObject_IsTrue(a[7])) stats = empty({B, N, 6}, at::kFloat, z.device());
         int64_t bytes = 0;
         check(lib.workspace_bytes(&in, &bytes), "spec_workspace_bytes");
-        const Scratch ws = scratch_of(a[8], bytes);        // holds the row cuts when truncating
+        const Scratch ws = scratch_of(a[8], bytes);        // holds the rows' records when truncating
         const int which = truncated(a[1]);
         float *pr = probs.defined() ? (float *)probs.data_ptr() : nullptr, *st = stats.defined() ? (float *)stats.data_ptr() : nullptr;
         void *stream = stream_of(a[9]);
