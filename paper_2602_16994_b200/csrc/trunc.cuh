@@ -376,7 +376,7 @@ struct Kept {
 };
 
 // Selection and kept sums of a row the one pass could not settle: radix levels over the row in L2.  total: mass
-// of the row in units of its largest e (top-p alone; it only narrows the first range).  Out of line: rare.
+// of the row in units of its largest e (top-p alone; it only narrows the first range; 0: not known).  Out of line: rare.
 template <int DT>
 __device__ __noinline__ Kept settle_from_row(Shared &S, uint32_t *bins, const stream::RowSpan row, int V, int top_k,
                                              float top_p, float m, float sf, float s_hi, float s_lo, double s_d, float of, double total)
@@ -703,7 +703,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
     };
     // ---- the row's maximum and mass; NaN / +inf ------------------------------------------------------------------
     float m;
-    double total = 0.0;                // sum over the row of 2^((z - m) s)
+    double total = 0.0;                // sum over the row of 2^((z - m) s); 0: not known
     {
         const bool nan = ps.tmax != ps.tmax;
         float wm = ps.tmax;
@@ -730,7 +730,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
                 RowPart r = {};
                 r.cut = -CUDART_INF_F; r.O = ROWPART_EMPTY; r.bad = 1;
                 *out = r;
-                    }
+            }
             __syncthreads();
             clear();
             if (tid == 0) { S.runmax = 0u; S.count = 0; S.odd = 0; }
@@ -740,9 +740,12 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
         if (TOTAL) {
             const int Om = __reduce_max_sync(0xffffffffu, Ok);
             total = warp_sum(lane < NW ? S.red[lane][0] * pow2d(max(Ok - Om, -1000)) : 0.0);
-            // from units of 2^Om to units of the row maximum: 2^(Om - m s), Om - m s in [0, 1]
-            const double d = (double)Om - (double)m * s_d;
-            total *= 1.4142135623730951 * exp2_frac(fmin(fmax(d, 0.0), 1.0) - 0.5);
+            // From units of 2^Om to units of the row maximum: 2^(Om - m s).  Om - m s lies in [0, 1] but for exponents beyond 2^24, where
+            // a reference is rounded to a float.  Beyond 1e9 references end and the sums overflow or vanish: such a mass is not known (0),
+            // and the row is settled without it.
+            const double d = (double)Om - (double)m * s_d, n = rint(d);
+            total *= exp2_frac(d - n) * pow2d((int)n);
+            if (!(total > 0.0 && total < CUDART_INF)) total = 0.0;
         }
     }
     const double Od = fmin(fmax(ceil((double)m * s_d), -1.0e9), 1.0e9);
@@ -808,12 +811,14 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             return S.verdict != 0;
         };
         settled = select(last_bin_above(ps.bound));
-        if (TOTAL && !settled) {
+        if (TOTAL && !settled && total > 0.0) {
             // The nucleus reaches below the bound.  All tokens more than log2(V / ((1 - top_p) total)) octaves
             // below the maximum together have no more than 1 - top_p of the mass: counted again, from L2, down
             // to there.
             const float wide = log2f((float)P.V / ((1.f - P.top_p) * (float)total)) + 0.01f;
-            const float bound2 = fmaxf(m - wide / sf, LOWEST);
+            // (never above the maximum, whatever `wide` is: count_unit raises lower logits to the keys just below the bound, which
+            // have bins because the maximum has one)
+            const float bound2 = fminf(m, fmaxf(m - wide / sf, LOWEST));
             const Counter C{bound_key(bound2)};
             const bool plain = C.plain() && m < HIGH;
             __syncthreads();

@@ -87,3 +87,23 @@ def test_a_value_beyond_the_bins_late_in_the_row():
     z = rows(40000, BF)
     z[0, 0, 30000], z[1, 2, 39999], z[1, 0, 100] = 600.0, 511.0, -700.0
     check(z, dict(top_p=0.95), T=200.0)
+
+
+# temperatures so low that z log2(e) / T leaves the range of the rows' references (1e9): the mass the pass has summed is not known then
+@pytest.mark.parametrize("V", [50, 8193, 40000])
+@pytest.mark.parametrize("dtype", [BF, F32], ids=["bf16", "f32"])
+@pytest.mark.parametrize("shift", [0.0, -40.0])
+@pytest.mark.parametrize("trunc", [dict(top_k=5), dict(top_p=0.95), dict(top_k=5, top_p=0.95)], ids=["k5", "p95", "k5p95"])
+def test_cuts_beyond_the_range_of_references(V, dtype, shift, trunc):
+    z = rows(V, dtype)
+    z = (z.float() + shift).to(dtype)
+    for T in (1e-7, 1e-9, 1e-12):
+        _, stats = binding.tree_probs(z, 0, temperature=T, want_probs=False, **trunc)
+        st, zd = stats.cpu().numpy(), z.float().cpu().numpy()
+        # a step between neighbouring logits is 13 octaves at least: the nucleus is the maximum and its ties
+        if "top_p" in trunc:
+            cut = zd.max(-1)
+        else:
+            cut = -np.sort(-zd, axis=-1)[..., trunc["top_k"] - 1]
+        np.testing.assert_array_equal(st[..., 5], cut)
+        np.testing.assert_array_equal(st[..., 2], (zd >= cut[..., None]).sum(-1))
