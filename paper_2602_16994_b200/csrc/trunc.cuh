@@ -46,7 +46,7 @@ constexpr float WINDOW_OCTAVES = 14.f;
 constexpr float SAMPLE_OCTAVES = 24.f;   // bf16 top-p: how far below its maximum the first slice is counted
 constexpr float SAMPLE_REST = 0.7f;      // safety factor of the bounds from a part of the row (mass_bound)
 constexpr float UNSET = -2.0e9f;
-constexpr float LOWEST = -3.3e38f;   // a bound that every finite logit passes and -inf does not
+constexpr float LOWEST = -3.3e38f;   // a bound that every finite logit passes but the lowest values of both types (masks: a row that keeps some of them is settled from L2)
 template <int DT> constexpr int K_FAST = DT == SPEC_BF16 ? UN * NT : NT;      // largest top-k the first slice can bound
 
 // bf16 value bins, largest value first: TB positive magnitudes, then TB negative ones; magnitudes below 2^-11

@@ -111,6 +111,25 @@ def test_strided_logits():
     np.testing.assert_array_equal(got.out_tokens.cpu().numpy(), ref.out_tokens)
 
 
+@pytest.mark.parametrize("algo", ALGOS)
+@pytest.mark.parametrize("mask", [-1e9, -1e10, -1e30, "lowest"])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("T", [0.3, 1.0])
+def test_finite_masks_below_top_k(algo, mask, dtype, T):
+    """20 ordinary tokens, the others masked with a finite value, top-k 50: the mask is the k-th largest logit."""
+    for V, shift in ((1000, 0.0), (6001, -30.0)):
+        w = Workload("masked", 3, V, dtype, 3, 1, 2, 1.0, temperature=T, top_k=50)
+        batch = make_batch(w, seed=1, device="cuda")
+        g = torch.Generator(device="cuda").manual_seed(2)
+        left = torch.randperm(V, generator=g, device="cuda")[:20]
+        for z in (batch.target_logits, batch.draft_logits):
+            ordinary = z[..., left].float() + shift
+            z.fill_(torch.finfo(z.dtype).min if mask == "lowest" else mask)
+            z[..., left] = ordinary.to(z.dtype)
+        batch.token[:, 1:] = left[torch.randint(20, batch.token[:, 1:].shape, generator=g, device="cuda")].int()
+        check_batch(batch, algo)
+
+
 def test_device_detected_errors_are_reported_not_trapped():
     w = small("bad", 500, "f32", 2, 0, 2, 4)
     batch = make_batch(w, seed=5, device="cuda")

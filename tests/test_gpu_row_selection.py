@@ -107,3 +107,27 @@ def test_cuts_beyond_the_range_of_references(V, dtype, shift, trunc):
             cut = -np.sort(-zd, axis=-1)[..., trunc["top_k"] - 1]
         np.testing.assert_array_equal(st[..., 5], cut)
         np.testing.assert_array_equal(st[..., 2], (zd >= cut[..., None]).sum(-1))
+
+
+# Masked vocabularies: fewer ordinary tokens than top_k, so that the k-th largest logit is the mask and all masked tokens are kept (with
+# probability 0).  V below and above the fp32 list's 4096.
+MASKS = [-1e9, -1e10, -1e30, "lowest"]
+
+
+def masked(z, left, value):
+    g = torch.Generator(device="cuda").manual_seed(z.shape[-1])
+    keep = torch.randperm(z.shape[-1], generator=g, device="cuda")[:left]
+    out = torch.full_like(z, torch.finfo(z.dtype).min if value == "lowest" else value)
+    out[..., keep] = z[..., keep]
+    return out, keep
+
+
+@pytest.mark.parametrize("mask", MASKS)
+@pytest.mark.parametrize("dtype", [BF, F32], ids=["bf16", "f32"])
+@pytest.mark.parametrize("V", [1000, 20003])
+@pytest.mark.parametrize("shift", [0.0, -30.0], ids=["max_above_0", "max_below_0"])
+def test_finite_masks(V, dtype, mask, shift):
+    z, _ = masked((rows(V, dtype).float() + shift).to(dtype), 20, mask)
+    for T in (0.3, 0.6, 1.0):
+        for trunc in (dict(top_k=50), dict(top_k=50, top_p=0.95), dict(top_p=0.95)):
+            check(z, trunc, T)
