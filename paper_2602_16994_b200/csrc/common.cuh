@@ -158,9 +158,9 @@ __device__ __forceinline__ double exp2_frac(double f)
     return fma(t8, fma(t4, p6, q2), fma(t4, q1, q0));
 }
 // 2^(z s - O) in fp64 (about 1e-15 relative); 0 for -inf and for exponents below the double range
-__device__ __forceinline__ double exp2_exact(float z, double s_d, int O)
+__device__ __forceinline__ double exp2_exact(double z, double s_d, double O)
 {
-    const double xd = (double)z * s_d - (double)O;
+    const double xd = z * s_d - O;
     if (!(xd > -1000.0)) return 0.0;
     const double nd = rint(xd);
     return exp2_frac(xd - nd) * pow2d((int)nd);

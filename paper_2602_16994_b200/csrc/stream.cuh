@@ -22,6 +22,8 @@ struct __align__(16) RowPart {
     int bad;           // 1: NaN or +inf seen; -1: row not read (draft row of a node without children)
 };
 constexpr int ROWPART_EMPTY = -(1 << 30);
+// exponents z s beyond which the fp32 product no longer has an integer part exact to 1/16: kept sums and distributions go by fp64 there
+constexpr double FAR_EXPONENT = 1048576.0;
 
 namespace stream {
 

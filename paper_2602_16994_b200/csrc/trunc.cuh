@@ -66,7 +66,7 @@ struct RParams {
     float T;
     const float *T_seq;
     RowPart *part;             // [B*N*2] the rows' statistics
-    int *kept;                 // [B*N*2] kept tokens of every row (spec_tree_probs; NULL: not wanted)
+    int *kept;                 // spec_tree_probs: number of kept tokens of every row and its largest logit as bits [B*N][2]; else NULL
     stream::NodeInit init;     // per-call words of the workspace to set (every-node verification)
 };
 
@@ -362,10 +362,14 @@ __device__ __forceinline__ void visit_row(const stream::RowSpan &row, F f)
     }
 }
 
+// The unit of a row's kept sums: exponents are (z - base) s - O.
+struct Unit {
+    double base, O;
+};
 // adds c tokens of logit z to a row's kept sums, in fp64: the sums are shared by all that is made of the row
-__device__ __forceinline__ void add_kept(float z, double c, double s_d, double O, double &Z, double &X)
+__device__ __forceinline__ void add_kept(float z, double c, double s_d, const Unit &u, double &Z, double &X)
 {
-    const double x = fmax((double)z * s_d - O, -200.0), n = rint(x), e = c * exp2_frac_once(x - n) * pow2d((int)n);
+    const double x = fmax(((double)z - u.base) * s_d - u.O, -200.0), n = rint(x), e = c * exp2_frac_once(x - n) * pow2d((int)n);
     Z += e;
     X += e * x;
 }
@@ -379,7 +383,7 @@ struct Kept {
 // of the row in units of its largest e (top-p alone; it only narrows the first range; 0: not known).  Out of line: rare.
 template <int DT>
 __device__ __noinline__ Kept settle_from_row(Shared &S, uint32_t *bins, const stream::RowSpan row, int V, int top_k,
-                                             float top_p, float m, float sf, float s_hi, float s_lo, double s_d, float of, double total)
+                                             float top_p, float m, float sf, float s_hi, float s_lo, double s_d, const Unit unit, double total)
 {
     uint32_t *lo = bins, *hi = bins + NB;
     const bool use_k = top_k > 0 && top_k < V, use_p = top_p < 1.f;
@@ -406,12 +410,14 @@ __device__ __noinline__ Kept settle_from_row(Shared &S, uint32_t *bins, const st
     const float cutv = r.key == 0u ? -CUDART_INF_F : cut::value_of(r.key);
     double Z = 0.0, X = 0.0;
     int n = 0;
+    const bool far = unit.base != 0.0 || fabs(unit.O) > FAR_EXPONENT;
+    const float of = (float)unit.O;
     visit_row<DT>(row, [&](float z) {
         if (z >= cutv) {
             const float x = fmaxf(fmaf(z, s_lo, fmaf(z, s_hi, -of)), -200.f);
             ++n;
-            if (x > -4.f) {                            // (there may be as many tokens as the row has: only the largest in fp64)
-                add_kept(z, 1.0, s_d, (double)of, Z, X);
+            if (far || x > -4.f) {                     // (there may be as many tokens as the row has: only the largest in fp64)
+                add_kept(z, 1.0, s_d, unit, Z, X);
             } else {
                 const float e = exp2_fine(z, s_hi, s_lo, (int)of);
                 Z += (double)e;
@@ -748,15 +754,20 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             if (!(total > 0.0 && total < CUDART_INF)) total = 0.0;
         }
     }
-    const double Od = fmin(fmax(ceil((double)m * s_d), -1.0e9), 1.0e9);
-    const float of = (float)Od;
+    // The row's reference.  For a verification an integer within 1e9 that is a float as well, because its kernels take it for one; the
+    // exponents of a row beyond that fit no fp32 e, and its sum is recorded as infinite, for which its sequence is reported.  A distribution
+    // with far exponents is referenced to the largest logit itself, before anything is rounded.
+    const double ms = (double)m * s_d, Oi = (double)(float)fmin(fmax(ceil(ms), -1.0e9), 1.0e9);
+    const bool own = P.kept && fabs(ms) > FAR_EXPONENT;
+    const Unit unit = {own ? (double)m : 0.0, own ? 0.0 : Oi};
+    const double top = own ? 0.0 : ms - Oi;             // the largest exponent
     auto write = [&](double Z, double X, float cutv, int kept) {
         RowPart r;
-        r.S = Z; r.X = X; r.O = (int)Od; r.cut = cutv;
-        r.xmax = (float)((double)m * s_d - (double)of);
+        r.S = fabs(top) < 126.0 ? Z : CUDART_INF; r.X = X; r.O = (int)Oi; r.cut = cutv;
+        r.xmax = (float)top;
         r.bad = 0;
         *out = r;
-        if (P.kept) P.kept[id] = kept;
+        if (P.kept) { P.kept[id] = kept; P.kept[id + 1] = __float_as_int(m); }
     };
     bool settled = false;
     if (DT == SPEC_BF16) {
@@ -777,7 +788,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             int n = 0;
             for (int i = b_max + lane; i <= b_cut; i += 32) {
                 const uint32_t c = bins[i];
-                if (c) add_kept(value_of_bin(i), (double)c, s_d, Od, Z, X);
+                if (c) add_kept(value_of_bin(i), (double)c, s_d, unit, Z, X);
                 n += (int)c;
             }
             Z = warp_sum(Z);
@@ -857,7 +868,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
         if (settled) {
             cutv = cut::value_of(key);
             for (int i = tid; i < n; i += NT)
-                if (keys[i] >= key) { add_kept(cut::value_of(keys[i]), 1.0, s_d, Od, Z, X); ++kept; }
+                if (keys[i] >= key) { add_kept(cut::value_of(keys[i]), 1.0, s_d, unit, Z, X); ++kept; }
         }
         if (P.kept) kept = (int)block_sum(S, (unsigned long long)kept);
         if (settled) {
@@ -875,7 +886,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
     }
     if (!settled) {
         __syncthreads();
-        const Kept kp = settle_from_row<DT>(S, bins, span_of<DT>(P, id), P.V, P.top_k, P.top_p, m, sf, s_hi, s_lo, s_d, of, total);
+        const Kept kp = settle_from_row<DT>(S, bins, span_of<DT>(P, id), P.V, P.top_k, P.top_p, m, sf, s_hi, s_lo, s_d, unit, total);
         if (tid == 0) write(kp.Z, kp.X, kp.key ? cut::value_of(kp.key) : -CUDART_INF_F, kp.n);
     }
     if (DT == SPEC_BF16) __syncthreads();                // the bins have been read

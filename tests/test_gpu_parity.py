@@ -130,6 +130,22 @@ def test_finite_masks_below_top_k(algo, mask, dtype, T):
         check_batch(batch, algo)
 
 
+@pytest.mark.parametrize("algo", ALGOS)
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("top_k,top_p", [(30, 1.0), (0, 0.95), (30, 0.95)])
+def test_far_exponents(algo, dtype, top_k, top_p):
+    """z log2(e) / T above 2^24, where the integers next to it are no floats any more; beyond 1e9 a sequence is reported."""
+    w = Workload("far", 4, 6001, dtype, 3, 1, 2, 1e-6, temperature=3e-7, top_k=top_k, top_p=top_p)
+    batch = make_batch(w, seed=1, device="cuda")
+    check_batch(batch, algo, full=False)
+    for z in (batch.target_logits, batch.draft_logits):
+        z.neg_()
+        z.add_(-30.0)
+    check_batch(batch, algo, full=False)
+    batch.workload = w = synth.shrink(w, temperature=1e-12)
+    assert (gpu_verify(batch, algo).status.cpu().numpy() == 3).all()
+
+
 def test_device_detected_errors_are_reported_not_trapped():
     w = small("bad", 500, "f32", 2, 0, 2, 4)
     batch = make_batch(w, seed=5, device="cuda")

@@ -131,3 +131,17 @@ def test_finite_masks(V, dtype, mask, shift):
     for T in (0.3, 0.6, 1.0):
         for trunc in (dict(top_k=50), dict(top_k=50, top_p=0.95), dict(top_p=0.95)):
             check(z, trunc, T)
+
+
+@pytest.mark.parametrize("V", [50, 20003])
+@pytest.mark.parametrize("dtype", [BF, F32], ids=["bf16", "f32"])
+@pytest.mark.parametrize("trunc", [dict(top_k=50), dict(top_k=25), dict(top_p=0.95), dict(top_k=25, top_p=0.95)], ids=["k50", "k25", "p95", "k25p95"])
+def test_distributions_with_far_exponents(V, dtype, trunc):
+    """z log2(e) / T beyond 2^20 (where fp32 loses the fraction), 2^24 (integers) and 1e9 (references): low temperatures, rows far from
+    zero, rows of a mask only."""
+    z = rows(V, dtype)
+    for shift, temperatures in ((0.0, (1e-5, 1e-6, 1e-7, 1e-9)), (-40.0, (1e-6, 1e-9)), (3e6, (1.0, 0.1)), (-3e7, (1.0, 0.1))):
+        for T in temperatures:
+            check((z.float() + shift).to(dtype), trunc, T)
+    for value in (-1e9, -1e30, torch.finfo(dtype).min, 1e30):
+        check(torch.full_like(z, value), trunc, 0.6)
