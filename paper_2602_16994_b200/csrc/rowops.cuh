@@ -453,7 +453,8 @@ struct BParams {
     int *token;
     float *margin;
 };
-// first lane with running sum > tau (and weight); else the last with weight and rest = inf; -1 where there is none
+// first lane with running sum > tau (and weight); else the last with weight and rest = inf; -1 where there is none.  (The sum ahead of the
+// lane is a difference: it may exceed tau by a rounding, and what is left of tau is then 0.)
 __device__ __forceinline__ int first_above(double v, double tau, double &rest)
 {
     const int lane = threadIdx.x & 31;
@@ -466,7 +467,7 @@ __device__ __forceinline__ int first_above(double v, double tau, double &rest)
     const unsigned hit = __ballot_sync(0xffffffffu, v > 0.0 && incl > tau), pos = __ballot_sync(0xffffffffu, v > 0.0);
     const int at = hit ? __ffs(hit) - 1 : 31 - __clz(pos);
     const double before = __shfl_sync(0xffffffffu, incl - v, at < 0 ? 0 : at);
-    rest = hit ? tau - before : CUDART_INF;
+    rest = hit ? fmax(tau - before, 0.0) : CUDART_INF;
     return pos ? at : -1;
 }
 // the lane's four consecutive weights of a tile; beyond the slice: 0
@@ -560,7 +561,7 @@ __global__ void __launch_bounds__(BN_NT) spec_bonus_kernel(const BParams P)
         const double before = run;
         run += (double)v[k];
         if (v[k] > 0.f) last = k;
-        if (found < 0 && run > tau3) { found = k; lo = tau3 - before; hi = run - tau3; }
+        if (found < 0 && v[k] > 0.f && run > tau3) { found = k; lo = tau3 - before; hi = run - tau3; }
     }
     P.token[r_id] = at + (found >= 0 ? found : last);
     if (P.margin) P.margin[r_id] = found >= 0 ? (float)(fmin(lo, hi) / all) : 0.f;

@@ -196,6 +196,17 @@ def test_tree_probs(V, dtype):
         np.testing.assert_allclose(st[..., 4], rs[..., 4], atol=PROB_TOL)
 
 
+def test_draw_within_rounding_of_a_boundary():
+    """Sums that round: 1 | 3/8 ulp | 0, 3/8 ulp | ... | 1.  The target 1 is reached in the third group, by a sum that was rounded up:
+    what lies ahead of the group then exceeds the target, and its first weight, 0, must not be named."""
+    w = torch.zeros((1, 128), device="cuda")
+    w[0, 0] = w[0, 124] = 1.0
+    w[0, 4] = w[0, 9] = 1.5 * 2.0 ** -54
+    token, margin = binding.sample_bonus(w, torch.tensor([0.5], device="cuda"), want_margin=True)
+    assert w[0, int(token[0])] > 0 and int(token[0]) in (4, 9)
+    assert float(margin[0]) >= 0.0
+
+
 @pytest.mark.parametrize("V,R", [(7, 64), (1000, 64), (50001, 64), (128256, 64), (300000, 64),
                                  (127, 6), (8192, 6), (16385, 700), (4096, 300)])        # slices and tiles: their edges, one CTA a row
 def test_sample_bonus(V, R):
