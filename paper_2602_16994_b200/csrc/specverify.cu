@@ -437,23 +437,34 @@ int row_statistics(const SpecIn *in, const SpecOut *out, unsigned char *w, const
                 : go(stream::spec_row_partial_kernel<SPEC_F32, false>, stream::Ring<SPEC_F32>::BYTES);
 }
 
+// The launch shape of the walk.
+// The walk keeps one cluster per sequence busy.  While all of them fit on the chip with one CTA per SM, a CTA has an SM to itself.
+// Larger batches run in rounds that way, and two CTAs on an SM (half of the registers, the first chunks in them) pay only
+// where a thread has few chunks of 16-bit logits and the clusters are no larger for it.  Calls with three nodes per path, us,
+// two CTAs against one: V = 50257 (7 chunks) B = 40 33.5 / 36.6, V = 100352 (7) B = 80 88 / 99, 128 127 / 148; but V = 128256 (8) B = 32
+// 57.7 / 53.0, 64 102 / 91, 128 180 / 167, V = 151936 (10) B = 32 73 / 62, V = 262144 B = 64 195 / 175, V = 65536 (cluster of 8 against
+// 4) B = 80 73 / 64, and fp32 V = 50257 B = 90 124 / 102.  With 8 chunks also for large truncated batches (few tokens left to evaluate:
+// top-k, V = 128256, B = 40 93 / 86, 90 156 / 162; 50 nodes, B = 128 711 / 729).
+struct WalkPlan {
+    VPlan pl;
+    bool two, big;       // two CTAs on an SM; chunks in registers as well
+};
+bool walk_plan(int V, int dtype, long long B, bool trunc, int sms, WalkPlan *w)
+{
+    VPlan one;
+    if (!one_cta_plan(V, 8, (int)sizeof(WHdr), &one, &w->big)) return false;
+    w->two = B * one.C > sms && dtype == SPEC_BF16 && two_cta_plan(V, (int)sizeof(WHdr), &w->pl) && w->pl.C == one.C &&
+             w->pl.slice_len <= (trunc && B * one.C >= 4ll * sms ? 8 : 7) * 256 * 8;
+    if (!w->two) w->pl = one;
+    return true;
+}
+
 // solver: -1 SpecInfer, otherwise the OTLP solver of spec_verify_otlp
 int verify_walk(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, bool trunc, cudaStream_t st, int solver = -1)
 {
-    // The walk keeps one cluster per sequence busy.  While all of them fit on the chip with one CTA per SM, a CTA has an SM to itself.
-    // Larger batches run in rounds that way, and two CTAs on an SM (half of the registers, the first chunks in them) pay only
-    // where a thread has few chunks of 16-bit logits and the clusters are no larger for it.  Calls with three nodes per path, us,
-    // two CTAs against one: V = 50257 (7 chunks) B = 40 33.5 / 36.6, V = 100352 (7) B = 80 88 / 99, 128 127 / 148; but V = 128256 (8) B = 32
-    // 57.7 / 53.0, 64 102 / 91, 128 180 / 167, V = 151936 (10) B = 32 73 / 62, V = 262144 B = 64 195 / 175, V = 65536 (cluster of 8 against
-    // 4) B = 80 73 / 64, and fp32 V = 50257 B = 90 124 / 102.  With 8 chunks also for large truncated batches (few tokens left to evaluate:
-    // top-k, V = 128256, B = 40 93 / 86, 90 156 / 162; 50 nodes, B = 128 711 / 729).
-    VPlan pl, one;
-    bool big;
-    const bool fits = one_cta_plan(in->V, 8, (int)sizeof(WHdr), &one, &big);
-    if (!fits) return SPEC_ERR_UNSUPPORTED;
-    const bool two = (long long)in->B * one.C > sm_count() && in->logits_dtype == SPEC_BF16 && two_cta_plan(in->V, (int)sizeof(WHdr), &pl) &&
-                     pl.C == one.C && pl.slice_len <= (trunc && (long long)in->B * one.C >= 4ll * sm_count() ? 8 : 7) * 256 * 8;
-    if (!two) pl = one;
+    WalkPlan plan;
+    if (!walk_plan(in->V, in->logits_dtype, in->B, trunc, sm_count(), &plan)) return SPEC_ERR_UNSUPPORTED;
+    const VPlan &pl = plan.pl;
     int rc = row_statistics(in, out, w, L, trunc, st);
     if (rc) return rc;
     WParams wp = {};
@@ -466,8 +477,8 @@ int verify_walk(const SpecIn *in, const SpecOut *out, unsigned char *w, const Ws
     const bool bf = in->logits_dtype == SPEC_BF16;
     auto go = [&](auto ot) {
         constexpr bool OT = decltype(ot)::value;
-        if (two) return launch_walk<SPEC_BF16, 8, 4, 2, OT>(pl, wp, st);
-        if (big) return bf ? launch_walk<SPEC_BF16, 8, 8, 1, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 8, 1, OT>(pl, wp, st);
+        if (plan.two) return launch_walk<SPEC_BF16, 8, 4, 2, OT>(pl, wp, st);
+        if (plan.big) return bf ? launch_walk<SPEC_BF16, 8, 8, 1, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 8, 1, OT>(pl, wp, st);
         return bf ? launch_walk<SPEC_BF16, 8, 0, 1, OT>(pl, wp, st) : launch_walk<SPEC_F32, 8, 0, 1, OT>(pl, wp, st);
     };
     return solver >= 0 ? go(std::true_type{}) : go(std::false_type{});
@@ -712,9 +723,9 @@ int32_t spec_query_plan(int32_t V, int32_t logits_dtype, int32_t *cluster_size, 
 {
     if (V <= 0) return SPEC_ERR_SHAPE;
     if (logits_dtype != SPEC_F32 && logits_dtype != SPEC_BF16) return SPEC_ERR_DTYPE;
-    VPlan pl;          // the walk of a batch that fills the chip
-    bool big;
-    if (!two_cta_plan(V, (int)sizeof(WHdr), &pl) && !one_cta_plan(V, 8, (int)sizeof(WHdr), &pl, &big)) return SPEC_ERR_UNSUPPORTED;
+    WalkPlan plan;
+    if (!walk_plan(V, logits_dtype, 1 << 20, true, 148, &plan)) return SPEC_ERR_UNSUPPORTED;
+    const VPlan &pl = plan.pl;
     if (cluster_size) *cluster_size = pl.C;
     if (slice_len) *slice_len = pl.slice_len;
     if (smem_bytes) *smem_bytes = pl.smem;

@@ -110,6 +110,15 @@ def test_query_plan():
     assert big["slice_len"] * big["cluster_size"] >= 262144 and big["smem_bytes"] <= 227 * 1024
 
 
+@pytest.mark.parametrize("V,dtype", [(128256, 0), (50257, 0), (151936, 1)])
+def test_query_plan_of_walks_with_an_sm_to_themselves(V, dtype):
+    """fp32 logits and more than 8 chunks per thread: never two CTAs per SM, whatever the batch."""
+    p = binding.query_plan(V, dtype)
+    chunks = -(-p["slice_len"] // 2048)
+    assert p["smem_bytes"] >= chunks * 16384                 # every chunk of the slice in shared memory, none in registers
+    assert p["slice_len"] * p["cluster_size"] >= V
+
+
 def test_binding_refuses_to_run_without_a_gpu():
     import torch
     if torch.cuda.is_available():
