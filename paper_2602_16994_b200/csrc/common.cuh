@@ -166,13 +166,12 @@ __device__ __forceinline__ double exp2_exact(double z, double s_d, double O)
     return exp2_frac(xd - nd) * pow2d((int)nd);
 }
 // 2^(z s - O) in fp32 to about half a unit in the last place, s = s_hi + s_lo (Taylor series of 2^f, |f| <= 0.5, to degree 7): unlike those of
-// ex2.approx, whose mean is -3e-8 to -5e-8, its errors average out.  0 below 2^-126 and for -inf: decided on the exponent itself, because
-// for a logit that stands for a mask (-1e10, the lowest value of its type) z s may overflow and its integer part fits no int.
+// ex2.approx, whose mean is -3e-8 to -5e-8, its errors average out.  0 below 2^-126 and for -inf: decided on the exponent itself, as a
+// float, because for a logit that stands for a mask (-1e10, the lowest value of its type) z s may overflow, its integer part fits no int and
+// f is no fraction.
 __device__ __forceinline__ float exp2_fine(float z, float s_hi, float s_lo, int O)
 {
-    const float t = z * s_hi;
-    if (!(t - (float)O > -126.f)) return 0.f;
-    const float n = rintf(t), f = fmaf(z, s_lo, fmaf(z, s_hi, -n));
+    const float n = rintf(z * s_hi), f = fmaf(z, s_lo, fmaf(z, s_hi, -n)), k = n - (float)O;
     float p = 1.5252734e-5f;
     p = fmaf(p, f, 1.5403530e-4f);
     p = fmaf(p, f, 1.3333558e-3f);
@@ -181,7 +180,7 @@ __device__ __forceinline__ float exp2_fine(float z, float s_hi, float s_lo, int 
     p = fmaf(p, f, 2.4022651e-1f);
     p = fmaf(p, f, 6.9314718e-1f);
     p = fmaf(p, f, 1.0f);
-    return p * pow2i((int)n - O);
+    return k > -127.f ? p * __int_as_float(((int)k + 127) << 23) : 0.f;          // (k is at most 1)
 }
 // fp32 pairs in one 64-bit register: packed fused multiply-add and add (sm_100)
 __device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi)

@@ -363,8 +363,16 @@ struct KParams {
     const int *kept;         // [rows][2]: kept tokens, largest logit as bits
     float *probs, *stats;
 };
-// of a token that is no less than 2^-4 of the unit of the row's sum, and of every token of a row with far exponents
-__device__ __noinline__ float heavy_prob(double z, double s_d, double O, double S) { return (float)(exp2_exact(z, s_d, O) / S); }
+// of a token that is no less than 2^-4 of the unit of the row's sum
+__device__ __noinline__ float heavy_prob(float z, double s_d, int O, double S) { return (float)(exp2_exact((double)z, s_d, (double)O) / S); }
+// tokens t0 .. t1 - 1 of a row with far exponents, whose unit is its largest logit m
+__device__ __noinline__ void write_far(const void *z, int dtype, float *out, int t0, int t1, float cut, float m, double s_d, double S)
+{
+    for (int t = t0 + (int)threadIdx.x; t < t1; t += KEPT_NT) {
+        const float v = load_logit(z, dtype, t);
+        out[t] = v >= cut ? (float)(exp2_exact((double)v - (double)m, s_d, 0.0) / S) : 0.f;
+    }
+}
 
 template <int DT>
 __global__ void __launch_bounds__(KEPT_NT, 4) spec_probs_kept_kernel(const KParams P)
@@ -377,17 +385,15 @@ __global__ void __launch_bounds__(KEPT_NT, 4) spec_probs_kept_kernel(const KPara
         const RowPart *rp = P.part + 2ll * row;
         const double T = (double)(P.T_seq ? __ldg(P.T_seq + b) : P.T), S = rp->S, s_d = 1.4426950408889634 / T;
         const int O = rp->O, bad = rp->bad;
-        const float cut = rp->cut, m = __int_as_float(P.kept[2ll * row + 1]);
-        const bool far = fabs((double)m * s_d) > FAR_EXPONENT;
-        const double base = far ? (double)m : 0.0, ref = far ? 0.0 : (double)O;      // exponents are (z - base) s - ref
+        const float cut = rp->cut;
         if (P.stats && part == 0 && tid == 0) {
             float *st = P.stats + 6ll * row;
-            if (bad) {
+            if (bad == 1) {
                 for (int i = 0; i < 6; ++i) st[i] = CUDART_NAN_F;
             } else {
                 // in units of the largest e, 2^xmax
                 const double x = (double)rp->xmax, Z = S * exp2(-x);
-                st[0] = (float)((double)m / T); st[1] = (float)Z; st[2] = (float)P.kept[2ll * row];
+                st[0] = (float)((double)__int_as_float(P.kept[2ll * row + 1]) / T); st[1] = (float)Z; st[2] = (float)P.kept[2ll * row];
                 st[3] = (float)(log(S) - 0.6931471805599453 * rp->X / S); st[4] = (float)(1.0 / Z); st[5] = cut;
             }
         }
@@ -398,10 +404,14 @@ __global__ void __launch_bounds__(KEPT_NT, 4) spec_probs_kept_kernel(const KPara
         const unsigned char *z = (const unsigned char *)P.z + ((long long)b * P.seq_stride + (long long)(row % P.N) * P.node_stride) * ESZ;
         float *out = P.probs + (long long)row * P.V;
         const int t0 = part * KEPT_PART, t1 = min(P.V, t0 + KEPT_PART);
-        const float near = far ? -CUDART_INF_F : (float)(((double)O - 4.0) / s_d);
+        if (bad == ROW_FAR) {
+            write_far(z, DT, out, t0, t1, cut, __int_as_float(P.kept[2ll * row + 1]), s_d, S);
+            continue;
+        }
+        const float near = (float)(((double)O - 4.0) / s_d);
         const auto prob = [&](float v) {
             if (!(v >= cut) || bad) return 0.f;
-            if (v >= near) return heavy_prob((double)v - base, s_d, ref, S);
+            if (v >= near) return heavy_prob(v, s_d, O, S);
             const float e = exp2_fine(v, s_hi, s_lo, O);
             return fmaf(e, inv_lo, e * inv_hi);
         };

@@ -24,6 +24,7 @@ struct __align__(16) RowPart {
 constexpr int ROWPART_EMPTY = -(1 << 30);
 // exponents z s beyond which the fp32 product no longer has an integer part exact to 1/16: kept sums and distributions go by fp64 there
 constexpr double FAR_EXPONENT = 1048576.0;
+constexpr int ROW_FAR = 2;         // RowPart::bad of such a row for which a distribution is wanted: S and X are in units of its largest e
 
 namespace stream {
 

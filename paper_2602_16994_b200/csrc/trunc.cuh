@@ -172,8 +172,8 @@ __device__ __forceinline__ void count_unit(const Counter &C, uint32_t bins, uint
         for (int k = 0; k < 4; ++k) {
             uint32_t v;
             asm("max.s16x2 %0, %1, %2;" : "=r"(v) : "r"(w[k]), "r"(floor));
-            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(__dp2a_lo((int)v, 0x00FC, base)));        // base - 4 low half
-            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(__dp2a_lo((int)v, 0xFC00, base)));        // base - 4 high half
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(__dp2a_lo((int)v, 0x00FC, base)) : "memory");     // base - 4 low half
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(__dp2a_lo((int)v, 0xFC00, base)) : "memory");     // base - 4 high half
         }
     } else {
         int seen = 0;
@@ -185,7 +185,7 @@ __device__ __forceinline__ void count_unit(const Counter &C, uint32_t bins, uint
             const int mag = key < 0 ? -1 - key : key;
             const int b = key >= 0 ? max(min(TB - 1 + M0 - key, TB - 1), 0) : min(max(TB - M0 + mag, TB), 2 * TB - 1);
             if (key >= C.kb) seen |= (mag - 1 < M0 && mag > 0 ? ODD_LOW : 0) | (mag >= M0 + TB - 1 ? ODD_HIGH : 0);
-            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(key >= C.kb ? bins + 4u * (uint32_t)b : dump));
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(key >= C.kb ? bins + 4u * (uint32_t)b : dump) : "memory");
         }
         if (seen) atomicOr(odd, seen);
     }
@@ -362,14 +362,10 @@ __device__ __forceinline__ void visit_row(const stream::RowSpan &row, F f)
     }
 }
 
-// The unit of a row's kept sums: exponents are (z - base) s - O.
-struct Unit {
-    double base, O;
-};
 // adds c tokens of logit z to a row's kept sums, in fp64: the sums are shared by all that is made of the row
-__device__ __forceinline__ void add_kept(float z, double c, double s_d, const Unit &u, double &Z, double &X)
+__device__ __forceinline__ void add_kept(double z, double c, double s_d, double O, double &Z, double &X)
 {
-    const double x = fmax(((double)z - u.base) * s_d - u.O, -200.0), n = rint(x), e = c * exp2_frac_once(x - n) * pow2d((int)n);
+    const double x = fmax(z * s_d - O, -200.0), n = rint(x), e = c * exp2_frac_once(x - n) * pow2d((int)n);
     Z += e;
     X += e * x;
 }
@@ -380,10 +376,11 @@ struct Kept {
 };
 
 // Selection and kept sums of a row the one pass could not settle: radix levels over the row in L2.  total: mass
-// of the row in units of its largest e (top-p alone; it only narrows the first range; 0: not known).  Out of line: rare.
+// of the row in units of its largest e (top-p alone; it only narrows the first range; 0: not known).  The sums are of 2^((z - base) s - O).
+// Out of line: rare.
 template <int DT>
 __device__ __noinline__ Kept settle_from_row(Shared &S, uint32_t *bins, const stream::RowSpan row, int V, int top_k,
-                                             float top_p, float m, float sf, float s_hi, float s_lo, double s_d, const Unit unit, double total)
+                                             float top_p, float m, float sf, float s_hi, float s_lo, double s_d, double base, double O, double total)
 {
     uint32_t *lo = bins, *hi = bins + NB;
     const bool use_k = top_k > 0 && top_k < V, use_p = top_p < 1.f;
@@ -410,14 +407,14 @@ __device__ __noinline__ Kept settle_from_row(Shared &S, uint32_t *bins, const st
     const float cutv = r.key == 0u ? -CUDART_INF_F : cut::value_of(r.key);
     double Z = 0.0, X = 0.0;
     int n = 0;
-    const bool far = unit.base != 0.0 || fabs(unit.O) > FAR_EXPONENT;
-    const float of = (float)unit.O;
+    const bool far = base != 0.0 || fabs(O) > FAR_EXPONENT;
+    const float of = (float)O;
     visit_row<DT>(row, [&](float z) {
         if (z >= cutv) {
             const float x = fmaxf(fmaf(z, s_lo, fmaf(z, s_hi, -of)), -200.f);
             ++n;
             if (far || x > -4.f) {                     // (there may be as many tokens as the row has: only the largest in fp64)
-                add_kept(z, 1.0, s_d, unit, Z, X);
+                add_kept((double)z - base, 1.0, s_d, O, Z, X);
             } else {
                 const float e = exp2_fine(z, s_hi, s_lo, (int)of);
                 Z += (double)e;
@@ -756,16 +753,14 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
     }
     // The row's reference.  For a verification an integer within 1e9 that is a float as well, because its kernels take it for one; the
     // exponents of a row beyond that fit no fp32 e, and its sum is recorded as infinite, for which its sequence is reported.  A distribution
-    // with far exponents is referenced to the largest logit itself, before anything is rounded.
-    const double ms = (double)m * s_d, Oi = (double)(float)fmin(fmax(ceil(ms), -1.0e9), 1.0e9);
+    // with far exponents is referenced to the largest logit itself, before anything is rounded (and settled from the row).
+    const double ms = (double)m * s_d, Od = (double)(float)fmin(fmax(ceil(ms), -1.0e9), 1.0e9);
     const bool own = P.kept && fabs(ms) > FAR_EXPONENT;
-    const Unit unit = {own ? (double)m : 0.0, own ? 0.0 : Oi};
-    const double top = own ? 0.0 : ms - Oi;             // the largest exponent
     auto write = [&](double Z, double X, float cutv, int kept) {
         RowPart r;
-        r.S = fabs(top) < 126.0 ? Z : CUDART_INF; r.X = X; r.O = (int)Oi; r.cut = cutv;
-        r.xmax = (float)top;
-        r.bad = 0;
+        r.S = own || fabs(ms - Od) < 126.0 ? Z : CUDART_INF; r.X = X; r.O = (int)Od; r.cut = cutv;
+        r.xmax = own ? 0.f : (float)(ms - Od);
+        r.bad = own ? ROW_FAR : 0;
         *out = r;
         if (P.kept) { P.kept[id] = kept; P.kept[id + 1] = __float_as_int(m); }
     };
@@ -788,7 +783,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             int n = 0;
             for (int i = b_max + lane; i <= b_cut; i += 32) {
                 const uint32_t c = bins[i];
-                if (c) add_kept(value_of_bin(i), (double)c, s_d, unit, Z, X);
+                if (c) add_kept(value_of_bin(i), (double)c, s_d, Od, Z, X);
                 n += (int)c;
             }
             Z = warp_sum(Z);
@@ -821,8 +816,8 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             __syncthreads();
             return S.verdict != 0;
         };
-        settled = select(last_bin_above(ps.bound));
-        if (TOTAL && !settled && total > 0.0) {
+        settled = !own && select(last_bin_above(ps.bound));
+        if (TOTAL && !own && !settled && total > 0.0) {
             // The nucleus reaches below the bound.  All tokens more than log2(V / ((1 - top_p) total)) octaves
             // below the maximum together have no more than 1 - top_p of the mass: counted again, from L2, down
             // to there.
@@ -847,7 +842,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
         float cutv = -CUDART_INF_F;
         double Z = 0.0, X = 0.0;
         int kept = 0;
-        settled = n <= CAP && (TOTAL || P.top_k <= K_FAST<DT>);
+        settled = !own && n <= CAP && (TOTAL || P.top_k <= K_FAST<DT>);
         // (at least k logits lie at or above the bound, so the k-th largest is in the list)
         if (settled && use_k) settled = radix_select<false>(S, bins, bins + NB, (double)P.top_k, 0u, cut::key_of(m), m, sf, key, visit);
         if (settled && use_p) {
@@ -868,7 +863,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
         if (settled) {
             cutv = cut::value_of(key);
             for (int i = tid; i < n; i += NT)
-                if (keys[i] >= key) { add_kept(cut::value_of(keys[i]), 1.0, s_d, unit, Z, X); ++kept; }
+                if (keys[i] >= key) { add_kept(cut::value_of(keys[i]), 1.0, s_d, Od, Z, X); ++kept; }
         }
         if (P.kept) kept = (int)block_sum(S, (unsigned long long)kept);
         if (settled) {
@@ -886,7 +881,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
     }
     if (!settled) {
         __syncthreads();
-        const Kept kp = settle_from_row<DT>(S, bins, span_of<DT>(P, id), P.V, P.top_k, P.top_p, m, sf, s_hi, s_lo, s_d, unit, total);
+        const Kept kp = settle_from_row<DT>(S, bins, span_of<DT>(P, id), P.V, P.top_k, P.top_p, m, sf, s_hi, s_lo, s_d, own ? (double)m : 0.0, own ? 0.0 : Od, total);
         if (tid == 0) write(kp.Z, kp.X, kp.key ? cut::value_of(kp.key) : -CUDART_INF_F, kp.n);
     }
     if (DT == SPEC_BF16) __syncthreads();                // the bins have been read
