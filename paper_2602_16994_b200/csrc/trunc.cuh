@@ -55,6 +55,8 @@ constexpr int TB = 20 * 128;
 constexpr int M0 = (127 - 11) << 7;
 constexpr float HIGH = 508.f;                 // below the outermost bin's value
 constexpr int PLAIN_KEY = M0 + 33;            // the smallest value that has 32 values with bins of their own below it, as bits
+constexpr int PLAIN_NEG = M0 + TB - 2 - 32;   // ... and, of negative ones, the largest magnitude
+constexpr float NEGATIVE = -4.8828125e-4f;    // -2^-11: the negative values below have bins of their own
 constexpr int ODD_LOW = 1, ODD_HIGH = 2;      // a candidate in such a shared bin (other than 0) was seen
 
 struct RParams {
@@ -147,8 +149,13 @@ __device__ __forceinline__ int bound_key(float bound)
 // What the counting of bf16 logits needs to know about a bound.
 struct Counter {
     int kb;                    // the bound as a key
-    // the bound and the 32 keys below it are positive values with bins of their own
-    __device__ __forceinline__ bool plain() const { return kb >= PLAIN_KEY; }
+    // Logits below this one are counted the plain way (count_unit): the bound and the 32 keys below it are values of one sign with
+    // bins of their own, and so are the candidates: positive ones below HIGH, or, where the bound is negative, negative ones.
+    __device__ __forceinline__ bool positive() const { return kb >= PLAIN_KEY; }
+    __device__ __forceinline__ float plain_below() const
+    {
+        return positive() ? HIGH : kb < -1 - M0 && kb >= -1 - PLAIN_NEG ? NEGATIVE : -CUDART_INF_F;
+    }
     // whether a unit with these maxima holds a candidate
     __device__ __forceinline__ bool reaches(uint32_t max_pair) const
     {
@@ -159,13 +166,25 @@ struct Counter {
 // Counts the 8 logits of a bf16 unit that are at or above the bound.  Every lane adds to some word for each of its logits: an
 // addition under a predicate is a branch to the compiler, and a slice of 8192 logits then takes 1310 cycles with no candidate
 // and 2150 with 9 to 49 % of them (one CTA of 8 warps on an SM); without, 675 and 760 to 900.
-// plain, and no logit of the unit reaches HIGH: positive values order like their bits, so a logit below the bound is raised to one of
-// the 32 keys below it, whose bins nobody reads any more (bounds only rise), and a pair of logits takes one maximum,
-// two multiply-adds and the two additions.
+// plain (no logit of the unit reaches plain_below): values of one sign order like their bits, or the other way round, so a logit below the
+// bound is raised to one of the 32 keys below it, whose bins nobody reads any more (bounds only rise), and a pair of
+// logits takes one maximum (negative: minimum), two multiply-adds and the two additions.  Logits that are all negative (log-probabilities),
+// counted one by one: 272 rows of 128256 shifted by -20, T 1, top-p 0.99: 124 us, 76 rows (T 0.8, top-p 0.9): 72; now 78 and 39.
 __device__ __forceinline__ void count_unit(const Counter &C, uint32_t bins, uint32_t dump, int *odd, const uint4 &r, bool plain)
 {
     const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-    if (plain) {
+    if (plain && C.kb < 0) {
+        // bits 0x8000 + magnitude, as a 16-bit integer magnitude - 0x8000
+        const int base = (int)bins + (TB - M0 + 0x8000) * 4;
+        const uint32_t ceiling = (uint32_t)(0x8000 - C.kb + (int)(threadIdx.x & 31)) * 0x10001u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            uint32_t v;
+            asm("min.s16x2 %0, %1, %2;" : "=r"(v) : "r"(w[k]), "r"(ceiling));
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(__dp2a_lo((int)v, 0x0004, base)) : "memory");     // base + 4 low half
+            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(__dp2a_lo((int)v, 0x0400, base)) : "memory");     // base + 4 high half
+        }
+    } else if (plain) {
         const int base = (int)bins + (TB - 1 + M0) * 4;
         const uint32_t floor = (uint32_t)(C.kb - 1 - (int)(threadIdx.x & 31)) * 0x10001u;
 #pragma unroll
@@ -623,7 +642,8 @@ __device__ __noinline__ float sample_bound(float ms)
     __syncthreads();
     return sample_floor();
 }
-// The first bound, from the first slice alone.  Of a row of several slices only positive logits have been counted: a cut below zero
+// The first bound, from the first slice alone.  Of a row of several slices with a positive logit in the first only positive ones have been
+// counted: a cut below zero
 // keeps more than half of a row of logits around zero.  Where they hold too little of the mass, the slice is counted again, from the
 // ring (stage: the warp's share), all of it that matters.
 __device__ __noinline__ float first_mass_bound(float tmax, float bound, float of, double Sd, float top_p, int n, int V, const uint4 *stage)
@@ -640,12 +660,14 @@ __device__ __noinline__ float first_mass_bound(float tmax, float bound, float of
     return mass_bound(tmax, loose, of, Sd, top_p, n, V);
 }
 
-// units of which some logits may be negative, or reach HIGH
-__device__ __noinline__ void count_pair(const Counter cnt, const uint4 r0, const uint4 r1)
+// Units of which some logits may be negative, or have no bins of their own; ms: the lane's maximum.  (Out of line: with the
+// negative bounds' way of counting in the loop over the slices as well, rows of both signs took 3 % longer.)
+__device__ __noinline__ void count_pair(const Counter cnt, const uint4 r0, const uint4 r1, float ms)
 {
     const Smem<SPEC_BF16> M;
-    M.count(cnt, r0, false);
-    M.count(cnt, r1, false);
+    const bool plain = !__any_sync(0xffffffffu, !(ms < cnt.plain_below()));
+    M.count(cnt, r0, plain);
+    M.count(cnt, r1, plain);
 }
 
 // what the pass over a row leaves in a thread (UNSET: no reference yet)
@@ -826,7 +848,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             // have bins because the maximum has one)
             const float bound2 = fminf(m, fmaxf(m - wide / sf, LOWEST));
             const Counter C{bound_key(bound2)};
-            const bool plain = C.plain() && m < HIGH;
+            const bool plain = m < C.plain_below();
             __syncthreads();
             clear();
             __syncthreads();
@@ -1007,7 +1029,7 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
 #pragma unroll
                     for (int c = 0; c < UN; ++c) m = stream::max_raw<DT>(m, stream::unit_max_raw<DT>(stage[c * NT + lane]));
                     ps.bound = sample_bound(stream::fold_max<DT>(m));
-                    if (nsl > 1) ps.bound = fmaxf(ps.bound, __uint_as_float((uint32_t)PLAIN_KEY << 16));
+                    if (nsl > 1 && cut::value_of(S.runmax) > 0.f) ps.bound = fmaxf(ps.bound, __uint_as_float((uint32_t)PLAIN_KEY << 16));
                     cnt.kb = bound_key(ps.bound);
                 }
                 // two units at a time: what a step needs fits the registers
@@ -1021,8 +1043,8 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
                     add_mass<DT, 2>(raw, ms, s_hi, s_lo, ps);
                     // A unit that holds a candidate anywhere in the warp is counted by all lanes.  Where all units of a slice did, those
                     // of the next three are not asked.
-                    if (!cnt.plain() || __any_sync(0xffffffffu, !(ms < HIGH))) {
-                        if (__any_sync(0xffffffffu, ms >= ps.bound)) count_pair(cnt, raw[0], raw[1]);
+                    if (!cnt.positive() || __any_sync(0xffffffffu, !(ms < HIGH))) {
+                        if (__any_sync(0xffffffffu, ms >= ps.bound)) count_pair(cnt, raw[0], raw[1], ms);
                     } else {
 #pragma unroll
                         for (int k = 0; k < 2; ++k) {

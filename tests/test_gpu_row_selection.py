@@ -145,3 +145,19 @@ def test_distributions_with_far_exponents(V, dtype, trunc):
             check((z.float() + shift).to(dtype), trunc, T)
     for value in (-1e9, -1e30, torch.finfo(dtype).min, 1e30):
         check(torch.full_like(z, value), trunc, 0.6)
+
+
+@pytest.mark.parametrize("V", [8192, 8193, 40000, 150001])
+@pytest.mark.parametrize("top,spread,T", [(-2.0 ** -11, 0.002, 1e-3),        # the largest logits at the edge of the bins that share values
+                                          (-0.25, 4.0, 1.0), (-9.0, 3.0, 0.6),
+                                          (-478.0, 3.0, 1.0), (-490.0, 3.0, 1.0),      # bounds whose 32 values below end at the outermost bin
+                                          (-505.0, 6.0, 1.0)])
+@pytest.mark.parametrize("p", [0.9, 0.99])
+def test_rows_of_negative_logits(V, top, spread, T, p):
+    g = torch.Generator(device="cuda").manual_seed(V)
+    z = (top - torch.rand((1, 4, V), generator=g, device="cuda") ** 2 * spread).to(BF)
+    if V > 8192:
+        z[0, 1, 8192:] = (z[0, 1, 8192:].float() * 0.5).to(BF)          # larger ones after the first slice
+        z[0, 2, V - 1] = 0.0                                            # a logit of the other kind late in the row
+        z[0, 3, V - 2] = 0.5
+    check(z, dict(top_p=p), T)
