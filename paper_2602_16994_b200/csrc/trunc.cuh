@@ -364,20 +364,32 @@ __device__ __forceinline__ void visit_units(const stream::RowSpan &row, F f)
         }
     }
 }
-// f(z) for every logit of a row
+// f(z) for every logit of a row.  fp32, whose wide nuclei are settled this way: the load of the unit after next is under way while a unit is
+// gone through; one at a time, a pass waited for L2 at every unit (T 1, top-p 0.99, 76 rows of 50257: 225 us, now 207; 272
+// rows of 128256: 1099, now 1000).  (For bf16, where it is rare, the registers that this takes are missing in the loop over the slices: 541
+// instead of 511 us on 2368 rows.)
 template <int DT, typename F>
 __device__ __forceinline__ void visit_row(const stream::RowSpan &row, F f)
 {
     constexpr int E = DT == SPEC_BF16 ? 8 : 4;
+    constexpr bool AHEAD = DT == SPEC_F32;
     const uint4 *src = reinterpret_cast<const uint4 *>(row.base);
-    for (int u = threadIdx.x; u < row.units; u += NT) {
-        const uint4 raw = __ldg(src + u);
+    int u = threadIdx.x;
+    uint4 raw = {}, next = {};
+    if (AHEAD && u < row.units) raw = __ldg(src + u);
+    if (AHEAD && u + NT < row.units) next = __ldg(src + u + NT);
+#pragma unroll 1
+    for (; u < row.units; u += NT) {
+        uint4 far = {};
+        if (!AHEAD) raw = __ldg(src + u);
+        else if (u + 2 * NT < row.units) far = __ldg(src + u + 2 * NT);
         const int e0 = u == 0 ? row.head : 0, e1 = u == row.units - 1 ? row.last : E;
         float z[E];
         stream::unpack_unit<DT>(raw, z);
 #pragma unroll
         for (int k = 0; k < E; ++k)
             if (k >= e0 && k < e1) f(z[k]);
+        if (AHEAD) { raw = next; next = far; }
     }
 }
 
