@@ -542,12 +542,22 @@ int launch_nodes(const SpecIn *in, NParams &np, bool analysis, cudaStream_t st)
     {
         // nodes with one child: more CTAs per node while few waves hold them all (with one CTA a node its passes, not their sum, are the
         // latency: traversal, batch 8, V = 128256, 152 nodes: 131 us with 1, 109 with 2, 94 with 4)
-        int C = 1;
+        int C = 1, bytes = smem;
         while (C < 8 && nodes * C * 2 <= 8 * sm_count() && in->V >= C * 8192) C <<= 1;
+        if (analysis) {
+            // The analysis' passes are arithmetic, and left alone three CTAs share an SM while others idle: with few nodes a CTA asks for so
+            // much shared memory that they spread, and clusters of 16 are taken where each of their CTAs finds an SM and 24 KB of the row.  Paths of six nodes,
+            // us, packed and spread: fp32 V = 262144 B = 1 123 and 64 (78 in clusters of 8), B = 2 129 and 78, B = 4 (two a SM) 136 and 110,
+            // V = 128256 B = 2 89 and 62, bf16 V = 262144 B = 1 70 and 57, V = 128256 B = 4 68 and 61; from three a SM on, packed is as it was
+            // (spread all the same, B = 8: 76 and 85).  Clusters of 16 for smaller rows: bf16 V = 128256 B = 1 46 and 48.
+            if (C == 8 && nodes * 16 <= sm_count() && (long long)in->V * (bf ? 2 : 4) >= 16 * 24 * 1024) C = 16;
+            const long long per_sm = (nodes * C + sm_count() - 1) / sm_count();
+            if (per_sm <= 2) bytes = per_sm == 1 ? 100 * 1024 : 62 * 1024;
+        }
         np.v.C = C;
         const auto go = [&](auto kernel) {
-            const int e = prepare_kernel(kernel, C, smem, true);
-            return e ? e : launch_clustered(kernel, (int)nodes * C, C, 256, smem, st, &np, true);
+            const int e = prepare_kernel(kernel, C, bytes, true);
+            return e ? e : launch_clustered(kernel, (int)nodes * C, C, 256, bytes, st, &np, true);
         };
         if (analysis) return bf ? go(spec_single_analysis_kernel<SPEC_BF16>) : go(spec_single_analysis_kernel<SPEC_F32>);
         rc = bf ? go(spec_single_kernel<SPEC_BF16>) : go(spec_single_kernel<SPEC_F32>);

@@ -29,6 +29,10 @@ SHAPES = [
     Workload("an_path_v2049_f32", 2, 2049, "f32", 1, 0, 3, 0.5, temperature=0.5),
     Workload("an_path_v65537", 1, 65537, "bf16", 1, 0, 4, 1.0),
     Workload("an_path_v65536_p", 1, 65536, "bf16", 1, 0, 4, 1.0, top_p=0.9),
+    # ... on clusters of 16, one CTA an SM, and two an SM
+    Workload("an_path_v200003", 1, 200003, "bf16", 1, 0, 4, 1.0),
+    Workload("an_path_v98305_f32", 1, 98305, "f32", 1, 0, 6, 1.0),
+    Workload("an_path_two_per_sm", 4, 70001, "f32", 1, 0, 6, 1.0),
 ]
 
 
