@@ -400,6 +400,9 @@ __device__ __forceinline__ void add_kept(double z, double c, double s_d, double 
     Z += e;
     X += e * x;
 }
+// a row's reference: an integer within 1e9 that is a float as well, because the verification kernels take it for one
+__device__ __forceinline__ double reference(double largest) { return (double)(float)fmin(fmax(ceil(largest), -1.0e9), 1.0e9); }
+
 struct Kept {
     uint32_t key;      // key of the cut (0: nothing is cut)
     double Z, X;       // sum over the kept tokens of e and e x
@@ -407,11 +410,11 @@ struct Kept {
 };
 
 // Selection and kept sums of a row the one pass could not settle: radix levels over the row in L2.  total: mass
-// of the row in units of its largest e (top-p alone; it only narrows the first range; 0: not known).  The sums are of 2^((z - base) s - O).
-// Out of line: rare.
+// of the row in units of its largest e (top-p alone; it only narrows the first range; 0: not known).  own: the sums' unit is the largest
+// e as well.  Out of line: rare.
 template <int DT>
 __device__ __noinline__ Kept settle_from_row(Shared &S, uint32_t *bins, const stream::RowSpan row, int V, int top_k,
-                                             float top_p, float m, float sf, float s_hi, float s_lo, double s_d, double base, double O, double total)
+                                             float top_p, float m, float sf, float s_hi, float s_lo, double s_d, bool own, double total)
 {
     uint32_t *lo = bins, *hi = bins + NB;
     const bool use_k = top_k > 0 && top_k < V, use_p = top_p < 1.f;
@@ -438,7 +441,8 @@ __device__ __noinline__ Kept settle_from_row(Shared &S, uint32_t *bins, const st
     const float cutv = r.key == 0u ? -CUDART_INF_F : cut::value_of(r.key);
     double Z = 0.0, X = 0.0;
     int n = 0;
-    const bool far = base != 0.0 || fabs(O) > FAR_EXPONENT;
+    const double base = own ? (double)m : 0.0, O = own ? 0.0 : reference((double)m * s_d);
+    const bool far = own || fabs(O) > FAR_EXPONENT;
     const float of = (float)O;
     visit_row<DT>(row, [&](float z) {
         if (z >= cutv) {
@@ -785,10 +789,10 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
             if (!(total > 0.0 && total < CUDART_INF)) total = 0.0;
         }
     }
-    // The row's reference.  For a verification an integer within 1e9 that is a float as well, because its kernels take it for one; the
-    // exponents of a row beyond that fit no fp32 e, and its sum is recorded as infinite, for which its sequence is reported.  A distribution
-    // with far exponents is referenced to the largest logit itself, before anything is rounded (and settled from the row).
-    const double ms = (double)m * s_d, Od = (double)(float)fmin(fmax(ceil(ms), -1.0e9), 1.0e9);
+    // The exponents of a row beyond the range of references fit no fp32 e; its sum is recorded as infinite, for which a verification reports
+    // its sequence.  A distribution with far exponents is referenced to the largest logit itself, before anything is rounded (and settled
+    // from the row).
+    const double ms = (double)m * s_d, Od = reference(ms);
     const bool own = P.kept && fabs(ms) > FAR_EXPONENT;
     auto write = [&](double Z, double X, float cutv, int kept) {
         RowPart r;
@@ -915,7 +919,7 @@ __device__ __noinline__ void finish_row(const RParams &P, int id, const Pass ps)
     }
     if (!settled) {
         __syncthreads();
-        const Kept kp = settle_from_row<DT>(S, bins, span_of<DT>(P, id), P.V, P.top_k, P.top_p, m, sf, s_hi, s_lo, s_d, own ? (double)m : 0.0, own ? 0.0 : Od, total);
+        const Kept kp = settle_from_row<DT>(S, bins, span_of<DT>(P, id), P.V, P.top_k, P.top_p, m, sf, s_hi, s_lo, s_d, own, total);
         if (tid == 0) write(kp.Z, kp.X, kp.key ? cut::value_of(kp.key) : -CUDART_INF_F, kp.n);
     }
     if (DT == SPEC_BF16) __syncthreads();                // the bins have been read
