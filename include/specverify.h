@@ -258,9 +258,9 @@ int32_t spec_host_staging_bytes(const SpecIn *in, int64_t *bytes);
 int32_t spec_verify_host(const SpecIn *in, const SpecOut *out, int32_t algorithm, void *dev_buf,
                          int64_t dev_bytes, void *stream);
 
-/* Launch plan of SpecInfer's walk for a vocabulary size and dtype, of a batch under top-k / top-p that fills
- * the device several times over (host-only query, for benchmarks and tests; smaller batches and batches
- * without truncation run the walk with one CTA per SM more often): CTAs per cluster, tokens per CTA slice,
+/* Launch plan of SpecInfer's walk for a vocabulary size and dtype, of a batch under top-k that fills the
+ * device several times over (host-only query, for benchmarks and tests; smaller batches and batches
+ * without top-k run the walk with one CTA per SM more often): CTAs per cluster, tokens per CTA slice,
  * dynamic shared memory bytes per CTA, threads per CTA. */
 int32_t spec_query_plan(int32_t V, int32_t logits_dtype, int32_t *cluster_size, int32_t *slice_len,
                         int32_t *smem_bytes, int32_t *threads);

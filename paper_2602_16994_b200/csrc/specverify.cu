@@ -443,18 +443,22 @@ int row_statistics(const SpecIn *in, const SpecOut *out, unsigned char *w, const
 // where a thread has few chunks of 16-bit logits and the clusters are no larger for it.  Calls with three nodes per path, us,
 // two CTAs against one: V = 50257 (7 chunks) B = 40 33.5 / 36.6, V = 100352 (7) B = 80 88 / 99, 128 127 / 148; but V = 128256 (8) B = 32
 // 57.7 / 53.0, 64 102 / 91, 128 180 / 167, V = 151936 (10) B = 32 73 / 62, V = 262144 B = 64 195 / 175, V = 65536 (cluster of 8 against
-// 4) B = 80 73 / 64, and fp32 V = 50257 B = 90 124 / 102.  With 8 chunks also for large truncated batches (few tokens left to evaluate:
-// top-k, V = 128256, B = 40 93 / 86, 90 156 / 162; 50 nodes, B = 128 711 / 729).
+// 4) B = 80 73 / 64, and fp32 V = 50257 B = 90 124 / 102.  With 8 chunks (up to V = 131072 on clusters of 8) also for large batches under
+// top-k, which leaves few tokens to evaluate: V = 114688 / 120064 / 128256 / 131072, two against one, B = 56 115 114 / 134 128 / 134 128 / 124
+// 122, B = 64 130 131 / 138 141 / 141 146 / 128 142, B = 96 181 181 / 187 197 / 191 199 / 182 196, B = 128 233 237 / 236 249 / 243 256 / 240
+// 248.  Under top-p alone neither is better throughout (T 0.6, 0.95: B = 80 225 221 / 233 236 / 242 222 / 240 226, B = 96 246 251 / 268 267 / 269
+// 270 / 276 271, B = 128 348 329 / 334 352 / 371 364 / 376 362): two from four CTAs per SM on, up to slices of 16384.
 struct WalkPlan {
     VPlan pl;
     bool two, big;       // two CTAs on an SM; chunks in registers as well
 };
-bool walk_plan(int V, int dtype, long long B, bool trunc, int sms, WalkPlan *w)
+bool walk_plan(int V, int dtype, long long B, bool top_k, bool top_p, int sms, WalkPlan *w)
 {
     VPlan one;
     if (!one_cta_plan(V, 8, (int)sizeof(WHdr), &one, &w->big)) return false;
     w->two = B * one.C > sms && dtype == SPEC_BF16 && two_cta_plan(V, (int)sizeof(WHdr), &w->pl) && w->pl.C == one.C &&
-             w->pl.slice_len <= (trunc && B * one.C >= 4ll * sms ? 8 : 7) * 256 * 8;
+             (w->pl.slice_len <= 7 * 256 * 8 || (top_k && 5 * B * one.C >= 17ll * sms && V <= 8 * 256 * 8 * one.C) ||
+              (top_p && B * one.C >= 4ll * sms && w->pl.slice_len <= 8 * 256 * 8));
     if (!w->two) w->pl = one;
     return true;
 }
@@ -463,7 +467,7 @@ bool walk_plan(int V, int dtype, long long B, bool trunc, int sms, WalkPlan *w)
 int verify_walk(const SpecIn *in, const SpecOut *out, unsigned char *w, const WsLayout &L, bool trunc, cudaStream_t st, int solver = -1)
 {
     WalkPlan plan;
-    if (!walk_plan(in->V, in->logits_dtype, in->B, trunc, sm_count(), &plan)) return SPEC_ERR_UNSUPPORTED;
+    if (!walk_plan(in->V, in->logits_dtype, in->B, in->top_k > 0 && in->top_k < in->V, in->top_p < 1.f, sm_count(), &plan)) return SPEC_ERR_UNSUPPORTED;
     const VPlan &pl = plan.pl;
     int rc = row_statistics(in, out, w, L, trunc, st);
     if (rc) return rc;
@@ -734,7 +738,7 @@ int32_t spec_query_plan(int32_t V, int32_t logits_dtype, int32_t *cluster_size, 
     if (V <= 0) return SPEC_ERR_SHAPE;
     if (logits_dtype != SPEC_F32 && logits_dtype != SPEC_BF16) return SPEC_ERR_DTYPE;
     WalkPlan plan;
-    if (!walk_plan(V, logits_dtype, 1 << 20, true, 148, &plan)) return SPEC_ERR_UNSUPPORTED;
+    if (!walk_plan(V, logits_dtype, 1 << 20, true, false, 148, &plan)) return SPEC_ERR_UNSUPPORTED;
     const VPlan &pl = plan.pl;
     if (cluster_size) *cluster_size = pl.C;
     if (slice_len) *slice_len = pl.slice_len;
