@@ -125,20 +125,24 @@ struct RowPlan {
 };
 constexpr int ROW_SMEM_BUDGET = 227 * 1024 - (int)sizeof(rowops::Shared) - 1024;
 
-// a row in the shared memory of a cluster: two CTAs per SM where eight CTAs are enough for that
-bool make_row_plan(int V, int bytes_per_token, RowPlan *p)
+// `rows` rows of fp32 values, each in the shared memory of a cluster: two CTAs per SM where eight CTAs are enough for that, but one
+// where all CTAs of clusters of four, and not of clusters of eight, have an SM to themselves (19 rows of 128256: 17.6 and 18.5 us; one CTA
+// against two does not pay: 76 rows of 32000 17.6 and 15.3).
+bool make_row_plan(int V, long long rows, int sms, RowPlan *p)
 {
-    for (const int budget : {ROW_SMEM_BUDGET / 2 - 4096, ROW_SMEM_BUDGET})
-        for (int C = 1; C <= (budget == ROW_SMEM_BUDGET ? rowops::CMAX : 8); C <<= 1) {
-            long long sl = ((long long)V + C - 1) / C;
-            sl = (sl + 63) / 64 * 64;
-            long long need = sl * bytes_per_token;
-            if (need <= budget) {
-                p->C = C; p->SL = (int)sl; p->smem = (int)need;
-                return true;
-            }
+    const auto plan = [&](int budget, int most) {
+        for (int C = 1; C <= most; C <<= 1) {
+            const long long sl = (((long long)V + C - 1) / C + 63) / 64 * 64, need = sl * 4;
+            if (need > budget) continue;
+            *p = RowPlan{C, (int)sl, (int)need};
+            return true;
         }
-    return false;
+        return false;
+    };
+    if (!plan(ROW_SMEM_BUDGET / 2 - 4096, 8)) return plan(ROW_SMEM_BUDGET, rowops::CMAX);
+    const RowPlan two = *p;
+    if (two.C == 8 && rows * two.C > sms && plan(ROW_SMEM_BUDGET, rowops::CMAX) && rows * p->C > sms) *p = two;
+    return true;
 }
 
 int check_in(const SpecIn *in, bool need_tree)
@@ -899,7 +903,7 @@ int32_t spec_tree_probs(const SpecIn *in, int32_t which, float *probs, float *ro
     if (!z || (!probs && !row_stats)) return SPEC_ERR_NULL;
     const bool trunc = (in->top_k > 0 && in->top_k < in->V) || in->top_p < 1.f;
     RowPlan pl;
-    if (!make_row_plan(in->V, 4, &pl)) return SPEC_ERR_UNSUPPORTED;
+    if (!make_row_plan(in->V, (long long)in->B * in->N, sm_count(), &pl)) return SPEC_ERR_UNSUPPORTED;
     if (trunc) {
         // the record of every row of the chosen side goes to the first of its pair in the workspace
         const WsLayout L = ws_layout(in);
@@ -933,7 +937,7 @@ int32_t spec_sample_bonus(const float *weights, int32_t R, int32_t V, const floa
     if (!weights || !u || !token) return SPEC_ERR_NULL;
     if (R <= 0 || V <= 0) return SPEC_ERR_SHAPE;
     RowPlan pl;
-    if (!make_row_plan(V, 4, &pl)) return SPEC_ERR_UNSUPPORTED;
+    if (!make_row_plan(V, R, sm_count(), &pl)) return SPEC_ERR_UNSUPPORTED;
     // CTAs for about four per SM, a slice of at least 4096 weights each, as many as the tiles' sums of a slice ask for
     int C = 1;
     while (C < rowops::BN_CMAX && (((long long)R * C < 4ll * sm_count() && V >= C * 8192) || (V + C - 1) / C > (rowops::BN_TILES - 1) * rowops::BN_TILE)) C <<= 1;

@@ -1,6 +1,6 @@
 // Streaming row statistics (no truncation): every logit row the verifiers may touch is read once from
 // HBM, straight into registers, and reduced to per-slice partial sums of the row's softmax normaliser.
-// No residency, no clusters: a CTA streams a row (or a part of it) in slices of 8192 logits, 32 per thread,
+// No residency: a CTA streams a row (or a part of it) in slices of 8192 logits, 32 per thread,
 // the asynchronous copies of the next slices in flight while the current one is exponentiated.
 //
 // A thread turns its logits into e = 2^(z s - o) (s = log2(e)/T, o = ceil of its own largest z s, an

@@ -46,7 +46,8 @@ constexpr float WINDOW_OCTAVES = 14.f;
 constexpr float SAMPLE_OCTAVES = 24.f;   // bf16 top-p: how far below its maximum the first slice is counted
 constexpr float SAMPLE_REST = 0.7f;      // safety factor of the bounds from a part of the row (mass_bound)
 constexpr float UNSET = -2.0e9f;
-constexpr float LOWEST = -3.3e38f;   // a bound that every finite logit passes but the lowest values of both types (masks: a row that keeps some of them is settled from L2)
+// a bound that every finite logit passes but the lowest values of both types (masks: a row that keeps some of them is settled from L2)
+constexpr float LOWEST = -3.3e38f;
 template <int DT> constexpr int K_FAST = DT == SPEC_BF16 ? UN * NT : NT;      // largest top-k the first slice can bound
 
 // bf16 value bins, largest value first: TB positive magnitudes, then TB negative ones; magnitudes below 2^-11
@@ -483,7 +484,10 @@ template <int DT> struct Smem {
           hits(dyn_smem + Layout<DT>::RING + (threadIdx.x >> 5) * UN * 32),
           bins(reinterpret_cast<uint32_t *>(dyn_smem + Layout<DT>::RING + Layout<DT>::HITS)), keys(bins + 2 * NB),
           S(*reinterpret_cast<Shared *>(dyn_smem + Layout<DT>::RING + Layout<DT>::HITS + Layout<DT>::BINS)) {}
-    __device__ __forceinline__ void count(const Counter &c, const uint4 &r, bool plain) const { count_unit(c, smem_u32(bins), smem_u32(hits) + (threadIdx.x & 31) * 4, &S.odd, r, plain); }
+    __device__ __forceinline__ void count(const Counter &c, const uint4 &r, bool plain) const
+    {
+        count_unit(c, smem_u32(bins), smem_u32(hits) + (threadIdx.x & 31) * 4, &S.odd, r, plain);
+    }
 };
 
 // row / N and row % N for row < 2^24
@@ -642,13 +646,14 @@ __device__ __noinline__ float mass_bound(float tmax, float bound, float of, doub
     }
     return kb > 0 && kb < 2 * TB - 1 && kb != TB && kb != TB - 1 ? fmaxf(bound, value_of_bin(kb)) : bound;
 }
-// How far down the first slice matters; ms: the thread's maximum.
+// How far down the first slice matters.
 __device__ __forceinline__ float sample_floor()
 {
     const Smem<SPEC_BF16> M;
     const float m = cut::value_of(M.S.runmax);
     return m > -CUDART_INF_F && m < CUDART_INF_F ? fmaxf(m - SAMPLE_OCTAVES / M.S.sc.sf, LOWEST) : LOWEST;
 }
+// Starts a row's state (runmax, verdict) from the threads' maxima of the first slice, ms; returns how far down that slice matters.
 __device__ __noinline__ float sample_bound(float ms)
 {
     const Smem<SPEC_BF16> M;
@@ -659,9 +664,8 @@ __device__ __noinline__ float sample_bound(float ms)
     return sample_floor();
 }
 // The first bound, from the first slice alone.  Of a row of several slices with a positive logit in the first only positive ones have been
-// counted: a cut below zero
-// keeps more than half of a row of logits around zero.  Where they hold too little of the mass, the slice is counted again, from the
-// ring (stage: the warp's share), all of it that matters.
+// counted: a cut below zero keeps more than half of a row of logits around zero.  Where they hold too little of the mass, the
+// slice is counted again, from the ring (stage: the warp's share), all of it that matters.
 __device__ __noinline__ float first_mass_bound(float tmax, float bound, float of, double Sd, float top_p, int n, int V, const uint4 *stage)
 {
     const Smem<SPEC_BF16> M;
@@ -995,7 +999,7 @@ __global__ void __launch_bounds__(NT, CTAS<DT>) spec_row_trunc_kernel(const __gr
                     RowPart r = {};
                     r.cut = -CUDART_INF_F; r.O = ROWPART_EMPTY; r.bad = -1;
                     P.part[id] = r;
-                                }
+                }
             }
             if (id == to) break;
         }
