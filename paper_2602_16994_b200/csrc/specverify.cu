@@ -330,8 +330,12 @@ int resident_clusters(K kernel, int C, int threads, int smem)
 
 // nodes with several children (AN: with any): a cluster each
 template <int DT, int RC, bool AN>
-int launch_branch(const VPlan &pl, NParams &np, cudaStream_t st)
+int launch_branch(VPlan pl, NParams &np, cudaStream_t st)
 {
+    // An SM's shared memory comes in configurations of ..., 132, 164, 196 and 228 KB (1 KB a CTA is the system's).  A CTA that nearly fills
+    // the 164 KB one leaves the CTAs of the kernels beside it no place until it is done; asking for more than that, it runs in a larger one.
+    // Traversal, V = 262144 (164 KB), us: B = 16 218 and 204, B = 8 134 and 128.
+    if (pl.smem > 160 * 1024 && pl.smem <= 163 * 1024) pl.smem = 163 * 1024 + 64;
     auto kernel = spec_recursion_kernel<DT, 7, RC, AN>;
     const int rc = prepare_kernel(kernel, pl.C, pl.smem, true);
     if (rc) return rc;

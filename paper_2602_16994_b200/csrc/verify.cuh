@@ -53,8 +53,7 @@ namespace specv {
 constexpr int CHMAX = 24;    // chunks per thread, in registers (RC of them) and shared memory
 constexpr int CMAX = 16;     // CTAs per cluster (above 8: non-portable size)
 constexpr int NWMAX = 8;     // consumer warps
-constexpr int NVMAX = 9;     // doubles per sum over the cluster (6 are used; with the smaller area the CTAs of the node kernels share SMs
-                             // differently: Traversal V = 262144, B = 16 232 instead of 205 us)
+constexpr int NVMAX = 6;     // doubles per sum over the cluster
 constexpr int FAST_N = 32;   // trees up to this size are finished warp-parallel
 constexpr int FIN_PENDING = -1;     // VParams::fin of a sequence whose nodes are not all done
 constexpr int FIN_FAULTY = -2;      // ... of a sequence with a device-detected fault: no bonus draw
