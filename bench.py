@@ -39,9 +39,9 @@ STAT_KERNEL = {False: "stream::spec_row_partial_kernel (row statistics: the one 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of that kernel, launched in a row, from the ncu
 # captures summarised under profiles/.  Workloads without a capture: null.
 TRAFFIC_BYTES = {"cfg2_llama3_b8": 69_770_000 + 100_000}
-# the same counters summed over the kernels of a whole call, captured in one pass without cache flushes between
-# the kernels (profiles/per_config.md): the later kernels of a call find most of their rows in L2
-TRAFFIC_CALL_BYTES = {"cfg2_llama3_b8": {"specinfer": 69_790_000 + 1_600_000, "traversal": 84_100_000 + 28_300_000}}
+# the same counters summed over the kernels of a whole call, calls of one kind in a row, captured in one pass without cache
+# flushes between the kernels (profiles/per_config.md): the later kernels of a call find most of their rows in L2
+TRAFFIC_CALL_BYTES = {"cfg2_llama3_b8": {"specinfer": 69_800_000 + 1_500_000, "traversal": 85_500_000 + 46_900_000}}
 
 
 def parse_args():

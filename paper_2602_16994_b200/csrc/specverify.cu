@@ -502,7 +502,7 @@ void fill_params(const SpecIn *in, const SpecOut *out, unsigned char *w, const W
     vp.B = in->B; vp.N = in->N; vp.V = in->V; vp.mode = mode;
     vp.all_thr = (out->node_thr != nullptr || out->margin != nullptr) ? 1 : 0;
     // Whether the finish kernel, a cluster per sequence for 15 us, lets the first kernel of the next call in while it runs (that kernel then
-    // waits for its end): where such a call's rows fill the chip (Traversal B = 8 92 -> 86 us, V = 262144 B = 16 219 -> 201).  Fewer CTAs
+    // waits for its end; it helps where calls of this library follow each other, and changes nothing for any other kernel that comes next): where such a call's rows fill the chip (Traversal B = 8 92 -> 86 us, V = 262144 B = 16 219 -> 201).  Fewer CTAs
     // would crowd onto the SMs that are free at that moment and leave the others idle, and so would the selection's
     // (wide nuclei, B = 8: 121 -> 127); nothing is gained after a walk (SpecInfer B = 8; top-k, B = 128: 708 -> 741).
     const bool trunc = (in->top_k > 0 && in->top_k < in->V) || in->top_p < 1.f;
