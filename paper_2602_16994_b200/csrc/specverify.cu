@@ -126,7 +126,7 @@ struct RowPlan {
 constexpr int ROW_SMEM_BUDGET = 227 * 1024 - (int)sizeof(rowops::Shared) - 1024;
 
 // `rows` rows of fp32 values, each in the shared memory of a cluster: two CTAs per SM where eight CTAs are enough for that, but one
-// where all CTAs of clusters of four, and not of clusters of eight, have an SM to themselves (19 rows of 128256: 17.6 and 18.5 us; one CTA
+// where all CTAs of clusters of four, and not of clusters of eight, have an SM to themselves (19 rows of 128256: 16.5 and 18.5 us; one CTA
 // against two does not pay: 76 rows of 32000 17.6 and 15.3).
 bool make_row_plan(int V, long long rows, int sms, RowPlan *p)
 {
@@ -558,13 +558,13 @@ int launch_nodes(const SpecIn *in, NParams &np, bool analysis, cudaStream_t st)
         while (C < 8 && nodes * C * 2 <= 8 * sm_count() && in->V >= C * 8192) C <<= 1;
         if (analysis) {
             // The analysis' passes are arithmetic, and left alone three CTAs share an SM while others idle: with few nodes a CTA asks for so
-            // much shared memory that they spread, and clusters of 16 are taken where each of their CTAs finds an SM and 24 KB of the row.  Paths of six nodes,
-            // us, packed and spread: fp32 V = 262144 B = 1 123 and 64 (78 in clusters of 8), B = 2 129 and 78, B = 4 (two a SM) 136 and 110,
+            // much shared memory that they spread, and clusters of 16 are taken where each of their CTAs finds an SM and 24 KB of the row.
+            // Paths of six nodes, us, packed and spread: fp32 V = 262144 B = 1 123 and 64 (78 in clusters of 8), B = 2 129 and 78, B = 4 (two a SM) 136 and 110,
             // V = 128256 B = 2 89 and 62, bf16 V = 262144 B = 1 70 and 57, V = 128256 B = 4 68 and 61; from three a SM on, packed is as it was
             // (spread all the same, B = 8: 76 and 85).  Clusters of 16 for smaller rows: bf16 V = 128256 B = 1 46 and 48.
             if (C == 8 && nodes * 16 <= sm_count() && (long long)in->V * (bf ? 2 : 4) >= 16 * 24 * 1024) C = 16;
             const long long per_sm = (nodes * C + sm_count() - 1) / sm_count();
-            if (per_sm <= 2) bytes = per_sm == 1 ? 100 * 1024 : 62 * 1024;
+            if (per_sm <= 2) bytes = per_sm == 1 ? 104 * 1024 : 66 * 1024;     // (with 14 KB of its own: one or two fit the 228 KB of an SM)
         }
         np.v.C = C;
         const auto go = [&](auto kernel) {
