@@ -502,7 +502,8 @@ void fill_params(const SpecIn *in, const SpecOut *out, unsigned char *w, const W
     vp.B = in->B; vp.N = in->N; vp.V = in->V; vp.mode = mode;
     vp.all_thr = (out->node_thr != nullptr || out->margin != nullptr) ? 1 : 0;
     // Whether the finish kernel, a cluster per sequence for 15 us, lets the first kernel of the next call in while it runs (that kernel then
-    // waits for its end; it helps where calls of this library follow each other, and changes nothing for any other kernel that comes next): where such a call's rows fill the chip (Traversal B = 8 92 -> 86 us, V = 262144 B = 16 219 -> 201).  Fewer CTAs
+    // waits for its end; it helps where calls of this library follow each other, and changes nothing for any other kernel that comes
+    // next): where such a call's rows fill the chip (Traversal B = 8 92 -> 86 us, V = 262144 B = 16 219 -> 201).  Fewer CTAs
     // would crowd onto the SMs that are free at that moment and leave the others idle, and so would the selection's
     // (wide nuclei, B = 8: 121 -> 127); nothing is gained after a walk (SpecInfer B = 8; top-k, B = 128: 708 -> 741).
     const bool trunc = (in->top_k > 0 && in->top_k < in->V) || in->top_p < 1.f;
@@ -564,7 +565,8 @@ int launch_nodes(const SpecIn *in, NParams &np, bool analysis, cudaStream_t st)
             // (spread all the same, B = 8: 76 and 85).  Clusters of 16 for smaller rows: bf16 V = 128256 B = 1 46 and 48.
             if (C == 8 && nodes * 16 <= sm_count() && (long long)in->V * (bf ? 2 : 4) >= 16 * 24 * 1024) C = 16;
             const long long per_sm = (nodes * C + sm_count() - 1) / sm_count();
-            if (per_sm <= 2) bytes = per_sm == 1 ? 104 * 1024 : 66 * 1024;     // (with 14 KB of its own: one or two fit the 228 KB of an SM)
+            // (with 14 KB of its own, one or two of them fit the 228 KB of an SM)
+            if (per_sm <= 2) bytes = per_sm == 1 ? 104 * 1024 : 66 * 1024;
         }
         np.v.C = C;
         const auto go = [&](auto kernel) {
